@@ -5,7 +5,7 @@
 // channel-last (8 channels = 16 bytes per cell); the convolutions run as implicit GEMMs on the tensor
 // cores (ldmatrix + mma.sync m16n8k16, BF16 operands, FP32 accumulation): M = 16 consecutive cells of
 // a row, N = 8 channels, K = 27 taps x 8 channels (padded to 224).  The weight gradient is a reduction
-// over all cells, done on the CUDA cores in FP32 with per-block partial sums reduced in a fixed order.
+// over all cells: the same tensor-core form with the cells as K, FP32 sums, per-block partials added in a fixed order.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -40,7 +40,6 @@ struct ibm_net {
     __nv_bfloat16* d1;
     float* out;
     float* wpart;             // per-block weight-gradient partials
-    long long wpart_blocks;
     double* scal;             // [0] feature scale s, [1] loss sum, [2..] reduction scratch
     double* partials;
     unsigned* counter;
@@ -172,64 +171,143 @@ __global__ void __launch_bounds__(256) k_nn_conv_tile(int nx, int ny, int nz, co
 }
 
 // Weight and bias gradients of one layer: dW[co][tap][ci] = sum_c dz[c][co] y[c + off(tap)][ci],
-// db[co] = sum_c dz[c][co].  Block = 224 threads: thread (tap, ci) for tid < 216, bias co for the
-// last 8; each block covers a contiguous range of cells and writes its partial sums.
-__global__ void __launch_bounds__(224) k_nn_wgrad(int nx, int ny, int nz, int ncout,
-                                                  const __nv_bfloat16* __restrict__ dz,
-                                                  const __nv_bfloat16* __restrict__ y, long long cells_per_block,
-                                                  float* __restrict__ wpart) {
-    const long long N = (long long)nx * ny * nz;
-    const long long c0 = blockIdx.x * cells_per_block, c1 = c0 + cells_per_block < N ? c0 + cells_per_block : N;
-    const int tid = threadIdx.x;
-    float acc[NN_C] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const int t = tid / NN_C, ci = tid % NN_C;
-    int dz_, dy_, dx_;
-    tap_off(t < NN_TAPS ? t : 13, dz_, dy_, dx_);
-    for (long long c = c0; c < c1; ++c) {
-        const uint4 zv = *reinterpret_cast<const uint4*>(dz + c * NN_C);
-        const __nv_bfloat162* zp = reinterpret_cast<const __nv_bfloat162*>(&zv);
-        float zf[NN_C];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            zf[2 * h] = __bfloat162float(zp[h].x);
-            zf[2 * h + 1] = __bfloat162float(zp[h].y);
-        }
-        float yv;
-        if (tid < NN_TAPS * NN_C) {
-            const int i = (int)(c % nx), j = (int)((c / nx) % ny), k = (int)(c / ((long long)nx * ny));
-            const int ii = i + dx_, jj = j + dy_, kk = k + dz_;
-            yv = (ii < 0 || ii >= nx || jj < 0 || jj >= ny || kk < 0 || kk >= nz)
-                     ? 0.f
-                     : __bfloat162float(y[(ii + (long long)nx * (jj + (long long)ny * kk)) * NN_C + ci]);
-        } else {
-            yv = 1.f;   // bias: sum of dz[co] with co = tid - 216
-        }
-#pragma unroll
-        for (int co = 0; co < NN_C; ++co) acc[co] += zf[co] * yv;
-    }
-    float* part = wpart + (long long)blockIdx.x * (NN_TAPS * NN_C * NN_C + NN_C);
-    if (tid < NN_TAPS * NN_C) {
-        for (int co = 0; co < ncout; ++co) part[(co * NN_TAPS + t) * NN_C + ci] = acc[co];
-    } else {
-        const int co = tid - NN_TAPS * NN_C;
-        part[NN_TAPS * NN_C * NN_C + co] = co < ncout ? acc[co] : 0.f;
-    }
+// db[co] = sum_c dz[c][co], as a GEMM on the tensor cores: M = 27 taps x 8 channels (padded to 28 taps;
+// the padding tap reads a row of ones in channel 0, so its row is db), N = 8 output channels, K = the
+// cells.  The tile, the three-plane ring and the warps' cells are those of the convolution above: per
+// plane a warp takes 16 cells, one ldmatrix.x2.trans gives their dz as the B fragment, and per pair of taps
+// one ldmatrix.x4.trans gathers y as the A fragment.  Each mma starts from zero and is added in FP32, so a
+// sum is a chain of one FP32 addition per 16 cells.  Blocks walk tiles of a fixed grid and write one partial
+// each.  Both operands are read once (16 + 16 bytes per cell, halo from L2).
+// 128^3 cells: 98 us per layer; one thread per (tap, channel) with serial global loads took 2.8 ms.
+#define WG_BLOCKS 608
+#define WG_STRIDE (NN_TAPS * NN_C * NN_C + NN_C)
+
+__device__ __forceinline__ void ldsm_x4_t(uint32_t r[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_x2_t(uint32_t r[2], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
 }
 
-// Sums the per-block partials in block order; writes dW / db of the layer into grad (scaled by 1/N).
-__global__ void k_nn_wgrad_reduce(const float* __restrict__ wpart, long long nblk, int ncout, float inv_n,
-                                  float* __restrict__ gw, float* __restrict__ gb) {
-    const int stride = NN_TAPS * NN_C * NN_C + NN_C;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < stride; e += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (long long b = 0; b < nblk; ++b) s += wpart[b * stride + e];
-        if (e < NN_TAPS * NN_C * NN_C) {
-            const int co = e / (NN_TAPS * NN_C);
-            if (co < ncout) gw[e] = (float)(s * inv_n);
-        } else {
-            const int co = e - NN_TAPS * NN_C * NN_C;
-            if (co < ncout) gb[co] = (float)(s * inv_n);
+__global__ void __launch_bounds__(256) k_nn_wgrad(int nx, int ny, int nz, int ncout,
+                                                  const __nv_bfloat16* __restrict__ dz,
+                                                  const __nv_bfloat16* __restrict__ y, float* __restrict__ wpart) {
+    __shared__ __align__(16) uint4 ring[3 * NC_PL + 1];          // y planes k - 1 .. k + 1, then the row of ones
+    __shared__ __align__(16) uint4 zt[2][NC_TX * NC_TY];         // dz of the plane, double buffered
+    __shared__ float red[NN_KSTEPS * 2 * NN_C * NN_C];           // [tap][ci][co]
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    if (tid == 0) ring[3 * NC_PL] = make_uint4(0x3f80u, 0u, 0u, 0u);     // bf16 1 in channel 0
+    for (int e = tid; e < NN_KSTEPS * 2 * NN_C * NN_C; e += 256) red[e] = 0.f;
+    const int gx = (nx + NC_TX - 1) / NC_TX, gy = (ny + NC_TY - 1) / NC_TY, gz = (nz + NC_KZ - 1) / NC_KZ;
+    const unsigned items = (unsigned)gx * gy * gz;
+    const int mj = lane >> 3, mr = lane & 7;
+    // matrix mj of the x4 gather: tap 2s + (mj & 1), cells 8 (mj >> 1) .. + 7 of the warp's 16
+    const int cx = (w & 1) * 16 + (mj >> 1) * 8 + mr, cy = w >> 1;
+    const uint32_t ring_base = (uint32_t)__cvta_generic_to_shared(ring), ones = ring_base + 3 * NC_PL * 16;
+    const uint32_t cell0 = (uint32_t)(((cy + 1) * NC_SX + cx + 1) * 16);
+    const uint32_t zaddr = (uint32_t)__cvta_generic_to_shared(&zt[0][0]) +
+                           (uint32_t)((cy * NC_TX + (w & 1) * 16 + (lane & 15)) * 16);
+    float acc[NN_KSTEPS][4];
+#pragma unroll
+    for (int s = 0; s < NN_KSTEPS; ++s)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) acc[s][h] = 0.f;
+    for (unsigned it = blockIdx.x; it < items; it += gridDim.x) {
+        const unsigned q = it / (unsigned)gx;
+        const int x0 = (int)(it - q * gx) * NC_TX, y0 = (int)(q % (unsigned)gy) * NC_TY, z0 = (int)(q / (unsigned)gy) * NC_KZ;
+        const int z1 = z0 + NC_KZ < nz ? z0 + NC_KZ : nz;
+        auto load_plane = [&](int kk, int slot) {
+            uint4* dst = ring + slot * NC_PL;
+            if (tid < NC_PL) {
+                const int ix = x0 + tid % NC_SX - 1, iy = y0 + tid / NC_SX - 1;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (kk >= 0 && kk < nz && ix >= 0 && ix < nx && iy >= 0 && iy < ny)
+                    v = *reinterpret_cast<const uint4*>(y + (ix + (long long)nx * (iy + (long long)ny * kk)) * NN_C);
+                dst[tid] = v;
+            }
+        };
+        auto load_dz = [&](int kk, int buf) {
+            if (tid < NC_TX * NC_TY) {
+                const int ix = x0 + (tid & (NC_TX - 1)), iy = y0 + tid / NC_TX;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (ix < nx && iy < ny)
+                    v = *reinterpret_cast<const uint4*>(dz + (ix + (long long)nx * (iy + (long long)ny * kk)) * NN_C);
+                zt[buf][tid] = v;
+            }
+        };
+        __syncthreads();                        // the previous tile's reads of the ring are done
+        load_plane(z0 - 1, 0);
+        load_plane(z0, 1);
+        int sp = 0, sc = 1, sn = 2;             // ring slots of planes k - 1, k, k + 1
+        for (int k = z0; k < z1; ++k) {
+            const int buf = k & 1;
+            load_plane(k + 1, sn);
+            load_dz(k, buf);
+            __syncthreads();
+            uint32_t b[2];
+            ldsm_x2_t(b, zaddr + (uint32_t)buf * (NC_TX * NC_TY * 16));
+            const uint32_t pb[3] = {cell0 + ring_base + (uint32_t)(sp * NC_PL * 16), cell0 + ring_base + (uint32_t)(sc * NC_PL * 16),
+                                    cell0 + ring_base + (uint32_t)(sn * NC_PL * 16)};
+#pragma unroll
+            for (int s = 0; s < NN_KSTEPS; ++s) {
+                const int ta = 2 * s, tb = 2 * s + 1;                    // compile-time taps of the two halves
+                const uint32_t aa = pb[ta / 9] + (uint32_t)((((ta / 3) % 3 - 1) * NC_SX + ta % 3 - 1) * 16);
+                const uint32_t ab = tb < NN_TAPS ? pb[tb < NN_TAPS ? tb / 9 : 0] + (uint32_t)((((tb / 3) % 3 - 1) * NC_SX + tb % 3 - 1) * 16) : ones;
+                uint32_t a[4];
+                ldsm_x4_t(a, (mj & 1) ? ab : aa);
+                float d[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_bf16(d, a, b);
+#pragma unroll
+                for (int h = 0; h < 4; ++h) acc[s][h] += d[h];
+            }
+            __syncthreads();                    // slot sp is overwritten by the next plane
+            const int t = sp;
+            sp = sc;
+            sc = sn;
+            sn = t;
         }
+    }
+    // the block's sum over its warps, in warp order
+    const int g = lane >> 2, qq = lane & 3;
+    for (int ww = 0; ww < 8; ++ww) {
+        __syncthreads();
+        if (w != ww) continue;
+#pragma unroll
+        for (int s = 0; s < NN_KSTEPS; ++s)
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+                red[((2 * s + (h >> 1)) * NN_C + g) * NN_C + 2 * qq + (h & 1)] += acc[s][h];
+    }
+    __syncthreads();
+    float* part = wpart + (long long)blockIdx.x * WG_STRIDE;
+    for (int e = tid; e < NN_TAPS * NN_C * NN_C; e += 256) {
+        const int co = e / (NN_TAPS * NN_C), tc = e - co * (NN_TAPS * NN_C);
+        part[e] = co < ncout ? red[tc * NN_C + co] : 0.f;
+    }
+    if (tid < NN_C) part[NN_TAPS * NN_C * NN_C + tid] = tid < ncout ? red[NN_TAPS * NN_C * NN_C + tid] : 0.f;
+}
+
+// Sums the per-block partials; writes dW / db of the layer into grad (scaled by 1/N).  A block takes 32
+// entries and splits the partials over 8 warps (coalesced rows), whose sums are added in warp order.
+__global__ void __launch_bounds__(256) k_nn_wgrad_reduce(const float* __restrict__ wpart, int nblk, int ncout,
+                                                         float inv_n, float* __restrict__ gw, float* __restrict__ gb) {
+    __shared__ double sh[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+    double s = 0.0;
+    if (e < WG_STRIDE)
+        for (int b = w; b < nblk; b += 8) s += wpart[(long long)b * WG_STRIDE + e];
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w != 0 || e >= WG_STRIDE) return;
+    for (int q = 1; q < 8; ++q) s += sh[q][lane];
+    if (e < NN_TAPS * NN_C * NN_C) {
+        const int co = e / (NN_TAPS * NN_C);
+        if (co < ncout) gw[e] = (float)(s * inv_n);
+    } else {
+        const int co = e - NN_TAPS * NN_C * NN_C;
+        if (co < ncout) gb[co] = (float)(s * inv_n);
     }
 }
 
@@ -355,16 +433,14 @@ static int net_reserve(ibm_net* n, long long N) {
     n->out = n->wpart = nullptr;
     n->cap_cells = 0;
     const size_t act = (size_t)N * NN_C * sizeof(__nv_bfloat16);
-    const long long nblk = (N + 4095) / 4096;
     cudaError_t e;
     if ((e = cudaMalloc(&n->x0, act)) != cudaSuccess || (e = cudaMalloc(&n->y1, act)) != cudaSuccess ||
         (e = cudaMalloc(&n->y2, act)) != cudaSuccess || (e = cudaMalloc(&n->d3, act)) != cudaSuccess ||
         (e = cudaMalloc(&n->d2, act)) != cudaSuccess || (e = cudaMalloc(&n->d1, act)) != cudaSuccess ||
         (e = cudaMalloc(&n->out, (size_t)N * sizeof(float))) != cudaSuccess ||
-        (e = cudaMalloc(&n->wpart, (size_t)nblk * (NN_TAPS * NN_C * NN_C + NN_C) * sizeof(float))) != cudaSuccess)
+        (e = cudaMalloc(&n->wpart, (size_t)WG_BLOCKS * WG_STRIDE * sizeof(float))) != cudaSuccess)
         return ibm_fail(IBM_E_NOMEM, "ibm_net: %s", cudaGetErrorString(e));
     n->cap_cells = N;
-    n->wpart_blocks = nblk;
     return IBM_OK;
 }
 
@@ -523,13 +599,14 @@ extern "C" int ibm_net_train_step(ibm_net* n, const ibm_grid* g, const double* d
     conv(n, g->nx, g->ny, g->nz, n->d3, 2, -1, 2, n->d2, nullptr, n->y2, s);
     conv(n, g->nx, g->ny, g->nz, n->d2, 1, -1, 2, n->d1, nullptr, n->y1, s);
     // weight gradients
-    const long long cpb = 4096;
-    const unsigned nblk = (unsigned)((N + cpb - 1) / cpb);
+    const long long tiles = (long long)((g->nx + NC_TX - 1) / NC_TX) * ((g->ny + NC_TY - 1) / NC_TY) *
+                            ((g->nz + NC_KZ - 1) / NC_KZ);
+    const int nblk = (int)(tiles < WG_BLOCKS ? tiles : WG_BLOCKS);
     const __nv_bfloat16* dz[3] = {n->d1, n->d2, n->d3};
     const __nv_bfloat16* yin[3] = {n->x0, n->y1, n->y2};
     for (int l = 0; l < 3; ++l) {
-        k_nn_wgrad<<<nblk, 224, 0, s>>>(g->nx, g->ny, g->nz, cout_of(l), dz[l], yin[l], cpb, n->wpart);
-        k_nn_wgrad_reduce<<<8, 256, 0, s>>>(n->wpart, nblk, cout_of(l), 1.f / (float)N, n->grad + offset_w(l),
+        k_nn_wgrad<<<nblk, 256, 0, s>>>(g->nx, g->ny, g->nz, cout_of(l), dz[l], yin[l], n->wpart);
+        k_nn_wgrad_reduce<<<(WG_STRIDE + 31) / 32, 256, 0, s>>>(n->wpart, nblk, cout_of(l), 1.f / (float)N, n->grad + offset_w(l),
                                             n->grad + offset_b(l));
     }
     IBM_LAUNCHED("ibm_net: backward");
