@@ -77,7 +77,7 @@ def bytes_per_cell(s, integrator="cn", sweeps=2, fused=False):
 # the kernel behind each single-kernel group (FP32 path with nx a multiple of 4)
 GROUP_KERNEL = {"csm": "k_csm", "predict": "k_cn_begin (tiled + general)", "faces": "k_faces",
                 "rhs": "k_rhs", "residual": "k_residual", "cg_dir_spmv": "k_cg_dir_spmv_x4",
-                "cg_update": "k_cg_update", "correct": "k_correct_cells + k_correct_faces",
+                "cg_update": "k_cg_update", "correct": "k_correct",
                 "mg_fine": "k_mg_smooth0_x4", "mg_transfer": "k_mg_restrict0_x4 + k_mg_prolong0_x4"}
 GROUP_KERNEL_FUSED = {"mg_fine": "k_mg_pre_fused + k_mg_post_fused", "mg_transfer": "k_mg_prolong0_x4"}
 

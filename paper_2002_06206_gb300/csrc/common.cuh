@@ -91,17 +91,6 @@ __device__ __forceinline__ T vel_across(const Dom& D, const T* __restrict__ u, i
     }
 }
 
-// Pressure read across link (a, s): Neumann on cut links and walls/inflow, p = 0 at outflow faces.
-template <class T>
-__device__ __forceinline__ T p_across(const Dom& D, const T* __restrict__ p, long long P, int xa,
-                                      unsigned fl, int a, int s) {
-    const int bit = link_bit(a, s);
-    if (fl & (1u << bit)) return p[P];
-    long long off;
-    if (nb_offset(D, a, s, xa, off)) return p[P + off];
-    return D.bc[bit] == IBM_BC_OUTFLOW ? -p[P] : p[P];
-}
-
 // Face offsets in the concatenated Ux | Uy | Uz vector.
 struct FaceLayout {
     long long off[3];

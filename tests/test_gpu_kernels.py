@@ -53,3 +53,48 @@ def test_weight_gradients_of_a_network_that_is_exact_in_bf16(L, shape):
     assert np.abs(ref).max() * N < 2 ** 24 and np.any(ref)
     np.testing.assert_allclose(net.grads().astype(np.float64), ref, rtol=1.3e-7, atol=0.0)
     net.close()
+
+
+@pytest.mark.parametrize("bc", [CHANNEL, PERIODIC])
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (33, 9, 17), (40, 8, 8), (64, 64, 33)])
+def test_correction_subtracts_fp64_pressures_of_any_size(L, shape, prec, bc):
+    """u = u* - c (p+ - p-), U = U* - 2 c (pR - pL) with u* = U* = 0: the result is the FP64 difference, rounded,
+    times the rounded factor -- five roundings of 2^-24 (2^-53 in FP64) at most, and 2^-47 of the pressure where it is held in two parts."""
+    nx, ny, nz = shape
+    N = nx * ny * nz
+    rng = np.random.default_rng(5)
+    p = rng.standard_normal(N) * 10.0 ** rng.integers(-3, 4, N) + 1.0
+    p[rng.random(N) < 0.1] = 0.0
+    p[rng.random(N) < 0.1] *= 1e-26            # below the range of the low part
+    p[rng.random(N) < 0.02] = 2.0 ** -130      # below the normal range of a float
+    p[rng.random(N) < 0.02] *= 1e30
+    dt = 0.2
+    s = L.Solver(L.make_grid(nx, ny, nz), 0.01, dt, bc, precision=prec)
+    z = torch.zeros(3 * N, dtype=s.dtype, device="cuda")
+    Z = torch.zeros(s.NF, dtype=s.dtype, device="cuda")
+    u, U = torch.full_like(z, 7.0), torch.full_like(Z, 7.0)
+    s.correct(z, Z, torch.from_numpy(p).cuda(), u, U)
+    P = p.reshape(nz, ny, nx)
+    eps = 2.0 ** -24 if prec else 2.0 ** -53
+    off = 0
+    for a, dim in ((0, 2), (1, 1), (2, 0)):
+        n = P.shape[dim]
+        lo = np.take(P, [-1 if bc[2 * a] == 0 else 0], dim)
+        hi = np.take(P, [0 if bc[2 * a] == 0 else -1], dim) * (-1.0 if bc[2 * a + 1] == 2 else 1.0)
+        E = np.concatenate([lo, P, hi], dim)
+        cut = lambda q0, q1: np.take(E, np.arange(q0, q1), dim)  # noqa: E731
+        for got, ref, big in ((u[a * N:(a + 1) * N].cpu().numpy().reshape(P.shape), -0.5 * dt * (cut(2, n + 2) - cut(0, n)),
+                               np.maximum(np.abs(cut(2, n + 2)), np.abs(cut(0, n)))),
+                              (U[off:off + (n + 1) * (N // n)].cpu().numpy().reshape(cut(0, n + 1).shape),
+                               -dt * (cut(1, n + 2) - cut(0, n + 1)), np.maximum(np.abs(cut(1, n + 2)), np.abs(cut(0, n + 1))))):
+            if got.shape != P.shape or bc[2 * a] != 0:
+                if got.shape != P.shape and bc[2 * a] != 0:                    # the wall and inflow faces keep U*
+                    keep = [0] + ([n] if bc[2 * a + 1] != 2 else [])
+                    assert np.all(np.take(got, keep, dim) == 0.0)
+                    inner = np.arange(1, n + (bc[2 * a + 1] == 2))
+                    got, ref, big = (np.take(v, inner, dim) for v in (got, ref, big))
+            tol = 5.0 * eps * np.abs(ref) + dt * 2.0 ** -47 * big + 2.0 ** -149
+            assert np.all(np.abs(got.astype(np.float64) - ref) <= tol)
+        off += (n + 1) * (N // n)
+    s.close()
