@@ -81,9 +81,9 @@ typedef struct {
     double mom_tol;      /* Crank-Nicolson: stop at ||r|| <= mom_tol ||dt L(u^n)|| (0 = 1e-6 in
                             FP32_REFINE64 mode, 1e-10 in FP64 mode) */
     int32_t mg_passes;   /* multigrid fine-grid passes: 0 = fused where the grid allows (FP32, mg_sweeps 2,
-                            nx a multiple of 16, no periodic axis, a body present: the four half-sweeps
-                            before the coarse correction and the restriction in one pass, the four after
-                            it and (r, z) in another), 1 = one kernel per half-sweep.  Same V-cycle. */
+                            nx a multiple of 4, no periodic axis: the four half-sweeps before the coarse
+                            correction and the restriction in one pass, the four after it and (r, z) in
+                            another), 1 = one kernel per half-sweep.  Same V-cycle. */
     int32_t reserved;
 } les_params;
 
@@ -226,7 +226,7 @@ int poisson_solve(les_state* st, const double* d_b, double* d_p, double tol, int
  * red-black SOR): d_z[N] = one V-cycle applied to d_r[N], in the state's working precision (float in
  * FP32_REFINE64 mode, double in FP64 mode), for the unscaled system  sum_links g (z_N - z_P) - d z_P =
  * dx^2 r  whose operator is dx^2 times the Eq. poisson operator.  Both arrays are 16-byte aligned and
- * distinct.  Needs a state created with precond = 1.  Synchronises (reads a device error word). */
+ * distinct.  Needs a state created with precond = 1.  Synchronises. */
 int poisson_precond(les_state* st, const void* d_r, void* d_z, void* stream);
 /* Multigrid hierarchy of a state (host, no synchronisation): out[0] = levels (0 without multigrid),
  * out[1] = 1 when the fused fine-grid passes are used, out[2 + l] = unknowns of level l (level 0 =

@@ -297,10 +297,7 @@ extern "C" int les_create(const ibm_grid* g, const les_params* p, const ibm_geom
         }
     }
     if (p->precond == 1) {
-        // MG holds 64-byte aligned tensor maps
-        const size_t mgb = (sizeof(MG) + 63) & ~(size_t)63;
-        MG* mg = (MG*)aligned_alloc(64, mgb);
-        if (mg) memset(mg, 0, mgb);
+        MG* mg = (MG*)calloc(1, sizeof(MG));
         if (!mg) {
             free_state(S);
             return ibm_fail(IBM_E_NOMEM, "les_create: host allocation");
@@ -492,9 +489,7 @@ extern "C" int poisson_precond(les_state* S, const void* r, void* z, void* strea
     int rc = S->c.prec == IBM_FP64 ? mg_vcycle<double>(S->c, *S->c.mg, (const double*)r, (double*)z, S->w.sc, s)
                                   : mg_vcycle<float>(S->c, *S->c.mg, (const float*)r, (float*)z, S->w.sc, s);
     if (rc) return rc;
-    IBM_CUDA(cudaMemcpyAsync(S->w.hsc, S->w.sc, sizeof(SolveScal), cudaMemcpyDeviceToHost, s));
     IBM_CUDA(cudaStreamSynchronize(s));
-    if (S->w.hsc->dev_error) return ibm_fail(IBM_E_CUDA, "poisson_precond: a multigrid shared-memory load timed out");
     return IBM_OK;
 }
 

@@ -19,10 +19,8 @@
 //
 // Equations are solved in the unscaled form  sum_links g (x_N - x_P) - d x_P = dx^2 r.
 #include <cooperative_groups.h>
-#include <cudaTypedefs.h>
 #include <string.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "scan.cuh"
@@ -229,509 +227,500 @@ __device__ __forceinline__ int fine_parts(const Dom& D, const unsigned (&fl)[8],
 
 // ---- fused fine-grid passes: all four red-black half-sweeps of a smoothing phase in one pass ------
 //
-// A block owns an (x, y) tile of FT_TX x FT_TY cells and marches along z over a chunk of planes.  It
-// keeps, for the tile plus a 4-cell halo, a ring of FT_NS planes of r, flags and z in shared memory;
-// the planes arrive by TMA (one elected thread issues cp.async.bulk.tensor loads one plane ahead; an
-// mbarrier per ring slot carries the byte count).  Step t takes plane t; the half-sweeps run at planes
-// t, t-1, t-2, t-3 (each needs its neighbours after the previous half-sweep, one plane and one halo
-// cell further out), so that after step t plane t-3 (pre-smoothing) or t-4 (post-smoothing) is final.
-// The halo shrinks by one cell per half-sweep, so the tile's own cells see exactly the values the
-// four separate passes compute.  Pre-smoothing starts from z = 0 (only r and the flags are read) and
-// ends with the residual and its restriction to level 1; post-smoothing reads z and ends with the
-// (r, z) product of the CG iteration.  Neighbouring chunks recompute each other's edge planes but
-// only write their own.
+// A block of 512 threads marches an (x, y) tile along z over a chunk of planes.  A thread owns a column of
+// 4 x 2 cells (a 16-byte quad in two rows) and keeps its planes in registers, so the neighbours above and
+// below cost nothing; the x neighbours within a quad are registers, across quads one shuffle, the y
+// neighbours the other row or, across threads, two values through shared memory.  At step t half-sweep s
+// (s = 1 .. 4) runs on plane t - s + 1: its in-plane neighbours were finished in step t - 1 and its upper
+// neighbour by half-sweep s - 1 of the same step in the same thread, so one barrier per plane orders
+// everything and the four half-sweeps are independent until they meet in the column.  Only the colour
+// just updated is published (two float2 per thread and half-sweep, double buffered by step parity); tile
+// origins and x quads are even, so which cells of a quad a half-sweep updates depends on the step's parity
+// alone and is known to the compiler.  The halo (4 cells) holds values that turn wrong one ring per
+// half-sweep from the outside; the tile's own cells see exactly the values of separate passes.  A tile at a
+// domain face has no halo there.
+//
+// Cells with no cut link and off the first and last plane take the plain form (s - scale r) * inv with inv
+// = 1 / (open links + outflow terms), fixed per column: neighbours outside the domain hold z = 0.  A warp
+// with a cut link in its plane takes the general form for that plane.
+//
+// The kernels are bound by instruction issue with shared memory close behind: about 300 instructions per
+// thread and plane for 8 cells.  512x256x256: 164 us (pre) and 150 us (post), 1.9 and 2.9 TB/s of the 9.1 and
+// 13 bytes per cell.  A ring of planes in shared memory filled by TMA with one barrier per half-sweep, the
+// form before, took 640 and 480 us: it issued 11 and 8.5 warp instructions per cell.
+#define FTP_NT 512
+#define FTP_RING 5
 
-#define FT_TX 48                    // tile along x (a multiple of 16: the flags box starts 16 cells left)
-#ifndef FT_TY
-#define FT_TY 16                    // tile along y (even: level-1 blocks are 2 x 2 x 2)
-#endif
-#ifndef FT_LA
-#define FT_LA 2                     // planes loaded ahead of the one a step consumes
-#endif
-#define FT_H 4                      // halo
-#define FT_RX (FT_TX + 2 * FT_H)    // r / z box along x (56 floats = 224 bytes)
-#define FT_RY (FT_TY + 2 * FT_H)    // box along y
-#define FT_FX (FT_TX + 32)          // flags box along x (80 bytes), starting 16 cells left of the tile
-#define FT_FOFF 12                  // flags column of r/z column 0
-#define FT_NS (6 + FT_LA)           // ring slots: planes t-5 .. t+FT_LA
-#define FT_QX (FT_RX / 4)           // 4-cell quads per ring row
-#define FT_NQ (FT_QX * FT_RY)       // quads of the ring plane
-#define FT_NT (((FT_NQ + 31) / 32) * 32)   // threads: one quad each
-#define FT_RBYTES (FT_RX * FT_RY * 4)
-#define FT_FBYTES (FT_FX * FT_RY)
-#define FT_FPAD (((FT_FBYTES + 127) / 128) * 128)
-#define FT_SLOT (2 * FT_RBYTES + FT_FPAD)             // r | z | flags
-#define FT_SMEM (FT_NS * FT_SLOT + 2 * FT_TX * FT_TY * 4 + 8 * FT_NS + 128)   // + alignment slack
-
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Waits for the phase of the given parity, for at most about a second (clock cycles); false on timeout.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
-        if (clock64() - t0 > 2000000000LL) return false;
-    return true;
-}
-__device__ __forceinline__ void tma_load3(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-
-struct FTSmem {
-    unsigned char* base;
-    __device__ float* r(int s) const { return reinterpret_cast<float*>(base + s * FT_SLOT); }
-    __device__ float* z(int s) const { return reinterpret_cast<float*>(base + s * FT_SLOT + FT_RBYTES); }
-    __device__ const uint8_t* f(int s) const { return base + s * FT_SLOT + 2 * FT_RBYTES; }
-    __device__ float* res(int parity) const { return reinterpret_cast<float*>(base + FT_NS * FT_SLOT) + parity * FT_TX * FT_TY; }
-    __device__ uint64_t* bar(int s) const {
-        return reinterpret_cast<uint64_t*>(base + FT_NS * FT_SLOT + 2 * FT_TX * FT_TY * 4) + s;
+template <int LX>
+struct FTile {
+    static constexpr int W = 4 * LX;               // cells along x, halo included
+    static constexpr int NRP = FTP_NT / LX;        // row pairs
+    static constexpr int H = 2 * NRP;              // rows, halo included
+    static constexpr int EXN = 2 * (NRP + 2) * LX; // float2 of one exchange buffer: two rows of every pair, padded
+    static constexpr size_t smem() {
+        return (size_t)8 * EXN * sizeof(float2) + (size_t)FTP_RING * FTP_NT * (2 * sizeof(float4) + sizeof(uint2)) +
+               16 * sizeof(float);
     }
 };
 
-struct FTPos {
-    int x0, y0, gx0, gy0;   // tile origin; global coordinates of ring column / row 0
-    int tlo;                // first plane loaded (ring slot 0, use 0)
+// A thread's column: constants of the march.
+struct FCol {
+    int xl;                 // quad within the row of the tile
+    int gx, gy;             // global coordinates of its first cell
+    bool in0, in1;          // rows inside the domain
+    bool own0, own1;        // rows of the tile's own cells
+    float inv[2][3];        // 1 / dg of the first, the middle two and the last cell of each row, 0 outside
+    int dg[2][3];
 };
 
-__device__ __forceinline__ int ft_slot(const FTPos& P, int t) { return (t - P.tlo) % FT_NS; }
-__device__ __forceinline__ unsigned ft_parity(const FTPos& P, int t) { return (unsigned)(((t - P.tlo) / FT_NS) & 1); }
-
-// Issues the TMA loads of plane t (r and flags, and z when `withz`) into its slot, or, for a plane
-// outside the domain, just completes the slot's phase.  One thread.
-__device__ __forceinline__ void ft_issue(const Dom& D, const FTSmem& S, const FTPos& P, int t, bool withz,
-                                         const CUtensorMap* tr, const CUtensorMap* tz, const CUtensorMap* tf) {
-    const int s = ft_slot(P, t);
-    uint64_t* b = S.bar(s);
-    if (t < 0 || t >= D.nz) {
-        mbar_arrive(b);
-        return;
+template <int LX>
+__device__ __forceinline__ FCol ftp_column(const Dom& D, int tx, int ty, int ntx, int nty) {
+    using T = FTile<LX>;
+    FCol c;
+    c.xl = threadIdx.x % LX;
+    const int rp = threadIdx.x / LX;
+    const int X0 = tx * (T::W - 8), Y0 = ty * (T::H - 8);
+    c.gx = X0 + 4 * c.xl;
+    c.gy = Y0 + 2 * rp;
+    const bool inx = c.gx < D.nx;                           // nx is a multiple of 4: a quad is inside or outside
+    c.in0 = inx && c.gy < D.ny;
+    c.in1 = inx && c.gy + 1 < D.ny;
+    const bool ox = (tx == 0 || c.xl > 0) && (tx == ntx - 1 || c.xl < LX - 1);
+    const bool oy = (ty == 0 || rp > 1) && (ty == nty - 1 || rp < T::NRP - 2);
+    c.own0 = c.in0 && ox && oy;
+    c.own1 = c.in1 && ox && oy;
+    auto term = [&](int f) { return D.bc[f] == IBM_BC_OUTFLOW ? 1 : -1; };   // a closed link, plus 2 at an outflow
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int y = c.gy + r;
+        const int d = 6 + (y == 0 ? term(2) : 0) + (y == D.ny - 1 ? term(3) : 0);
+        const bool in = r ? c.in1 : c.in0;
+        c.dg[r][0] = in ? d + (c.gx == 0 ? term(0) : 0) : 0;
+        c.dg[r][1] = in ? d : 0;
+        c.dg[r][2] = in ? d + (c.gx + 4 == D.nx ? term(1) : 0) : 0;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) c.inv[r][m] = c.dg[r][m] > 0 ? 1.f / (float)c.dg[r][m] : 0.f;
     }
-    mbar_expect_tx(b, (withz ? 2 : 1) * FT_RBYTES + FT_FBYTES);
-    tma_load3(S.r(s), tr, P.gx0, P.gy0, t, b);
-    if (withz) tma_load3(S.z(s), tz, P.gx0, P.gy0, t, b);
-    tma_load3((void*)S.f(s), tf, P.gx0 - FT_FOFF, P.gy0, t, b);
+    return c;
 }
 
-// Per-thread cells: thread q < FT_NQ owns the quad of 4 consecutive ring cells (ry, 4 qx .. 4 qx + 3),
-// fixed for the whole march; the quads line up with the tile (its x-range starts at ring column 4).
-// Cell masks (bit m for cell m): in the domain; interior (its in-plane neighbours are in the domain,
-// which the plain form of the update needs); within distance e of the tile (the half-sweeps of halo
-// e update those), for e = 0 .. 3.
-struct FTQuad {
-    int c;          // ring index of cell 0
-    int f;          // flags-ring index of cell 0 (a multiple of 4)
-    int gx, gy;     // global coordinates of cell 0
-    int par;        // (gx + gy) & 1
-    int tile;       // index of cell 0 in the tile (tile quads), -1 otherwise
-    unsigned dom, inter, halo;   // halo: 4 bits per e
+// Sum of z over the open links of a cell with flags f.
+__device__ __forceinline__ float ftp_open_sum(unsigned f, float xm, float xp, float ym, float yp, float zm, float zp) {
+    const float sx = ((f & 1u) ? 0.f : xm) + ((f & 2u) ? 0.f : xp);
+    const float sy = ((f & 4u) ? 0.f : ym) + ((f & 8u) ? 0.f : yp);
+    const float sz = ((f & 16u) ? 0.f : zm) + ((f & 32u) ? 0.f : zp);
+    return (sx + sy) + sz;
+}
+
+// x neighbours of the cells D0, D0 + 2 of row 0 and 1 - D0, 3 - D0 of row 1 that lie in another quad.
+template <int LX, int D0>
+__device__ __forceinline__ void ftp_xside(const FCol& c, const float (&zc)[2][4], float& e0, float& e1) {
+    const float a = D0 == 0 ? __shfl_up_sync(0xffffffffu, zc[0][3], 1) : __shfl_down_sync(0xffffffffu, zc[0][0], 1);
+    const float b = D0 == 0 ? __shfl_down_sync(0xffffffffu, zc[1][0], 1) : __shfl_up_sync(0xffffffffu, zc[1][3], 1);
+    const bool first = c.xl == 0, last = c.xl == LX - 1;
+    e0 = (D0 == 0 ? first : last) ? 0.f : a;
+    e1 = (D0 == 0 ? last : first) ? 0.f : b;
+}
+
+// The two cells D, D + 2 of row `zr` and their neighbours: calls f(cell, xm, xp, ym, yp, zm, zp, which).
+template <int D, class Fn>
+__device__ __forceinline__ void ftp_pair(const float (&zr)[4], float e, float ym0, float ym1, float yp0, float yp1,
+                                         const float (&zm)[4], const float (&zp)[4], Fn f) {
+    f(D, D == 0 ? e : zr[0], zr[D + 1], ym0, yp0, zm[D], zp[D], 0);
+    f(D + 2, zr[D + 1], D == 0 ? zr[3] : e, ym1, yp1, zm[D + 2], zp[D + 2], 1);
+}
+
+// One half-sweep on a thread's cells of one plane: cells D0, D0 + 2 of row 0 and 1 - D0, 3 - D0 of row 1.
+// yb, yt: the rows below and above (another thread's); r0, r1: the right-hand side at the updated cells.
+template <int LX, int D0>
+__device__ __forceinline__ void ftp_sweep(const FCol& c, float (&zc)[2][4], const float (&zm)[2][4], const float (&zp)[2][4],
+                                          float2 yb, float2 yt, float2 r0, float2 r1, float scale, bool general,
+                                          const uint2* fl, int zadj, const float* rcp) {
+    float e0, e1;
+    ftp_xside<LX, D0>(c, zc, e0, e1);
+    constexpr int D1 = 1 - D0;
+    float v0[2], v1[2];
+    if (!general) {
+        ftp_pair<D0>(zc[0], e0, yb.x, yb.y, zc[1][D0], zc[1][D0 + 2], zm[0], zp[0],
+                     [&](int m, float a, float b, float p, float q, float l, float u, int w) {
+                         v0[w] = fmaf(-scale, w ? r0.y : r0.x, ((a + b) + (p + q)) + (l + u)) * c.inv[0][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+                     });
+        ftp_pair<D1>(zc[1], e1, zc[0][D1], zc[0][D1 + 2], yt.x, yt.y, zm[1], zp[1],
+                     [&](int m, float a, float b, float p, float q, float l, float u, int w) {
+                         v1[w] = fmaf(-scale, w ? r1.y : r1.x, ((a + b) + (p + q)) + (l + u)) * c.inv[1][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+                     });
+    } else {
+        const uint2 ff = *fl;
+        auto cell = [&](int row, int m, float s, unsigned f, float r) {
+            const int d = c.dg[row][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+            return fmaf(-scale, r, s) * rcp[d ? d + zadj - __popc(f & 63u) : 0];
+        };
+        ftp_pair<D0>(zc[0], e0, yb.x, yb.y, zc[1][D0], zc[1][D0 + 2], zm[0], zp[0],
+                     [&](int m, float a, float b, float p, float q, float l, float u, int w) {
+                         const unsigned f = ff.x >> (8 * m);
+                         v0[w] = cell(0, m, ftp_open_sum(f, a, b, p, q, l, u), f, w ? r0.y : r0.x);
+                     });
+        ftp_pair<D1>(zc[1], e1, zc[0][D1], zc[0][D1 + 2], yt.x, yt.y, zm[1], zp[1],
+                     [&](int m, float a, float b, float p, float q, float l, float u, int w) {
+                         const unsigned f = ff.y >> (8 * m);
+                         v1[w] = cell(1, m, ftp_open_sum(f, a, b, p, q, l, u), f, w ? r1.y : r1.x);
+                     });
+    }
+    zc[0][D0] = v0[0];
+    zc[0][D0 + 2] = v0[1];
+    zc[1][D1] = v1[0];
+    zc[1][D1 + 2] = v1[1];
+}
+
+__device__ __forceinline__ void ftp_zero(float (&z)[2][4]) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) z[r][m] = 0.f;
+}
+__device__ __forceinline__ void ftp_copy(float (&a)[2][4], const float (&b)[2][4]) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) a[r][m] = b[r][m];
+}
+__device__ __forceinline__ void ftp_set(float (&a)[2][4], float4 x, float4 y) {
+    a[0][0] = x.x; a[0][1] = x.y; a[0][2] = x.z; a[0][3] = x.w;
+    a[1][0] = y.x; a[1][1] = y.y; a[1][2] = y.z; a[1][3] = y.w;
+}
+
+// Shared memory of a block and the thread's places in it.
+template <int LX>
+struct FShared {
+    float2* ex;          // [buffer 0 .. 3][step parity][row][pair + 1][quad]
+    float4* r;           // [slot][row][thread]: right-hand side, colour 0 then colour 1 (two cells each)
+    uint2* f;            // [slot][thread]: flags of the two quads
+    float* rcp;          // 1 / n, 0 for n = 0
+    int mine;            // index of the thread's pair and quad in a buffer row
+    __device__ __forceinline__ float2* at(int b, int par, int row, int dpair) const {
+        return ex + ((b * 2 + par) * 2 + row) * ((FTile<LX>::NRP + 2) * LX) + mine + dpair * LX;
+    }
+    __device__ __forceinline__ void publish(int b, int par, const float (&z)[2][4], int d0) const {
+        *at(b, par, 0, 0) = d0 ? make_float2(z[0][1], z[0][3]) : make_float2(z[0][0], z[0][2]);
+        *at(b, par, 1, 0) = d0 ? make_float2(z[1][0], z[1][2]) : make_float2(z[1][1], z[1][3]);
+    }
+    __device__ __forceinline__ float2 below(int b, int par) const { return *at(b, par, 1, -1); }
+    __device__ __forceinline__ float2 above(int b, int par) const { return *at(b, par, 0, 1); }
+    __device__ __forceinline__ float2 rhs(int slot, int row, int col) const {
+        return reinterpret_cast<const float2*>(r + (slot * 2 + row) * FTP_NT + threadIdx.x)[col];
+    }
 };
 
-__device__ __forceinline__ FTQuad ft_quad(const Dom& D, const FTPos& P, int q) {
-    FTQuad a;
-    a.c = a.f = a.gx = a.gy = a.par = 0;
-    a.tile = -1;
-    a.dom = a.inter = a.halo = 0u;
-    if (q >= FT_NQ) return a;
-    const int ry = q / FT_QX, rx = 4 * (q % FT_QX);
-    a.c = ry * FT_RX + rx;
-    a.f = ry * FT_FX + rx + FT_FOFF;
-    a.gx = P.gx0 + rx;
-    a.gy = P.gy0 + ry;
-    a.par = (a.gx + a.gy) & 1;
-    const int dy = max(max(FT_H - ry, ry - (FT_H + FT_TY - 1)), 0);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int x = rx + m, gx = a.gx + m;
-        const int dx = max(max(FT_H - x, x - (FT_H + FT_TX - 1)), 0);
-        const bool in = gx >= 0 && gx < D.nx && a.gy >= 0 && a.gy < D.ny;
-        const bool inter = gx > 0 && gx < D.nx - 1 && a.gy > 0 && a.gy < D.ny - 1;
-        const int d = max(dx, dy);
-        a.dom |= (in ? 1u : 0u) << m;
-        a.inter |= (inter ? 1u : 0u) << m;
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (in && d <= e) a.halo |= 1u << (4 * e + m);
-    }
-    if (dy == 0 && rx >= FT_H && rx < FT_H + FT_TX) a.tile = (ry - FT_H) * FT_TX + (rx - FT_H);
-    return a;
+template <int LX>
+__device__ __forceinline__ FShared<LX> ftp_shared(unsigned char* base) {
+    using T = FTile<LX>;
+    FShared<LX> S;
+    S.ex = reinterpret_cast<float2*>(base);
+    S.r = reinterpret_cast<float4*>(S.ex + 8 * T::EXN);
+    S.f = reinterpret_cast<uint2*>(S.r + FTP_RING * 2 * FTP_NT);
+    S.rcp = reinterpret_cast<float*>(S.f + FTP_RING * FTP_NT);
+    S.mine = (threadIdx.x / LX + 1) * LX + threadIdx.x % LX;
+    for (int e = threadIdx.x; e < 8 * T::EXN; e += FTP_NT) S.ex[e] = make_float2(0.f, 0.f);
+    if (threadIdx.x < 16) S.rcp[threadIdx.x] = threadIdx.x ? 1.f / (float)threadIdx.x : 0.f;
+    __syncthreads();
+    return S;
 }
 
-__device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float f4e(const float4& v, int m) { return m == 0 ? v.x : (m == 1 ? v.y : (m == 2 ? v.z : v.w)); }
+__device__ __forceinline__ int ftp_back(int slot, int k) { return slot >= k ? slot - k : slot - k + FTP_RING; }
 
-// Gauss-Seidel value of a ring cell in the generic case (a cut link or a domain face next to it):
-// (sum of z over the open links - sr) / dg, dg = open links + the outflow terms.
-__device__ __forceinline__ float ft_gs_generic(const Dom& D, int c, int gx, int gy, int t, unsigned fl, float sr,
-                                               const float* zm, const float* zc, const float* zp) {
-    const int g[3] = {gx, gy, t}, n[3] = {D.nx, D.ny, D.nz};
-    float s = 0.f, dg = 0.f;
-#pragma unroll
-    for (int b = 0; b < 6; ++b) {
-        const int a = b >> 1, sd = (b & 1) ? 1 : -1;
-        const bool in = g[a] + sd >= 0 && g[a] + sd < n[a];
-        if (in && !(fl & (1u << b))) {
-            dg += 1.f;
-            s += a == 0 ? zc[c + sd] : (a == 1 ? zc[c + sd * FT_RX] : (sd < 0 ? zm[c] : zp[c]));
-        } else if (!in && D.bc[b] == IBM_BC_OUTFLOW) {
-            dg += 2.f;
-        }
-    }
-    return dg == 0.f ? 0.f : (s - sr) / dg;
+// Extra diagonal of the first and last plane.
+__device__ __forceinline__ int ftp_zadj(const Dom& D, int p) {
+    return (p == 0 ? (D.bc[4] == IBM_BC_OUTFLOW ? 1 : -1) : 0) + (p == D.nz - 1 ? (D.bc[5] == IBM_BC_OUTFLOW ? 1 : -1) : 0);
 }
 
-// A z at a ring cell in the generic case, unscaled form  sum_open (z_N - z_P) - d z_P.
-__device__ __forceinline__ float ft_az_generic(const Dom& D, int c, int gx, int gy, int t, unsigned fl,
-                                               const float* zm, const float* zc, const float* zp) {
-    const float zP = zc[c];
-    const int g[3] = {gx, gy, t}, n[3] = {D.nx, D.ny, D.nz};
-    float s = 0.f;
-#pragma unroll
-    for (int b = 0; b < 6; ++b) {
-        const int a = b >> 1, sd = (b & 1) ? 1 : -1;
-        const bool in = g[a] + sd >= 0 && g[a] + sd < n[a];
-        if (in && !(fl & (1u << b)))
-            s += (a == 0 ? zc[c + sd] : (a == 1 ? zc[c + sd * FT_RX] : (sd < 0 ? zm[c] : zp[c]))) - zP;
-        else if (!in && D.bc[b] == IBM_BC_OUTFLOW)
-            s += -zP - zP;
-    }
-    return s;
-}
-
-// The ring planes of one step: slot of plane t - k for k = 0 .. 5 (one modulo per step).
-struct FTRing {
-    int sl[6];
-    __device__ __forceinline__ FTRing(const FTPos& P, int t) {
-        sl[0] = (t - P.tlo) % FT_NS;
-#pragma unroll
-        for (int k = 1; k < 6; ++k) sl[k] = sl[k - 1] == 0 ? FT_NS - 1 : sl[k - 1] - 1;
-    }
-};
-
-// One half-sweep of colour `col` on plane t = step - k (ring slot R.sl[k]) over the thread's cells
-// within `e` of the tile.  The k-th half-sweep of a pass runs only on planes t >= tlo + k: below that
-// its inputs (the previous half-sweep on plane t - 1) were never formed in this block, and nothing it
-// would produce is needed.  The quad's two cells of colour col are d and d + 2; a cell with no cut
-// link whose neighbours lie in the domain takes the six-neighbour sum from 16-byte loads.
-__device__ __forceinline__ void ft_half_sweep(const Dom& D, const FTSmem& S, const FTPos& P, const FTQuad& Q,
-                                              const FTRing& R, int k, int t, int col, int e, float scale, int kind) {
-    if (t < P.tlo + kind || t < 0 || t >= D.nz) return;     // the same for the whole block
-    const int d = (col + Q.par + t) & 1;
-    const unsigned act = (Q.halo >> (4 * e)) & (5u << d);
-    float* zc = S.z(R.sl[k]);
-    const float* zm = S.z(R.sl[k + 1]);           // planes outside the domain are never read (links closed)
-    const float* zp = S.z(k > 0 ? R.sl[k - 1] : R.sl[k]);
-    const float* rc = S.r(R.sl[k]);
-    const unsigned fl4 = *reinterpret_cast<const unsigned*>(S.f(R.sl[k]) + Q.f);
-    const bool tint = t > 0 && t < D.nz - 1;
-    const unsigned fa = (fl4 >> (8 * d)) & 0xffu, fb = (fl4 >> (8 * (d + 2))) & 0xffu;
-    const bool onA = (act >> d) & 1u, onB = (act >> (d + 2)) & 1u;
-    const bool plainA = fa == 0u && tint && ((Q.inter >> d) & 1u);
-    const bool plainB = fb == 0u && tint && ((Q.inter >> (d + 2)) & 1u);
-    // a warp without a generic cell skips the generic form altogether
-    const bool generic = __any_sync(0xffffffffu, (onA && !plainA) || (onB && !plainB));
-    if (!act) return;
-    const int c = Q.c;
-    const float4 z4 = lds4(zc + c), r4 = lds4(rc + c);
-    const float4 ym = lds4(zc + c - FT_RX), yp = lds4(zc + c + FT_RX);
-    const float4 zl = lds4(zm + c), zu = lds4(zp + c);
-    const bool odd = d != 0;
-    // cells A = d and B = d + 2 and their x-neighbours (the cell left of the quad and the one right of
-    // it lie in the same ring row: an active quad is never in the ring's first or last column)
-    const float left = zc[c - 1], right = zc[c + 4];
-    const float xa_l = odd ? z4.x : left, xa_r = odd ? z4.z : z4.y;
-    const float xb_l = xa_r, xb_r = odd ? right : z4.w;
-    const float sa = ((xa_l + xa_r) + ((odd ? ym.y : ym.x) + (odd ? yp.y : yp.x))) + ((odd ? zl.y : zl.x) + (odd ? zu.y : zu.x));
-    const float sb = ((xb_l + xb_r) + ((odd ? ym.w : ym.z) + (odd ? yp.w : yp.z))) + ((odd ? zl.w : zl.z) + (odd ? zu.w : zu.z));
-    const float ra = odd ? r4.y : r4.x, rb = odd ? r4.w : r4.z;
-    float va = (sa - scale * ra) * (1.f / 6.f), vb = (sb - scale * rb) * (1.f / 6.f);
-    if (generic) {
-        if (onA && !plainA) va = ft_gs_generic(D, c + d, Q.gx + d, Q.gy, t, fa, scale * ra, zm, zc, zp);
-        if (onB && !plainB) vb = ft_gs_generic(D, c + d + 2, Q.gx + d + 2, Q.gy, t, fb, scale * rb, zm, zc, zp);
-    }
-    if (onA) zc[c + d] = va;
-    if (onB) zc[c + d + 2] = vb;
-}
-
-// Pre-smoothing (from z = 0, colours 0, 1, 0, 1) + restriction of  scale r - A z  to the parts of the
-// level-1 blocks.  Writes z on its chunk's planes [k0, k1) and b_1.
-__global__ void __launch_bounds__(FT_NT, 2) k_mg_pre_fused(Dom D, float* __restrict__ z, float scale, MGLev C1,
-                                                          int kchunk, SolveScal* sc,
-                                                          const __grid_constant__ CUtensorMap tmr,
-                                                          const __grid_constant__ CUtensorMap tmf) {
+// Pre-smoothing (from z = 0, colours 0, 1, 0, 1) and the restriction of  scale r - A z  to the parts of the
+// level-1 blocks.  Writes z on its chunk's planes [k0, k1) and b_1.  The last half-sweep leaves the residual
+// of colour 1 zero, so only colour 0 is evaluated (one plane behind the last half-sweep).
+template <int LX>
+__global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* __restrict__ rg, float* __restrict__ zg,
+                                                            float scale, MGLev C1, int kchunk, const SolveScal* sc) {
     if (sc->done) return;
-    extern __shared__ __align__(128) unsigned char ft_smem[];
-    __shared__ int abort_flag;
-    FTSmem S{reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(ft_smem) + 127) & ~(uintptr_t)127)};
-    FTPos P;
-    P.x0 = blockIdx.x * FT_TX;
-    P.y0 = blockIdx.y * FT_TY;
-    P.gx0 = P.x0 - FT_H;
-    P.gy0 = P.y0 - FT_H;
+    extern __shared__ __align__(16) unsigned char ftp_raw[];
+    const FShared<LX> S = ftp_shared<LX>(ftp_raw);
+    const FCol c = ftp_column<LX>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
     const int k0 = blockIdx.z * kchunk, k1 = min(D.nz, k0 + kchunk);
-    P.tlo = k0 - 4;
-    const int thi = k1 + 3;
+    const int tlo = max(0, k0 - 4), thi = k1 + 3;
     float* __restrict__ b1 = (float*)C1.b;
-    const FTQuad Q = ft_quad(D, P, threadIdx.x);
-    if (threadIdx.x == 0) {
-        abort_flag = 0;
-        for (int s = 0; s < FT_NS; ++s) mbar_init(S.bar(s), 1);
-        fence_barrier_init();
-    }
-    __syncthreads();
-    int issued = P.tlo - 1;
-    if (threadIdx.x == 0)
-        for (int u = P.tlo; u < P.tlo + FT_LA && u <= thi; ++u) {
-            ft_issue(D, S, P, u, false, &tmr, nullptr, &tmf);
-            issued = u;
+    const int row0 = c.gx + D.sy * c.gy;
+    float Z[6][2][4];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) ftp_zero(Z[q]);
+    float4 nr0 = make_float4(0.f, 0.f, 0.f, 0.f), nr1 = nr0;
+    unsigned nf0 = 0u, nf1 = 0u;
+    auto fetch = [&](int t) {
+        nr0 = nr1 = make_float4(0.f, 0.f, 0.f, 0.f);
+        nf0 = nf1 = 0u;
+        if (t >= D.nz) return;
+        const long long P = row0 + D.sz * t;
+        if (c.in0) {
+            nr0 = *reinterpret_cast<const float4*>(rg + P);
+            if (D.flags) nf0 = *reinterpret_cast<const unsigned*>(D.flags + P);
         }
-    for (int t = P.tlo; t <= thi; ++t) {
-        if (threadIdx.x == 0) {
-            if (t + FT_LA <= thi) {
-                ft_issue(D, S, P, t + FT_LA, false, &tmr, nullptr, &tmf);
-                issued = t + FT_LA;
-            }
-            if (!mbar_wait(S.bar(ft_slot(P, t)), ft_parity(P, t))) abort_flag = 1;
+        if (c.in1) {
+            nr1 = *reinterpret_cast<const float4*>(rg + P + D.sy);
+            if (D.flags) nf1 = *reinterpret_cast<const unsigned*>(D.flags + P + D.sy);
         }
-        __syncthreads();
-        if (abort_flag) break;
-        const FTRing R(P, t);
-        // h1 on plane t: z = -scale r / dg on colour 0, 0 on colour 1 (z = 0 before the first pass)
-        if (t >= 0 && t < D.nz) {
-            const int s = R.sl[0];
-            const float4 r4 = lds4(S.r(s) + Q.c);
-            const unsigned fl4 = *reinterpret_cast<const unsigned*>(S.f(s) + Q.f);
-            const bool tint = t > 0 && t < D.nz - 1;
-            unsigned on = 0u, gen = 0u;
+    };
+    fetch(tlo);
+    unsigned gen = 0u;                  // bit k: plane t - k takes the general form in this warp
+    int slot = 0;                       // ring slot of plane t
+    float er[2][2] = {{0.f, 0.f}, {0.f, 0.f}};       // residuals of the even plane [row][position]
+    auto step = [&](auto par, int t) {
+        constexpr int D0 = decltype(par)::value;      // = t & 1
+        const int pw = D0, pr = 1 - D0;                // exchange buffers written and read in this step
+        // plane t arrives: right-hand side and flags into the ring, colour 0 first
+        const float4 c0 = D0 ? make_float4(nr0.y, nr0.w, nr0.x, nr0.z) : make_float4(nr0.x, nr0.z, nr0.y, nr0.w);
+        const float4 c1 = D0 ? make_float4(nr1.x, nr1.z, nr1.y, nr1.w) : make_float4(nr1.y, nr1.w, nr1.x, nr1.z);
+        S.r[(slot * 2 + 0) * FTP_NT + threadIdx.x] = c0;
+        S.r[(slot * 2 + 1) * FTP_NT + threadIdx.x] = c1;
+        const uint2 ft = make_uint2(nf0, nf1);
+        S.f[slot * FTP_NT + threadIdx.x] = ft;
+        gen = (gen << 1) | ((__any_sync(0xffffffffu, ((nf0 | nf1) & 0x3f3f3f3fu) != 0u) || t == 0 || t == D.nz - 1) ? 1u : 0u);
+        fetch(t + 1);
+        // half-sweep 1 on plane t, from z = 0
+        ftp_zero(Z[0]);
+        if (t < D.nz) {
+            const float q[2][2] = {{-scale * c0.x, -scale * c0.y}, {-scale * c1.x, -scale * c1.y}};
+            const int zadj = (gen & 1u) ? ftp_zadj(D, t) : 0;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const bool o = ((Q.dom >> m) & 1u) && !((Q.par + m + t) & 1);
-                const bool plain = ((fl4 >> (8 * m)) & 0xffu) == 0u && tint && ((Q.inter >> m) & 1u);
-                on |= (o ? 1u : 0u) << m;
-                gen |= (o && !plain ? 1u : 0u) << m;
-            }
-            float v[4];
+            for (int row = 0; row < 2; ++row)
 #pragma unroll
-            for (int m = 0; m < 4; ++m) v[m] = ((on >> m) & 1u) ? (0.f - scale * f4e(r4, m)) * (1.f / 6.f) : 0.f;
-            if (__any_sync(0xffffffffu, gen != 0u)) {
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    if (!((gen >> m) & 1u)) continue;
-                    const unsigned fl = (fl4 >> (8 * m)) & 0xffu;
-                    const int g[3] = {Q.gx + m, Q.gy, t}, n[3] = {D.nx, D.ny, D.nz};
-                    float dg = 0.f;
-#pragma unroll
-                    for (int b = 0; b < 6; ++b) {
-                        const int a = b >> 1, sd = (b & 1) ? 1 : -1;
-                        const bool in = g[a] + sd >= 0 && g[a] + sd < n[a];
-                        if (in && !(fl & (1u << b))) dg += 1.f;
-                        else if (!in && D.bc[b] == IBM_BC_OUTFLOW) dg += 2.f;
+                for (int w = 0; w < 2; ++w) {
+                    const int m = (row ? 1 - D0 : D0) + 2 * w, mi = m == 0 ? 0 : (m == 3 ? 2 : 1);
+                    float iv = c.inv[row][mi];
+                    if (gen & 1u) {
+                        const unsigned f = (row ? ft.y : ft.x) >> (8 * m);
+                        const int d = c.dg[row][mi];
+                        iv = S.rcp[d ? d + zadj - __popc(f & 63u) : 0];
                     }
-                    v[m] = dg == 0.f ? 0.f : (0.f - scale * f4e(r4, m)) / dg;
+                    Z[0][row][m] = q[row][w] * iv;
                 }
-            }
-            if (threadIdx.x < FT_NQ)
-                *reinterpret_cast<float4*>(S.z(s) + Q.c) = make_float4(v[0], v[1], v[2], v[3]);
+            S.publish(0, pw, Z[0], D0);
         }
-        __syncthreads();
-        ft_half_sweep(D, S, P, Q, R, 1, t - 1, 1, 3, scale, 1);
-        __syncthreads();
-        ft_half_sweep(D, S, P, Q, R, 2, t - 2, 0, 2, scale, 2);
-        __syncthreads();
-        ft_half_sweep(D, S, P, Q, R, 3, t - 3, 1, 1, scale, 3);
-        __syncthreads();
-        // plane t-3 is final: store the tile; residual of plane t-4 (its neighbours are final)
-        const int tw = t - 3, tr = t - 4;
-        if (tw >= k0 && tw < k1 && Q.tile >= 0 && Q.dom == 0xfu)
-            *reinterpret_cast<float4*>(z + Q.gx + (long long)D.sy * Q.gy + D.sz * tw) = lds4(S.z(R.sl[3]) + Q.c);
+        // half-sweeps 2, 3, 4 on planes t - 1, t - 2, t - 3 (colours 1, 0, 1)
+#pragma unroll
+        for (int k = 1; k <= 3; ++k) {
+            const int p = t - k;
+            if (p >= tlo && p < D.nz) {
+                const int sl = ftp_back(slot, k);
+                const bool g = (gen >> k) & 1u;
+                ftp_sweep<LX, D0>(c, Z[k], Z[k + 1], Z[k - 1], S.below(k - 1, pr), S.above(k - 1, pr), S.rhs(sl, 0, k & 1),
+                                  S.rhs(sl, 1, k & 1), scale, g, S.f + sl * FTP_NT + threadIdx.x, g ? ftp_zadj(D, p) : 0, S.rcp);
+                S.publish(k, pw, Z[k], D0);
+            }
+        }
+        // plane t - 3 is final
+        const int tw = t - 3;
+        if (tw >= k0 && tw < k1) {
+            float* zo = zg + row0 + D.sz * tw;
+            if (c.own0) *reinterpret_cast<float4*>(zo) = make_float4(Z[3][0][0], Z[3][0][1], Z[3][0][2], Z[3][0][3]);
+            if (c.own1) *reinterpret_cast<float4*>(zo + D.sy) = make_float4(Z[3][1][0], Z[3][1][1], Z[3][1][2], Z[3][1][3]);
+        }
+        // residual of colour 0 on plane t - 4
+        const int tr = t - 4;
         if (tr >= k0 && tr < k1) {
-            {
-                const int s = R.sl[4];
-                const float* zc = S.z(s);
-                const float* zm = S.z(R.sl[5]);
-                const float* zp = S.z(R.sl[3]);
-                const int c = Q.c;
-                const unsigned fl4 = *reinterpret_cast<const unsigned*>(S.f(s) + Q.f);
-                const bool tint = tr > 0 && tr < D.nz - 1;
-                const bool tq = Q.tile >= 0 && Q.dom != 0u;
-                unsigned gen = 0u;
+            const int sl = ftp_back(slot, 4);
+            const bool g = (gen >> 4) & 1u;
+            const float2 yb = S.below(3, pr), yt = S.above(3, pr), r0 = S.rhs(sl, 0, 0), r1 = S.rhs(sl, 1, 0);
+            float e0, e1;
+            ftp_xside<LX, D0>(c, Z[4], e0, e1);
+            const uint2 ff = g ? S.f[sl * FTP_NT + threadIdx.x] : make_uint2(0u, 0u);
+            const int zadj = g ? ftp_zadj(D, tr) : 0;
+            float res[2][2];
+            auto cell = [&](int row, int m, float a, float b, float p, float q, float l, float u, float r) {
+                int d = c.dg[row][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+                float s;
+                if (!g) {
+                    s = ((a + b) + (p + q)) + (l + u);
+                } else {
+                    const unsigned f = (row ? ff.y : ff.x) >> (8 * m);
+                    s = ftp_open_sum(f, a, b, p, q, l, u);
+                    d += zadj - __popc(f & 63u);
+                }
+                return scale * r - (s - (float)d * Z[4][row][m]);
+            };
+            constexpr int D1 = 1 - D0;
+            ftp_pair<D0>(Z[4][0], e0, yb.x, yb.y, Z[4][1][D0], Z[4][1][D0 + 2], Z[5][0], Z[3][0],
+                         [&](int m, float a, float b, float p, float q, float l, float u, int w) {
+                             res[0][w] = cell(0, m, a, b, p, q, l, u, w ? r0.y : r0.x);
+                         });
+            ftp_pair<D1>(Z[4][1], e1, Z[4][0][D1], Z[4][0][D1 + 2], yt.x, yt.y, Z[5][1], Z[3][1],
+                         [&](int m, float a, float b, float p, float q, float l, float u, int w) {
+                             res[1][w] = cell(1, m, a, b, p, q, l, u, w ? r1.y : r1.x);
+                         });
+            if (!c.in1) res[1][0] = res[1][1] = 0.f;
+            const bool lastp = tr == D.nz - 1;
+            if (D0 == 0) {              // an even plane (tr and t have the same parity)
 #pragma unroll
-                for (int m = 0; m < 4; ++m)
-                    if (tq && !(((fl4 >> (8 * m)) & 0xffu) == 0u && tint && ((Q.inter >> m) & 1u))) gen |= 1u << m;
-                // a warp without a generic cell skips the generic form altogether
-                const bool generic = __any_sync(0xffffffffu, gen != 0u);
-                if (Q.tile >= 0) {
-                    float v[4] = {0.f, 0.f, 0.f, 0.f};
-                    if (Q.dom) {
-                        const float4 z4 = lds4(zc + c), r4 = lds4(S.r(s) + c);
-                        const float4 ym = lds4(zc + c - FT_RX), yp = lds4(zc + c + FT_RX);
-                        const float4 zl = lds4(zm + c), zu = lds4(zp + c);
-                        const float left = zc[c - 1], right = zc[c + 4];
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            const float xm = m == 0 ? left : f4e(z4, m - 1);
-                            const float xp = m == 3 ? right : f4e(z4, m + 1);
-                            float az = ((xm + xp) + (f4e(ym, m) + f4e(yp, m))) + (f4e(zl, m) + f4e(zu, m)) - 6.f * f4e(z4, m);
-                            if (generic && ((gen >> m) & 1u))
-                                az = ft_az_generic(D, c + m, Q.gx + m, Q.gy, tr, (fl4 >> (8 * m)) & 0xffu, zm, zc, zp);
-                            v[m] = scale * f4e(r4, m) - az;
-                        }
-                    }
-                    *reinterpret_cast<float4*>(S.res(tr & 1) + Q.tile) = make_float4(v[0], v[1], v[2], v[3]);
+                for (int w = 0; w < 2; ++w) {
+                    er[0][w] = res[0][w];
+                    er[1][w] = res[1][w];
                 }
             }
-            if ((tr & 1) || tr == D.nz - 1) {
-                __syncthreads();
-                // restriction: the level-1 blocks of planes (tr & ~1, tr | 1)
-                const int ke = tr & ~1;
-                const int Z = ke >> 1;
-                const bool both = ke + 1 < D.nz;
-                // tr odd: the pair is (tr - 1, tr) in slots 5, 4; tr even (the last plane of an odd count): tr alone
-                const uint8_t* fe = S.f((tr & 1) ? R.sl[5] : R.sl[4]);
-                const uint8_t* fo = both ? S.f(R.sl[4]) : fe;
-                const float* re = S.res(0);
-                const float* ro = S.res(1);
-                for (int q = threadIdx.x; q < (FT_TX / 2) * (FT_TY / 2); q += FT_NT) {
-                    const int bx = q % (FT_TX / 2), by = q / (FT_TX / 2);
-                    const int X = (P.x0 >> 1) + bx, Y = (P.y0 >> 1) + by;
-                    if (X >= C1.px || Y >= C1.py) continue;
-                    const bool yok = 2 * Y + 1 < D.ny;           // x: nx is even, so both columns exist
-                    unsigned fl[8];
-                    float rv[8];
-                    unsigned in = 0;
-                    const int fi = (FT_H + 2 * by) * FT_FX + FT_H + 2 * bx + FT_FOFF;
-                    const int ri = (2 * by) * FT_TX + 2 * bx;
+            if ((D0 == 1 || lastp) && c.own0) {
+                const long long q = (c.gx >> 1) + (long long)C1.px * ((c.gy >> 1) + (long long)C1.py * (tr >> 1));
+                const int2 o = *reinterpret_cast<const int2*>(C1.off + q);
+                const bool odd = D0 == 1;                // both planes of the block are there
+                // a warp without a cut link in the two planes: whole blocks
+                if (!((gen >> 4) & 1u) && !(odd && ((gen >> 5) & 1u))) {
+                    b1[o.x] = odd ? (er[0][0] + er[1][0]) + (res[0][0] + res[1][0]) : er[0][0] + er[1][0];
+                    b1[o.y] = odd ? (er[0][1] + er[1][1]) + (res[0][1] + res[1][1]) : er[0][1] + er[1][1];
+                } else {
+                    const long long Pe = row0 + D.sz * (tr & ~1);
+                    unsigned fe[2], fo[2];
+                    fe[0] = D.flags ? *reinterpret_cast<const unsigned*>(D.flags + Pe) : 0u;
+                    fe[1] = D.flags && c.in1 ? *reinterpret_cast<const unsigned*>(D.flags + Pe + D.sy) : 0u;
+                    fo[0] = D.flags && odd ? *reinterpret_cast<const unsigned*>(D.flags + Pe + D.sz) : 0u;
+                    fo[1] = D.flags && odd && c.in1 ? *reinterpret_cast<const unsigned*>(D.flags + Pe + D.sz + D.sy) : 0u;
 #pragma unroll
-                    for (int m = 0; m < 8; ++m) {
-                        const int di = m & 1, dj = (m >> 1) & 1, dk = m >> 2;
-                        const bool ok = (dj == 0 || yok) && (dk == 0 || both);
-                        fl[m] = ok ? (unsigned)(dk ? fo : fe)[fi + dj * FT_FX + di] : 0u;
-                        rv[m] = ok ? (dk ? ro : re)[ri + dj * FT_TX + di] : 0.f;
-                        in |= (ok ? 1u : 0u) << m;
+                    for (int h = 0; h < 2; ++h) {
+                        unsigned fl[8], in = 0;
+                        float rv[8];
+#pragma unroll
+                        for (int m = 0; m < 8; ++m) {
+                            const int di = m & 1, dj = (m >> 1) & 1, dk = m >> 2;
+                            const bool ok = (dj == 0 || c.in1) && (dk == 0 || odd);
+                            fl[m] = ok ? ((dk ? fo[dj] : fe[dj]) >> (8 * (2 * h + di))) & 0xffu : 0u;
+                            in |= (ok ? 1u : 0u) << m;
+                            // colour 0: x + y + z even within the block
+                            rv[m] = ((di + dj + dk) & 1) ? 0.f : (dk ? res[dj][h] : er[dj][h]);
+                        }
+                        int part[8];
+                        const int np = fine_parts(D, fl, in, part);
+                        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                        for (int m = 0; m < 8; ++m)
+#pragma unroll
+                            for (int s2 = 0; s2 < 8; ++s2) acc[s2] += (((in >> m) & 1u) && part[m] == s2) ? rv[m] : 0.f;
+                        const int oo = h ? o.y : o.x;
+#pragma unroll
+                        for (int s2 = 0; s2 < 8; ++s2)
+                            if (s2 < np) b1[oo + s2] = acc[s2];
                     }
-                    int part[8];
-                    const int np = fine_parts(D, fl, in, part);
-                    const int o = C1.off[X + (long long)C1.px * (Y + (long long)C1.py * Z)];
-                    if (np == 1) {
-                        b1[o] = ((rv[0] + rv[1]) + (rv[2] + rv[3])) + ((rv[4] + rv[5]) + (rv[6] + rv[7]));
-                        continue;
-                    }
-                    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int m = 0; m < 8; ++m)
-#pragma unroll
-                        for (int s2 = 0; s2 < 8; ++s2) acc[s2] += part[m] == s2 ? rv[m] : 0.f;
-#pragma unroll
-                    for (int s2 = 0; s2 < 8; ++s2)
-                        if (s2 < np) b1[o + s2] = acc[s2];
                 }
             }
         }
-        fence_proxy_async();
+#pragma unroll
+        for (int q = 5; q > 0; --q) ftp_copy(Z[q], Z[q - 1]);
+        slot = slot == FTP_RING - 1 ? 0 : slot + 1;
         __syncthreads();
-    }
-    if (abort_flag && threadIdx.x == 0) {
-        // let the loads already issued land before the block's shared memory goes away
-        for (int u = issued; u > issued - FT_NS && u >= P.tlo; --u) mbar_wait(S.bar(ft_slot(P, u)), ft_parity(P, u));
-        atomicExch(&sc->dev_error, 1);
+    };
+    for (int t = tlo; t <= thi; t += 2) {
+        step(std::integral_constant<int, 0>{}, t);
+        step(std::integral_constant<int, 1>{}, t + 1);
     }
 }
 
-// Post-smoothing (colours 1, 0, 1, 0) of the iterate the coarse correction left (read through the
-// `tmz` map from an array this pass does not write), into z; then (r, z) over the grid:
+// Post-smoothing (colours 1, 0, 1, 0) of the iterate the coarse correction left, read from zin (an array
+// this pass does not write: neighbouring tiles read each other's cells), into z; then (r, z) over the grid:
 // rz_old = rz, rz = (r, z).
-__global__ void __launch_bounds__(FT_NT, 2) k_mg_post_fused(Dom D, float* __restrict__ z, float scale, int kchunk,
-                                                           SolveScal* sc, double* partials, unsigned* counter,
-                                                           const __grid_constant__ CUtensorMap tmr,
-                                                           const __grid_constant__ CUtensorMap tmz,
-                                                           const __grid_constant__ CUtensorMap tmf) {
+template <int LX>
+__global__ void __launch_bounds__(FTP_NT, 1) k_mg_post_fused(Dom D, const float* __restrict__ rg, const float* __restrict__ zin,
+                                                             float* __restrict__ zg, float scale, int kchunk, SolveScal* sc,
+                                                             double* partials, unsigned* counter) {
     if (sc->done) return;
-    extern __shared__ __align__(128) unsigned char ft_smem[];
-    __shared__ int abort_flag;
-    FTSmem S{reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(ft_smem) + 127) & ~(uintptr_t)127)};
-    FTPos P;
-    P.x0 = blockIdx.x * FT_TX;
-    P.y0 = blockIdx.y * FT_TY;
-    P.gx0 = P.x0 - FT_H;
-    P.gy0 = P.y0 - FT_H;
+    extern __shared__ __align__(16) unsigned char ftp_raw[];
+    const FShared<LX> S = ftp_shared<LX>(ftp_raw);
+    const FCol c = ftp_column<LX>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
     const int k0 = blockIdx.z * kchunk, k1 = min(D.nz, k0 + kchunk);
-    P.tlo = k0 - 4;
-    const int thi = k1 + 3;
-    const FTQuad Q = ft_quad(D, P, threadIdx.x);
-    if (threadIdx.x == 0) {
-        abort_flag = 0;
-        for (int s = 0; s < FT_NS; ++s) mbar_init(S.bar(s), 1);
-        fence_barrier_init();
-    }
+    const int tlo = max(0, k0 - 4), thi = k1 + 2;
+    const int row0 = c.gx + D.sy * c.gy;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float Z[5][2][4], zn[2][4];          // planes t .. t - 4 and t + 1
+    float4 nr0, nr1, nz0, nz1;           // r of plane t + 1 and z of plane t + 2, in flight
+    unsigned nf0, nf1;
+    auto fetch_r = [&](int t) {
+        nr0 = nr1 = zero4;
+        nf0 = nf1 = 0u;
+        if (t >= D.nz) return;
+        const long long P = row0 + D.sz * t;
+        if (c.in0) {
+            nr0 = *reinterpret_cast<const float4*>(rg + P);
+            if (D.flags) nf0 = *reinterpret_cast<const unsigned*>(D.flags + P);
+        }
+        if (c.in1) {
+            nr1 = *reinterpret_cast<const float4*>(rg + P + D.sy);
+            if (D.flags) nf1 = *reinterpret_cast<const unsigned*>(D.flags + P + D.sy);
+        }
+    };
+    auto fetch_z = [&](int t) {
+        nz0 = nz1 = zero4;
+        if (t >= D.nz) return;
+        const long long P = row0 + D.sz * t;
+        if (c.in0) nz0 = *reinterpret_cast<const float4*>(zin + P);
+        if (c.in1) nz1 = *reinterpret_cast<const float4*>(zin + P + D.sy);
+    };
+#pragma unroll
+    for (int q = 1; q < 5; ++q) ftp_zero(Z[q]);
+    fetch_z(tlo);
+    ftp_set(Z[0], nz0, nz1);
+    // colour 0 of plane tlo, read by step tlo (even) from the buffers of odd steps
+    S.publish(0, 1, Z[0], 0);
+    fetch_z(tlo + 1);
+    ftp_set(zn, nz0, nz1);
+    fetch_z(tlo + 2);
+    fetch_r(tlo);
     __syncthreads();
-    int issued = P.tlo - 1;
-    if (threadIdx.x == 0)
-        for (int u = P.tlo; u < P.tlo + FT_LA && u <= thi; ++u) {
-            ft_issue(D, S, P, u, true, &tmr, &tmz, &tmf);
-            issued = u;
-        }
+    unsigned gen = 0u;
+    int slot = 0;
     float part = 0.f;
-    for (int t = P.tlo; t <= thi; ++t) {
-        if (threadIdx.x == 0) {
-            if (t + FT_LA <= thi) {
-                ft_issue(D, S, P, t + FT_LA, true, &tmr, &tmz, &tmf);
-                issued = t + FT_LA;
+    auto step = [&](auto par, int t) {
+        constexpr int PT = decltype(par)::value;      // t & 1
+        constexpr int D0 = 1 - PT;                    // cells of row 0 the step's half-sweeps update
+        const int pw = PT, pr = 1 - PT;
+        const float4 c0 = PT ? make_float4(nr0.y, nr0.w, nr0.x, nr0.z) : make_float4(nr0.x, nr0.z, nr0.y, nr0.w);
+        const float4 c1 = PT ? make_float4(nr1.x, nr1.z, nr1.y, nr1.w) : make_float4(nr1.y, nr1.w, nr1.x, nr1.z);
+        S.r[(slot * 2 + 0) * FTP_NT + threadIdx.x] = c0;
+        S.r[(slot * 2 + 1) * FTP_NT + threadIdx.x] = c1;
+        S.f[slot * FTP_NT + threadIdx.x] = make_uint2(nf0, nf1);
+        gen = (gen << 1) | ((__any_sync(0xffffffffu, ((nf0 | nf1) & 0x3f3f3f3fu) != 0u) || t == 0 || t == D.nz - 1) ? 1u : 0u);
+        fetch_r(t + 1);
+        S.publish(0, pw, zn, D0);                     // colour 0 of plane t + 1
+        // half-sweeps 1 .. 4 on planes t .. t - 3 (colours 1, 0, 1, 0)
+#pragma unroll
+        for (int k = 0; k <= 3; ++k) {
+            const int p = t - k;
+            if (p >= tlo && p < D.nz) {
+                const int sl = ftp_back(slot, k);
+                const bool g = (gen >> k) & 1u;
+                ftp_sweep<LX, D0>(c, Z[k], Z[k + 1], k ? Z[k > 0 ? k - 1 : 0] : zn, S.below(k, pr), S.above(k, pr),
+                                  S.rhs(sl, 0, (k + 1) & 1), S.rhs(sl, 1, (k + 1) & 1), scale, g,
+                                  S.f + sl * FTP_NT + threadIdx.x, g ? ftp_zadj(D, p) : 0, S.rcp);
+                if (k < 3) S.publish(k + 1, pw, Z[k], D0);
             }
-            if (!mbar_wait(S.bar(ft_slot(P, t)), ft_parity(P, t))) abort_flag = 1;
         }
-        __syncthreads();
-        if (abort_flag) break;
-        const FTRing R(P, t);
-        ft_half_sweep(D, S, P, Q, R, 1, t - 1, 1, 3, scale, 1);
-        __syncthreads();
-        ft_half_sweep(D, S, P, Q, R, 2, t - 2, 0, 2, scale, 2);
-        __syncthreads();
-        ft_half_sweep(D, S, P, Q, R, 3, t - 3, 1, 1, scale, 3);
-        __syncthreads();
-        // last half-sweep on plane t-4 (colour 0, the tile only); each thread then stores its quad and
-        // adds r z of its four cells to the product
-        const int tf = t - 4;
-        // every lane takes part (the half-sweep votes across the warp); with halo 0 only the tile's
-        // cells in the domain change
-        if (tf >= k0 && tf < k1) ft_half_sweep(D, S, P, Q, R, 4, tf, 0, 0, scale, 4);
-        if (tf >= k0 && tf < k1 && Q.tile >= 0 && Q.dom == 0xfu) {
-            const int s = R.sl[4];
-            const float4 z4 = lds4(S.z(s) + Q.c), r4 = lds4(S.r(s) + Q.c);
-            *reinterpret_cast<float4*>(z + Q.gx + (long long)D.sy * Q.gy + D.sz * tf) = z4;
-            part += (r4.x * z4.x + r4.y * z4.y) + (r4.z * z4.z + r4.w * z4.w);
+        const int tf = t - 3;
+        if (tf >= k0 && tf < k1) {
+            const int sl = ftp_back(slot, 3);
+            float* zo = zg + row0 + D.sz * tf;
+            // row 0 of plane t - 3: colour 0 holds the cells D0, D0 + 2; row 1 the others
+            if (c.own0) {
+                *reinterpret_cast<float4*>(zo) = make_float4(Z[3][0][0], Z[3][0][1], Z[3][0][2], Z[3][0][3]);
+                const float2 a = S.rhs(sl, 0, 0), b = S.rhs(sl, 0, 1);
+                part += (a.x * Z[3][0][D0] + a.y * Z[3][0][D0 + 2]) + (b.x * Z[3][0][1 - D0] + b.y * Z[3][0][3 - D0]);
+            }
+            if (c.own1) {
+                *reinterpret_cast<float4*>(zo + D.sy) = make_float4(Z[3][1][0], Z[3][1][1], Z[3][1][2], Z[3][1][3]);
+                const float2 a = S.rhs(sl, 1, 0), b = S.rhs(sl, 1, 1);
+                part += (a.x * Z[3][1][1 - D0] + a.y * Z[3][1][3 - D0]) + (b.x * Z[3][1][D0] + b.y * Z[3][1][D0 + 2]);
+            }
         }
-        fence_proxy_async();
+#pragma unroll
+        for (int q = 4; q > 0; --q) ftp_copy(Z[q], Z[q - 1]);
+        ftp_copy(Z[0], zn);
+        ftp_set(zn, nz0, nz1);
+        fetch_z(t + 3);
+        slot = slot == FTP_RING - 1 ? 0 : slot + 1;
         __syncthreads();
-    }
-    if (abort_flag) {
-        if (threadIdx.x == 0) {
-            for (int u = issued; u > issued - FT_NS && u >= P.tlo; --u) mbar_wait(S.bar(ft_slot(P, u)), ft_parity(P, u));
-            atomicExch(&sc->dev_error, 1);
-        }
-        part = 0.f;
+    };
+    for (int t = tlo; t <= thi; t += 2) {
+        step(std::integral_constant<int, 0>{}, t);
+        step(std::integral_constant<int, 1>{}, t + 1);
     }
     decltype(part) acc[1] = {part};
     grid_reduce<1>(acc, partials, counter, [&](double* tt) {
@@ -1360,66 +1349,34 @@ unsigned lin_blocks(long long n) {
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-// ---- tensor maps of the fused passes -------------------------------------------------------------
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-    });
-    return fn;
-}
-
-// 3-D map of an nx x ny x nz array of `esize`-byte elements, box (boxx, FT_RY, 1): one plane of a
-// tile plus its halo per load.  Elements outside the array read as zero.
-int make_plane_map(CUtensorMap* out, const Dom& D, const void* ptr, CUtensorMapDataType dt, int esize, int boxx) {
-    PFN_cuTensorMapEncodeTiled_v12000 fn = encode_tiled();
-    if (!fn) return ibm_fail(IBM_E_CUDA, "multigrid: cuTensorMapEncodeTiled is not available");
-    alignas(64) CUtensorMap m;
-    cuuint64_t dims[3] = {(cuuint64_t)D.nx, (cuuint64_t)D.ny, (cuuint64_t)D.nz};
-    cuuint64_t strides[2] = {(cuuint64_t)D.nx * esize, (cuuint64_t)D.nx * D.ny * esize};
-    cuuint32_t box[3] = {(cuuint32_t)boxx, (cuuint32_t)FT_RY, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(&m, dt, 3, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return ibm_fail(IBM_E_CUDA, "multigrid: cuTensorMapEncodeTiled failed (%d)", (int)r);
-    memcpy(out, &m, sizeof(m));
-    return IBM_OK;
-}
-
-// Whether the fused passes apply, and their launch shape: tiles of FT_TX x FT_TY and the z-chunk that
-// minimises waves x (chunk + 8 planes of pipeline) with two resident blocks per SM.
+// Whether the fused passes apply, and their launch shape: of the two tile widths (64 x 64 or 128 x 32 cells,
+// halo included) and the z-chunks, the one with the fewest plane steps over all waves (one block per SM; a
+// chunk of k planes takes k + 8 steps).  64 x 64 has the smaller halo, 128 x 32 fits some grids better.
 void fused_plan(const LesCtx& c, MG& mg, int sb) {
     const Dom& D = c.D;
     bool per = false;
     for (int f = 0; f < 6; ++f) per = per || D.bc[f] == IBM_BC_PERIODIC;
-    mg.fused = mg.allow_fused && sb == 4 && mg.sweeps == 2 && mg.nlev > 1 && D.flags != nullptr && !per && D.nx % 16 == 0 &&
-               D.nx >= 16 && D.ny >= 2 && D.nz >= 2 && encode_tiled() != nullptr;
+    mg.fused = mg.allow_fused && sb == 4 && mg.sweeps == 2 && mg.nlev > 1 && !per && D.nx % 4 == 0;
     if (!mg.fused) return;
-    const long long tx = (D.nx + FT_TX - 1) / FT_TX, ty = (D.ny + FT_TY - 1) / FT_TY;
-    const long long slots = 2LL * IBM_NSM;
     long long best = -1;
-    int best_k = D.nz + (D.nz & 1);
-    for (int ch = 1; ch <= 64; ++ch) {
-        int k = (D.nz + ch - 1) / ch;
-        k += k & 1;
-        if (k < 8 && ch > 1) break;
-        const long long nchunk = (D.nz + k - 1) / k;
-        const long long waves = (tx * ty * nchunk + slots - 1) / slots;
-        const long long cost = waves * (k + 8);
-        if (best < 0 || cost < best) {
-            best = cost;
-            best_k = k;
+    for (int lx = 16; lx <= 32; lx *= 2) {
+        const int w = 4 * lx, h = 2 * (FTP_NT / lx);
+        const long long tx = D.nx > w ? (D.nx - 8 + w - 9) / (w - 8) : 1, ty = D.ny > h ? (D.ny - 8 + h - 9) / (h - 8) : 1;
+        for (int ch = 1; ch <= 64; ++ch) {
+            int k = (D.nz + ch - 1) / ch;
+            k += k & 1;
+            if (k < 4 && ch > 1) break;
+            const long long nchunk = (D.nz + k - 1) / k;
+            const long long waves = (tx * ty * nchunk + IBM_NSM - 1) / IBM_NSM;
+            const long long cost = waves * (k + 8);
+            if (best < 0 || cost < best) {
+                best = cost;
+                mg.fz_chunk = k;
+                mg.flx = lx;
+                mg.fgrid = dim3((unsigned)tx, (unsigned)ty, (unsigned)nchunk);
+            }
         }
     }
-    mg.fz_chunk = best_k;
-    mg.fgrid = dim3((unsigned)tx, (unsigned)ty, (unsigned)((D.nz + best_k - 1) / best_k));
-    mg.tm_r_ptr = nullptr;
 }
 
 // ---- host side of the set-up --------------------------------------------------------------------
@@ -1635,22 +1592,14 @@ static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStrea
 
 // V-cycle with the fused fine-grid passes: pre-smoothing + restriction, the coarse levels,
 // prolongation, post-smoothing + (r, z).
-static int vcycle_fused(const LesCtx& c, MG& mg, const float* r, float* z, SolveScal* sc, cudaStream_t s) {
-    if (mg.tm_r_ptr != r) {
-        int rc = make_plane_map(&mg.tm_r, c.D, r, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, FT_RX);
-        if (rc) return rc;
-        mg.tm_r_ptr = r;
-    }
-    alignas(64) CUtensorMap tr, tz, tf;
-    memcpy(&tr, &mg.tm_r, sizeof(tr));
-    memcpy(&tz, &mg.tm_z2, sizeof(tz));
-    memcpy(&tf, &mg.tm_f, sizeof(tf));
+static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z, SolveScal* sc, cudaStream_t s) {
     float* z2 = (float*)mg.z2;
     const float scale = (float)(c.D.dx * c.D.dx);
     const MGLev& L1 = mg.lev[1];
     int launches = 0;
     prof_begin(c.prof, PS_MG_FINE, s);
-    k_mg_pre_fused<<<mg.fgrid, FT_NT, FT_SMEM, s>>>(c.D, z2, scale, L1, mg.fz_chunk, sc, tr, tf);
+    if (mg.flx == 16) k_mg_pre_fused<16><<<mg.fgrid, FTP_NT, FTile<16>::smem(), s>>>(c.D, r, z2, scale, L1, mg.fz_chunk, sc);
+    else k_mg_pre_fused<32><<<mg.fgrid, FTP_NT, FTile<32>::smem(), s>>>(c.D, r, z2, scale, L1, mg.fz_chunk, sc);
     prof_end(c.prof, PS_MG_FINE, s);
     ++launches;
     prof_begin(c.prof, PS_MG_COARSE, s);
@@ -1662,7 +1611,10 @@ static int vcycle_fused(const LesCtx& c, MG& mg, const float* r, float* z, Solve
     prof_end(c.prof, PS_MG_TRANSFER, s);
     ++launches;
     prof_begin(c.prof, PS_MG_FINE, s);
-    k_mg_post_fused<<<mg.fgrid, FT_NT, FT_SMEM, s>>>(c.D, z, scale, mg.fz_chunk, sc, c.partials, c.counter, tr, tz, tf);
+    if (mg.flx == 16)
+        k_mg_post_fused<16><<<mg.fgrid, FTP_NT, FTile<16>::smem(), s>>>(c.D, r, z2, z, scale, mg.fz_chunk, sc, c.partials, c.counter);
+    else
+        k_mg_post_fused<32><<<mg.fgrid, FTP_NT, FTile<32>::smem(), s>>>(c.D, r, z2, z, scale, mg.fz_chunk, sc, c.partials, c.counter);
     prof_end(c.prof, PS_MG_FINE, s);
     ++launches;
     IBM_LAUNCHED("mg_vcycle (fused)");
@@ -1705,11 +1657,11 @@ int mg_setup(const LesCtx& c, MG& mg, int sb) {
     }
     fused_plan(c, mg, sb);
     if (mg.fused) {
-        IBM_CUDA(cudaFuncSetAttribute(k_mg_pre_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, FT_SMEM));
-        IBM_CUDA(cudaFuncSetAttribute(k_mg_post_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, FT_SMEM));
-        if ((rc = make_plane_map(&mg.tm_f, c.D, c.D.flags, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, FT_FX))) return rc;
         MG_ALLOCB(mg.z2, c.D.N * 4);
-        if ((rc = make_plane_map(&mg.tm_z2, c.D, mg.z2, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, FT_RX))) return rc;
+        IBM_CUDA(cudaFuncSetAttribute(k_mg_pre_fused<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<16>::smem()));
+        IBM_CUDA(cudaFuncSetAttribute(k_mg_pre_fused<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<32>::smem()));
+        IBM_CUDA(cudaFuncSetAttribute(k_mg_post_fused<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<16>::smem()));
+        IBM_CUDA(cudaFuncSetAttribute(k_mg_post_fused<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<32>::smem()));
     }
     return IBM_OK;
 }
@@ -1728,7 +1680,7 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
     bool vec = false;
     if constexpr (std::is_same<T, float>::value) vec = x4_ok(c);
     if constexpr (std::is_same<T, float>::value) {
-        if (mg.fused) return vcycle_fused(c, const_cast<MG&>(mg), r, z, sc, s);
+        if (mg.fused) return vcycle_fused(c, mg, r, z, sc, s);
     }
     auto fine = [&](int col, int zero) {
         prof_begin(c.prof, PS_MG_FINE, s);

@@ -111,7 +111,6 @@ __global__ void k_reset(SolveScal* sc) {
     sc->iters = 0;
     sc->nonfinite = 0;
     sc->done = 0;
-    sc->dev_error = 0;
 }
 
 // CG, first half: direction p = r + beta p_old (recomputed where a neighbour needs it, so p never
@@ -593,7 +592,6 @@ int run_poisson(const LesCtx& c, PoissonWork& w, const double* b, double* x, dou
         IBM_COUNT(c, 1);
         if ((rc = read_scalars(w, s))) return rc;
         const SolveScal h = *w.hsc;
-        if (h.dev_error) return ibm_fail(IBM_E_CUDA, "poisson_solve: a multigrid shared-memory load timed out");
         out.bnorm = sqrt(h.bb);
         out.relres = h.bb > 0.0 ? sqrt(h.res2 / h.bb) : 0.0;
         out.iters = h.iters;
