@@ -31,16 +31,16 @@ namespace cg = cooperative_groups;
 namespace {
 
 #define MG_TAIL_CTAS 8          // portable cluster size
-#define MG_TAIL_MAX (1LL << 13) // levels with at most this many unknowns run in the one-launch tail
+#define MG_TAIL_MAX (1LL << 14) // levels with at most this many unknowns run in the one-launch tail
 #define MG_COARSE_TARGET 1024   // coarsening stops at this many unknowns (or one position)
-#define MG_MAXCH 64             // unknowns of a block whose internal links are followed (more: singletons)
-#define MG_MAXE 256             // internal links followed per block
+#define MG_ELL 6                // links of an unknown kept in the padded rows (more: its CSR row)
+#define MG_SMEM_MAX 3500        // unknowns of a coarsest level that is solved in shared memory
 #define MG_MAXL 64              // distinct neighbours of a coarse unknown (more: the level is dropped)
 #define MG_L1L 24               // level 1: a 2x2x2 block has at most 24 links leaving it
 
 struct MGTail {
     MGLev lev[IBM_MG_MAXLEV];
-    int first, nlev, sweeps, coarse_sweeps;
+    int first, nlev, coarse_sweeps;
     double omega;
 };
 
@@ -223,6 +223,13 @@ __device__ __forceinline__ int fine_parts(const Dom& D, const unsigned (&fl)[8],
 #pragma unroll
     for (int m = 0; m < 8; ++m) part[m] = __popc(roots & ((1u << lab[m]) - 1u));
     return __popc(roots);
+}
+
+// Level-1 right-hand side of unknown u, with the first half-sweep of that level from x = 0.
+template <class T>
+__device__ __forceinline__ void put_b1(const MGLev& C, int u, T b) {
+    ((T*)C.b)[u] = b;
+    ((T*)C.x)[u] = -b * (T)C.invdg[u];
 }
 
 // ---- fused fine-grid passes: all four red-black half-sweeps of a smoothing phase in one pass ------
@@ -445,7 +452,6 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
     const FCol c = ftp_column<LX>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
     const int k0 = blockIdx.z * kchunk, k1 = min(D.nz, k0 + kchunk);
     const int tlo = max(0, k0 - 4), thi = k1 + 3;
-    float* __restrict__ b1 = (float*)C1.b;
     const int row0 = c.gx + D.sy * c.gy;
     float Z[6][2][4];
 #pragma unroll
@@ -568,8 +574,8 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
                 const bool odd = D0 == 1;                // both planes of the block are there
                 // a warp without a cut link in the two planes: whole blocks
                 if (!((gen >> 4) & 1u) && !(odd && ((gen >> 5) & 1u))) {
-                    b1[o.x] = odd ? (er[0][0] + er[1][0]) + (res[0][0] + res[1][0]) : er[0][0] + er[1][0];
-                    b1[o.y] = odd ? (er[0][1] + er[1][1]) + (res[0][1] + res[1][1]) : er[0][1] + er[1][1];
+                    put_b1<float>(C1, o.x, odd ? (er[0][0] + er[1][0]) + (res[0][0] + res[1][0]) : er[0][0] + er[1][0]);
+                    put_b1<float>(C1, o.y, odd ? (er[0][1] + er[1][1]) + (res[0][1] + res[1][1]) : er[0][1] + er[1][1]);
                 } else {
                     const long long Pe = row0 + D.sz * (tr & ~1);
                     unsigned fe[2], fo[2];
@@ -600,7 +606,7 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
                         const int oo = h ? o.y : o.x;
 #pragma unroll
                         for (int s2 = 0; s2 < 8; ++s2)
-                            if (s2 < np) b1[oo + s2] = acc[s2];
+                            if (s2 < np) put_b1<float>(C1, oo + s2, acc[s2]);
                     }
                 }
             }
@@ -837,85 +843,68 @@ __global__ void k_links1(Dom D, MGLev L, const uint8_t* __restrict__ sub0, int f
     }
 }
 
-// Children of coarse position Y: the unknowns of the (up to) 8 positions of level F below it, in
-// position order.  Returns how many there are; the first MG_MAXCH go into list.
-__device__ __forceinline__ int block_children(const MGLev& F, const int Y[3], int (&list)[MG_MAXCH]) {
-    int n = 0;
-    for (int m = 0; m < 8; ++m) {
-        const int X[3] = {2 * Y[0] + (m & 1), 2 * Y[1] + ((m >> 1) & 1), 2 * Y[2] + (m >> 2)};
-        if (X[0] >= F.px || X[1] >= F.py || X[2] >= F.pz) continue;
-        const long long q = pos_index(F, X);
-        const int o = F.off[q], c = F.cnt[q];
-        for (int k = 0; k < c; ++k, ++n)
-            if (n < MG_MAXCH) list[n] = o + k;
+// Level l + 1 from level l (= F): the parts of each block of 8 positions are the connected components of its
+// unknowns under the links inside the block.  Lock-free union of every such link over all unknowns at once
+// (the larger root is hung below the smaller, so a component's root is its smallest unknown whatever the
+// order of the threads), however many unknowns a block holds: if some were left out they would become parts
+// of their own, linked inside one position, and the two colours would no longer separate neighbours.
+__device__ __forceinline__ int uf_find(const int* lab, int u) {
+    int p = ((const volatile int*)lab)[u];
+    while (p != u) {
+        u = p;
+        p = ((const volatile int*)lab)[u];
     }
-    return n;
+    return u;
 }
 
-// Level l + 1 from level l (= F): parts of each block of 8 positions.  F.parent[u] receives the part
-// of u within its block (made global by k_parent_next).  Children beyond MG_MAXCH, and internal links
-// beyond MG_MAXE, are not followed: such children stay parts of their own (a finer partition is as
-// valid an aggregation).
-__global__ void k_parts_next(MGLev F, MGLev C) {
+__global__ void k_uf_init(long long n, int* __restrict__ lab, int* __restrict__ num) {
+    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x) {
+        lab[u] = (int)u;
+        num[u] = -1;
+    }
+}
+
+__global__ void k_uf_union(MGLev F, int* lab) {
+    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < F.M; u += (long long)gridDim.x * blockDim.x) {
+        int X[3];
+        coords3(F.pos[u], F.px, F.py, X);
+        for (int e = F.rp[u]; e < F.rp[u + 1]; ++e) {
+            const int w = F.col[e];
+            if (w > u) continue;                           // each link once
+            int Y[3];
+            coords3(F.pos[w], F.px, F.py, Y);
+            if ((Y[0] >> 1) != (X[0] >> 1) || (Y[1] >> 1) != (X[1] >> 1) || (Y[2] >> 1) != (X[2] >> 1)) continue;
+            int a = uf_find(lab, (int)u), b = uf_find(lab, w);
+            while (a != b) {
+                if (a < b) { const int t = a; a = b; b = t; }
+                const int old = atomicCAS(&lab[a], a, b);  // hang root a below b
+                if (old == a) break;
+                a = uf_find(lab, a);
+                b = uf_find(lab, b);
+            }
+        }
+    }
+}
+
+// Numbers the parts of a block in the order in which its unknowns (by position) first meet them;
+// F.parent[u] receives the part of u within its block (made global by k_parent_next).
+__global__ void k_parts_next(MGLev F, MGLev C, const int* __restrict__ lab, int* __restrict__ num) {
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < C.P; q += (long long)gridDim.x * blockDim.x) {
         int Y[3];
         coords3(q, C.px, C.py, Y);
-        int list[MG_MAXCH];
-        const int ntot = block_children(F, Y, list);
-        const int n = ntot < MG_MAXCH ? ntot : MG_MAXCH;
-        uint8_t ea[MG_MAXE], eb[MG_MAXE];
-        int ne = 0;
-        for (int k = 0; k < n; ++k) {
-            const int u = list[k];
-            for (int e = F.rp[u]; e < F.rp[u + 1]; ++e) {
-                const int w = F.col[e];
-                if (w < u) continue;                       // each internal link once
-                int Xw[3];
-                coords3(F.pos[w], F.px, F.py, Xw);
-                if ((Xw[0] >> 1) != Y[0] || (Xw[1] >> 1) != Y[1] || (Xw[2] >> 1) != Y[2]) continue;
-                int kw = -1;
-                for (int t = 0; t < n; ++t)
-                    if (list[t] == w) {
-                        kw = t;
-                        break;
-                    }
-                if (kw < 0 || ne == MG_MAXE) continue;
-                ea[ne] = (uint8_t)k;
-                eb[ne] = (uint8_t)kw;
-                ++ne;
+        int n = 0;
+        for (int m = 0; m < 8; ++m) {
+            const int X[3] = {2 * Y[0] + (m & 1), 2 * Y[1] + ((m >> 1) & 1), 2 * Y[2] + (m >> 2)};
+            if (X[0] >= F.px || X[1] >= F.py || X[2] >= F.pz) continue;
+            const long long qx = pos_index(F, X);
+            for (int u = F.off[qx]; u < F.off[qx] + F.cnt[qx]; ++u) {
+                const int r = uf_find(lab, u);             // a component lies in one block: no other thread
+                int k = num[r];
+                if (k < 0) num[r] = k = n++;
+                F.parent[u] = k;
             }
         }
-        uint8_t lab[MG_MAXCH];
-        for (int k = 0; k < n; ++k) lab[k] = (uint8_t)k;
-        for (int it = 0; it < n; ++it) {
-            bool changed = false;
-            for (int e = 0; e < ne; ++e) {
-                const uint8_t lo = lab[ea[e]] < lab[eb[e]] ? lab[ea[e]] : lab[eb[e]];
-                if (lab[ea[e]] != lo || lab[eb[e]] != lo) {
-                    lab[ea[e]] = lo;
-                    lab[eb[e]] = lo;
-                    changed = true;
-                }
-            }
-            if (!changed) break;
-        }
-        // part numbers: roots in list order, then the children that were not followed
-        int nroot = 0;
-        uint8_t rank[MG_MAXCH];
-        for (int k = 0; k < n; ++k)
-            if (lab[k] == k) rank[k] = (uint8_t)nroot++;
-        for (int k = 0; k < n; ++k) F.parent[list[k]] = rank[lab[k]];
-        if (ntot > n) {
-            int extra = 0;
-            for (int m = 0; m < 8; ++m) {
-                const int X[3] = {2 * Y[0] + (m & 1), 2 * Y[1] + ((m >> 1) & 1), 2 * Y[2] + (m >> 2)};
-                if (X[0] >= F.px || X[1] >= F.py || X[2] >= F.pz) continue;
-                const long long qx = pos_index(F, X);
-                for (int k = 0; k < F.cnt[qx]; ++k, ++extra)
-                    if (extra >= MG_MAXCH) F.parent[F.off[qx] + k] = nroot + (extra - MG_MAXCH);
-            }
-        }
-        C.cnt[q] = nroot + (ntot - n);
+        C.cnt[q] = n;
     }
 }
 
@@ -928,9 +917,8 @@ __global__ void k_parent_next(MGLev F, MGLev C) {
     }
 }
 
-// Level l + 1 links (Galerkin sums) and children lists.  Count pass: rp[v] = distinct neighbours,
-// cp[v] = children, d, pos.  Fill pass: sorted rows, invdg, children.
-__global__ void k_links_next(MGLev F, MGLev C, int fill, int* ovf) {
+// Level l + 1 links (Galerkin sums) and lists of the children: of colour 0, or `all` (see grestrict).  Count pass: rp[v] = distinct neighbours, cp[v] = children, d, pos.  Fill pass: sorted rows, invdg, children.
+__global__ void k_links_next(MGLev F, MGLev C, int fill, int all, int* ovf) {
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < C.P; q += (long long)gridDim.x * blockDim.x) {
         int Y[3];
         coords3(q, C.px, C.py, Y);
@@ -947,8 +935,10 @@ __global__ void k_links_next(MGLev F, MGLev C, int fill, int* ovf) {
                 const long long qx = pos_index(F, X);
                 for (int u = F.off[qx]; u < F.off[qx] + F.cnt[qx]; ++u) {
                     if (F.parent[u] != v) continue;
-                    if (fill) C.ch[C.cp[v] + nch] = u;
-                    ++nch;
+                    if (all || u < F.M0) {
+                        if (fill) C.ch[C.cp[v] + nch] = u;
+                        ++nch;
+                    }
                     dsum += F.d[u];
                     for (int e = F.rp[u]; e < F.rp[u + 1]; ++e) {
                         const int pw = F.parent[F.col[e]];
@@ -1001,58 +991,103 @@ struct ArrEmit {
     __device__ void operator()(long long i, long long o, long long) const { a[i] = (int32_t)o; }
 };
 
-// ---- the V-cycle on the coarse levels -----------------------------------------------------------
-
-// One red-black pass of colour `col` over the unknowns t0, t0 + nt, ... of that colour.  With `zero`
-// the iterate is taken as 0: colour `col` gets -b / dg and the other colour is cleared.
-template <class T>
-__device__ __forceinline__ void gsmooth(const MGLev& L, int col, bool zero, long long t0, long long nt) {
-    const T* __restrict__ b = (const T*)L.b;
-    T* x = (T*)L.x;
-    if (zero) {
-        for (long long u = t0; u < L.M; u += nt) {
-            const bool mine = (u < L.M0) == (col == 0);
-            x[u] = mine ? -b[u] * (T)L.invdg[u] : (T)0;
+// Padded rows of the V-cycle: link e of unknown u at [e M + u], so a warp's rows are read whole; padding has
+// g = 0.  A row with more than MG_ELL links stores -1 as its first column and is read from the CSR arrays.
+__global__ void k_ell(MGLev L) {
+    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < L.M; u += (long long)gridDim.x * blockDim.x) {
+        const int k0 = L.rp[u], n = L.rp[u + 1] - k0;
+        for (int e = 0; e < MG_ELL; ++e) {
+            L.ecol[e * L.M + u] = n > MG_ELL ? -1 : (e < n ? L.col[k0 + e] : (int)u);
+            L.eg[e * L.M + u] = n <= MG_ELL && e < n ? L.g[k0 + e] : 0.f;
         }
-        return;
-    }
-    const long long lo = col ? L.M0 : 0, hi = col ? L.M : L.M0;
-    for (long long u = lo + t0; u < hi; u += nt) {
-        T s = 0;
-        for (int e = L.rp[u]; e < L.rp[u + 1]; ++e) s += (T)L.g[e] * x[L.col[e]];
-        x[u] = (s - b[u]) * (T)L.invdg[u];
     }
 }
 
-// b_C[v] = sum over the children u of v of the level-F residual  b_u - (sum g (x_w - x_u) - d_u x_u).
+// ---- the V-cycle on the coarse levels -----------------------------------------------------------
+//
+// One red-black sweep before and after the coarse correction.  From x = 0 the first colour is x = -b / dg,
+// written with b by whoever forms b; the residual of colour 0 after colour 1 is then  -sum g x_w  and that
+// of colour 1 is zero, so the restriction reads colour 0 only.  After the correction colour 1 reads its
+// neighbours' prolongated values on the fly and colour 0 reads colour 1: neither needs its own old value,
+// so no pass adds the correction.  Four passes per level: colour 1, restriction, colour 1, colour 0.
+
+// sum over the links of u of g f(neighbour).
+template <class T, class Fn>
+__device__ __forceinline__ T row_sum(const MGLev& L, long long u, Fn f) {
+    T s = 0;
+    int c[MG_ELL];
+    float g[MG_ELL];
+#pragma unroll
+    for (int e = 0; e < MG_ELL; ++e) {
+        c[e] = L.ecol[e * L.M + u];
+        g[e] = L.eg[e * L.M + u];
+    }
+    if (c[0] < 0) {
+        for (int e = L.rp[u]; e < L.rp[u + 1]; ++e) s += (T)L.g[e] * f(L.col[e]);
+        return s;
+    }
+#pragma unroll
+    for (int e = 0; e < MG_ELL; ++e)
+        if (g[e] != 0.f) s += (T)g[e] * f(c[e]);
+    return s;
+}
+
+// Colour `col` from its neighbours.
+template <class T>
+__device__ __forceinline__ void gsmooth(const MGLev& L, int col, long long t0, long long nt) {
+    const T* b = (const T*)L.b;
+    T* x = (T*)L.x;
+    const long long lo = col ? L.M0 : 0, hi = col ? L.M : L.M0;
+    for (long long u = lo + t0; u < hi; u += nt)
+        x[u] = (row_sum<T>(L, u, [&](int w) { return x[w]; }) - b[u]) * (T)L.invdg[u];
+}
+
+// Colour 1 after the coarse correction: the neighbours (colour 0) count with x + omega x_C(parent).
+template <class T>
+__device__ __forceinline__ void gup(const MGLev& L, const MGLev& C, T omega, long long t0, long long nt) {
+    const T* b = (const T*)L.b;
+    T* x = (T*)L.x;
+    const T* xc = (const T*)C.x;
+    for (long long u = L.M0 + t0; u < L.M; u += nt)
+        x[u] = (row_sum<T>(L, u, [&](int w) { return x[w] + omega * xc[L.parent[w]]; }) - b[u]) * (T)L.invdg[u];
+}
+
+// b_C[v] = -sum over the children u of v of colour 0 of  sum g x_w; x_C = -b_C / dg.  Four lanes per coarse
+// unknown (a plain 2x2x2 block has four children of each colour).  The thread count is a multiple of 32.
+// FP64: 1 / dg is stored in FP32, so the smoothed residuals vanish to 2^-24 only; they are evaluated in full
+// over all children.
 template <class T>
 __device__ __forceinline__ void grestrict(const MGLev& F, const MGLev& C, long long t0, long long nt) {
-    const T* __restrict__ bf = (const T*)F.b;
-    const T* __restrict__ xf = (const T*)F.x;
-    T* __restrict__ bc = (T*)C.b;
-    for (long long v = t0; v < C.M; v += nt) {
+    const T* xf = (const T*)F.x;
+    T* bc = (T*)C.b;
+    T* xc = (T*)C.x;
+    const int lane = (int)(t0 & 3);
+    const long long rounds = (4 * C.M + nt - 1) / nt;
+    for (long long q = 0; q < rounds; ++q) {
+        const long long v = (t0 + q * nt) >> 2;
         T acc = 0;
-        for (int k = C.cp[v]; k < C.cp[v + 1]; ++k) {
-            const int u = C.ch[k];
-            const T xu = xf[u];
-            T ax = -(T)F.d[u] * xu;
-            for (int e = F.rp[u]; e < F.rp[u + 1]; ++e) ax += (T)F.g[e] * (xf[F.col[e]] - xu);
-            acc += bf[u] - ax;
+        if (v < C.M)
+            for (int k = C.cp[v] + lane; k < C.cp[v + 1]; k += 4) {
+                const int u = C.ch[k];
+                if constexpr (std::is_same<T, double>::value) {
+                    const T xu = xf[u];
+                    acc += ((const T*)F.b)[u] - (row_sum<T>(F, u, [&](int w) { return xf[w] - xu; }) - (T)F.d[u] * xu);
+                } else {
+                    acc -= row_sum<T>(F, u, [&](int w) { return xf[w]; });
+                }
+            }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (v < C.M && lane == 0) {
+            bc[v] = acc;
+            xc[v] = -acc * (T)C.invdg[v];
         }
-        bc[v] = acc;
     }
 }
 
-// x_F[u] += omega x_C[parent of u].
-template <class T>
-__device__ __forceinline__ void gprolong(const MGLev& F, const MGLev& C, T omega, long long t0, long long nt) {
-    T* __restrict__ xf = (T*)F.x;
-    const T* __restrict__ xc = (const T*)C.x;
-    for (long long u = t0; u < F.M; u += nt) xf[u] = xf[u] + omega * xc[F.parent[u]];
-}
-
-// Coarsest level, one block: x = 0, then `sweeps` red-black passes and as many black-red (a
-// symmetric operator).  The iterate stays in global memory; __syncthreads orders the passes.
+// Coarsest level, one block: x = 0, then `sweeps` red-black passes and as many black-red (a symmetric
+// operator), __syncthreads between the passes; in global memory, or (gcoarsest_load first) with the rows, b
+// and x in shared memory: the passes are a chain of 4 * sweeps barriers, each about an L2 round trip otherwise.
 template <class T>
 __device__ __forceinline__ void gcoarsest(const MGLev& L, int sweeps) {
     T* x = (T*)L.x;
@@ -1060,15 +1095,70 @@ __device__ __forceinline__ void gcoarsest(const MGLev& L, int sweeps) {
     __syncthreads();
     for (int pass = 0; pass < 4 * sweeps; ++pass) {
         const int half = pass / (2 * sweeps);
-        gsmooth<T>(L, (pass & 1) ^ half, false, threadIdx.x, blockDim.x);
+        gsmooth<T>(L, (pass & 1) ^ half, threadIdx.x, blockDim.x);
         __syncthreads();
     }
 }
 
 template <class T>
-__global__ void __launch_bounds__(256) k_gsmooth(MGLev L, int col, int zero, const SolveScal* sc) {
+struct CoarseSmem {
+    T *x, *b;
+    float *eg, *invdg;
+    int16_t* ecol;
+    __host__ __device__ static size_t bytes(long long M) { return (size_t)M * (2 * sizeof(T) + MG_ELL * 6 + 4) + 16; }
+    __device__ __forceinline__ CoarseSmem(unsigned char* p, long long M) {
+        x = reinterpret_cast<T*>(p);
+        b = x + M;
+        eg = reinterpret_cast<float*>(b + M);
+        invdg = eg + MG_ELL * M;
+        ecol = reinterpret_cast<int16_t*>(invdg + M);
+    }
+};
+
+template <class T>
+__device__ __forceinline__ void gcoarsest_load(const MGLev& L, CoarseSmem<T>& S) {
+    for (int e = threadIdx.x; e < MG_ELL * (int)L.M; e += blockDim.x) {
+        S.ecol[e] = (int16_t)L.ecol[e];
+        S.eg[e] = L.eg[e];
+    }
+    for (int u = threadIdx.x; u < (int)L.M; u += blockDim.x) S.invdg[u] = L.invdg[u];
+}
+
+template <class T>
+__device__ __forceinline__ void gcoarsest_smem(const MGLev& L, CoarseSmem<T>& S, int sweeps) {
+    const int M = (int)L.M, M0 = (int)L.M0;
+    const T* bg = (const T*)L.b;
+    T* xg = (T*)L.x;
+    for (int u = threadIdx.x; u < M; u += blockDim.x) {
+        S.b[u] = bg[u];
+        S.x[u] = (T)0;
+    }
+    __syncthreads();
+    for (int pass = 0; pass < 4 * sweeps; ++pass) {
+        const int col = (pass & 1) ^ (pass / (2 * sweeps));
+        const int lo = col ? M0 : 0, hi = col ? M : M0;
+        for (int u = lo + threadIdx.x; u < hi; u += blockDim.x) {
+            T s = 0;
+            if (S.ecol[u] < 0) {
+                for (int e = L.rp[u]; e < L.rp[u + 1]; ++e) s += (T)L.g[e] * S.x[L.col[e]];
+            } else {
+#pragma unroll
+                for (int e = 0; e < MG_ELL; ++e) {
+                    const float g = S.eg[e * M + u];
+                    if (g != 0.f) s += (T)g * S.x[S.ecol[e * M + u]];
+                }
+            }
+            S.x[u] = (s - S.b[u]) * (T)S.invdg[u];
+        }
+        __syncthreads();
+    }
+    for (int u = threadIdx.x; u < M; u += blockDim.x) xg[u] = S.x[u];
+}
+
+template <class T>
+__global__ void __launch_bounds__(256) k_gsmooth(MGLev L, int col, const SolveScal* sc) {
     if (sc->done) return;
-    gsmooth<T>(L, col, zero != 0, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
+    gsmooth<T>(L, col, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
 template <class T>
@@ -1078,25 +1168,20 @@ __global__ void __launch_bounds__(256) k_grestrict(MGLev F, MGLev C, const Solve
 }
 
 template <class T>
-__global__ void __launch_bounds__(256) k_gprolong(MGLev F, MGLev C, T omega, const SolveScal* sc) {
+__global__ void __launch_bounds__(256) k_gup(MGLev F, MGLev C, T omega, const SolveScal* sc) {
     if (sc->done) return;
-    gprolong<T>(F, C, omega, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
-}
-
-template <class T>
-__global__ void __launch_bounds__(1024) k_gcoarsest(MGLev L, int sweeps, const SolveScal* sc) {
-    if (sc->done) return;
-    gcoarsest<T>(L, sweeps);
+    gup<T>(F, C, omega, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
 // The small levels first .. nlev-1 of a V-cycle in one launch: one cluster of MG_TAIL_CTAS blocks of
-// 1024 threads walks the descent (smoothing, restriction), the coarsest solve (block 0) and the
-// ascent (prolongation, smoothing), with a cluster barrier (hardware, release/acquire at cluster
-// scope) between dependent passes.  These levels are small and stay in L2; as separate kernels each
-// pass would cost a launch for a few microseconds of work.
+// 1024 threads walks the descent (smoothing, restriction), the coarsest solve (block 0, in shared memory
+// where it fits, its rows loaded before the descent) and the ascent, with a cluster barrier (hardware,
+// release/acquire at cluster scope) between dependent passes.  These levels stay in L2; as separate kernels
+// each pass would cost a launch for a few microseconds of work.
 template <class T>
 __global__ void __launch_bounds__(1024) k_mg_tail(MGTail M, const SolveScal* sc) {
     if (sc->done) return;                       // the flag is uniform: set by an earlier kernel
+    extern __shared__ __align__(16) unsigned char tail_smem[];
     cg::cluster_group cl = cg::this_cluster();
     const long long t0 = (long long)cl.block_rank() * blockDim.x + threadIdx.x;
     const long long nt = (long long)cl.num_blocks() * blockDim.x;
@@ -1105,38 +1190,36 @@ __global__ void __launch_bounds__(1024) k_mg_tail(MGTail M, const SolveScal* sc)
         cl.sync();
     };
     const int last = M.nlev - 1;
+    const bool insm = M.lev[last].M <= MG_SMEM_MAX;
+    CoarseSmem<T> S(tail_smem, M.lev[last].M);
+    if (insm && cl.block_rank() == 0) gcoarsest_load<T>(M.lev[last], S);
     for (int l = M.first; l < last; ++l) {
-        for (int q = 0; q < M.sweeps; ++q) {
-            gsmooth<T>(M.lev[l], 0, q == 0, t0, nt);
-            bar();
-            gsmooth<T>(M.lev[l], 1, false, t0, nt);
-            bar();
-        }
+        gsmooth<T>(M.lev[l], 1, t0, nt);
+        bar();
         grestrict<T>(M.lev[l], M.lev[l + 1], t0, nt);
         bar();
     }
-    if (cl.block_rank() == 0) gcoarsest<T>(M.lev[last], M.coarse_sweeps);
+    if (cl.block_rank() == 0) {
+        if (insm) gcoarsest_smem<T>(M.lev[last], S, M.coarse_sweeps);
+        else gcoarsest<T>(M.lev[last], M.coarse_sweeps);
+    }
     bar();
     for (int l = last - 1; l >= M.first; --l) {
-        gprolong<T>(M.lev[l], M.lev[l + 1], (T)M.omega, t0, nt);
+        gup<T>(M.lev[l], M.lev[l + 1], (T)M.omega, t0, nt);
         bar();
-        for (int q = 0; q < M.sweeps; ++q) {
-            gsmooth<T>(M.lev[l], 1, false, t0, nt);
-            bar();
-            gsmooth<T>(M.lev[l], 0, false, t0, nt);
-            bar();
-        }
+        gsmooth<T>(M.lev[l], 0, t0, nt);
+        if (l > M.first) bar();
     }
 }
 
 // ---- transfer between the fine grid and level 1 -------------------------------------------------
 
-// b_1 of each part of a level-1 block = the sum of the fine residuals  scale r - (A z)  of its cells.
+// b_1 of each part of a level-1 block = the sum of the fine residuals  scale r - (A z)  of its cells, and the
+// first half-sweep of level 1, x_1 = -b_1 / dg.
 template <class T>
 __global__ void __launch_bounds__(256) k_mg_restrict0(Dom D, const T* __restrict__ r, const T* __restrict__ z, T scale,
                                                       MGLev C, const SolveScal* sc) {
     if (sc->done) return;
-    T* __restrict__ bc = (T*)C.b;
     auto zv = [&](long long c) { return z[c]; };
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < C.P; q += (long long)gridDim.x * blockDim.x) {
         int X[3];
@@ -1158,7 +1241,7 @@ __global__ void __launch_bounds__(256) k_mg_restrict0(Dom D, const T* __restrict
         const int o = C.off[q];
 #pragma unroll
         for (int s = 0; s < 8; ++s)
-            if (s < np) bc[o + s] = acc[s];
+            if (s < np) put_b1<T>(C, o + s, acc[s]);
     }
 }
 
@@ -1203,7 +1286,6 @@ __global__ void __launch_bounds__(256) k_mg_restrict0_x4(Dom D, const float* __r
                                                          const float* __restrict__ z, float scale, MGLev C,
                                                          const SolveScal* sc) {
     if (sc->done) return;
-    float* __restrict__ bc = (float*)C.b;
     const int px = D.nx / 4;
     const long long npairs = (long long)px * C.py * C.pz;
     auto zv = [&](long long c) { return z[c]; };
@@ -1272,7 +1354,7 @@ __global__ void __launch_bounds__(256) k_mg_restrict0_x4(Dom D, const float* __r
             const int o = C.off[(2 * xp + h) + (long long)C.px * (Y + (long long)C.py * Z)];
 #pragma unroll
             for (int s = 0; s < 8; ++s)
-                if (s < np) bc[o + s] = acc[s];
+                if (s < np) put_b1<float>(C, o + s, acc[s]);
         }
     }
 }
@@ -1386,7 +1468,11 @@ struct SetupTmp {
     long long nt = 0;
     int* ovf = nullptr;
     uint8_t* sub0 = nullptr;
+    int* lab = nullptr;             // union-find labels and part numbers of a level's unknowns
+    int* num = nullptr;
     ~SetupTmp() {
+        cudaFree(lab);
+        cudaFree(num);
         cudaFree(tiles);
         cudaFree(ovf);
         cudaFree(sub0);
@@ -1395,7 +1481,7 @@ struct SetupTmp {
 
 void free_level(MGLev& L) {
     cudaFree(L.off); cudaFree(L.cnt); cudaFree(L.pos); cudaFree(L.rp); cudaFree(L.col); cudaFree(L.g);
-    cudaFree(L.d); cudaFree(L.invdg); cudaFree(L.parent); cudaFree(L.cp); cudaFree(L.ch); cudaFree(L.b);
+    cudaFree(L.ecol); cudaFree(L.eg); cudaFree(L.d); cudaFree(L.invdg); cudaFree(L.parent); cudaFree(L.cp); cudaFree(L.ch); cudaFree(L.b);
     cudaFree(L.x);
     const int px = L.px, py = L.py, pz = L.pz;
     const long long P = L.P;
@@ -1444,6 +1530,14 @@ int scan_in_place(int32_t* a, long long n, SetupTmp& t, long long* total) {
     return IBM_OK;
 }
 
+int build_ell(MGLev& L) {
+    MG_ALLOC(L.ecol, MG_ELL * L.M);
+    MG_ALLOC(L.eg, MG_ELL * L.M);
+    k_ell<<<lin_blocks(L.M), 256>>>(L);
+    IBM_LAUNCHED("k_ell");
+    return IBM_OK;
+}
+
 int build_level1(const LesCtx& c, MGLev& L, int sb, SetupTmp& t) {
     const Dom& D = c.D;
     L.px = (D.nx + 1) / 2;
@@ -1475,7 +1569,9 @@ int build_level1(const LesCtx& c, MGLev& L, int sb, SetupTmp& t) {
     int h = 0;
     IBM_CUDA(cudaMemcpy(&h, t.ovf, sizeof(int), cudaMemcpyDeviceToHost));
     if (h) return ibm_fail(IBM_E_INVALID, "multigrid set-up: a level-1 block has too many links");
-    return IBM_OK;
+    MG_ALLOC(t.lab, L.M);           // the largest level: reused by the others
+    MG_ALLOC(t.num, L.M);
+    return build_ell(L);
 }
 
 // Level C from level F; returns 1 (and leaves C empty) when the level would not shrink enough or
@@ -1487,7 +1583,9 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
     C.P = (long long)C.px * C.py * C.pz;
     MG_ALLOC(C.off, C.P);
     MG_ALLOC(C.cnt, C.P);
-    k_parts_next<<<lin_blocks(C.P), 256>>>(F, C);
+    k_uf_init<<<lin_blocks(F.M), 256>>>(F.M, t.lab, t.num);
+    k_uf_union<<<lin_blocks(F.M), 256>>>(F, t.lab);
+    k_parts_next<<<lin_blocks(C.P), 256>>>(F, C, t.lab, t.num);
     IBM_LAUNCHED("k_parts_next");
     int rc = number_unknowns(C, t);
     if (rc) return -rc;
@@ -1500,14 +1598,16 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
     MG_ALLOC(C.pos, C.M);
     MG_ALLOC(C.rp, C.M + 1);
     MG_ALLOC(C.cp, C.M + 1);
-    MG_ALLOC(C.ch, F.M);
+    const int all = sb == 8;
+    const long long nchild = all ? F.M : F.M0;
+    MG_ALLOC(C.ch, nchild);
     MG_ALLOC(C.d, C.M);
     MG_ALLOC(C.invdg, C.M);
     MG_ALLOC(C.parent, C.M);
     MG_ALLOCB(C.b, C.M * sb);
     MG_ALLOCB(C.x, C.M * sb);
     IBM_CUDA(cudaMemset(t.ovf, 0, sizeof(int)));
-    k_links_next<<<lin_blocks(C.P), 256>>>(F, C, 0, t.ovf);
+    k_links_next<<<lin_blocks(C.P), 256>>>(F, C, 0, all, t.ovf);
     IBM_LAUNCHED("k_links_next");
     IBM_CUDA(cudaDeviceSynchronize());
     int h = 0;
@@ -1519,73 +1619,61 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
     long long nch = 0;
     if ((rc = scan_in_place(C.rp, C.M, t, &C.nnz))) return -rc;
     if ((rc = scan_in_place(C.cp, C.M, t, &nch))) return -rc;
-    if (nch != F.M) return -ibm_fail(IBM_E_INVALID, "multigrid set-up: children do not cover the level");
+    if (nch != nchild) return -ibm_fail(IBM_E_INVALID, "multigrid set-up: children do not cover the level");
     MG_ALLOC(C.col, C.nnz);
     MG_ALLOC(C.g, C.nnz);
-    k_links_next<<<lin_blocks(C.P), 256>>>(F, C, 1, t.ovf);
+    k_links_next<<<lin_blocks(C.P), 256>>>(F, C, 1, all, t.ovf);
     IBM_LAUNCHED("k_links_next");
+    if ((rc = build_ell(C))) return -rc;
     IBM_CUDA(cudaDeviceSynchronize());
     return 0;
 }
 
 }  // namespace
 
-// Coarse levels of a V-cycle (level 1 holds the restricted residual; on return level 1 holds the
-// coarse correction): descent, coarsest solve and ascent, as separate kernels on the large levels
-// and one cluster launch for the small ones.
+// Coarse levels of a V-cycle (level 1 holds the restricted residual and its first half-sweep; on return level 1
+// holds the coarse correction): descent, coarsest solve and ascent, as separate kernels on the large levels
+// and one cluster launch for the small ones (and always for the coarsest).
 template <class T>
 static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStream_t s, int& launches) {
     const T om = (T)mg.omega;
-    const int SC = mg.sweeps > 0 ? 1 : 0;
-    int tf = mg.nlev;
-    for (int l = 1; l + 1 < mg.nlev; ++l)
+    const int last = mg.nlev - 1;
+    int tf = last;
+    for (int l = 1; l < last; ++l)
         if (mg.lev[l].M <= MG_TAIL_MAX) { tf = l; break; }
-    const int top = tf < mg.nlev ? tf : mg.nlev - 1;
-    for (int l = 1; l < top; ++l) {
+    for (int l = 1; l < tf; ++l) {
         const MGLev& L = mg.lev[l];
-        for (int q = 0; q < SC; ++q) {
-            k_gsmooth<T><<<lin_blocks(q == 0 ? L.M : L.M0), 256, 0, s>>>(L, 0, q == 0, sc);
-            k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, 0, sc);
-            launches += 2;
-        }
-        k_grestrict<T><<<lin_blocks(mg.lev[l + 1].M), 256, 0, s>>>(L, mg.lev[l + 1], sc);
-        ++launches;
+        k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, sc);
+        k_grestrict<T><<<lin_blocks(4 * mg.lev[l + 1].M), 256, 0, s>>>(L, mg.lev[l + 1], sc);
+        launches += 2;
     }
-    if (tf < mg.nlev) {
+    {
         MGTail M;
         for (int l = 0; l < IBM_MG_MAXLEV; ++l) M.lev[l] = mg.lev[l];
         M.first = tf;
         M.nlev = mg.nlev;
-        M.sweeps = SC;
         M.coarse_sweeps = mg.coarse_sweeps;
         M.omega = mg.omega;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(MG_TAIL_CTAS);
+        cfg.gridDim = dim3(tf < last ? MG_TAIL_CTAS : 1);
         cfg.blockDim = dim3(1024);
-        cfg.dynamicSmemBytes = 0;
+        cfg.dynamicSmemBytes = mg.lev[last].M <= MG_SMEM_MAX ? CoarseSmem<T>::bytes(mg.lev[last].M) : 0;
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = MG_TAIL_CTAS;
+        at[0].val.clusterDim.x = cfg.gridDim.x;
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
         IBM_CUDA(cudaLaunchKernelEx(&cfg, k_mg_tail<T>, M, (const SolveScal*)sc));
         ++launches;
-    } else {
-        k_gcoarsest<T><<<1, 1024, 0, s>>>(mg.lev[mg.nlev - 1], mg.coarse_sweeps, sc);
-        ++launches;
     }
-    for (int l = top - 1; l >= 1; --l) {
+    for (int l = tf - 1; l >= 1; --l) {
         const MGLev& L = mg.lev[l];
-        k_gprolong<T><<<lin_blocks(L.M), 256, 0, s>>>(L, mg.lev[l + 1], om, sc);
-        ++launches;
-        for (int q = 0; q < SC; ++q) {
-            k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, 0, sc);
-            k_gsmooth<T><<<lin_blocks(L.M0), 256, 0, s>>>(L, 0, 0, sc);
-            launches += 2;
-        }
+        k_gup<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, mg.lev[l + 1], om, sc);
+        k_gsmooth<T><<<lin_blocks(L.M0), 256, 0, s>>>(L, 0, sc);
+        launches += 2;
     }
     return IBM_OK;
 }
@@ -1655,6 +1743,8 @@ int mg_setup(const LesCtx& c, MG& mg, int sb) {
         if (r2 > 0) break;
         mg.nlev = l + 2;
     }
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CoarseSmem<float>::bytes(MG_SMEM_MAX)));
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CoarseSmem<double>::bytes(MG_SMEM_MAX)));
     fused_plan(c, mg, sb);
     if (mg.fused) {
         MG_ALLOCB(mg.z2, c.D.N * 4);
@@ -1672,9 +1762,6 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
     const T scale = (T)(c.D.dx * c.D.dx);
     const T om = (T)mg.omega;
     const int S = mg.sweeps;
-    // one sweep before and after on the coarse levels: measured faster overall on the dirty sphere than
-    // S there too (a few more outer iterations, much less coarse-level work)
-    const int SC = S > 0 ? 1 : 0;
     const CellGrid& g = c.cg;
     int launches = 0;
     bool vec = false;
@@ -1709,57 +1796,8 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
         prof_end(c.prof, PS_MG_TRANSFER, s);
         ++launches;
         prof_begin(c.prof, PS_MG_COARSE, s);
-        // levels >= tf (if any) run in one cluster launch; separate kernels above them
-        int tf = mg.nlev;
-        for (int l = 1; l + 1 < mg.nlev; ++l)
-            if (mg.lev[l].M <= MG_TAIL_MAX) { tf = l; break; }
-        const int top = tf < mg.nlev ? tf : mg.nlev - 1;
-        for (int l = 1; l < top; ++l) {
-            const MGLev& L = mg.lev[l];
-            for (int q = 0; q < SC; ++q) {
-                k_gsmooth<T><<<lin_blocks(q == 0 ? L.M : L.M0), 256, 0, s>>>(L, 0, q == 0, sc);
-                k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, 0, sc);
-                launches += 2;
-            }
-            k_grestrict<T><<<lin_blocks(mg.lev[l + 1].M), 256, 0, s>>>(L, mg.lev[l + 1], sc);
-            ++launches;
-        }
-        if (tf < mg.nlev) {
-            MGTail M;
-            for (int l = 0; l < IBM_MG_MAXLEV; ++l) M.lev[l] = mg.lev[l];
-            M.first = tf;
-            M.nlev = mg.nlev;
-            M.sweeps = SC;
-            M.coarse_sweeps = mg.coarse_sweeps;
-            M.omega = mg.omega;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(MG_TAIL_CTAS);
-            cfg.blockDim = dim3(1024);
-            cfg.dynamicSmemBytes = 0;
-            cfg.stream = s;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = MG_TAIL_CTAS;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            IBM_CUDA(cudaLaunchKernelEx(&cfg, k_mg_tail<T>, M, (const SolveScal*)sc));
-            ++launches;
-        } else {
-            k_gcoarsest<T><<<1, 1024, 0, s>>>(mg.lev[mg.nlev - 1], mg.coarse_sweeps, sc);
-            ++launches;
-        }
-        for (int l = top - 1; l >= 1; --l) {
-            const MGLev& L = mg.lev[l];
-            k_gprolong<T><<<lin_blocks(L.M), 256, 0, s>>>(L, mg.lev[l + 1], om, sc);
-            ++launches;
-            for (int q = 0; q < SC; ++q) {
-                k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, 0, sc);
-                k_gsmooth<T><<<lin_blocks(L.M0), 256, 0, s>>>(L, 0, 0, sc);
-                launches += 2;
-            }
-        }
+        int rc = coarse_levels<T>(c, mg, sc, s, launches);
+        if (rc) return rc;
         prof_end(c.prof, PS_MG_COARSE, s);
         prof_begin(c.prof, PS_MG_TRANSFER, s);
         if constexpr (std::is_same<T, float>::value) {

@@ -47,11 +47,13 @@ struct MGLev {
     int32_t* rp;         // [M + 1] first link of each unknown
     int32_t* col;        // [nnz] neighbour unknown
     float* g;            // [nnz] conductance: sum of the fine conductances between the two aggregates
+    int32_t* ecol;       // padded rows read by the V-cycle (mg.cu), column-major
+    float* eg;
     float* d;            // [M] Dirichlet (outflow) diagonal term
     float* invdg;        // [M] 1 / (sum of g + d), 0 for an isolated unknown
     int32_t* parent;     // [M] unknown of level l + 1 that contains this one
-    int32_t* cp;         // [M + 1] first child (levels >= 2: children are unknowns of level l - 1)
-    int32_t* ch;         // [M of level l - 1] children, grouped by parent
+    int32_t* cp;         // [M + 1] first child (levels >= 2: unknowns of level l - 1, in FP32 those of colour 0)
+    int32_t* ch;         // children, grouped by parent
     void* b;             // right-hand side (working precision)
     void* x;             // iterate
 };
