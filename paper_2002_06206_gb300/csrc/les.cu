@@ -6,6 +6,8 @@
 // Cell kernels use a 32 x 8 thread tile over (x, y) so that consecutive threads touch consecutive
 // cells (coalesced rows); the momentum flux walks z-marching tiles staged in shared memory, with the
 // cells next to cut links in a separate general kernel.
+#include <type_traits>
+
 #include "solver.cuh"
 
 #ifndef IBM_FLUX_GEN_MINB
@@ -119,31 +121,38 @@ __device__ __forceinline__ bool fast_cell(const Dom& D, long long P, int i, int 
     return (m & 63u) == 0u;
 }
 
-// Fast cells run in z-marching tiles: a block of 32 x 8 threads owns an (x, y) tile and walks FT_KZ
-// planes; u (three components) and nu_t of the planes k-2 .. k+2 over the tile plus a two-cell halo
-// sit in a five-plane ring in shared memory, so every neighbour read of the flux is a shared-memory
-// load at a fixed offset.  Halo positions across a periodic seam hold the wrapped cell; one cell
-// beyond a non-periodic domain face they hold the boundary ghost of vel_across (a function of the
-// cell across that face alone), so cells on the domain faces are fast too.  Links through a domain
-// face take the boundary forms of flux_general (near-cell nu_t and cross derivative, central advected
-// value).  Cells that are not fast_cell are skipped (the general kernel takes them).
+// Fast cells run in z-marching tiles: a block of 32 x 8 threads owns an (x, y) tile and walks D.tile_z planes.  u (three components) and nu_t of the planes k-1 .. k+2 over the tile plus a two-cell halo sit in a
+// ring in shared memory; a thread holds its own column in registers.  Halo positions across a periodic
+// seam hold the wrapped cell; one cell beyond a non-periodic domain face they hold the boundary ghost of
+// vel_across (a function of the cell across that face alone), so cells on the domain faces are fast too.
+// A domain face takes the near cell's nu_t and cross derivative and the central advected value: weights
+// (0, 2) or (2, 0) in place of (1, 1) and no QUICK share, so every face runs the same instructions.  Cells
+// that are not fast_cell are skipped (the general kernel takes them).
 //
 // The flux form is conservative: the face between L and R = L + e_a gives L the term Phi and R the
 // term -Phi, so the march evaluates every face once.  Each thread takes its cell's -x, -y and +z
 // faces (two warps add the tile's last x column and y row); the x and y faces meet in shared memory,
 // the z face stays in registers for the next plane.  A plane's sums run one step later, so a single
 // barrier per plane orders both the face buffers (two of them, by plane parity) and the ring.
+//
+// Bound by instruction issue.  Per face and component: the advected value is c0 (u_L + u_R) + kq (3 (u_L +
+// u_R + u_up) - u_far), the scale factors of the differences are taken out of the components, addresses are a
+// block-uniform plane plus a fixed thread offset.  512x256x256 FP32, Crank-Nicolson operator: 660 us (530
+// thread instructions per cell, 2.6 per cycle and SM; its 41 bytes per cell would take 205 us), 1540 us with
+// per-component face forms, 64-bit face indexes and velocities loaded where they are used.  Two rows per
+// thread (455 instructions, 16 resident warps) and four blocks per SM (64 registers) measured 660 and 694 us.
+// FP64: 212 us at 128x64x64, three quarters of the FP64 rate for its 160 operations per cell.
 #define FT_X 32
 #define FT_Y 8
 #define FT_H 2
 #define FT_SX (FT_X + 2 * FT_H)
-#define FT_SY (FT_Y + 2 * FT_H)
-#define FT_PL (FT_SX * FT_SY)
 #define FT_NV 4
-#define FT_KZ 16
-#define FT_RING 6
-#define FT_FXN (FT_Y * (FT_X + 1))   // x faces of a tile plane, per component
-#define FT_FYN ((FT_Y + 1) * FT_X)   // y faces
+#define FT_RING 5
+#define FT_SY (FT_Y + 2 * FT_H)
+#define FT_PL (FT_SX * FT_SY)          // halo-tile positions of a plane
+#define FT_NT (FT_X * FT_Y)
+#define FT_FXN (FT_Y * (FT_X + 1))     // x faces of a tile plane, per component
+#define FT_FYN ((FT_Y + 1) * FT_X)     // y faces
 
 // Domain-boundary ghost of component c across face (a, s) of the cell holding v (vel_across's rules).
 template <class T>
@@ -156,177 +165,256 @@ __device__ __forceinline__ T bc_ghost(const Dom& D, int a, int s, int c, T v) {
     }
 }
 
+// Coefficients of the faces of one axis at one place.
+template <class T>
+struct FaceW {
+    T wl, wr;      // weights of the two cells in the cross derivatives (sum 2)
+    T c0, kq;      // central and QUICK coefficients of the advected value
+};
+
+template <class T>
+struct FaceK {
+    T c0, kq;              // interior faces
+    T nui, h, e;           // nu / dx, 1 / (2 dx), 1 / (8 dx)
+};
+
+template <class T>
+__device__ __forceinline__ FaceW<T> face_w(const FaceK<T>& K, bool dlo, bool dhi) {
+    FaceW<T> w;
+    w.wl = dlo ? (T)0 : (dhi ? (T)2 : (T)1);
+    w.wr = dlo ? (T)2 : (dhi ? (T)0 : (T)1);
+    w.c0 = dlo || dhi ? (T)0.5 : K.c0;
+    w.kq = dlo || dhi ? (T)0 : K.kq;
+    return w;
+}
+
 // Phi of the face between L = R - e_A and R, per component: the term of L's flux sum (R takes -Phi).
-// S[d] is ring plane k + d - 2; R sits at in-plane ring index c0 of plane k + ZR and at global (g0, g1,
-// g2), g_A = 0 .. n_A naming the face.  A face on a non-periodic domain side (R or L outside) takes the
-// boundary forms of the cell inside.  Positions outside the domain give unused values (U reads 0).
-template <class T, int A, int ZR>
-__device__ __forceinline__ void ft_face(const Dom& D, const FaceLayout& F, const T* __restrict__ U,
-                                        const T* const (&S)[5], int c0, int g0, int g1, int g2, T nu, T gam,
-                                        T inv2dx, T invdx, T (&phi)[3]) {
-    constexpr int EX = A == 0, EY = A == 1, EZ = A == 2;
-    // variable v at R + (dx, dy, dz)
-    auto V = [&](int v, int dx, int dy, int dz) -> T { return S[ZR + 2 + dz][v * FT_PL + c0 + dy * FT_SX + dx]; };
-    const int g[3] = {g0, g1, g2}, n[3] = {D.nx, D.ny, D.nz};
-    const bool per = D.bc[2 * A] == IBM_BC_PERIODIC;
-    const bool dlo = !per && g[A] == 0, dhi = !per && g[A] == n[A];
-    bool valid = g[A] >= 0 && g[A] <= n[A];
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-        if (b != A) valid = valid && g[b] >= 0 && g[b] < n[b];
-    const T Uf = valid ? U[F.index(A, g0, g1, g2)] : (T)0;
-    const T nutL = V(3, -EX, -EY, -EZ), nutR = V(3, 0, 0, 0);
-    const T nutf = dlo ? nutR : (dhi ? nutL : (T)0.5 * (nutL + nutR));
-    const T nuf = nu + nutf;
-    const bool quick = gam != (T)0 && !dlo && !dhi;
+// far: the cell beyond the upwind one; d0, d1: wl dL + wr dR of the undivided central differences of u_A along
+// the other two axes (in axis order); nn: nu_t of both cells, summed (a ghost holds the near cell's); Uf: the
+// face velocity.
+template <class T, int A>
+__device__ __forceinline__ void face_phi(const FaceW<T>& w, const FaceK<T>& K, T Uf, const T (&l)[3], const T (&r)[3],
+                                         const T (&far)[3], T d0, T d1, T nn, T (&phi)[3]) {
+    const T a = K.nui + K.h * nn, x = K.e * nn, aa = a + K.h * nn;
+    const T uc = Uf * w.c0, uq = Uf * w.kq;
+    const bool up = Uf >= (T)0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const T uL = V(c, -EX, -EY, -EZ), uR = V(c, 0, 0, 0);
-        const T D1 = (uR - uL) * invdx;
-        T Tt = D1;
-        if (c != A) {
-            // d u_A / d x_c at L and at R (central)
-            const int cx = c == 0, cy = c == 1, cz = c == 2;
-            const T gL = (V(A, cx - EX, cy - EY, cz - EZ) - V(A, -cx - EX, -cy - EY, -cz - EZ)) * inv2dx;
-            const T gR = (V(A, cx, cy, cz) - V(A, -cx, -cy, -cz)) * inv2dx;
-            Tt = dlo ? gR : (dhi ? gL : (T)0.5 * (gL + gR));
-        }
-        T adv = (T)0.5 * (uL + uR);
-        if (quick) {
-            // far upwind: L - e_A for U >= 0, R + e_A otherwise
-            const bool up = Uf >= (T)0;
-            const T far = up ? V(c, -2 * EX, -2 * EY, -2 * EZ) : V(c, EX, EY, EZ);
-            const T q = up ? ((T)6 * uL + (T)3 * uR - far) / (T)8 : ((T)6 * uR + (T)3 * uL - far) / (T)8;
-            adv = ((T)1 - gam) * adv + gam * q;
-        }
-        phi[c] = -Uf * adv + nuf * D1 + nutf * Tt;
+        const T s = l[c] + r[c];
+        const T q = (T)3 * (s + (up ? l[c] : r[c])) - far[c];
+        T v = (c == A ? aa : a) * (r[c] - l[c]) - uc * s;
+        v -= uq * q;
+        if (c != A) v += x * (c == (A == 0 ? 1 : 0) ? d0 : d1);
+        phi[c] = v;
     }
 }
 
+// The x (A = 0) or y (A = 1) face between ring position q - e_A and q of plane k.  S0: plane k, Sm, Sp: its
+// neighbours; r: u at q; dz: undivided z difference of u_A at q.
+template <class T, int A>
+__device__ __forceinline__ void face_inplane(const FaceW<T>& w, const FaceK<T>& K, T Uf, const T* S0, const T* Sm,
+                                             const T* Sp, int q, const T (&r)[3], T nr, T dz, T (&phi)[3]) {
+    constexpr int E = A == 0 ? 1 : FT_SX, B = A == 0 ? FT_SX : 1;
+    T l[3], far[3];
+    const T* sf = S0 + q + (Uf >= (T)0 ? -2 * E : E);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        l[c] = S0[c * FT_PL + q - E];
+        far[c] = sf[c * FT_PL];
+    }
+    const T* s = S0 + A * FT_PL + q;
+    const T db = w.wl * (s[B - E] - s[-B - E]) + w.wr * (s[B] - s[-B]);
+    const T dzs = w.wl * (Sp[A * FT_PL + q - E] - Sm[A * FT_PL + q - E]) + w.wr * dz;
+    face_phi<T, A>(w, K, Uf, l, r, far, db, dzs, S0[3 * FT_PL + q - E] + nr, phi);
+}
+
+// base is the same for the whole block, the byte offset within a plane fixed per thread (a plane has less
+// than 2^31/3 cells: 32 bits for FP32): one add per access.
+template <class T>
+using Off = std::conditional_t<sizeof(T) == 4, unsigned, unsigned long long>;
+
+template <class T>
+__device__ __forceinline__ T at_off(const T* base, Off<T> off) {
+    return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
+}
+
+template <class T>
+__device__ __forceinline__ void to_off(T* base, Off<T> off, T v) {
+    *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off) = v;
+}
+
+// Calls epi(plane, off, h, u, w) for the fast cells: the cell is plane + off / sizeof(T), plane uniform; w holds
+// the three values of `wv` at the cell (loaded a step ahead; unset where wv is null).
 template <class T, class Epi>
 __device__ __forceinline__ void fast_tile_march(const Dom& D, const FaceLayout& F, const T* __restrict__ u,
                                                 const T* __restrict__ U, const T* __restrict__ nut, T nu, T gam,
-                                                Epi epi) {
+                                                const T* wv, Epi epi) {
     extern __shared__ __align__(16) unsigned char ft_raw[];
     T* sm = reinterpret_cast<T*>(ft_raw);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + FT_X * ty;
-    const T inv2dx = (T)0.5 * dom_idx<T>(D), invdx = dom_idx<T>(D);
-    auto slot = [](int kk) { return ((kk % FT_RING) + FT_RING) % FT_RING; };
+    const T invdx = dom_idx<T>(D);
+    FaceK<T> K;
+    K.c0 = (T)0.5 * ((T)1 - gam);
+    K.kq = gam * (T)0.125;
+    K.nui = nu * invdx;
+    K.h = (T)0.5 * invdx;
+    K.e = (T)0.125 * invdx;
     const int n[3] = {D.nx, D.ny, D.nz};
-    const int gx = (D.nx + FT_X - 1) / FT_X, gy = (D.ny + FT_Y - 1) / FT_Y, gz = (D.nz + FT_KZ - 1) / FT_KZ;
+    const unsigned gx = (D.nx + FT_X - 1) / FT_X, gy = (D.ny + FT_Y - 1) / FT_Y, gz = (D.nz + D.tile_z - 1) / D.tile_z;
     const long long items = (long long)gx * gy * gz;
-    // the planes' values a thread stages: FT_PL <= 2 * 256 halo-tile positions per plane
+    // the planes' values a thread stages: two halo-tile positions (the second only where it exists), where they
+    // are read from (byte offset within a plane: the wrapped cell across a periodic seam, the cell at the
+    // face beyond a domain face) and what becomes of them: 0 as read, 1 + face: the ghost beyond that face, 7:
+    // zero (corners and second ghost layers, which no fast cell reads)
     T pf[2][FT_NV];
     int x0 = 0, y0 = 0;
-    // the thread's halo-tile positions (fixed) and whether the tile's halo box lies inside the domain
-    // in x and y (then a plane inside the domain needs no boundary logic)
-    const int ex0 = tid % FT_SX - FT_H, ey0 = tid / FT_SX - FT_H;
-    const int ex1 = (tid + FT_X * FT_Y) % FT_SX - FT_H, ey1 = (tid + FT_X * FT_Y) / FT_SX - FT_H;
-    bool inner = false;
-    auto fetch = [&](int kk) {
-        if (inner && kk >= 0 && kk < D.nz) {
-            const long long base = x0 + (long long)D.sy * y0 + D.sz * kk;
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                const int e = tid + t * (FT_X * FT_Y);
-                pf[t][0] = pf[t][1] = pf[t][2] = pf[t][3] = (T)0;
-                if (e >= FT_PL) continue;
-                const long long c = base + (t ? ex1 : ex0) + (long long)D.sy * (t ? ey1 : ey0);
-                pf[t][0] = u[c];
-                pf[t][1] = u[D.N + c];
-                pf[t][2] = u[2 * D.N + c];
-                pf[t][3] = nut[c];
-            }
-            return;
+    Off<T> eo[2];
+    unsigned kind = 0;
+    const bool has1 = tid + FT_NT < FT_PL;
+    // domain position along axis a of a coordinate beyond it
+    auto beyond = [&](int a, int& g) -> unsigned {
+        if (g >= 0 && g < n[a]) return 0u;
+        if (D.bc[2 * a] == IBM_BC_PERIODIC) {
+            g = ((g % n[a]) + n[a]) % n[a];
+            return 0u;
         }
+        const unsigned k = g == -1 ? 1u + 2 * a : (g == n[a] ? 2u + 2 * a : 7u);
+        g = g < 0 ? 0 : n[a] - 1;
+        return k;
+    };
+    auto places = [&]() {
+        kind = 0;
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-            const int e = tid + t * (FT_X * FT_Y);
-            pf[t][0] = pf[t][1] = pf[t][2] = pf[t][3] = (T)0;
-            if (e >= FT_PL) continue;
-            int g[3] = {x0 + e % FT_SX - FT_H, y0 + e / FT_SX - FT_H, kk};
-            int out = 0, oa = 0, os = 0, depth = 0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (g[a] >= 0 && g[a] < n[a]) continue;
-                if (D.bc[2 * a] == IBM_BC_PERIODIC) {
-                    g[a] = ((g[a] % n[a]) + n[a]) % n[a];
-                    continue;
-                }
-                ++out;
-                oa = a;
-                os = g[a] < 0 ? -1 : 1;
-                depth = g[a] < 0 ? -g[a] : g[a] - n[a] + 1;
-                g[a] = g[a] < 0 ? 0 : n[a] - 1;
-            }
-            // corners and second ghost layers are never read by a fast cell
-            if (out > 1 || depth > 1 || g[0] < 0 || g[0] >= n[0] || g[1] < 0 || g[1] >= n[1] || g[2] < 0 ||
-                g[2] >= n[2])
-                continue;
-            const long long c = g[0] + (long long)D.sy * g[1] + D.sz * g[2];
-            T v0 = u[c], v1 = u[D.N + c], v2 = u[2 * D.N + c];
-            if (out) {
-                v0 = bc_ghost(D, oa, os, 0, v0);
-                v1 = bc_ghost(D, oa, os, 1, v1);
-                v2 = bc_ghost(D, oa, os, 2, v2);
-            }
-            pf[t][0] = v0;
-            pf[t][1] = v1;
-            pf[t][2] = v2;
-            pf[t][3] = nut[c];
+            const int e = tid + t * FT_NT;
+            int i = x0 + e % FT_SX - FT_H, j = y0 + e / FT_SX - FT_H;
+            const unsigned kx = beyond(0, i), ky = beyond(1, j);
+            kind |= (kx && ky ? 7u : kx | ky) << (4 * t);
+            eo[t] = ((Off<T>)i + (Off<T>)D.sy * j) * sizeof(T);
         }
     };
-    auto commit = [&](int kk) {
-        T* dst = sm + slot(kk) * (FT_NV * FT_PL);
+    auto fetch = [&](int kk) {
+        const unsigned kz = beyond(2, kk);
+        const long long base = D.sz * kk;
+        const T *b0 = u + base, *b1 = b0 + D.N, *b2 = b1 + D.N, *b3 = nut + base;
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-            const int e = tid + t * (FT_X * FT_Y);
-            if (e >= FT_PL) continue;
+            if (t == 1 && !has1) break;
+            pf[t][0] = at_off(b0, eo[t]);
+            pf[t][1] = at_off(b1, eo[t]);
+            pf[t][2] = at_off(b2, eo[t]);
+            pf[t][3] = at_off(b3, eo[t]);
+        }
+        if (kind | kz) {
 #pragma unroll
-            for (int v = 0; v < FT_NV; ++v) dst[v * FT_PL + e] = pf[t][v];
+            for (int t = 0; t < 2; ++t) {
+                const unsigned kt = (kind >> (4 * t)) & 7u;
+                const unsigned k = kt && kz ? 7u : kt | kz;
+                if (k == 0u) continue;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) pf[t][c] = k == 7u ? (T)0 : bc_ghost(D, (int)(k - 1) >> 1, (k & 1u) ? -1 : 1, c, pf[t][c]);
+                if (k == 7u) pf[t][3] = (T)0;
+            }
+        }
+    };
+    auto commit = [&](T* dst) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            if (t == 1 && !has1) break;
+#pragma unroll
+            for (int v = 0; v < FT_NV; ++v) dst[v * FT_PL + tid + t * FT_NT] = pf[t][v];
         }
     };
     const int cidx = (ty + FT_H) * FT_SX + (tx + FT_H);
-    T* const fxs = sm + FT_RING * FT_NV * FT_PL;     // [parity][component][FT_Y][FT_X + 1]
-    T* const fys = fxs + 2 * 3 * FT_FXN;               // [parity][component][FT_Y + 1][FT_X]
+    T* const fxs = sm + FT_RING * FT_NV * FT_PL;                // [parity][component][FT_Y][FT_X + 1]
+    T* const fys = fxs + 2 * 3 * FT_FXN;                        // [parity][component][FT_Y + 1][FT_X]
+    const bool per0 = D.bc[0] == IBM_BC_PERIODIC, per1 = D.bc[2] == IBM_BC_PERIODIC, per2 = D.bc[4] == IBM_BC_PERIODIC;
+    const long long sUx = (long long)F.dim[0][0] * F.dim[0][1], sUy = (long long)F.dim[1][0] * F.dim[1][1];
+    const Off<T> row = (Off<T>)D.sy, rowx = (Off<T>)F.dim[0][0];
     for (long long item = blockIdx.x; item < items; item += gridDim.x) {
-        x0 = (int)(item % gx) * FT_X;
-        y0 = (int)((item / gx) % gy) * FT_Y;
-        inner = x0 >= FT_H && x0 + FT_X + FT_H <= D.nx && y0 >= FT_H && y0 + FT_Y + FT_H <= D.ny;
-        const int z0 = (int)(item / ((long long)gx * gy)) * FT_KZ;
-        const int z1 = z0 + FT_KZ < D.nz ? z0 + FT_KZ : D.nz;
-        for (int kk = z0 - 2; kk <= z0 + 2; ++kk) {
-            fetch(kk);
-            commit(kk);
+        // tiles of a grid of < 2^31 cells; a row of tiles starts one further along than the last, so that a
+        // block does not come back to the same (slower) tiles at the domain faces
+        const unsigned it = (unsigned)item, itx = it / gx;
+        x0 = (int)((it + itx) % gx) * FT_X;
+        y0 = (int)(itx % gy) * FT_Y;
+        places();
+        const int z0 = (int)(itx / gy) * D.tile_z;
+        const int z1 = min(z0 + D.tile_z, D.nz);
+        // ring planes of step k: k - 2 (then k + 3), k - 1, k, k + 1, k + 2
+        T *Sa = sm, *Sm = sm + FT_NV * FT_PL, *S0 = sm + 2 * FT_NV * FT_PL, *Sp = sm + 3 * FT_NV * FT_PL, *Sq = sm + 4 * FT_NV * FT_PL;
+        for (int q = 0; q < 5; ++q) {
+            fetch(z0 - 2 + q);
+            commit(sm + q * (FT_NV * FT_PL));
         }
         if (z0 + 3 <= z1 + 1) fetch(z0 + 3);
         __syncthreads();
+        // faces of the thread: -x and -y of its cell (also of the first cell beyond the domain), +z; and the
+        // face of the tile's last row (warp 0) or column (warp 1) it adds
         const int i = x0 + tx, j = y0 + ty;
-        const bool inxy = i < D.nx && j < D.ny;
-        // the cell of the plane whose sums are pending: fast, index, u; its -z and +z faces
-        bool pf_fast = false;
-        long long pP = 0;
-        T pu[3] = {0, 0, 0}, zlo[3] = {0, 0, 0}, zhi[3] = {0, 0, 0};
-        int s0 = slot(z0 - 2);          // ring slot of plane k - 2, advanced with k (no division per cell)
-        for (int k = z0; k <= z1; ++k, s0 = s0 + 1 == FT_RING ? 0 : s0 + 1) {
+        const bool in = i < D.nx && j < D.ny;
+        const FaceW<T> wx = face_w(K, !per0 && i == 0, !per0 && i == D.nx), wy = face_w(K, !per1 && j == 0, !per1 && j == D.ny);
+        // byte offsets from the tile's origin of a plane; places outside the domain read the origin (unused)
+        const Off<T> oP = in ? (tx + row * ty) * sizeof(T) : 0;
+        const Off<T> oUx = i <= D.nx && j < D.ny ? (tx + rowx * ty) * sizeof(T) : 0;
+        const Off<T> oUy = i < D.nx && j <= D.ny ? (tx + row * ty) * sizeof(T) : 0;
+        const bool exrow = ty == 0, excol = ty == 1 && tx < FT_Y;
+        const int ei = x0 + FT_X, ej = exrow ? y0 + FT_Y : y0 + tx;
+        const bool exin = exrow ? (i < D.nx && ej <= D.ny) : (excol && ei <= D.nx && ej < D.ny);
+        const FaceW<T> we = exrow ? face_w(K, false, !per1 && ej == D.ny) : face_w(K, false, !per0 && ei == D.nx);
+        const int eidx = exrow ? (FT_Y + FT_H) * FT_SX + tx + FT_H : (tx + FT_H) * FT_SX + FT_X + FT_H;
+        const Off<T> oUe = exin ? (exrow ? tx + row * FT_Y : FT_X + rowx * tx) * sizeof(T) : 0;
+        const T* Ux = U + F.index(0, x0, y0, z0);
+        const T* Uy = U + F.index(1, x0, y0, z0);
+        const T* Uz = U + F.index(2, x0, y0, z0);
+        long long P = x0 + (long long)D.sy * y0 + D.sz * z0;
+        // the thread's column: u of the planes k - 1 .. k + 1, nu_t of k, undivided in-plane differences of
+        // u_z on plane k
+        T um[3], uc[3], up[3], zlo[3], zhi[3] = {0, 0, 0}, nc, ex, ey;
+        {
+            const FaceW<T> wz = face_w(K, !per2 && z0 == 0, false);
+            T far[3];
+            const T Uf = at_off(Uz, oP);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                um[c] = Sm[c * FT_PL + cidx];
+                uc[c] = S0[c * FT_PL + cidx];
+                up[c] = Sp[c * FT_PL + cidx];
+                far[c] = Uf >= (T)0 ? Sa[c * FT_PL + cidx] : up[c];
+            }
+            nc = S0[3 * FT_PL + cidx];
+            const T *m = Sm + 2 * FT_PL + cidx, *o = S0 + 2 * FT_PL + cidx;
+            ex = o[1] - o[-1];
+            ey = o[FT_SX] - o[-FT_SX];
+            face_phi<T, 2>(wz, K, Uf, um, uc, far, wz.wl * (m[1] - m[-1]) + wz.wr * ex,
+                           wz.wl * (m[FT_SX] - m[-FT_SX]) + wz.wr * ey, Sm[3 * FT_PL + cidx] + nc, zlo);
+        }
+        // face velocities of the step's faces, loaded a step ahead
+        T Ufx, Ufy, Ufz, Ufe;
+        auto faces = [&]() {
+            Ufx = at_off(Ux, oUx);
+            Ufy = at_off(Uy, oUy);
+            Ufz = at_off(Uz + D.sz, oP);
+            Ufe = at_off(exrow ? Uy : Ux, oUe);
+            Ux += sUx;
+            Uy += sUy;
+            Uz += D.sz;
+        };
+        faces();
+        __syncthreads();                // the ring slot of plane z0 - 2 is free
+        bool fast = false;
+        T wq[3] = {};
+        for (int k = z0; k <= z1; ++k, P += D.sz) {
             // plane k + 3, fetched into registers during the previous step, goes into the ring slot that
-            // plane k - 3 left (the previous barrier ended every read of it); then plane k + 4 is fetched,
+            // plane k - 2 left (the previous barrier ended every read of it); then plane k + 4 is fetched,
             // so each load has a whole step and a barrier to land.  The barrier at the end of the step
             // publishes plane k + 3.
             if (k < z1 && k + 3 <= z1 + 1) {
-                T* dst = sm + (s0 == 0 ? FT_RING - 1 : s0 - 1) * (FT_NV * FT_PL);   // slot of k - 3 = s0 - 1
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    const int e = tid + t * (FT_X * FT_Y);
-                    if (e >= FT_PL) continue;
-#pragma unroll
-                    for (int v = 0; v < FT_NV; ++v) dst[v * FT_PL + e] = pf[t][v];
-                }
+                commit(Sa);
                 if (k + 4 <= z1 + 1) fetch(k + 4);
             }
             if (k > z0) {
                 // sums of plane k - 1, whose faces the previous step wrote
-                if (pf_fast) {
+                if (fast) {
                     const int pb = (k - 1) & 1;
                     const T* fx = fxs + pb * 3 * FT_FXN + ty * (FT_X + 1) + tx;
                     const T* fy = fys + pb * 3 * FT_FYN + ty * FT_X + tx;
@@ -335,48 +423,73 @@ __device__ __forceinline__ void fast_tile_march(const Dom& D, const FaceLayout& 
                     for (int c = 0; c < 3; ++c)
                         h[c] = ((fx[c * FT_FXN + 1] - fx[c * FT_FXN]) + (fy[c * FT_FYN + FT_X] - fy[c * FT_FYN]) +
                                 (zhi[c] - zlo[c])) * invdx;
-                    epi(pP, h, pu);
+                    epi(P - D.sz, oP, h, um, wq);
                 }
 #pragma unroll
                 for (int c = 0; c < 3; ++c) zlo[c] = zhi[c];
             }
             if (k == z1) break;
-            const T* S[5];
-#pragma unroll
-            for (int d = 0; d < 5; ++d) {
-                const int sd = s0 + d;
-                S[d] = sm + (sd >= FT_RING ? sd - FT_RING : sd) * (FT_NV * FT_PL);
-            }
-            const long long P = i + (long long)D.sy * j + D.sz * k;
-            pf_fast = inxy && (D.fast ? D.fast[P] != 0 : fast_cell(D, P, i, j, k));
-            pP = P;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) pu[c] = S[2][c * FT_PL + cidx];
-            if (k == z0) ft_face<T, 2, 0>(D, F, U, S, cidx, i, j, k, nu, gam, inv2dx, invdx, zlo);
-            ft_face<T, 2, 1>(D, F, U, S, cidx, i, j, k + 1, nu, gam, inv2dx, invdx, zhi);
+            fast = in && (D.fast ? D.fast[P + oP / sizeof(T)] != 0 : fast_cell(D, P + oP / sizeof(T), i, j, k));
             const int b = k & 1;
-            T* fx = fxs + b * 3 * FT_FXN;
-            T* fy = fys + b * 3 * FT_FYN;
+            T* fx = fxs + b * 3 * FT_FXN + ty * (FT_X + 1) + tx;
+            T* fy = fys + b * 3 * FT_FYN + ty * FT_X + tx;
             T ph[3];
-            ft_face<T, 0, 0>(D, F, U, S, cidx, i, j, k, nu, gam, inv2dx, invdx, ph);
+            face_inplane<T, 0>(wx, K, Ufx, S0, Sm, Sp, cidx, uc, nc, up[0] - um[0], ph);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) fx[c * FT_FXN + ty * (FT_X + 1) + tx] = ph[c];
-            ft_face<T, 1, 0>(D, F, U, S, cidx, i, j, k, nu, gam, inv2dx, invdx, ph);
+            for (int c = 0; c < 3; ++c) fx[c * FT_FXN] = ph[c];
+            face_inplane<T, 1>(wy, K, Ufy, S0, Sm, Sp, cidx, uc, nc, up[1] - um[1], ph);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) fy[c * FT_FYN + ty * FT_X + tx] = ph[c];
-            if (ty == 0) {
-                // the +y faces of the tile's last row
-                ft_face<T, 1, 0>(D, F, U, S, (FT_Y + FT_H) * FT_SX + tx + FT_H, i, y0 + FT_Y, k, nu, gam, inv2dx,
-                                 invdx, ph);
+            for (int c = 0; c < 3; ++c) fy[c * FT_FYN] = ph[c];
+            {
+                // the +z face
+                const FaceW<T> wz = face_w(K, false, !per2 && k + 1 == D.nz);
+                T uq[3], far[3];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) fy[c * FT_FYN + FT_Y * FT_X + tx] = ph[c];
-            } else if (ty == 1 && tx < FT_Y) {
-                // the +x faces of the tile's last column (row tx)
-                ft_face<T, 0, 0>(D, F, U, S, (tx + FT_H) * FT_SX + FT_X + FT_H, x0 + FT_X, y0 + tx, k, nu, gam,
-                                 inv2dx, invdx, ph);
+                for (int c = 0; c < 3; ++c) {
+                    uq[c] = Sq[c * FT_PL + cidx];
+                    far[c] = Ufz >= (T)0 ? um[c] : uq[c];
+                }
+                const T np = Sp[3 * FT_PL + cidx];
+                const T* o = Sp + 2 * FT_PL + cidx;
+                const T nx_ = o[1] - o[-1], ny_ = o[FT_SX] - o[-FT_SX];
+                face_phi<T, 2>(wz, K, Ufz, uc, up, far, wz.wl * ex + wz.wr * nx_, wz.wl * ey + wz.wr * ny_, nc + np, zhi);
+                ex = nx_;
+                ey = ny_;
+                nc = np;
 #pragma unroll
-                for (int c = 0; c < 3; ++c) fx[c * FT_FXN + tx * (FT_X + 1) + FT_X] = ph[c];
+                for (int c = 0; c < 3; ++c) {
+                    um[c] = uc[c];
+                    uc[c] = up[c];
+                    up[c] = uq[c];
+                }
             }
+            if (ty < 2) {
+                // the +y faces of the tile's last row (ty = 0), the +x faces of its last column (ty = 1, row tx)
+                T r[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) r[c] = S0[c * FT_PL + eidx];
+                if (exrow) {
+                    face_inplane<T, 1>(we, K, Ufe, S0, Sm, Sp, eidx, r, S0[3 * FT_PL + eidx], Sp[FT_PL + eidx] - Sm[FT_PL + eidx], ph);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) fy[c * FT_FYN + FT_Y * FT_X] = ph[c];
+                } else if (excol) {
+                    face_inplane<T, 0>(we, K, Ufe, S0, Sm, Sp, eidx, r, S0[3 * FT_PL + eidx], Sp[eidx] - Sm[eidx], ph);
+                    T* fe = fxs + b * 3 * FT_FXN + tx * (FT_X + 1) + FT_X;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) fe[c * FT_FXN] = ph[c];
+                }
+            }
+            if (k + 1 < z1) faces();
+            if (wv) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) wq[c] = at_off(wv + c * D.N + P, oP);
+            }
+            T* const t = Sa;
+            Sa = Sm;
+            Sm = S0;
+            S0 = Sp;
+            Sp = Sq;
+            Sq = t;
             __syncthreads();
         }
     }
@@ -461,21 +574,24 @@ __device__ __forceinline__ void for_general_cells(const Dom& D, const int32_t* _
     }
 }
 
-// Runs epi(P, h, u_P) over the kernel's cells: z-marching shared-memory tiles of fast cells, or the
+// Runs epi(plane, off, h, u, w) over the kernel's cells (cell = plane + off / sizeof(T), w = wv there): z-marching shared-memory tiles of fast cells, or the
 // general list.
 template <bool GENERAL, class T, class Epi>
 __device__ __forceinline__ void flux_cells(const Dom& D, const FaceLayout& F, const T* __restrict__ u,
                                            const T* __restrict__ U, const T* __restrict__ nut, T nu, T gam,
-                                           const int32_t* __restrict__ list, long long nlist, Epi epi) {
+                                           const int32_t* __restrict__ list, long long nlist, const T* wv, Epi epi) {
     if constexpr (GENERAL) {
         for_general_cells(D, list, nlist, [&](long long P, int i, int j, int k) {
             T h[3];
             flux_general(D, F, u, U, nut, P, i, j, k, nu, gam, h);
             const T uc[3] = {u[P], u[D.N + P], u[2 * D.N + P]};
-            epi(P, h, uc);
+            T wq[3] = {};
+            if (wv)
+                for (int c = 0; c < 3; ++c) wq[c] = wv[c * D.N + P];
+            epi(P, 0, h, uc, wq);
         });
     } else {
-        fast_tile_march<T>(D, F, u, U, nut, nu, gam, epi);
+        fast_tile_march<T>(D, F, u, U, nut, nu, gam, wv, epi);
     }
 }
 
@@ -491,14 +607,15 @@ __global__ void __launch_bounds__(256, (FluxOcc<T, GENERAL>::value)) k_predict(D
                                                  const T* __restrict__ nut, const T* Hprev, T* H,
                                                  T* __restrict__ ustar, T nu, T dt, int first, T gam,
                                                  const int32_t* __restrict__ list, long long nlist) {
-    flux_cells<GENERAL, T>(D, F, u, U, nut, nu, gam, list, nlist, [&](long long P, const T (&h)[3], const T (&uc)[3]) {
+    flux_cells<GENERAL, T>(D, F, u, U, nut, nu, gam, list, nlist, first ? nullptr : Hprev,
+                           [&](long long P, Off<T> o, const T (&h)[3], const T (&uc)[3], const T (&w)[3]) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const long long oc = c * D.N + P;
             const T hc = h[c];
-            const T hp = first ? (T)0 : Hprev[oc];
-            H[oc] = hc;
-            ustar[oc] = first ? uc[c] + dt * hc : uc[c] + dt * ((T)1.5 * hc - (T)0.5 * hp);
+            const T hp = first ? (T)0 : w[c];
+            to_off(H + oc, o, hc);
+            to_off(ustar + oc, o, first ? uc[c] + dt * hc : uc[c] + dt * ((T)1.5 * hc - (T)0.5 * hp));
         }
     });
 }
@@ -959,15 +1076,16 @@ __global__ void __launch_bounds__(256, (FluxOcc<T, GENERAL>::value)) k_cn_begin(
                                                   int maxit, int keepx, SolveScal* sc, double* partials, unsigned* counter,
                                                   const int32_t* __restrict__ list, long long nlist) {
     T a0 = 0;
-    flux_cells<GENERAL, T>(D, F, u, U, nut, nu, gam, list, nlist, [&](long long P, const T (&h)[3], const T (&uc)[3]) {
+    flux_cells<GENERAL, T>(D, F, u, U, nut, nu, gam, list, nlist, (const T*)nullptr,
+                           [&](long long P, Off<T> o, const T (&h)[3], const T (&)[3], const T (&)[3]) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const long long q = c * D.N + P;
             const T b = dt * h[c];
-            H[q] = h[c];
-            r[q] = b;
-            rh[q] = b;
-            if (!keepx) x[q] = (T)0;
+            to_off(H + q, o, h[c]);
+            to_off(r + q, o, b);
+            to_off(rh + q, o, b);
+            if (!keepx) to_off(x + q, o, (T)0);
             a0 += b * b;
         }
     });
@@ -1008,30 +1126,31 @@ __global__ void k_cn_p(long long n, const T* __restrict__ r, T* __restrict__ p, 
 // y = M xin = xin - (dt/2) L_0(xin).  mode 0: (w, y) -> alpha = rho / (r_hat, v).  mode 1 (xin = s):
 // (y, s), (y, y) -> omega.  mode 2 (warm start, xin = the previous increment): r = b - M xin with b
 // read from and r written to r2, r_hat = r in y, (r, r) -> rr = rho.
-template <class T, bool GENERAL>
+template <class T, bool GENERAL, int mode>
 __global__ void __launch_bounds__(256, (FluxOcc<T, GENERAL>::value)) k_cn_apply(Dom D, FaceLayout F, const T* __restrict__ xin,
                                                   const T* __restrict__ U, const T* __restrict__ nut,
                                                   T* __restrict__ y, const T* __restrict__ w, T* r2, T nu, T gam,
-                                                  T hdt, int mode, SolveScal* sc, double* partials,
+                                                  T hdt, SolveScal* sc, double* partials,
                                                   unsigned* counter, const int32_t* __restrict__ list, long long nlist) {
     if (sc->done) return;
     T a0 = 0, a1 = 0;
-    flux_cells<GENERAL, T>(D, F, xin, U, nut, nu, gam, list, nlist, [&](long long P, const T (&h)[3], const T (&uc)[3]) {
+    flux_cells<GENERAL, T>(D, F, xin, U, nut, nu, gam, list, nlist, mode == 0 ? w : (mode == 2 ? (const T*)r2 : nullptr),
+                           [&](long long P, Off<T> o, const T (&h)[3], const T (&uc)[3], const T (&wq)[3]) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const long long q = c * D.N + P;
             const T xv = uc[c];
             const T yv = xv - hdt * h[c];
             if (mode == 2) {
-                const T rn = r2[q] - yv;
-                r2[q] = rn;
-                y[q] = rn;
+                const T rn = wq[c] - yv;
+                to_off(r2 + q, o, rn);
+                to_off(y + q, o, rn);
                 a0 += rn * rn;
                 continue;
             }
-            y[q] = yv;
+            to_off(y + q, o, yv);
             if (mode == 0) {
-                a0 += w[q] * yv;
+                a0 += wq[c] * yv;
             } else {
                 a0 += yv * xv;
                 a1 += yv * yv;
@@ -1123,9 +1242,29 @@ int g_tile_blocks[2] = {2 * IBM_NSM, 2 * IBM_NSM};   // FP32, FP64
 template <class T>
 dim3 tile_grid(const LesCtx& c) {
     const long long items = (long long)((c.D.nx + FT_X - 1) / FT_X) * ((c.D.ny + FT_Y - 1) / FT_Y) *
-                            ((c.D.nz + FT_KZ - 1) / FT_KZ);
+                            ((c.D.nz + c.D.tile_z - 1) / c.D.tile_z);
     const long long cap = g_tile_blocks[sizeof(T) == 8];
     return dim3((unsigned)(items < cap ? items : cap));
+}
+
+// Planes per tile of the march: the fewest plane steps over all rounds of the persistent blocks (a tile of
+// k planes takes about k + 4: five are staged before its first).
+template <class T>
+int tile_planes(const Dom& D) {
+    const long long xy = (long long)((D.nx + FT_X - 1) / FT_X) * ((D.ny + FT_Y - 1) / FT_Y);
+    const long long cap = g_tile_blocks[sizeof(T) == 8];
+    long long best = -1;
+    int best_k = D.nz;
+    for (int ch = 1; ch <= D.nz; ++ch) {
+        const int k = (D.nz + ch - 1) / ch;
+        if ((k < 4 || k > 64) && ch > 1 && best >= 0) { if (k < 4) break; else continue; }
+        const long long cost = ((xy * ((D.nz + k - 1) / k) + cap - 1) / cap) * (k + 4);
+        if (best < 0 || cost < best || best_k > 64) {
+            best = cost;
+            best_k = k;
+        }
+    }
+    return best_k;
 }
 
 template <class T>
@@ -1148,25 +1287,26 @@ int predict_cn_t(const LesCtx& c, const T* u, const T* U, const T* nut, T* H, T*
     prof_end(c.prof, PS_PREDICT, s);
     IBM_LAUNCHED("k_cn_begin");
     IBM_COUNT(c, 2);
-    auto apply = [&](const T* in, T* out, int mode) {
+    auto apply = [&](const T* in, T* out, auto m) {
+        constexpr int mode = decltype(m)::value;
         const T* wv = mode == 2 ? nullptr : rh;
         T* r2 = mode == 2 ? r : nullptr;
-        k_cn_apply<T, false><<<tile_grid<T>(c), dim3(FT_X, FT_Y), fast_tile_smem<T>(), s>>>(Dh, c.F, in, U, nut, out, wv, r2, nu, gam, hdt, mode, w.sc,
-                                                            c.partials, c.counter, nullptr, 0);
-        k_cn_apply<T, true><<<ngen, 256, 0, s>>>(Dh, c.F, in, U, nut, out, wv, r2, nu, gam, hdt, mode, w.sc, c.partials,
-                                                 c.counter, c.general, c.n_general);
+        k_cn_apply<T, false, mode><<<tile_grid<T>(c), dim3(FT_X, FT_Y), fast_tile_smem<T>(), s>>>(
+            Dh, c.F, in, U, nut, out, wv, r2, nu, gam, hdt, w.sc, c.partials, c.counter, nullptr, 0);
+        k_cn_apply<T, true, mode><<<ngen, 256, 0, s>>>(Dh, c.F, in, U, nut, out, wv, r2, nu, gam, hdt, w.sc, c.partials,
+                                                       c.counter, c.general, c.n_general);
     };
     if (keepx) {
-        apply(x, rh, 2);
+        apply(x, rh, std::integral_constant<int, 2>{});
         IBM_COUNT(c, 2);
     }
     for (;;) {
         prof_begin(c.prof, PS_MOMENTUM, s);
         for (int it = 0; it < 4; ++it) {
             k_cn_p<T><<<nbv, 256, 0, s>>>(n3, r, p, v, w.sc);
-            apply(p, v, 0);
+            apply(p, v, std::integral_constant<int, 0>{});
             k_cn_s<T><<<nbv, 256, 0, s>>>(n3, r, v, sv, w.sc);
-            apply(sv, tv, 1);
+            apply(sv, tv, std::integral_constant<int, 1>{});
             k_cn_xr<T><<<nbv, 256, 0, s>>>(n3, p, sv, tv, rh, x, r, w.sc, c.partials, c.counter);
         }
         prof_end(c.prof, PS_MOMENTUM, s);
@@ -1241,16 +1381,20 @@ int flux_kernels_setup() {
     const int bytes = (int)fast_tile_smem<double>(), bytesf = (int)fast_tile_smem<float>();
     IBM_CUDA(cudaFuncSetAttribute(k_predict<false, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     IBM_CUDA(cudaFuncSetAttribute(k_cn_begin<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<double, false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<double, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<double, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     IBM_CUDA(cudaFuncSetAttribute(k_predict<false, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytesf));
     IBM_CUDA(cudaFuncSetAttribute(k_cn_begin<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytesf));
-    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytesf));
+    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<float, false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytesf));
+    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<float, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytesf));
+    IBM_CUDA(cudaFuncSetAttribute(k_cn_apply<float, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytesf));
     int dev = 0, nsm = IBM_NSM, bf = 0, bd = 0;
     IBM_CUDA(cudaGetDevice(&dev));
     IBM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    IBM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_cn_apply<float, false>, FT_X * FT_Y,
+    IBM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_cn_apply<float, false, 0>, FT_NT,
                                                            fast_tile_smem<float>()));
-    IBM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bd, k_cn_apply<double, false>, FT_X * FT_Y,
+    IBM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bd, k_cn_apply<double, false, 0>, FT_NT,
                                                            fast_tile_smem<double>()));
     g_tile_blocks[0] = (bf > 0 ? bf : 1) * nsm;
     g_tile_blocks[1] = (bd > 0 ? bd : 1) * nsm;
@@ -1282,6 +1426,7 @@ int build_general_list(LesCtx& c, cudaStream_t s) {
     if (e != cudaSuccess) return ibm_cuda_check(e, "momentum flux: general-cell list");
     c.n_general = (long long)total;
     c.D.fast = c.fastmask;
+    c.D.tile_z = c.prec == IBM_FP64 ? tile_planes<double>(c.D) : tile_planes<float>(c.D);
     return IBM_OK;
 }
 
