@@ -17,19 +17,6 @@ constexpr unsigned long long kEmpty = 0xffffffffffffffffULL;
 
 struct Tri { double v[3][3]; };
 
-__device__ __forceinline__ bool load_tri(const float* __restrict__ t, Tri& T) {
-    bool ok = true;
-#pragma unroll
-    for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            double x = (double)t[3 * p + d];
-            T.v[p][d] = x;
-            ok = ok && isfinite(x);
-        }
-    return ok;
-}
-
 __device__ __forceinline__ long long clamp_line(double v, long long n) {
     if (!(v > -1.0)) return -1;
     if (v > (double)n) return n;
@@ -43,15 +30,6 @@ __device__ __forceinline__ void line_range(double mn, double mx, long long n, lo
     lo = l < 0.0 ? 0 : clamp_line(l, n);
     hi = clamp_line(h, n);
     if (hi > n - 1) hi = n - 1;
-}
-
-__device__ __forceinline__ void tri_lines(const Tri& T, int a, const long long n[3], long long& jb0,
-                                          long long& jb1, long long& jc0, long long& jc1) {
-    const int b = (a + 1) % 3, c = (a + 2) % 3;
-    line_range(fmin(fmin(T.v[0][b], T.v[1][b]), T.v[2][b]), fmax(fmax(T.v[0][b], T.v[1][b]), T.v[2][b]),
-               n[b], jb0, jb1);
-    line_range(fmin(fmin(T.v[0][c], T.v[1][c]), T.v[2][c]), fmax(fmax(T.v[0][c], T.v[1][c]), T.v[2][c]),
-               n[c], jc0, jc1);
 }
 
 // Twice the signed area of (P, Q, q) in the (b, c) projection.
@@ -83,122 +61,389 @@ __device__ __forceinline__ bool line_hit(const Tri& T, int a, double qb, double 
     return true;
 }
 
-__global__ void k_fill_u64(unsigned long long* __restrict__ p, long long n, unsigned long long v) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        p[i] = v;
+// One hit of a grid line parallel to axis a: the interior face it belongs to and its position t on it.  The
+// triangle's coordinates come in the order a, a + 1, a + 2.
+__device__ __forceinline__ bool face_hit(const Tri& T, int a, int jb, int jc, const int n[3], double eps_edge, double eps_det,
+                                         long long& fid, unsigned long long& bits) {
+    double xh;
+    if (!line_hit(T, 0, (double)jb + 0.5, (double)jc + 0.5, eps_edge, eps_det, xh)) return false;
+    const double xm = __dsub_rn(xh, 0.5);
+    const double f = floor(xm);
+    const int na = a == 0 ? n[0] : (a == 1 ? n[1] : n[2]);
+    if (!(f >= 0.0 && f <= (double)(na - 2))) return false;
+    const double t = __dsub_rn(xm, f);
+    const int xa = (int)f;
+    const int x = a == 0 ? xa : (a == 1 ? jc : jb), y = a == 0 ? jb : (a == 1 ? xa : jc), z = a == 0 ? jc : (a == 1 ? jb : xa);
+    fid = a * ((long long)n[0] * n[1] * n[2]) + x + n[0] * (y + (long long)n[1] * z);
+    bits = (unsigned long long)__double_as_longlong(t);
+    return true;
 }
 
-struct LineCount {
+// FP32 test of the same line that only ever says "certainly outside": two of the barycentric weights differ
+// in sign by more than the FP32 error (every difference and product is good to a few 2^-24 of the absolute
+// products) and the edge tolerance, so the FP64 predicate rejects the line whatever the sign of their sum.
+__device__ __forceinline__ bool surely_outside(float Ab, float Ac, float Bb, float Bc, float Cb, float Cc, float qb, float qc,
+                                               float eps) {
+    const float ab = qb - Ab, ac = qc - Ac, bb = qb - Bb, bc = qc - Bc, cb = qb - Cb, cc = qc - Cc;
+    float hi = -1.f, lo = 1.f, sum = 0.f, w[3], e[3];
+    const float P[3] = {(Cb - Bb) * bc, (Ab - Cb) * cc, (Bb - Ab) * ac}, Q[3] = {(Cc - Bc) * bb, (Ac - Cc) * cb, (Bc - Ac) * ab};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        w[i] = P[i] - Q[i];
+        e[i] = 1e-6f * (fabsf(P[i]) + fabsf(Q[i]));      // 16 * 2^-24
+        sum += fabsf(w[i]) + e[i];
+    }
+    const float thr = eps * sum;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        hi = fmaxf(hi, w[i] > e[i] + thr ? 1.f : -1.f);
+        lo = fminf(lo, w[i] < -(e[i] + thr) ? -1.f : 1.f);
+    }
+    return hi > 0.f && lo < 0.f;
+}
+
+// Hits found by the marking pass, kept where the soup's size leaves room (else they are found again).
+struct HitList {
+    unsigned long long* t;
+    unsigned* fid;                 // face ids stay below 2^32 (grids of at most 2^31/3 cells)
+    long long cap;
+    unsigned long long* count;
+};
+
+struct TestArgs {
     const float* tri;
-    long long n[3];
-    __device__ long long operator()(long long item) const {
-        Tri T;
-        if (!load_tri(tri + 9 * (item / 3), T)) return 0;
-        long long jb0, jb1, jc0, jc1;
-        tri_lines(T, (int)(item % 3), n, jb0, jb1, jc0, jc1);
-        if (jb1 < jb0 || jc1 < jc0) return 0;
-        return (jb1 - jb0 + 1) * (jc1 - jc0 + 1);
-    }
+    long long ntri;
+    int n[3];
+    double eps_edge, eps_det;
+    uint8_t* flags;
+    unsigned long long *tmin, *tmax, *tests;
+    HitList hits;
 };
 
-struct StoreOffset {
-    long long* off;
-    __device__ void operator()(long long i, long long o, long long) const { off[i] = o; }
-};
+__device__ __forceinline__ void or_byte(uint8_t* p, unsigned bit) {
+    // the aligned word around a byte lies in the same allocation; its other bytes are or-ed with 0
+    const uintptr_t q = (uintptr_t)p;
+    atomicOr(reinterpret_cast<unsigned*>(q & ~(uintptr_t)3), bit << (8 * (q & 3)));
+}
 
-// One thread per (triangle, axis, line) test; the owning (triangle, axis) item is found by binary
-// search in the exclusive offsets.  Hits update the per-face min/max of t through 64-bit integer
-// atomics on the bit patterns of t >= 0 (their order is the order of the values), so the result
-// does not depend on the order in which threads run.
-__global__ void __launch_bounds__(256) k_test_lines(const float* __restrict__ tri, long long nitems,
-                                                    const long long* __restrict__ off, const long long* __restrict__ total,
-                                                    long long nx, long long ny, long long nz, double eps_edge,
-                                                    double eps_det, unsigned long long* __restrict__ tmin,
-                                                    unsigned long long* __restrict__ tmax) {
-    const long long ntests = *total;
-    const long long n[3] = {nx, ny, nz};
-    const long long N = nx * ny * nz;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < ntests;
-         g += (long long)gridDim.x * blockDim.x) {
-        long long lo = 0, hi = nitems - 1;        // last item with off[item] <= g
-        while (lo < hi) {
-            long long mid = (lo + hi + 1) >> 1;
-            if (off[mid] <= g) lo = mid; else hi = mid - 1;
-        }
-        const long long item = lo;
-        const int a = (int)(item % 3);
-        Tri T;
-        load_tri(tri + 9 * (item / 3), T);
-        long long jb0, jb1, jc0, jc1;
-        tri_lines(T, a, n, jb0, jb1, jc0, jc1);
-        const long long l = g - off[item];
-        const long long nb = jb1 - jb0 + 1;
-        const long long jb = jb0 + l % nb, jc = jc0 + l / nb;
-        double xh;
-        if (!line_hit(T, a, (double)jb + 0.5, (double)jc + 0.5, eps_edge, eps_det, xh)) continue;
-        double xm = __dsub_rn(xh, 0.5);
-        double f = floor(xm);
-        if (!(f >= 0.0 && f <= (double)(n[a] - 2))) continue;
-        double t = __dsub_rn(xm, f);
-        const int b = (a + 1) % 3, c = (a + 2) % 3;
-        long long x[3];
-        x[a] = (long long)f;
-        x[b] = jb;
-        x[c] = jc;
-        const long long fid = a * N + x[0] + nx * (x[1] + ny * x[2]);
-        const unsigned long long bits = (unsigned long long)__double_as_longlong(t);
-        atomicMin(&tmin[fid], bits);
-        atomicMax(&tmax[fid], bits);
+// The marking pass (PASS 1) sets the two link bits of every hit face and gives its min/max slot its start
+// values (every writer stores the same); the second forms the min/max of t through 64-bit integer atomics on
+// the bit patterns of t >= 0 (their order is the order of the values), so nothing depends on the order of the
+// threads, and faces without a hit cost nothing.
+template <int PASS>
+__device__ __forceinline__ void use_hit(const TestArgs& A, long long fid, unsigned long long bits) {
+    if (PASS == 1) {
+        const long long N = (long long)A.n[0] * A.n[1] * A.n[2];
+        const int a = fid >= 2 * N ? 2 : (fid >= N ? 1 : 0);
+        const long long c = fid - a * N, st = a == 0 ? 1 : (a == 1 ? (long long)A.n[0] : (long long)A.n[0] * A.n[1]);
+        or_byte(A.flags + c, 2u << (2 * a));
+        or_byte(A.flags + c + st, 1u << (2 * a));
+        A.tmin[fid] = kEmpty;
+        A.tmax[fid] = 0ULL;
+    } else {
+        atomicMin(&A.tmin[fid], bits);
+        atomicMax(&A.tmax[fid], bits);
     }
 }
 
-// Flags bits 0-5 from the per-face hit table (bits 6-7 cleared).
-__global__ void k_cut_flags(int nx, int ny, int nz, const unsigned long long* __restrict__ tmin,
-                            uint8_t* __restrict__ flags) {
-    const long long N = (long long)nx * ny * nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(c % nx);
-        const int j = (int)((c / nx) % ny);
-        const int k = (int)(c / ((long long)nx * ny));
-        const int x[3] = {i, j, k};
-        const long long st[3] = {1, nx, (long long)nx * ny};
-        unsigned f = 0;
+// Every (triangle, axis, grid line) test whose line lies in the triangle's widened projected box.  A warp takes
+// 32 triangles, lays the tests of one axis end to end (a warp scan of the line counts) and gives each lane
+// one test, the owner found by a search over the scan: a soup of small triangles needs no list of tests in
+// memory and no idle lanes.  Tests that FP32 cannot rule out wait in a queue of the warp until 32 lanes can
+// take the FP64 predicate together: the pass is bound by its FP64 instructions (about 80 with the
+// conversions and the division).  An item of more than kBigItem tests goes to the whole block; gridDim.y
+// slices share such items when the soup has few triangles.
+// Vehicle assembly (2.03 M triangles, 6.0 M tests): 1.01 ms, 2.4 ms without the FP32 test and the queue; one
+// thread per test with offsets in memory took 1.07 ms after 1.3 ms of counting and 1.4 ms of table clearing.
+constexpr int kBigItem = 1024;
+
+template <int PASS>
+__global__ void __launch_bounds__(256) k_test_lines(TestArgs A, int tpb) {
+    if (PASS == 2 && (long long)*A.hits.count <= A.hits.cap) return;       // the list has them all
+    __shared__ int big[3 * 256];
+    __shared__ int nbig;
+    __shared__ unsigned queue[8][64][2];              // [warp]: owner lane | axis << 5, line within the item
+    if (threadIdx.x == 0) nbig = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long n3[3] = {A.n[0], A.n[1], A.n[2]};
+    const long long t0 = (long long)blockIdx.x * tpb;
+    const int mine = w * 32 + lane;
+    float v[3][3] = {};             // vertices stay FP32 until a test needs them (conversions cost an FP64 slot)
+    int lo[3] = {0, 0, 0}, len[3] = {0, 0, 0};
+    if (mine < tpb && t0 + mine < A.ntri) {
+        const float* t = A.tri + 9 * (t0 + mine);
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            v[q / 3][q % 3] = t[q];
+            ok = ok && isfinite(v[q / 3][q % 3]);
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            long long l, h;
+            line_range((double)fminf(fminf(v[0][d], v[1][d]), v[2][d]), (double)fmaxf(fmaxf(v[0][d], v[1][d]), v[2][d]), n3[d], l, h);
+            if (ok && h >= l) {
+                lo[d] = (int)l;
+                len[d] = (int)(h - l + 1);
+            }
+        }
+    }
+    unsigned long long ntests = 0;
+    auto store = [&](bool hit, long long fid, unsigned long long bits) {
+        if (PASS == 1) {
+            const unsigned m = __ballot_sync(0xffffffffu, hit);
+            if (!m) return;
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(A.hits.count, (unsigned long long)__popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            const long long pos = (long long)base + __popc(m & ((1u << lane) - 1u));
+            if (hit && pos < A.hits.cap) {
+                A.hits.t[pos] = bits;
+                A.hits.fid[pos] = (unsigned)fid;
+            }
+        }
+        if (hit) use_hit<PASS>(A, fid, bits);
+    };
+    if (w * 32 < tpb) {
+        int nq = 0;
+        // takes the first min(32, nq) entries of the queue
+        auto drain = [&]() {
+            const bool on = lane < nq;
+            const unsigned e = on ? queue[w][lane][0] : 0u, l = on ? queue[w][lane][1] : 0u;
+            const int own = (int)(e & 31u), a = (int)(e >> 5);
+            float r[9];
+#pragma unroll
+            for (int q = 0; q < 9; ++q) r[q] = __shfl_sync(0xffffffffu, v[q / 3][q % 3], own);
+            int o3[3], l3[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                o3[d] = __shfl_sync(0xffffffffu, lo[d], own);
+                l3[d] = __shfl_sync(0xffffffffu, len[d], own);
+            }
+            Tri Q;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                const float x = r[3 * p], y = r[3 * p + 1], z = r[3 * p + 2];
+                Q.v[p][0] = (double)(a == 0 ? x : (a == 1 ? y : z));
+                Q.v[p][1] = (double)(a == 0 ? y : (a == 1 ? z : x));
+                Q.v[p][2] = (double)(a == 0 ? z : (a == 1 ? x : y));
+            }
+            const unsigned nb = (unsigned)(a == 0 ? l3[1] : (a == 1 ? l3[2] : l3[0])), jc = nb ? l / nb : 0u;
+            const int b0 = a == 0 ? o3[1] : (a == 1 ? o3[2] : o3[0]), c0 = a == 0 ? o3[2] : (a == 1 ? o3[0] : o3[1]);
+            long long fid = 0;
+            unsigned long long bits = 0;
+            const bool hit = on && face_hit(Q, a, b0 + (int)(l - jc * nb), c0 + (int)jc, A.n, A.eps_edge, A.eps_det, fid, bits);
+            store(hit, fid, bits);
+            nq -= nq < 32 ? nq : 32;
+        };
+        const float epsf = (float)A.eps_edge * 1.0001f;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            if (tmin[a * N + c] != kEmpty) f |= 1u << (2 * a + 1);
-            if (x[a] > 0 && tmin[a * N + c - st[a]] != kEmpty) f |= 1u << (2 * a);
+            const int b = (a + 1) % 3, c = (a + 2) % 3;
+            const long long all = (long long)len[b] * len[c];
+            int cnt = 0;
+            if (all > kBigItem) big[atomicAdd(&nbig, 1)] = 3 * mine + a;
+            else cnt = (int)all;
+            ntests += (unsigned long long)all;
+            if (blockIdx.y != 0) continue;
+            int incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int total = __shfl_sync(0xffffffffu, incl, 31), excl = incl - cnt;
+            for (int g0 = 0; g0 < total; g0 += 32) {
+                const int g = g0 + lane;
+                int own = 0;                              // last lane with excl <= g (empty ones before it end there too)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const int e = __shfl_sync(0xffffffffu, excl, own + o);
+                    if (e <= g) own += o;
+                }
+                float q[6];
+#pragma unroll
+                for (int p = 0; p < 3; ++p) {
+                    q[2 * p] = __shfl_sync(0xffffffffu, v[p][b], own);
+                    q[2 * p + 1] = __shfl_sync(0xffffffffu, v[p][c], own);
+                }
+                const int e0 = __shfl_sync(0xffffffffu, excl, own), nb = __shfl_sync(0xffffffffu, len[b], own);
+                const int b0 = __shfl_sync(0xffffffffu, lo[b], own), c0 = __shfl_sync(0xffffffffu, lo[c], own);
+                bool may = false;
+                unsigned l = 0;
+                if (g < total) {
+                    l = (unsigned)(g - e0);
+                    const int jc = (int)(l / (unsigned)nb), jb = (int)l - jc * nb;
+                    may = !surely_outside(q[0], q[1], q[2], q[3], q[4], q[5], (float)(b0 + jb) + 0.5f, (float)(c0 + jc) + 0.5f, epsf);
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, may);
+                if (may) {
+                    const int pos = nq + __popc(m & ((1u << lane) - 1u));
+                    queue[w][pos][0] = (unsigned)own | ((unsigned)a << 5);
+                    queue[w][pos][1] = l;
+                }
+                nq += __popc(m);
+                __syncwarp();
+                if (nq >= 32) {
+                    const int rest = nq - 32;
+                    drain();
+                    // the entries beyond the first 32 move to the front
+                    unsigned t0 = 0, t1 = 0;
+                    if (lane < rest) {
+                        t0 = queue[w][32 + lane][0];
+                        t1 = queue[w][32 + lane][1];
+                    }
+                    __syncwarp();
+                    if (lane < rest) {
+                        queue[w][lane][0] = t0;
+                        queue[w][lane][1] = t1;
+                    }
+                    __syncwarp();
+                }
+            }
         }
-        flags[c] = (uint8_t)f;
+        if (nq > 0) drain();
+    }
+    if (PASS == 1 && blockIdx.y == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ntests += __shfl_down_sync(0xffffffffu, ntests, o);
+        if (lane == 0 && ntests) atomicAdd(A.tests, ntests);
+    }
+    __syncthreads();
+    for (int q = 0; q < nbig; ++q) {
+        const int item = big[q], a = item % 3, b = (a + 1) % 3, c = (a + 2) % 3;
+        const float* t = A.tri + 9 * (t0 + item / 3);
+        Tri Q;
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            Q.v[p][0] = (double)t[3 * p + a];
+            Q.v[p][1] = (double)t[3 * p + b];
+            Q.v[p][2] = (double)t[3 * p + c];
+        }
+        long long bl, bh, cl, ch;
+        line_range(fmin(fmin(Q.v[0][1], Q.v[1][1]), Q.v[2][1]), fmax(fmax(Q.v[0][1], Q.v[1][1]), Q.v[2][1]), n3[b], bl, bh);
+        line_range(fmin(fmin(Q.v[0][2], Q.v[1][2]), Q.v[2][2]), fmax(fmax(Q.v[0][2], Q.v[1][2]), Q.v[2][2]), n3[c], cl, ch);
+        const long long nb = bh - bl + 1, total = nb * (ch - cl + 1);
+        for (long long g0 = (long long)blockIdx.y * 256; g0 < total; g0 += (long long)gridDim.y * 256) {
+            const long long g = g0 + threadIdx.x;
+            long long fid = 0;
+            unsigned long long bits = 0;
+            bool hit = false;
+            if (g < total) {
+                const unsigned jc = (unsigned)g / (unsigned)nb;           // lines of one axis: fewer than 2^31
+                hit = face_hit(Q, a, (int)(bl + (g - jc * nb)), (int)(cl + jc), A.n, A.eps_edge, A.eps_det, fid, bits);
+            }
+            store(hit, fid, bits);
+        }
     }
 }
 
-struct FaceHit {
-    const unsigned long long* tmin;
-    __device__ long long operator()(long long f) const { return tmin[f] != kEmpty ? 1 : 0; }
-};
+__global__ void __launch_bounds__(256) k_apply_hits(TestArgs A) {
+    const long long n = (long long)*A.hits.count;
+    if (n > A.hits.cap) return;
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
+        use_hit<2>(A, (long long)A.hits.fid[q], A.hits.t[q]);
+}
 
-struct EmitCut {
-    const unsigned long long* tmin;
-    const unsigned long long* tmax;
-    int64_t* face_id;
-    double* t_lo;
-    double* t_hi;
-    long long cap;
-    __device__ void operator()(long long f, long long o, long long c) const {
-        if (c && o < cap) {
-            face_id[o] = f;
-            t_lo[o] = __longlong_as_double((long long)tmin[f]);
-            t_hi[o] = __longlong_as_double((long long)tmax[f]);
+// ---- lists from the flags -----------------------------------------------------------------------
+//
+// A block takes a tile of 256 * CPT cells, a thread CPT (16 or 64) consecutive ones as 16-byte loads; almost
+// all are zero, so the passes cost the flags' bytes (one per cell) and not the tables behind them.
+constexpr int kListThreads = IBM_SCAN_NT;
+
+template <int CPT>
+struct FlagChunk {
+    uint32_t w[CPT / 4];
+    __device__ __forceinline__ FlagChunk(const uint8_t* __restrict__ f, long long c0, long long N) {
+#pragma unroll
+        for (int q = 0; q < CPT / 16; ++q) {
+            const long long c = c0 + 16 * q;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (c + 16 <= N && ((uintptr_t)(f + c) & 15u) == 0) {
+                v = *reinterpret_cast<const uint4*>(f + c);
+            } else if (c < N) {
+                unsigned t[4] = {0u, 0u, 0u, 0u};
+                for (int m = 0; m < 16 && c + m < N; ++m) t[m >> 2] |= (unsigned)f[c + m] << (8 * (m & 3));
+                v = make_uint4(t[0], t[1], t[2], t[3]);
+            }
+            w[4 * q] = v.x;
+            w[4 * q + 1] = v.y;
+            w[4 * q + 2] = v.z;
+            w[4 * q + 3] = v.w;
         }
     }
 };
+
+// Cut faces of the three axes, 20 bits each (a tile has at most 16384 of each).
+template <int CPT>
+__device__ __forceinline__ long long face_counts(const FlagChunk<CPT>& F) {
+    int n0 = 0, n1 = 0, n2 = 0;
+#pragma unroll
+    for (int q = 0; q < CPT / 4; ++q) {
+        n0 += __popc(F.w[q] & 0x02020202u);
+        n1 += __popc(F.w[q] & 0x08080808u);
+        n2 += __popc(F.w[q] & 0x20202020u);
+    }
+    return (long long)n0 | ((long long)n1 << 20) | ((long long)n2 << 40);
+}
+
+template <int CPT>
+__global__ void __launch_bounds__(kListThreads) k_face_counts(const uint8_t* __restrict__ flags, long long N, long long nt,
+                                                              long long* __restrict__ tiles) {
+    const FlagChunk<CPT> F(flags, ((long long)blockIdx.x * kListThreads + threadIdx.x) * CPT, N);
+    long long tot;
+    block_exscan(face_counts(F), tot);
+    if (threadIdx.x < 3) tiles[threadIdx.x * nt + blockIdx.x] = (tot >> (20 * threadIdx.x)) & 0xfffff;
+}
+
+template <int CPT>
+__global__ void __launch_bounds__(kListThreads) k_emit_faces(const uint8_t* __restrict__ flags, long long N, long long nt,
+                                                             const long long* __restrict__ tiles,
+                                                             const unsigned long long* __restrict__ tmin,
+                                                             const unsigned long long* __restrict__ tmax,
+                                                             int64_t* __restrict__ face_id, double* __restrict__ t_lo,
+                                                             double* __restrict__ t_hi, long long cap) {
+    const long long c0 = ((long long)blockIdx.x * kListThreads + threadIdx.x) * CPT;
+    const FlagChunk<CPT> F(flags, c0, N);
+    const long long cnt = face_counts(F);
+    if (!__syncthreads_or(cnt != 0)) return;
+    long long tot;
+    const long long off = block_exscan(cnt, tot);
+    if (!cnt) return;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        long long o = tiles[a * nt + blockIdx.x] + ((off >> (20 * a)) & 0xfffff);
+#pragma unroll
+        for (int q = 0; q < CPT / 4; ++q) {
+            unsigned m = F.w[q] & (0x02020202u << (2 * a));
+            while (m) {
+                const int bit = __ffs(m) - 1;
+                m &= m - 1;
+                if (o < cap) {
+                    const long long f = a * N + c0 + 4 * q + (bit >> 3);
+                    face_id[o] = f;
+                    t_lo[o] = __longlong_as_double((long long)tmin[f]);
+                    t_hi[o] = __longlong_as_double((long long)tmax[f]);
+                }
+                ++o;
+            }
+        }
+    }
+}
+
+inline bool wide_tiles(long long N) { return N >= (4LL << 20); }      // 64 cells per thread (else 16)
+inline long long list_tiles(long long N) {
+    const long long t = (long long)kListThreads * (wide_tiles(N) ? 64 : 16);
+    return (N + t - 1) / t;
+}
 
 struct Workspace {
     unsigned long long* tmin;
     unsigned long long* tmax;
-    long long* item_off;
+    unsigned char* hits;   // 8 (3 ntri + 1) bytes
     long long* tiles;
-    long long* scalars;   // [0] tests, [1] cut faces
+    long long* scalars;    // [0] tests, [1] cut faces, [2] hits
     size_t bytes;
 };
 
@@ -211,7 +456,7 @@ Workspace carve(void* base, long long N, long long ntri) {
     const long long nt = scan_tiles(3 * N > 3 * ntri ? 3 * N : 3 * ntri) + 1;
     w.tmin = (unsigned long long*)(p + o); o += align256(sizeof(unsigned long long) * 3 * N);
     w.tmax = (unsigned long long*)(p + o); o += align256(sizeof(unsigned long long) * 3 * N);
-    w.item_off = (long long*)(p + o); o += align256(sizeof(long long) * (3 * ntri + 1));
+    w.hits = (unsigned char*)(p + o); o += align256(sizeof(long long) * (3 * ntri + 1));
     w.tiles = (long long*)(p + o); o += align256(sizeof(long long) * nt);
     w.scalars = (long long*)(p + o); o += align256(sizeof(long long) * 4);
     w.bytes = o;
@@ -247,24 +492,43 @@ extern "C" int ibm_classify(const ibm_grid* g, const float* d_tri, int64_t ntri,
     if (!d_ws || ws_bytes < w.bytes)
         return ibm_fail(IBM_E_INVALID, "ibm_classify: workspace of %zu bytes, %zu needed", ws_bytes, w.bytes);
     cudaStream_t s = (cudaStream_t)stream;
-    k_fill_u64<<<blocks_for(3 * N, 256), 256, 0, s>>>(w.tmin, 3 * N, kEmpty);
-    k_fill_u64<<<blocks_for(3 * N, 256), 256, 0, s>>>(w.tmax, 3 * N, 0ULL);
-    IBM_LAUNCHED("ibm_classify: fill");
-    const long long nitems = 3 * ntri;
-    if (nitems > 0) {
-        LineCount lc{d_tri, {g->nx, g->ny, g->nz}};
-        IBM_CUDA(scan_emit(nitems, lc, StoreOffset{w.item_off}, w.tiles, w.scalars + 0, s));
-        k_test_lines<<<32 * IBM_NSM, 256, 0, s>>>(d_tri, nitems, w.item_off, w.scalars + 0, g->nx, g->ny, g->nz,
-                                                  gp->eps_edge, gp->eps_det, w.tmin, w.tmax);
+    IBM_CUDA(cudaMemsetAsync(d_flags, 0, (size_t)N, s));
+    IBM_CUDA(cudaMemsetAsync(w.scalars, 0, 4 * sizeof(long long), s));
+    if (ntri > 0) {
+        TestArgs A;
+        A.tri = d_tri;
+        A.ntri = ntri;
+        A.n[0] = g->nx; A.n[1] = g->ny; A.n[2] = g->nz;
+        A.eps_edge = gp->eps_edge;
+        A.eps_det = gp->eps_det;
+        A.flags = d_flags;
+        A.tmin = w.tmin;
+        A.tmax = w.tmax;
+        A.tests = (unsigned long long*)w.scalars;
+        A.hits.cap = 8 * (3 * ntri + 1) / 12;
+        A.hits.t = (unsigned long long*)w.hits;
+        A.hits.fid = (unsigned*)(A.hits.t + A.hits.cap);
+        A.hits.count = (unsigned long long*)w.scalars + 2;
+        // triangles per block: all SMs for a small soup, then whole blocks; slices where few triangles may be large
+        long long tpb = ntri / (4 * IBM_NSM);
+        tpb = tpb < 1 ? 1 : (tpb > 256 ? 256 : tpb);
+        const long long nb = (ntri + tpb - 1) / tpb;
+        const dim3 grid((unsigned)nb, (unsigned)(nb < IBM_NSM ? 8 : 1));
+        k_test_lines<1><<<grid, 256, 0, s>>>(A, (int)tpb);
+        k_apply_hits<<<8 * IBM_NSM, 256, 0, s>>>(A);
+        k_test_lines<2><<<grid, 256, 0, s>>>(A, (int)tpb);
         IBM_LAUNCHED("ibm_classify: k_test_lines");
-    } else {
-        IBM_CUDA(cudaMemsetAsync(w.scalars, 0, sizeof(long long), s));
     }
-    k_cut_flags<<<blocks_for(N, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, w.tmin, d_flags);
-    IBM_LAUNCHED("ibm_classify: k_cut_flags");
-    // count first; the list is only written when it fits
-    IBM_CUDA(scan_emit(3 * N, FaceHit{w.tmin}, EmitCut{w.tmin, w.tmax, d_face_id, d_t_lo, d_t_hi, cap},
-                       w.tiles, w.scalars + 1, s));
+    // count first; the list is only written as far as it fits
+    const long long nt = list_tiles(N);
+    if (wide_tiles(N)) k_face_counts<64><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, N, nt, w.tiles);
+    else k_face_counts<16><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, N, nt, w.tiles);
+    k_scan_tile_totals<<<1, IBM_SCAN_NT, 0, s>>>(w.tiles, 3 * nt, w.scalars + 1);
+    if (wide_tiles(N))
+        k_emit_faces<64><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, N, nt, w.tiles, w.tmin, w.tmax, d_face_id, d_t_lo, d_t_hi, cap);
+    else
+        k_emit_faces<16><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, N, nt, w.tiles, w.tmin, w.tmax, d_face_id, d_t_lo, d_t_hi, cap);
+    IBM_LAUNCHED("ibm_classify: cut faces");
     long long host[2];
     IBM_CUDA(cudaMemcpyAsync(host, w.scalars, sizeof(host), cudaMemcpyDeviceToHost, s));
     IBM_CUDA(cudaStreamSynchronize(s));
@@ -285,105 +549,135 @@ struct ibm_geom {
     long long n_cut, n_rec, n_inc;
     uint8_t* flags;        // caller-owned
     int32_t* cellrec;      // [N]
-    int32_t* inc;          // [n_inc] Omega_inc cells in index order
     LinkRec* rec;          // [n_rec]
+    int32_t* inc;          // [n_inc] Omega_inc cells in index order (behind rec in its allocation)
 };
 
 namespace {
 
-__global__ void k_region_bits(int nx, int ny, int nz, uint8_t* __restrict__ flags) {
-    const long long N = (long long)nx * ny * nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        const unsigned f = flags[c] & 63u;
-        unsigned out = f;
-        if (f) {
-            out |= 64u;
-        } else {
-            const int x[3] = {(int)(c % nx), (int)((c / nx) % ny), (int)(c / ((long long)nx * ny))};
-            const int n[3] = {nx, ny, nz};
-            const long long st[3] = {1, nx, (long long)nx * ny};
-            bool adj = false;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (x[a] > 0 && (flags[c - st[a]] & 63u)) adj = true;
-                if (x[a] < n[a] - 1 && (flags[c + st[a]] & 63u)) adj = true;
-            }
-            if (adj) out |= 128u;
-        }
-        flags[c] = (uint8_t)out;
+// Omega_inc (bit 6) and Omega_adj (bit 7).  W cells per thread (4 as one word where rows are whole words);
+// words that come out as they were (nearly all are 0) are not written.
+template <int W>
+__global__ void __launch_bounds__(256) k_region_bits(int nx, int ny, int nz, uint8_t* flags) {
+    const long long N = (long long)nx * ny * nz, nxy = (long long)nx * ny;
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < N / W; q += (long long)gridDim.x * blockDim.x) {
+        const unsigned c = (unsigned)(q * W), r = c / (unsigned)nx;       // grids of fewer than 2^31 cells
+        const int i = (int)(c - r * (unsigned)nx), j = (int)(r % (unsigned)ny), k = (int)(r / (unsigned)ny);
+        auto cut = [&](long long o) -> unsigned {                           // 1 in the byte of every cell with a cut link
+            if (W == 4) return ((*reinterpret_cast<const unsigned*>(flags + c + o) & 0x3f3f3f3fu) + 0x3f3f3f3fu) >> 6 & 0x01010101u;
+            return (flags[c + o] & 63u) ? 1u : 0u;
+        };
+        const unsigned own = cut(0);
+        unsigned nb = 0;
+        if (j > 0) nb |= cut(-nx);
+        if (j < ny - 1) nb |= cut(nx);
+        if (k > 0) nb |= cut(-nxy);
+        if (k < nz - 1) nb |= cut(nxy);
+        if (W == 4) nb |= (own << 8) | (own >> 8);
+        if (i > 0 && (flags[c - 1] & 63u)) nb |= 1u;
+        if (i + W < nx && (flags[c + W] & 63u)) nb |= 1u << (8 * (W - 1));
+        const unsigned raw = W == 4 ? *reinterpret_cast<const unsigned*>(flags + c) : flags[c];
+        const unsigned out = (raw & 0x3f3f3f3fu) | (own << 6) | ((nb & ~own) << 7);
+        if (out == raw) continue;
+        if (W == 4) *reinterpret_cast<unsigned*>(flags + c) = out;
+        else flags[c] = (uint8_t)out;
     }
 }
 
-// Packed count per cell: records in the low 32 bits, one Omega_inc slot in the high bits.
-struct RecCount {
-    const uint8_t* flags;
-    __device__ long long operator()(long long c) const {
-        const unsigned f = flags[c] & 63u;
-        return f ? ((1LL << 32) | (long long)__popc(f)) : 0;
+// Records (low 32 bits) and Omega_inc cells (high bits) of a thread's cells.
+template <int CPT>
+__device__ __forceinline__ long long rec_counts(const FlagChunk<CPT>& F) {
+    int nr = 0, ni = 0;
+#pragma unroll
+    for (int q = 0; q < CPT / 4; ++q) {
+        const unsigned m = F.w[q] & 0x3f3f3f3fu;
+        nr += __popc(m);
+        ni += __popc((m + 0x3f3f3f3fu) & 0x40404040u);
     }
-};
+    return (long long)nr | ((long long)ni << 32);
+}
 
-struct EmitCellrec {
-    int32_t* cellrec;
-    int32_t* inc;
-    __device__ void operator()(long long c, long long o, long long cnt) const {
-        if (cnt) {
+template <int CPT>
+__global__ void __launch_bounds__(kListThreads) k_rec_counts(const uint8_t* __restrict__ flags, long long N,
+                                                             long long* __restrict__ tiles) {
+    const FlagChunk<CPT> F(flags, ((long long)blockIdx.x * kListThreads + threadIdx.x) * CPT, N);
+    long long tot;
+    block_exscan(rec_counts(F), tot);
+    if (threadIdx.x == 0) tiles[blockIdx.x] = tot;
+}
+
+// First record of every Omega_inc cell (cellrec holds -1 before) and the list of these cells.
+template <int CPT>
+__global__ void __launch_bounds__(kListThreads) k_emit_cellrec(const uint8_t* __restrict__ flags, long long N,
+                                                               const long long* __restrict__ tiles,
+                                                               int32_t* __restrict__ cellrec, int32_t* __restrict__ inc) {
+    const long long c0 = ((long long)blockIdx.x * kListThreads + threadIdx.x) * CPT;
+    const FlagChunk<CPT> F(flags, c0, N);
+    const long long cnt = rec_counts(F);
+    if (!__syncthreads_or(cnt != 0)) return;
+    long long tot;
+    long long o = tiles[blockIdx.x] + block_exscan(cnt, tot);
+    if (!cnt) return;
+#pragma unroll
+    for (int q = 0; q < CPT / 4; ++q) {
+        if (!(F.w[q] & 0x3f3f3f3fu)) continue;
+        for (int m = 0; m < 4; ++m) {
+            const unsigned f = (F.w[q] >> (8 * m)) & 63u;
+            if (!f) continue;
+            const long long c = c0 + 4 * q + m;
             cellrec[c] = (int32_t)(o & 0xffffffffLL);
             inc[o >> 32] = (int32_t)c;
-        } else {
-            cellrec[c] = -1;
+            o += (1LL << 32) | (long long)__popc(f);
         }
     }
-};
-
-__device__ __forceinline__ long long find_face(const int64_t* __restrict__ fid, long long n, long long key) {
-    long long lo = 0, hi = n - 1;
-    while (lo <= hi) {
-        long long mid = lo + ((hi - lo) >> 1);
-        long long v = fid[mid];
-        if (v == key) return mid;
-        if (v < key) lo = mid + 1; else hi = mid - 1;
-    }
-    return -1;
 }
 
 // Eq. q_axis: upper branch (Dx/d) q_IB + ((d - Dx)/d) q_P on d/Dx >= 1/2; lower branch
 // 2 q_IB + ((2d - Dx)/Dx) q_O - (2d/Dx) q_P on d/Dx < 1/2 when the opposite neighbour O is usable;
 // otherwise the upper branch at d = 1/2.  Eq. distribution_function weights with the near distance d.
-__global__ void k_build_records(int nx, int ny, int nz, const uint8_t* __restrict__ flags,
-                                const int32_t* __restrict__ inc, long long n_inc,
-                                const int32_t* __restrict__ cellrec, const int64_t* __restrict__ fid,
-                                const double* __restrict__ t_lo, const double* __restrict__ t_hi, long long n_cut,
-                                LinkRec* __restrict__ rec, int* __restrict__ err) {
+//
+// One thread per cut face writes the records of its two cells: a record's place follows from its cell's first
+// record and flags, so nothing is searched.  The flags name 2 n_cut links (checked before); a list whose ids
+// rise strictly and whose every face is flagged from both of its cells therefore covers each link once.
+// Vehicle assembly: 0.29 ms, 2.3 ms with a binary search of the list per record.
+__global__ void __launch_bounds__(128) k_build_records(int nx, int ny, int nz, const uint8_t* __restrict__ flags,
+                                                       const int32_t* __restrict__ cellrec, const int64_t* __restrict__ fid,
+                                                       const double* __restrict__ t_lo, const double* __restrict__ t_hi,
+                                                       long long n_cut, LinkRec* __restrict__ rec, int* __restrict__ err) {
     const long long N = (long long)nx * ny * nz;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n_inc; q += (long long)gridDim.x * blockDim.x) {
-        const long long P = inc[q];
-        const unsigned f = flags[P] & 63u;
-        const int x[3] = {(int)(P % nx), (int)((P / nx) % ny), (int)(P / ((long long)nx * ny))};
-        const int n[3] = {nx, ny, nz};
-        const long long st[3] = {1, nx, (long long)nx * ny};
-        int k = cellrec[P];
-        for (int bit = 0; bit < 6; ++bit) {
-            if (!((f >> bit) & 1u)) continue;
-            const int a = bit >> 1, s = (bit & 1) ? 1 : -1;
-            const long long lower = s > 0 ? P : P - st[a];
-            const long long idx = find_face(fid, n_cut, a * N + lower);
+    const long long stb[3] = {1, nx, (long long)nx * ny};
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n_cut; q += (long long)gridDim.x * blockDim.x) {
+        const long long id = fid[q];
+        bool ok = id >= 0 && id < 3 * N && (q == 0 || fid[q - 1] < id);
+        int a = 0, xa = 0, na = 1;
+        long long c = 0, st = 1;
+        if (ok) {
+            a = id >= 2 * N ? 2 : (id >= N ? 1 : 0);
+            c = id - a * N;
+            st = stb[a];
+            na = a == 0 ? nx : (a == 1 ? ny : nz);
+            const unsigned u = (unsigned)c, r = u / (unsigned)nx;
+            xa = a == 0 ? (int)(u - r * (unsigned)nx) : (a == 1 ? (int)(r % (unsigned)ny) : (int)(r / (unsigned)ny));
+            ok = xa + 1 < na && ((flags[c] >> (2 * a + 1)) & 1u) && ((flags[c + st] >> (2 * a)) & 1u);
+        }
+        if (!ok) {
+            atomicExch(err, 1);
+            continue;
+        }
+        for (int s = 1; s >= -1; s -= 2) {
+            const long long P = s > 0 ? c : c + st;
+            const int bit = 2 * a + (s > 0), x = s > 0 ? xa : xa + 1;
+            const unsigned f = flags[P] & 63u;
+            const double d = s > 0 ? t_lo[q] : __dsub_rn(1.0, t_hi[q]);
             LinkRec r;
-            if (idx < 0) {
-                atomicExch(err, 1);
-                r = LinkRec{};
-                rec[k++] = r;
-                continue;
-            }
-            const double d = s > 0 ? t_lo[idx] : __dsub_rn(1.0, t_hi[idx]);
             r.cell = (int32_t)P;
-            r.far = (int32_t)(P + s * st[a]);
+            r.far = (int32_t)(P + s * st);
             r.axis = (int8_t)a;
             r.side = (int8_t)s;
             r.pad = 0;
             r.d = d;
-            const int yo = x[a] - s;
-            const bool o_ok = yo >= 0 && yo < n[a] && !((f >> (2 * a + (s > 0 ? 0 : 1))) & 1u);
+            const int yo = x - s;
+            const bool o_ok = yo >= 0 && yo < na && !((f >> (2 * a + (s > 0 ? 0 : 1))) & 1u);
             if (d >= 0.5) {
                 r.branch = 0;
                 r.opp = -1;
@@ -392,7 +686,7 @@ __global__ void k_build_records(int nx, int ny, int nz, const uint8_t* __restric
                 r.c_o = 0.0;
             } else if (o_ok) {
                 r.branch = 1;
-                r.opp = (int32_t)(P - s * st[a]);
+                r.opp = (int32_t)(P - s * st);
                 r.c_ib = 2.0;
                 r.c_o = __dsub_rn(__dmul_rn(2.0, d), 1.0);
                 r.c_p = -__dmul_rn(2.0, d);
@@ -407,7 +701,7 @@ __global__ void k_build_records(int nx, int ny, int nz, const uint8_t* __restric
             r.w_fluid = __ddiv_rn(d, den);
             r.w_ghost = __ddiv_rn(__dsub_rn(1.0, d), den);
             r.uib[0] = r.uib[1] = r.uib[2] = 0.0;
-            rec[k++] = r;
+            rec[cellrec[P] + __popc(f & ((1u << bit) - 1u))] = r;
         }
     }
 }
@@ -450,7 +744,6 @@ __global__ void k_set_uib(LinkRec* __restrict__ rec, long long n, const double* 
 extern "C" void ibm_geom_destroy(ibm_geom* G) {
     if (!G) return;
     cudaFree(G->cellrec);
-    cudaFree(G->inc);
     cudaFree(G->rec);
     free(G);
 }
@@ -470,47 +763,45 @@ extern "C" int ibm_setup(const ibm_grid* g, const ibm_geom_params* gp, uint8_t* 
     G->N = (long long)g->nx * g->ny * g->nz;
     G->n_cut = n_cut;
     G->flags = d_flags;
-    long long* tiles = nullptr;
-    int* d_err = nullptr;
-    long long host[2] = {0, 0};
+    long long* tiles = nullptr;                 // tile totals, their sum, the error word
+    long long host = 0;
     int herr = 0;
-    const long long nt = scan_tiles(G->N) + 1;
+    const long long nt = list_tiles(G->N);
     cudaError_t e;
-    if ((e = cudaMalloc(&G->cellrec, sizeof(int32_t) * G->N)) != cudaSuccess ||
-        (e = cudaMalloc(&tiles, sizeof(long long) * (nt + 2))) != cudaSuccess ||
-        (e = cudaMalloc(&d_err, sizeof(int))) != cudaSuccess) {
-        cudaFree(tiles);
-        cudaFree(d_err);
-        ibm_geom_destroy(G);
-        return ibm_fail(IBM_E_NOMEM, "ibm_setup: %s", cudaGetErrorString(e));
-    }
-    // inc list sized after the count is known: count into a scratch of N int32 first
-    if ((e = cudaMalloc(&G->inc, sizeof(int32_t) * (G->N > 0 ? G->N : 1))) != cudaSuccess) goto nomem;
-    k_region_bits<<<blocks_for(G->N, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, d_flags);
-    if ((e = scan_emit(G->N, RecCount{d_flags}, EmitCellrec{G->cellrec, G->inc}, tiles, tiles + nt, s)) != cudaSuccess)
-        goto cuda_err;
-    if ((e = cudaMemcpyAsync(host, tiles + nt, sizeof(long long), cudaMemcpyDeviceToHost, s)) != cudaSuccess) goto cuda_err;
+    const bool words = g->nx % 4 == 0 && ((uintptr_t)d_flags & 3u) == 0;
+    // one allocation for the cell table with the scan's tile totals behind it, one for the cell list and records
+    const size_t cellb = (sizeof(int32_t) * (size_t)G->N + 15) & ~(size_t)15;
+    if ((e = cudaMalloc(&G->cellrec, cellb + sizeof(long long) * (nt + 2))) != cudaSuccess) goto nomem;
+    tiles = (long long*)((char*)G->cellrec + cellb);
+    if (words) k_region_bits<4><<<blocks_for(G->N / 4, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, d_flags);
+    else k_region_bits<1><<<blocks_for(G->N, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, d_flags);
+    if (wide_tiles(G->N)) k_rec_counts<64><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, G->N, tiles);
+    else k_rec_counts<16><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, G->N, tiles);
+    k_scan_tile_totals<<<1, IBM_SCAN_NT, 0, s>>>(tiles, nt, tiles + nt);
+    if ((e = cudaGetLastError()) != cudaSuccess) goto cuda_err;
+    if ((e = cudaMemcpyAsync(&host, tiles + nt, sizeof(long long), cudaMemcpyDeviceToHost, s)) != cudaSuccess) goto cuda_err;
+    if ((e = cudaMemsetAsync(G->cellrec, 0xff, sizeof(int32_t) * G->N, s)) != cudaSuccess) goto cuda_err;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) goto cuda_err;
-    G->n_rec = host[0] & 0xffffffffLL;
-    G->n_inc = host[0] >> 32;
+    G->n_rec = host & 0xffffffffLL;
+    G->n_inc = host >> 32;
     if (G->n_rec != 2 * n_cut) {
-        cudaFree(tiles);
-        cudaFree(d_err);
         ibm_geom_destroy(G);
         return ibm_fail(IBM_E_INVALID, "ibm_setup: flags name %lld cut links but the list has %lld faces",
-                        (long long)host[0] & 0xffffffffLL, (long long)n_cut);
+                        host & 0xffffffffLL, (long long)n_cut);
     }
-    if ((e = cudaMalloc(&G->rec, sizeof(LinkRec) * (G->n_rec > 0 ? G->n_rec : 1))) != cudaSuccess) goto nomem;
-    if ((e = cudaMemsetAsync(d_err, 0, sizeof(int), s)) != cudaSuccess) goto cuda_err;
-    if (G->n_inc > 0)
-        k_build_records<<<blocks_for(G->n_inc, 128), 128, 0, s>>>(g->nx, g->ny, g->nz, d_flags, G->inc, G->n_inc,
-                                                                  G->cellrec, d_face_id, d_t_lo, d_t_hi, n_cut,
-                                                                  G->rec, d_err);
-    if ((e = cudaGetLastError()) != cudaSuccess) goto cuda_err;
-    if ((e = cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) goto cuda_err;
+    if ((e = cudaMalloc(&G->rec, sizeof(LinkRec) * (size_t)G->n_rec + sizeof(int32_t) * (size_t)(G->n_inc + 4))) != cudaSuccess) goto nomem;
+    G->inc = (int32_t*)(G->rec + G->n_rec);
+    if (n_cut > 0) {
+        int* const d_err = (int*)(tiles + nt + 1);
+        if ((e = cudaMemsetAsync(d_err, 0, sizeof(int), s)) != cudaSuccess) goto cuda_err;
+        if (wide_tiles(G->N)) k_emit_cellrec<64><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, G->N, tiles, G->cellrec, G->inc);
+        else k_emit_cellrec<16><<<(unsigned)nt, kListThreads, 0, s>>>(d_flags, G->N, tiles, G->cellrec, G->inc);
+        k_build_records<<<blocks_for(n_cut, 128), 128, 0, s>>>(g->nx, g->ny, g->nz, d_flags, G->cellrec, d_face_id, d_t_lo,
+                                                               d_t_hi, n_cut, G->rec, d_err);
+        if ((e = cudaGetLastError()) != cudaSuccess) goto cuda_err;
+        if ((e = cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) goto cuda_err;
+    }
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) goto cuda_err;
-    cudaFree(tiles);
-    cudaFree(d_err);
     if (herr) {
         ibm_geom_destroy(G);
         return ibm_fail(IBM_E_INVALID, "ibm_setup: a cut link has no entry in the cut-face list");
@@ -518,13 +809,9 @@ extern "C" int ibm_setup(const ibm_grid* g, const ibm_geom_params* gp, uint8_t* 
     *out = G;
     return IBM_OK;
 nomem:
-    cudaFree(tiles);
-    cudaFree(d_err);
     ibm_geom_destroy(G);
     return ibm_fail(IBM_E_NOMEM, "ibm_setup: %s", cudaGetErrorString(e));
 cuda_err:
-    cudaFree(tiles);
-    cudaFree(d_err);
     ibm_geom_destroy(G);
     return ibm_cuda_check(e, "ibm_setup");
 }

@@ -126,3 +126,61 @@ def test_fused_smoothing_is_the_separate_half_sweeps(L, shape, bc, body):
     assert np.linalg.norm(a - b) <= 20 * 2.0 ** -24 * np.linalg.norm(b) * 8
     for v in s:
         v.close()
+
+
+@pytest.mark.parametrize("shape", [(70, 45, 37), (68, 44, 40), (33, 1, 5), (1, 1, 1), (260, 130, 128)])
+@pytest.mark.parametrize("kind", ["large", "small", "both", "none"])
+def test_classification_of_any_triangle_size_is_the_oracles(L, shape, kind):
+    """Flags, cut faces and positions bit for bit, with triangles of more tests than a warp takes (they go to the
+    block and, in a small soup, to slices of the grid), more hits than the list holds (found twice), several
+    warps and blocks of small ones, a flags array that starts off a word boundary and holds old bits, and grids
+    on both sides of the wide list tiles."""
+    import ctypes as C
+
+    import oracle
+    import workloads as W
+    nx, ny, nz = shape
+    rng = np.random.default_rng(12)
+    n = np.array(shape, float)
+    big = [(np.array([[-5, -5, 0.3], [2.5, -5, 0.4], [-5, 2.5, 0.5]]) * n),
+           (np.array([[0.2, -3, -3], [0.7, 4, -3], [0.3, -3, 4]]) * n), (np.array([[-1, 0.6, -1], [3, 0.55, -1], [-1, 0.62, 3]]) * n)]
+    small = W.random_soup(700, (0, 0, 0), shape, 2.0, seed=9)
+    small[::97] = np.nan
+    soup = {"large": np.array(big), "small": small, "both": np.concatenate([small, np.array(big)]), "none": small[:0]}[kind].astype(np.float32)
+    N = nx * ny * nz
+    g = L.make_grid(nx, ny, nz)
+    gp = L.GeomParams(1e-9, 0.0, 0, 0)
+    tri = torch.from_numpy(soup).cuda()
+    buf = torch.from_numpy(rng.integers(0, 256, N + 8).astype(np.uint8)).cuda()
+    before = buf.cpu().numpy()
+    ws = torch.empty(int(L.lib().ibm_classify_workspace_bytes(C.byref(g), len(soup))), dtype=torch.uint8, device="cuda")
+    cap = 3 * N
+    fid = torch.empty(cap, dtype=torch.int64, device="cuda")
+    lo, hi = (torch.empty(cap, dtype=torch.float64, device="cuda") for _ in range(2))
+    n_cut, n_tests = C.c_int64(), C.c_int64()
+    p = lambda t, o=0: C.c_void_p(t.data_ptr() + o)  # noqa: E731
+    assert L.lib().ibm_classify(C.byref(g), p(tri), len(soup), C.byref(gp), p(buf, 3), p(fid), p(lo), p(hi), cap, C.byref(n_cut),
+                                C.byref(n_tests), p(ws), ws.numel(), None) == 0, L.lib().ibm_last_error()
+    ref = oracle.Case(nx, ny, nz)
+    ref.classify(soup)
+    got = buf.cpu().numpy()
+    assert np.array_equal(got[3:3 + N], ref.flags & 63)
+    assert np.array_equal(got[:3], before[:3]) and np.array_equal(got[3 + N:], before[3 + N:])
+    k = n_cut.value
+    for t, r in zip((fid, lo, hi), ref.cut):
+        assert np.array_equal(t[:k].cpu().numpy(), r)
+    if kind == "large" and nx > 60:
+        assert k > 8 * (3 * len(soup) + 1) // 12 and n_tests.value > 3 * 1024
+    # set-up: region bits and records on the odd pointer, with old bits in the flags
+    buf |= torch.from_numpy((rng.integers(0, 4, N + 8) << 6).astype(np.uint8)).cuda()
+    h = C.c_void_p()
+    assert L.lib().ibm_setup(C.byref(g), C.byref(gp), p(buf, 3), p(fid), p(lo), p(hi), k, C.byref(h), None) == 0
+    ref.set_geometry(soup)
+    assert np.array_equal(buf.cpu().numpy()[3:3 + N], ref.flags)
+    L.lib().ibm_geom_destroy(h)
+    # a list that is not the flags' is refused: out of order, a face twice, a face beyond the grid
+    if k > 2:
+        for bad in ([1, 0], [0, 0], [2 ** 40, 1]):
+            f2 = fid.clone()
+            f2[:2] = torch.tensor([int(fid[b]) if b < 2 ** 40 else b for b in bad], device="cuda")
+            assert L.lib().ibm_setup(C.byref(g), C.byref(gp), p(buf, 3), p(f2), p(lo), p(hi), k, C.byref(h), None) == L.E_INVALID
