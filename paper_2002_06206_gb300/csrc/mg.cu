@@ -19,6 +19,7 @@
 //
 // Equations are solved in the unscaled form  sum_links g (x_N - x_P) - d x_P = dx^2 r.
 #include <cooperative_groups.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <type_traits>
@@ -28,21 +29,33 @@
 
 namespace cg = cooperative_groups;
 
+// Levels first .. nlev - 1 of the one-launch tail (see k_mg_tail), with each level's share of a block.
+struct MGTailLev {
+    int M, M0;               // unknowns; the first M0 have colour 0
+    int s0, s1;              // unknowns of either colour per block (all of them for the coarsest: block 0)
+    unsigned i0, i1;         // floor(2^32 / s) + 1
+    int x, b, t;             // byte offsets of its arrays in shared memory: iterate, right-hand side, residual,
+    int col, pc, g, dg, d;   // neighbours' places, their parents' places, conductances, 1 / dg, Dirichlet term,
+    int cv, ch;              // children of its unknowns (start | count << 18, places on the level below),
+    int oc, op, og;          // links of rows longer than MG_ELL: places, parents' places, conductances
+};
+struct MGTail {
+    MGTailLev t[IBM_MG_MAXLEV];
+    MGLev lev[IBM_MG_MAXLEV];
+    int first, nlev, coarse_sweeps;
+    int image;               // bytes of a block's constant arrays (the first in its shared memory)
+    const uint4* img;        // their image in global memory, block after block
+    double omega;
+};
+
 namespace {
 
 #define MG_TAIL_CTAS 8          // portable cluster size
 #define MG_TAIL_MAX (1LL << 14) // levels with at most this many unknowns run in the one-launch tail
 #define MG_COARSE_TARGET 1024   // coarsening stops at this many unknowns (or one position)
 #define MG_ELL 6                // links of an unknown kept in the padded rows (more: its CSR row)
-#define MG_SMEM_MAX 3500        // unknowns of a coarsest level that is solved in shared memory
 #define MG_MAXL 64              // distinct neighbours of a coarse unknown (more: the level is dropped)
 #define MG_L1L 24               // level 1: a 2x2x2 block has at most 24 links leaving it
-
-struct MGTail {
-    MGLev lev[IBM_MG_MAXLEV];
-    int first, nlev, coarse_sweeps;
-    double omega;
-};
 
 __device__ __forceinline__ unsigned flags_at(const Dom& D, long long P) { return D.flags ? (unsigned)D.flags[P] : 0u; }
 
@@ -1026,9 +1039,12 @@ __device__ __forceinline__ T row_sum(const MGLev& L, long long u, Fn f) {
         for (int e = L.rp[u]; e < L.rp[u + 1]; ++e) s += (T)L.g[e] * f(L.col[e]);
         return s;
     }
+    // padding points at the unknown itself with g = 0 (its value is always set): the reads do not wait for one another
+    T v[MG_ELL];
 #pragma unroll
-    for (int e = 0; e < MG_ELL; ++e)
-        if (g[e] != 0.f) s += (T)g[e] * f(c[e]);
+    for (int e = 0; e < MG_ELL; ++e) v[e] = f(c[e]);
+#pragma unroll
+    for (int e = 0; e < MG_ELL; ++e) s += (T)g[e] * v[e];
     return s;
 }
 
@@ -1085,11 +1101,11 @@ __device__ __forceinline__ void grestrict(const MGLev& F, const MGLev& C, long l
     }
 }
 
-// Coarsest level, one block: x = 0, then `sweeps` red-black passes and as many black-red (a symmetric
-// operator), __syncthreads between the passes; in global memory, or (gcoarsest_load first) with the rows, b
-// and x in shared memory: the passes are a chain of 4 * sweeps barriers, each about an L2 round trip otherwise.
+// Coarsest level, one block, in global memory: x = 0, then `sweeps` red-black passes and as many black-red (a
+// symmetric operator).
 template <class T>
-__device__ __forceinline__ void gcoarsest(const MGLev& L, int sweeps) {
+__global__ void __launch_bounds__(1024) k_gcoarsest(MGLev L, int sweeps, const SolveScal* sc) {
+    if (sc->done) return;
     T* x = (T*)L.x;
     for (long long u = threadIdx.x; u < L.M; u += blockDim.x) x[u] = (T)0;
     __syncthreads();
@@ -1098,61 +1114,6 @@ __device__ __forceinline__ void gcoarsest(const MGLev& L, int sweeps) {
         gsmooth<T>(L, (pass & 1) ^ half, threadIdx.x, blockDim.x);
         __syncthreads();
     }
-}
-
-template <class T>
-struct CoarseSmem {
-    T *x, *b;
-    float *eg, *invdg;
-    int16_t* ecol;
-    __host__ __device__ static size_t bytes(long long M) { return (size_t)M * (2 * sizeof(T) + MG_ELL * 6 + 4) + 16; }
-    __device__ __forceinline__ CoarseSmem(unsigned char* p, long long M) {
-        x = reinterpret_cast<T*>(p);
-        b = x + M;
-        eg = reinterpret_cast<float*>(b + M);
-        invdg = eg + MG_ELL * M;
-        ecol = reinterpret_cast<int16_t*>(invdg + M);
-    }
-};
-
-template <class T>
-__device__ __forceinline__ void gcoarsest_load(const MGLev& L, CoarseSmem<T>& S) {
-    for (int e = threadIdx.x; e < MG_ELL * (int)L.M; e += blockDim.x) {
-        S.ecol[e] = (int16_t)L.ecol[e];
-        S.eg[e] = L.eg[e];
-    }
-    for (int u = threadIdx.x; u < (int)L.M; u += blockDim.x) S.invdg[u] = L.invdg[u];
-}
-
-template <class T>
-__device__ __forceinline__ void gcoarsest_smem(const MGLev& L, CoarseSmem<T>& S, int sweeps) {
-    const int M = (int)L.M, M0 = (int)L.M0;
-    const T* bg = (const T*)L.b;
-    T* xg = (T*)L.x;
-    for (int u = threadIdx.x; u < M; u += blockDim.x) {
-        S.b[u] = bg[u];
-        S.x[u] = (T)0;
-    }
-    __syncthreads();
-    for (int pass = 0; pass < 4 * sweeps; ++pass) {
-        const int col = (pass & 1) ^ (pass / (2 * sweeps));
-        const int lo = col ? M0 : 0, hi = col ? M : M0;
-        for (int u = lo + threadIdx.x; u < hi; u += blockDim.x) {
-            T s = 0;
-            if (S.ecol[u] < 0) {
-                for (int e = L.rp[u]; e < L.rp[u + 1]; ++e) s += (T)L.g[e] * S.x[L.col[e]];
-            } else {
-#pragma unroll
-                for (int e = 0; e < MG_ELL; ++e) {
-                    const float g = S.eg[e * M + u];
-                    if (g != 0.f) s += (T)g * S.x[S.ecol[e * M + u]];
-                }
-            }
-            S.x[u] = (s - S.b[u]) * (T)S.invdg[u];
-        }
-        __syncthreads();
-    }
-    for (int u = threadIdx.x; u < M; u += blockDim.x) xg[u] = S.x[u];
 }
 
 template <class T>
@@ -1173,43 +1134,296 @@ __global__ void __launch_bounds__(256) k_gup(MGLev F, MGLev C, T omega, const So
     gup<T>(F, C, omega, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
-// The small levels first .. nlev-1 of a V-cycle in one launch: one cluster of MG_TAIL_CTAS blocks of
-// 1024 threads walks the descent (smoothing, restriction), the coarsest solve (block 0, in shared memory
-// where it fits, its rows loaded before the descent) and the ascent, with a cluster barrier (hardware,
-// release/acquire at cluster scope) between dependent passes.  These levels stay in L2; as separate kernels
-// each pass would cost a launch for a few microseconds of work.
+// The small levels first .. nlev-1 of a V-cycle in one launch of one cluster of MG_TAIL_CTAS blocks.  Every
+// block keeps its share of each level (half of it of either colour) in shared memory; neighbours are read
+// from the other blocks' shared memory and a cluster barrier (hardware, release/acquire at cluster scope)
+// separates dependent passes.  The coarsest level belongs to block 0 as a whole and is solved there with
+// barriers of the warps it needs, its rows in registers.  All of it is latency: five passes per level and 32
+// on the coarsest.  So everything that does not change between V-cycles (rows, parents of neighbours,
+// children, as places: block << 13 | index) is laid out once as an image of the blocks' shared memory and
+// copied in by 16-byte loads that are all in flight at once, and a row's reads do not wait for one another.
+// Levels of 8227, 1032 and 136 unknowns: 20 us (FP64 38), 48 us through L2 with device-wide fences and rows read
+// where they are used (FP64 80).
+#define MG_TAIL_NT 512
+#define MG_FAR 0xffffu          // first place of a row with more than MG_ELL links: start and count follow
+
+struct TailPlace {
+    MGTailLev t;
+    __device__ __forceinline__ unsigned operator()(int u) const {
+        const bool c = u >= t.M0;
+        const unsigned w = (unsigned)(c ? u - t.M0 : u), s = (unsigned)(c ? t.s1 : t.s0);
+        const unsigned r = __umulhi(w, c ? t.i1 : t.i0);
+        return r << 13 | ((c ? (unsigned)t.s0 : 0u) + w - r * s);
+    }
+};
+
 template <class T>
-__global__ void __launch_bounds__(1024) k_mg_tail(MGTail M, const SolveScal* sc) {
+struct TailLevel {
+    MGTailLev t;
+    unsigned char* sm;
+    int rank;
+    __device__ __forceinline__ TailLevel(const MGTail& M, int l, unsigned char* s, int r) : t(M.t[l]), sm(s), rank(r) {}
+    template <class V>
+    __device__ __forceinline__ V* arr(int o) const { return reinterpret_cast<V*>(sm + o); }
+    __device__ __forceinline__ T* x() const { return arr<T>(t.x); }
+    __device__ __forceinline__ T* b() const { return arr<T>(t.b); }
+    __device__ __forceinline__ T* tmp() const { return arr<T>(t.t); }
+    __device__ __forceinline__ T* dg() const { return arr<T>(t.dg); }
+    __device__ __forceinline__ T* d() const { return arr<T>(t.d); }
+    // the block's unknowns of colour c: local [base, base + n), global from lo
+    __device__ __forceinline__ void span(int c, int& base, int& n, int& lo) const {
+        const int s = c ? t.s1 : t.s0, all = c ? t.M - t.M0 : t.M0;
+        base = c ? t.s0 : 0;
+        const int f = rank * s;
+        n = f < all ? (all - f < s ? all - f : s) : 0;
+        lo = (c ? t.M0 : 0) + f;
+    }
+    // value of an array (a pointer into this block's shared memory) at a place
+    __device__ __forceinline__ T at(const T* a, unsigned place) const {
+        return *cg::this_cluster().map_shared_rank(const_cast<T*>(a) + (place & 8191u), place >> 13);
+    }
+    // sum over the links of local unknown i of g f(place of the neighbour, place of its parent)
+    template <bool PARENT, class Fn>
+    __device__ __forceinline__ T row(int i, Fn f) const {
+        const int S = t.s0 + t.s1;
+        unsigned c[MG_ELL], p[MG_ELL];
+        T g[MG_ELL], v[MG_ELL];
+#pragma unroll
+        for (int e = 0; e < MG_ELL; ++e) {
+            c[e] = arr<uint16_t>(t.col)[e * S + i];
+            p[e] = PARENT ? arr<uint16_t>(t.pc)[e * S + i] : 0u;
+            g[e] = arr<T>(t.g)[e * S + i];
+        }
+        if (c[0] == MG_FAR) {
+            T s = 0;
+            for (unsigned k = c[1]; k < c[1] + c[2]; ++k)
+                s += arr<T>(t.og)[k] * f((unsigned)arr<uint16_t>(t.oc)[k], PARENT ? (unsigned)arr<uint16_t>(t.op)[k] : 0u);
+            return s;
+        }
+        // padding points at the unknown itself with g = 0
+#pragma unroll
+        for (int e = 0; e < MG_ELL; ++e) v[e] = f(c[e], p[e]);
+        T s = 0;
+#pragma unroll
+        for (int e = 0; e < MG_ELL; ++e) s += g[e] * v[e];
+        return s;
+    }
+};
+
+// The constant arrays of every block's shares, in the layout of its shared memory (set-up; 32-bit cursors of
+// the long rows in `cur`, zero before).
+template <class T>
+__global__ void __launch_bounds__(256) k_tail_image(MGTail M, unsigned char* img, int* cur) {
+    const int rank = blockIdx.x, last = M.nlev - 1;
+    unsigned char* sm = img + (size_t)rank * M.image;
+    for (int l = M.first; l <= last; ++l) {
+        const TailLevel<T> A(M, l, sm, rank);
+        const MGLev& L = M.lev[l];
+        const TailPlace here{A.t}, up{M.t[l < last ? l + 1 : l]}, below{M.t[l > M.first ? l - 1 : l]};
+        const int S = A.t.s0 + A.t.s1;
+        int nch = 0;
+        for (int c = 0; c < 2; ++c) {
+            int base, n, lo;
+            A.span(c, base, n, lo);
+            const int k0 = l > M.first && n > 0 ? L.cp[lo] : 0, k1 = l > M.first && n > 0 ? L.cp[lo + n] : 0;
+            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                const int u = lo + i, r0 = L.rp[u], nr = L.rp[u + 1] - r0;
+                A.dg()[base + i] = (T)L.invdg[u];
+                if (sizeof(T) == 8) A.d()[base + i] = (T)L.d[u];
+                int at = 0;
+                if (nr > MG_ELL) {
+                    at = atomicAdd(&cur[rank * IBM_MG_MAXLEV + l], nr);
+                    for (int e = 0; e < nr; ++e) {
+                        const int w = L.col[r0 + e];
+                        A.template arr<uint16_t>(A.t.oc)[at + e] = (uint16_t)here(w);
+                        if (l < last) A.template arr<uint16_t>(A.t.op)[at + e] = (uint16_t)up(L.parent[w]);
+                        A.template arr<T>(A.t.og)[at + e] = (T)L.g[r0 + e];
+                    }
+                }
+                for (int e = 0; e < MG_ELL; ++e) {
+                    const int w = e < nr ? L.col[r0 + e] : u;
+                    unsigned q = here(w);
+                    if (nr > MG_ELL) q = e == 0 ? MG_FAR : (unsigned)(e == 1 ? at : nr);
+                    A.template arr<uint16_t>(A.t.col)[e * S + base + i] = (uint16_t)q;
+                    if (l < last) A.template arr<uint16_t>(A.t.pc)[e * S + base + i] = (uint16_t)up(L.parent[w]);
+                    A.template arr<T>(A.t.g)[e * S + base + i] = e < nr ? (T)L.g[r0 + e] : (T)0;
+                }
+                if (l > M.first) A.template arr<int>(A.t.cv)[base + i] = (nch + L.cp[u] - k0) | (L.cp[u + 1] - L.cp[u]) << 18;
+            }
+            for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x)
+                A.template arr<uint16_t>(A.t.ch)[nch + k - k0] = (uint16_t)below(L.ch[k]);
+            nch += k1 - k0;
+        }
+    }
+}
+
+template <class T>
+__global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant__ MGTail M, const SolveScal* sc) {
     if (sc->done) return;                       // the flag is uniform: set by an earlier kernel
     extern __shared__ __align__(16) unsigned char tail_smem[];
     cg::cluster_group cl = cg::this_cluster();
-    const long long t0 = (long long)cl.block_rank() * blockDim.x + threadIdx.x;
-    const long long nt = (long long)cl.num_blocks() * blockDim.x;
-    auto bar = [&]() {
-        __threadfence();
-        cl.sync();
+    const int rank = (int)cl.block_rank(), last = M.nlev - 1, tid = threadIdx.x;
+    {
+        const uint4* __restrict__ src = M.img + (size_t)rank * (M.image / 16);
+        uint4* dst = reinterpret_cast<uint4*>(tail_smem);
+        const int n = M.image / 16;
+        for (int q0 = tid; q0 < n; q0 += 8 * MG_TAIL_NT) {
+            uint4 v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q0 + q * MG_TAIL_NT < n) v[q] = src[q0 + q * MG_TAIL_NT];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q0 + q * MG_TAIL_NT < n) dst[q0 + q * MG_TAIL_NT] = v[q];
+        }
+        // b and x of the first level from global memory, x = 0 on the coarsest (also where padding is read)
+        const TailLevel<T> A(M, M.first, tail_smem, rank);
+        for (int c = 0; c < 2; ++c) {
+            int base, nn, lo;
+            A.span(c, base, nn, lo);
+            const T *bg = (const T*)M.lev[M.first].b, *xg = (const T*)M.lev[M.first].x;
+            for (int i = tid; i < nn; i += MG_TAIL_NT) {
+                A.b()[base + i] = bg[lo + i];
+                if (M.first < last) A.x()[base + i] = xg[lo + i];
+            }
+        }
+        const TailLevel<T> C(M, last, tail_smem, rank);
+        if (rank == 0)
+            for (int i = tid; i < C.t.M; i += MG_TAIL_NT) C.x()[i] = (T)0;
+    }
+    cl.sync();
+    // colour c of a level from its neighbours
+    auto smooth = [&](const TailLevel<T>& A, int c) {
+        int base, n, lo;
+        A.span(c, base, n, lo);
+        T* x = A.x();
+        for (int i = base + tid; i < base + n; i += MG_TAIL_NT)
+            x[i] = (A.template row<false>(i, [&](unsigned q, unsigned) { return A.at(x, q); }) - A.b()[i]) * A.dg()[i];
     };
-    const int last = M.nlev - 1;
-    const bool insm = M.lev[last].M <= MG_SMEM_MAX;
-    CoarseSmem<T> S(tail_smem, M.lev[last].M);
-    if (insm && cl.block_rank() == 0) gcoarsest_load<T>(M.lev[last], S);
     for (int l = M.first; l < last; ++l) {
-        gsmooth<T>(M.lev[l], 1, t0, nt);
-        bar();
-        grestrict<T>(M.lev[l], M.lev[l + 1], t0, nt);
-        bar();
+        const TailLevel<T> A(M, l, tail_smem, rank), C(M, l + 1, tail_smem, rank);
+        T* x = A.x();
+        smooth(A, 1);
+        cl.sync();
+        // residuals (FP64: of both colours, see grestrict)
+        for (int c = 0; c < (sizeof(T) == 8 ? 2 : 1); ++c) {
+            int base, n, lo;
+            A.span(c, base, n, lo);
+            for (int i = base + tid; i < base + n; i += MG_TAIL_NT) {
+                const T xu = x[i];
+                if (sizeof(T) == 8)
+                    A.tmp()[i] = A.b()[i] - (A.template row<false>(i, [&](unsigned q, unsigned) { return A.at(x, q) - xu; }) - A.d()[i] * xu);
+                else
+                    A.tmp()[i] = -A.template row<false>(i, [&](unsigned q, unsigned) { return A.at(x, q); });
+            }
+        }
+        cl.sync();
+        // b of the next level and its first half-sweep: four lanes per unknown
+        for (int c = 0; c < 2; ++c) {
+            int base, n, lo;
+            C.span(c, base, n, lo);
+            for (int q = 0; q < (4 * n + MG_TAIL_NT - 1) / MG_TAIL_NT; ++q) {
+                const int i = (tid + q * MG_TAIL_NT) >> 2;
+                T acc = 0;
+                if (i < n) {
+                    const int v = C.template arr<int>(C.t.cv)[base + i], k0 = v & 0x3ffff, nk = v >> 18;
+                    for (int k = tid & 3; k < nk; k += 4) acc += A.at(A.tmp(), C.template arr<uint16_t>(C.t.ch)[k0 + k]);
+                }
+                acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+                if (i < n && (tid & 3) == 0) {
+                    C.b()[base + i] = acc;
+                    if (l + 1 < last) C.x()[base + i] = -acc * C.dg()[base + i];
+                }
+            }
+        }
+        cl.sync();
     }
-    if (cl.block_rank() == 0) {
-        if (insm) gcoarsest_smem<T>(M.lev[last], S, M.coarse_sweeps);
-        else gcoarsest<T>(M.lev[last], M.coarse_sweeps);
+    if (rank == 0) {
+        // coarsest level: x = 0, then sweeps red-black passes and as many black-red (a symmetric operator)
+        const TailLevel<T> A(M, last, tail_smem, 0);
+        const int most = max(A.t.s0, A.t.s1), nth = min(MG_TAIL_NT, (most + 31) & ~31), S = A.t.s0 + A.t.s1;
+        T* x = A.x();
+        if (most <= MG_TAIL_NT && tid < nth) {
+            // one row of either colour per thread, in registers
+            unsigned q[2][MG_ELL];
+            T g[2][MG_ELL], b[2] = {0, 0}, dg[2] = {0, 0};
+            bool on[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                on[c] = tid < (c ? A.t.M - A.t.M0 : A.t.M0);
+                const int i = (c ? A.t.s0 : 0) + (on[c] ? tid : 0);
+                if (on[c]) {
+                    b[c] = A.b()[i];
+                    dg[c] = A.dg()[i];
+                }
+#pragma unroll
+                for (int e = 0; e < MG_ELL; ++e) {
+                    q[c][e] = on[c] ? A.template arr<uint16_t>(A.t.col)[e * S + i] : 0u;
+                    g[c][e] = on[c] ? A.template arr<T>(A.t.g)[e * S + i] : (T)0;
+                }
+            }
+            for (int pass = 0; pass < 2 * M.coarse_sweeps; ++pass) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    auto colour = [&](auto cc) {
+                        constexpr int c = decltype(cc)::value;
+                        if (!on[c]) return;
+                        const int i = (c ? A.t.s0 : 0) + tid;
+                        T s = 0;
+                        if (q[c][0] == MG_FAR) {
+                            s = A.template row<false>(i, [&](unsigned p, unsigned) { return x[p]; });
+                        } else {
+                            T v[MG_ELL];
+#pragma unroll
+                            for (int e = 0; e < MG_ELL; ++e) v[e] = x[q[c][e]];
+#pragma unroll
+                            for (int e = 0; e < MG_ELL; ++e) s += g[c][e] * v[e];
+                        }
+                        x[i] = (s - b[c]) * dg[c];
+                    };
+                    if (h ^ (pass >= M.coarse_sweeps ? 1 : 0)) colour(std::integral_constant<int, 1>{});
+                    else colour(std::integral_constant<int, 0>{});
+                    asm volatile("bar.sync 1, %0;" ::"r"(nth) : "memory");
+                }
+            }
+        } else if (most > MG_TAIL_NT) {
+            for (int pass = 0; pass < 4 * M.coarse_sweeps; ++pass) {
+                const int c = (pass & 1) ^ (pass / (2 * M.coarse_sweeps));
+                const int lo = c ? A.t.M0 : 0, hi = c ? A.t.M : A.t.M0;
+                for (int i = lo + tid; i < hi; i += MG_TAIL_NT)
+                    x[i] = (A.template row<false>(i, [&](unsigned p, unsigned) { return x[p]; }) - A.b()[i]) * A.dg()[i];
+                __syncthreads();
+            }
+        }
     }
-    bar();
+    cl.sync();
     for (int l = last - 1; l >= M.first; --l) {
-        gup<T>(M.lev[l], M.lev[l + 1], (T)M.omega, t0, nt);
-        bar();
-        gsmooth<T>(M.lev[l], 0, t0, nt);
-        if (l > M.first) bar();
+        const TailLevel<T> A(M, l, tail_smem, rank), C(M, l + 1, tail_smem, rank);
+        {
+            // colour 1: the neighbours count with their prolongated correction
+            int base, n, lo;
+            A.span(1, base, n, lo);
+            T* x = A.x();
+            const T om = (T)M.omega;
+            for (int i = base + tid; i < base + n; i += MG_TAIL_NT)
+                x[i] = (A.template row<true>(i, [&](unsigned q, unsigned p) { return A.at(x, q) + om * C.at(C.x(), p); }) - A.b()[i]) *
+                       A.dg()[i];
+        }
+        cl.sync();
+        smooth(A, 0);
+        if (l > M.first) cl.sync();
     }
+    {
+        const TailLevel<T> A(M, M.first, tail_smem, rank);
+        __syncthreads();
+        for (int c = 0; c < 2; ++c) {
+            int base, n, lo;
+            A.span(c, base, n, lo);
+            for (int i = tid; i < n; i += MG_TAIL_NT) ((T*)M.lev[M.first].x)[lo + i] = A.x()[base + i];
+        }
+    }
+    cl.sync();                                  // no block leaves while others may read its shared memory
 }
 
 // ---- transfer between the fine grid and level 1 -------------------------------------------------
@@ -1538,6 +1752,132 @@ int build_ell(MGLev& L) {
     return IBM_OK;
 }
 
+// Shares and shared-memory layout of the tail for levels first .. nlev - 1; its bytes per block (0: too large).
+long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
+    const int last = mg.nlev - 1, blocks = first < last ? MG_TAIL_CTAS : 1;
+    long long o = 0;
+    auto take = [&](long long bytes) {
+        const long long at = o;
+        o += (bytes + 15) & ~15LL;
+        return (int)at;
+    };
+    rc = IBM_OK;
+    for (int l = first; l <= last; ++l) {
+        const MGLev& L = mg.lev[l];
+        MGTailLev& t = M.t[l];
+        const long long M1 = L.M - L.M0;
+        if (L.M > 8191LL * MG_TAIL_CTAS || (l == last && L.M > 8191)) return 0;
+        t.M = (int)L.M;
+        t.M0 = (int)L.M0;
+        const int nb = l < last ? blocks : 1;
+        t.s0 = (int)((L.M0 + nb - 1) / nb);
+        t.s1 = (int)((M1 + nb - 1) / nb);
+        if (t.s0 < 1) t.s0 = 1;
+        if (t.s1 < 1) t.s1 = 1;
+        t.i0 = (unsigned)(0x100000000ULL / (unsigned)t.s0 + 1);      // s = 1 gives 2^32 + 1 = 1: see below
+        t.i1 = (unsigned)(0x100000000ULL / (unsigned)t.s1 + 1);
+        if ((t.s0 == 1 && L.M0 > 1) || (t.s1 == 1 && M1 > 1)) return 0;   // (a share of one: no such level is built)
+        if (t.s0 == 1) t.i0 = 0;
+        if (t.s1 == 1) t.i1 = 0;
+        const long long S = t.s0 + t.s1;
+        if (S > 8191) return 0;
+        t.col = take(S * 2 * MG_ELL);
+        t.pc = take(l < last ? S * 2 * MG_ELL : 0);
+        t.g = take(S * sb * MG_ELL);
+        t.dg = take(S * sb);
+        t.d = take(sb == 8 ? S * 8 : 0);
+        // the most children and the most links of long rows that any block holds
+        int32_t *cp = nullptr, *rp = (int32_t*)malloc(sizeof(int32_t) * (L.M + 1));
+        if (l > first) cp = (int32_t*)malloc(sizeof(int32_t) * (L.M + 1));
+        cudaError_t e = cudaSuccess;
+        if (rp) e = cudaMemcpy(rp, L.rp, sizeof(int32_t) * (L.M + 1), cudaMemcpyDeviceToHost);
+        if (cp && e == cudaSuccess) e = cudaMemcpy(cp, L.cp, sizeof(int32_t) * (L.M + 1), cudaMemcpyDeviceToHost);
+        long long children = 0, links = 0;
+        bool fits = rp && (l == first || cp) && e == cudaSuccess;
+        for (int r = 0; fits && r < nb; ++r) {
+            long long nc = 0, nl = 0;
+            for (int c = 0; c < 2; ++c) {
+                const long long s1 = c ? t.s1 : t.s0, end = c ? L.M : L.M0, u0 = (c ? L.M0 : 0) + r * s1;
+                for (long long u = u0; u < u0 + s1 && u < end; ++u) {
+                    const int n = rp[u + 1] - rp[u];
+                    if (n > MG_ELL) nl += n;
+                    if (cp) {
+                        nc += cp[u + 1] - cp[u];
+                        fits = fits && cp[u + 1] - cp[u] < (1 << 13);
+                    }
+                }
+            }
+            children = nc > children ? nc : children;
+            links = nl > links ? nl : links;
+        }
+        if (!rp || (l > first && !cp)) rc = ibm_fail(IBM_E_NOMEM, "multigrid set-up: host allocation");
+        else if (e != cudaSuccess) rc = ibm_cuda_check(e, "multigrid set-up: tail");
+        free(rp);
+        free(cp);
+        if (!fits || children >= (1 << 18) || links >= 65536) return 0;
+        t.cv = take(l > first ? S * 4 : 0);
+        t.ch = take(children * 2);
+        t.oc = take(links * 2);
+        t.op = take(l < last ? links * 2 : 0);
+        t.og = take(links * sb);
+    }
+    M.image = (int)o;
+    for (int l = first; l <= last; ++l) {
+        MGTailLev& t = M.t[l];
+        const long long S = t.s0 + t.s1;
+        t.x = take(S * sb);
+        t.b = take(S * sb);
+        t.t = take(l < last ? S * sb : 0);
+    }
+    return o <= 220 * 1024 ? o : 0;
+}
+
+// The tail starts at the first level whose shares fit, of those with at most MG_TAIL_MAX unknowns; a coarsest
+// level too large for one block's shared memory runs from global memory (tail_smem = 0).
+int tail_plan(MG& mg, int sb) {
+    const int last = mg.nlev - 1;
+    mg.tail_first = last;
+    mg.tail_smem = 0;
+    if (last < 1) return IBM_OK;
+    mg.tail = (MGTail*)calloc(1, sizeof(MGTail));
+    if (!mg.tail) return ibm_fail(IBM_E_NOMEM, "multigrid set-up: host allocation");
+    for (int l = 0; l < IBM_MG_MAXLEV; ++l) mg.tail->lev[l] = mg.lev[l];
+    mg.tail->nlev = mg.nlev;
+    mg.tail->coarse_sweeps = mg.coarse_sweeps;
+    mg.tail->omega = mg.omega;
+    for (int l = 1; l <= last; ++l) {
+        if (l < last && mg.lev[l].M > MG_TAIL_MAX) continue;
+        int rc;
+        const long long bytes = tail_layout(mg, *mg.tail, l, sb, rc);
+        if (rc) return rc;
+        if (bytes > 0) {
+            mg.tail->first = mg.tail_first = l;
+            mg.tail_smem = (int)bytes;
+            break;
+        }
+    }
+    if (mg.tail_smem > 0) {
+        const int blocks = mg.tail_first < last ? MG_TAIL_CTAS : 1;
+        int* cur = nullptr;
+        MG_ALLOCB(mg.tail_img, (size_t)blocks * mg.tail->image);
+        MG_ALLOC(cur, MG_TAIL_CTAS * IBM_MG_MAXLEV);
+        cudaError_t e = cudaMemset(cur, 0, sizeof(int) * MG_TAIL_CTAS * IBM_MG_MAXLEV);
+        if (e == cudaSuccess) e = cudaMemset(mg.tail_img, 0, (size_t)blocks * mg.tail->image);
+        if (e == cudaSuccess) {
+            mg.tail->img = (const uint4*)mg.tail_img;
+            if (sb == 8) k_tail_image<double><<<blocks, 256>>>(*mg.tail, (unsigned char*)mg.tail_img, cur);
+            else k_tail_image<float><<<blocks, 256>>>(*mg.tail, (unsigned char*)mg.tail_img, cur);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        cudaFree(cur);
+        if (e != cudaSuccess) return ibm_cuda_check(e, "multigrid set-up: tail");
+    }
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    return IBM_OK;
+}
+
 int build_level1(const LesCtx& c, MGLev& L, int sb, SetupTmp& t) {
     const Dom& D = c.D;
     L.px = (D.nx + 1) / 2;
@@ -1637,27 +1977,18 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
 template <class T>
 static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStream_t s, int& launches) {
     const T om = (T)mg.omega;
-    const int last = mg.nlev - 1;
-    int tf = last;
-    for (int l = 1; l < last; ++l)
-        if (mg.lev[l].M <= MG_TAIL_MAX) { tf = l; break; }
+    const int last = mg.nlev - 1, tf = mg.tail_first;
     for (int l = 1; l < tf; ++l) {
         const MGLev& L = mg.lev[l];
         k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, sc);
         k_grestrict<T><<<lin_blocks(4 * mg.lev[l + 1].M), 256, 0, s>>>(L, mg.lev[l + 1], sc);
         launches += 2;
     }
-    {
-        MGTail M;
-        for (int l = 0; l < IBM_MG_MAXLEV; ++l) M.lev[l] = mg.lev[l];
-        M.first = tf;
-        M.nlev = mg.nlev;
-        M.coarse_sweeps = mg.coarse_sweeps;
-        M.omega = mg.omega;
+    if (mg.tail_smem > 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(tf < last ? MG_TAIL_CTAS : 1);
-        cfg.blockDim = dim3(1024);
-        cfg.dynamicSmemBytes = mg.lev[last].M <= MG_SMEM_MAX ? CoarseSmem<T>::bytes(mg.lev[last].M) : 0;
+        cfg.blockDim = dim3(MG_TAIL_NT);
+        cfg.dynamicSmemBytes = mg.tail_smem;
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1666,9 +1997,11 @@ static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStrea
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        IBM_CUDA(cudaLaunchKernelEx(&cfg, k_mg_tail<T>, M, (const SolveScal*)sc));
-        ++launches;
+        IBM_CUDA(cudaLaunchKernelEx(&cfg, k_mg_tail<T>, *mg.tail, (const SolveScal*)sc));
+    } else {
+        k_gcoarsest<T><<<1, 1024, 0, s>>>(mg.lev[last], mg.coarse_sweeps, sc);
     }
+    ++launches;
     for (int l = tf - 1; l >= 1; --l) {
         const MGLev& L = mg.lev[l];
         k_gup<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, mg.lev[l + 1], om, sc);
@@ -1713,6 +2046,10 @@ static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z,
 void mg_free(MG& mg) {
     for (int l = 1; l < IBM_MG_MAXLEV; ++l) free_level(mg.lev[l]);
     cudaFree(mg.z2);
+    cudaFree(mg.tail_img);
+    mg.tail_img = nullptr;
+    free(mg.tail);
+    mg.tail = nullptr;
     mg.z2 = nullptr;
     mg.nlev = 1;
 }
@@ -1743,8 +2080,7 @@ int mg_setup(const LesCtx& c, MG& mg, int sb) {
         if (r2 > 0) break;
         mg.nlev = l + 2;
     }
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CoarseSmem<float>::bytes(MG_SMEM_MAX)));
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CoarseSmem<double>::bytes(MG_SMEM_MAX)));
+    if ((rc = tail_plan(mg, sb))) return rc;
     fused_plan(c, mg, sb);
     if (mg.fused) {
         MG_ALLOCB(mg.z2, c.D.N * 4);

@@ -57,12 +57,16 @@ struct MGLev {
     void* b;             // right-hand side (working precision)
     void* x;             // iterate
 };
+struct MGTail;
 struct MG {
     int nlev;
     int sweeps;          // red-black passes before and after the coarse correction on the fine grid
     int coarse_sweeps;   // symmetric sweeps on the coarsest level
     double omega;        // coarse-correction factor, 0 < omega < 2
     MGLev lev[IBM_MG_MAXLEV];
+    struct MGTail* tail; // small levels in one launch: first level, shared memory per block (0: not used) and layout
+    int tail_first, tail_smem;
+    void* tail_img;      // the blocks' constant shared memory
     // fused fine-grid passes (FP32, two sweeps, nx a multiple of 4, no periodic axis)
     int allow_fused;     // les_params.mg_passes == 0
     int fused;           // 1: the fused kernels apply to this grid and configuration
