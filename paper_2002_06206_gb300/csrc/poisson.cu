@@ -121,11 +121,12 @@ __global__ void __launch_bounds__(256) k_cg_dir_spmv(Dom D, const T* __restrict_
                                                      T* __restrict__ pnew, T* __restrict__ q, T idx2, SolveScal* sc,
                                                      double* partials, unsigned* counter, int pcg) {
     if (sc->done) return;
-    const T beta = sc->restart ? (T)0 : (T)(pcg ? sc->rz / sc->rz_old : sc->rr / sc->rr_old);
+    const bool first = sc->restart != 0;        // p_old holds nothing then (it may hold anything)
+    const T beta = first ? (T)0 : (T)(pcg ? sc->rz / sc->rz_old : sc->rr / sc->rr_old);
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
     const int kb = blockIdx.z * IBM_KU;
     const bool active = i < D.nx && j < D.ny;
-    auto pv = [&](long long c) { return r[c] + beta * pold[c]; };
+    auto pv = [&](long long c) { return first ? r[c] : r[c] + beta * pold[c]; };
     T part = 0;       // per-thread partial sum in the working precision (FP64 arithmetic is slow here)
 #pragma unroll
     for (int u = 0; u < IBM_KU; ++u) {

@@ -44,9 +44,11 @@ __global__ void __launch_bounds__(256, 4) k_cg_dir_spmv_x4(Dom D, const float* _
                                                         float* __restrict__ q, float idx2, SolveScal* sc,
                                                         double* partials, unsigned* counter, int pcg) {
     if (sc->done) return;
-    const float beta = sc->restart ? 0.f : (float)(pcg ? sc->rz / sc->rz_old : sc->rr / sc->rr_old);
+    const bool first = sc->restart != 0;        // p_old holds nothing then (it may hold anything)
+    const float beta = first ? 0.f : (float)(pcg ? sc->rz / sc->rz_old : sc->rr / sc->rr_old);
     float part = 0.f;
-    auto pv = [&](long long c) { return r[c] + beta * pold[c]; };
+    auto old4 = [&](long long c) { return first ? make_float4(0.f, 0.f, 0.f, 0.f) : ld4(pold + c); };
+    auto pv = [&](long long c) { return first ? r[c] : r[c] + beta * pold[c]; };
     X4_TILE_LOOP_BEGIN
 #pragma unroll
     for (int u = 0; u < IBM_KU; ++u) {
@@ -54,14 +56,14 @@ __global__ void __launch_bounds__(256, 4) k_cg_dir_spmv_x4(Dom D, const float* _
         if (!active || k >= D.nz) continue;
         const long long P = i0 + (long long)D.sy * j + D.sz * k;
         const unsigned fl4 = flags4(D, P);
-        const float4 r4 = ld4(r + P), o4 = ld4(pold + P);
+        const float4 r4 = ld4(r + P), o4 = old4(P);
         float pc[4] = {r4.x + beta * o4.x, r4.y + beta * o4.y, r4.z + beta * o4.z, r4.w + beta * o4.w};
         float qv[4];
         if (plain_chunk(D, i0, j, k, fl4)) {
-            const float4 ym = ld4(r + P - D.sy), ymo = ld4(pold + P - D.sy);
-            const float4 yp = ld4(r + P + D.sy), ypo = ld4(pold + P + D.sy);
-            const float4 zm = ld4(r + P - D.sz), zmo = ld4(pold + P - D.sz);
-            const float4 zp = ld4(r + P + D.sz), zpo = ld4(pold + P + D.sz);
+            const float4 ym = ld4(r + P - D.sy), ymo = old4(P - D.sy);
+            const float4 yp = ld4(r + P + D.sy), ypo = old4(P + D.sy);
+            const float4 zm = ld4(r + P - D.sz), zmo = old4(P - D.sz);
+            const float4 zp = ld4(r + P + D.sz), zpo = old4(P + D.sz);
             const float xl = pv(P - 1), xr = pv(P + 4);
 #pragma unroll
             for (int m = 0; m < 4; ++m) {

@@ -184,3 +184,51 @@ def test_classification_of_any_triangle_size_is_the_oracles(L, shape, kind):
             f2 = fid.clone()
             f2[:2] = torch.tensor([int(fid[b]) if b < 2 ** 40 else b for b in bad], device="cuda")
             assert L.lib().ibm_setup(C.byref(g), C.byref(gp), p(buf, 3), p(f2), p(lo), p(hi), k, C.byref(h), None) == L.E_INVALID
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("nx", [36, 37])
+def test_the_first_direction_of_a_solve_is_its_residual(L, nx, prec):
+    """What the workspaces hold before the first solve is not read: they are made from memory that held NaN."""
+    N = nx * 20 * 12
+    g = L.make_grid(nx, 20, 12)
+    b = torch.from_numpy(np.random.default_rng(2).standard_normal(N)).cuda()
+    p = torch.zeros(N, dtype=torch.float64, device="cuda")
+    nan = [torch.full((1 << k,), float("nan"), device="cuda") for k in range(12, 24)]
+    torch.cuda.synchronize()
+    del nan
+    torch.cuda.empty_cache()
+    sol = L.Solver(g, 0.01, 0.2, CHANNEL, precision=prec, precond=0)
+    assert sol.solve(b, p, 1e-6, 1000, 0).status == 0
+    assert bool(torch.isfinite(p).all())
+    sol.close()
+
+
+@pytest.mark.parametrize("shape", [(4, 1, 3), (4, 17, 5), (36, 33, 12), (132, 16, 9), (256, 47, 70)])
+@pytest.mark.parametrize("bc", [CHANNEL, (1, 2, 0, 0, 0, 0), (0, 0, 3, 4, 1, 2), (2, 2, 1, 1, 2, 1)])
+@pytest.mark.parametrize("body", [False, True])
+def test_cg_on_quads_of_cells_takes_the_iterations_of_fp64(L, shape, bc, body):
+    """Conjugate gradients on 16-byte quads against FP64 cell by cell, one cycle to 1e-4: a neighbour taken from the
+    wrong place leaves a true residual above the target, which costs another cycle.  Rounding alone moves the count by
+    a few."""
+    import workloads as W
+    nx, ny, nz = shape
+    N = nx * ny * nz
+    g = L.make_grid(nx, ny, nz)
+    geo = None
+    if body:
+        soup = W.random_soup(60, (0.5, 0.5, 0.5), (nx - 0.5, ny - 0.5, nz - 0.5), 4.0, seed=8)
+        geo = L.Geometry(g, torch.from_numpy(soup).cuda())
+    rng = np.random.default_rng(6)
+    x = torch.from_numpy(rng.standard_normal(N)).cuda()
+    its = []
+    for prec in (0, 1):
+        sol = L.Solver(g, 0.01, 0.2, bc, precision=prec, geometry=geo, precond=0)
+        b = torch.empty_like(x)
+        sol.apply(x, b)
+        p = torch.zeros_like(x)
+        st = sol.solve(b, p, 1e-4, 20000, 0)
+        assert st.status == 0
+        its.append(st.iters)
+        sol.close()
+    assert abs(its[1] - its[0]) <= 2 + 0.1 * its[0], its
