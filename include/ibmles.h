@@ -80,10 +80,10 @@ typedef struct {
     int32_t mom_max_iter;/* Crank-Nicolson: BiCGStab iteration cap per step (0 = 200) */
     double mom_tol;      /* Crank-Nicolson: stop at ||r|| <= mom_tol ||dt L(u^n)|| (0 = 1e-6 in
                             FP32_REFINE64 mode, 1e-10 in FP64 mode) */
-    int32_t mg_passes;   /* multigrid fine-grid passes: 0 = fused where the grid allows (FP32, mg_sweeps 2,
-                            nx a multiple of 4, no periodic axis: the four half-sweeps before the coarse
-                            correction and the restriction in one pass, the four after it and (r, z) in
-                            another), 1 = one kernel per half-sweep.  Same V-cycle. */
+    int32_t mg_passes;   /* multigrid fine-grid passes: 0 = fused where the grid allows (FP32, mg_sweeps 2, no
+                            periodic axis: the four half-sweeps before the coarse correction and the
+                            restriction in one pass, the four after it and (r, z) in another), 1 = one
+                            kernel per half-sweep.  Same V-cycle. */
     int32_t reserved;
 } les_params;
 

@@ -283,26 +283,29 @@ struct FTile {
     }
 };
 
-// A thread's column: constants of the march.
+// A thread's column: constants of the march (NI = 3: nx a multiple of 4, else 4).
+template <int NI>
 struct FCol {
     int xl;                 // quad within the row of the tile
     int gx, gy;             // global coordinates of its first cell
     bool in0, in1;          // rows inside the domain
     bool own0, own1;        // rows of the tile's own cells
-    float inv[2][3];        // 1 / dg of the first, the middle two and the last cell of each row, 0 outside
-    int dg[2][3];
+    float inv[2][NI];       // 1 / dg per row and cell, 0 outside the domain
+    int dg[2][NI];
+    // a quad of a grid with nx a multiple of 4 lies inside or outside as a whole: its middle cells share a value
+    static __device__ __forceinline__ constexpr int at(int m) { return NI == 4 ? m : (m == 0 ? 0 : (m == 3 ? 2 : 1)); }
 };
 
-template <int LX>
-__device__ __forceinline__ FCol ftp_column(const Dom& D, int tx, int ty, int ntx, int nty) {
+template <int LX, int NI>
+__device__ __forceinline__ FCol<NI> ftp_column(const Dom& D, int tx, int ty, int ntx, int nty) {
     using T = FTile<LX>;
-    FCol c;
+    FCol<NI> c;
     c.xl = threadIdx.x % LX;
     const int rp = threadIdx.x / LX;
     const int X0 = tx * (T::W - 8), Y0 = ty * (T::H - 8);
     c.gx = X0 + 4 * c.xl;
     c.gy = Y0 + 2 * rp;
-    const bool inx = c.gx < D.nx;                           // nx is a multiple of 4: a quad is inside or outside
+    const bool inx = c.gx < D.nx;
     c.in0 = inx && c.gy < D.ny;
     c.in1 = inx && c.gy + 1 < D.ny;
     const bool ox = (tx == 0 || c.xl > 0) && (tx == ntx - 1 || c.xl < LX - 1);
@@ -315,11 +318,12 @@ __device__ __forceinline__ FCol ftp_column(const Dom& D, int tx, int ty, int ntx
         const int y = c.gy + r;
         const int d = 6 + (y == 0 ? term(2) : 0) + (y == D.ny - 1 ? term(3) : 0);
         const bool in = r ? c.in1 : c.in0;
-        c.dg[r][0] = in ? d + (c.gx == 0 ? term(0) : 0) : 0;
-        c.dg[r][1] = in ? d : 0;
-        c.dg[r][2] = in ? d + (c.gx + 4 == D.nx ? term(1) : 0) : 0;
 #pragma unroll
-        for (int m = 0; m < 3; ++m) c.inv[r][m] = c.dg[r][m] > 0 ? 1.f / (float)c.dg[r][m] : 0.f;
+        for (int m = 0; m < NI; ++m) {
+            const int x = c.gx + (NI == 3 && m == 2 ? 3 : m);
+            c.dg[r][m] = in && x < D.nx ? d + (x == 0 ? term(0) : 0) + (x == D.nx - 1 ? term(1) : 0) : 0;
+            c.inv[r][m] = c.dg[r][m] > 0 ? 1.f / (float)c.dg[r][m] : 0.f;
+        }
     }
     return c;
 }
@@ -333,8 +337,8 @@ __device__ __forceinline__ float ftp_open_sum(unsigned f, float xm, float xp, fl
 }
 
 // x neighbours of the cells D0, D0 + 2 of row 0 and 1 - D0, 3 - D0 of row 1 that lie in another quad.
-template <int LX, int D0>
-__device__ __forceinline__ void ftp_xside(const FCol& c, const float (&zc)[2][4], float& e0, float& e1) {
+template <int LX, int D0, int NI>
+__device__ __forceinline__ void ftp_xside(const FCol<NI>& c, const float (&zc)[2][4], float& e0, float& e1) {
     const float a = D0 == 0 ? __shfl_up_sync(0xffffffffu, zc[0][3], 1) : __shfl_down_sync(0xffffffffu, zc[0][0], 1);
     const float b = D0 == 0 ? __shfl_down_sync(0xffffffffu, zc[1][0], 1) : __shfl_up_sync(0xffffffffu, zc[1][3], 1);
     const bool first = c.xl == 0, last = c.xl == LX - 1;
@@ -352,27 +356,27 @@ __device__ __forceinline__ void ftp_pair(const float (&zr)[4], float e, float ym
 
 // One half-sweep on a thread's cells of one plane: cells D0, D0 + 2 of row 0 and 1 - D0, 3 - D0 of row 1.
 // yb, yt: the rows below and above (another thread's); r0, r1: the right-hand side at the updated cells.
-template <int LX, int D0>
-__device__ __forceinline__ void ftp_sweep(const FCol& c, float (&zc)[2][4], const float (&zm)[2][4], const float (&zp)[2][4],
+template <int LX, int D0, int NI>
+__device__ __forceinline__ void ftp_sweep(const FCol<NI>& c, float (&zc)[2][4], const float (&zm)[2][4], const float (&zp)[2][4],
                                           float2 yb, float2 yt, float2 r0, float2 r1, float scale, bool general,
                                           const uint2* fl, int zadj, const float* rcp) {
     float e0, e1;
-    ftp_xside<LX, D0>(c, zc, e0, e1);
+    ftp_xside<LX, D0, NI>(c, zc, e0, e1);
     constexpr int D1 = 1 - D0;
     float v0[2], v1[2];
     if (!general) {
         ftp_pair<D0>(zc[0], e0, yb.x, yb.y, zc[1][D0], zc[1][D0 + 2], zm[0], zp[0],
                      [&](int m, float a, float b, float p, float q, float l, float u, int w) {
-                         v0[w] = fmaf(-scale, w ? r0.y : r0.x, ((a + b) + (p + q)) + (l + u)) * c.inv[0][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+                         v0[w] = fmaf(-scale, w ? r0.y : r0.x, ((a + b) + (p + q)) + (l + u)) * c.inv[0][FCol<NI>::at(m)];
                      });
         ftp_pair<D1>(zc[1], e1, zc[0][D1], zc[0][D1 + 2], yt.x, yt.y, zm[1], zp[1],
                      [&](int m, float a, float b, float p, float q, float l, float u, int w) {
-                         v1[w] = fmaf(-scale, w ? r1.y : r1.x, ((a + b) + (p + q)) + (l + u)) * c.inv[1][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+                         v1[w] = fmaf(-scale, w ? r1.y : r1.x, ((a + b) + (p + q)) + (l + u)) * c.inv[1][FCol<NI>::at(m)];
                      });
     } else {
         const uint2 ff = *fl;
         auto cell = [&](int row, int m, float s, unsigned f, float r) {
-            const int d = c.dg[row][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+            const int d = c.dg[row][FCol<NI>::at(m)];
             return fmaf(-scale, r, s) * rcp[d ? d + zadj - __popc(f & 63u) : 0];
         };
         ftp_pair<D0>(zc[0], e0, yb.x, yb.y, zc[1][D0], zc[1][D0 + 2], zm[0], zp[0],
@@ -407,6 +411,29 @@ __device__ __forceinline__ void ftp_copy(float (&a)[2][4], const float (&b)[2][4
 __device__ __forceinline__ void ftp_set(float (&a)[2][4], float4 x, float4 y) {
     a[0][0] = x.x; a[0][1] = x.y; a[0][2] = x.z; a[0][3] = x.w;
     a[1][0] = y.x; a[1][1] = y.y; a[1][2] = y.z; a[1][3] = y.w;
+}
+
+// A quad of a row: 16 bytes where rows start on 16-byte boundaries (NI = 3), cell by cell within the domain.
+template <int NI>
+__device__ __forceinline__ float4 ftp_load(const float* p, int left) {
+    if (NI == 3) return *reinterpret_cast<const float4*>(p);
+    return make_float4(p[0], left > 1 ? p[1] : 0.f, left > 2 ? p[2] : 0.f, left > 3 ? p[3] : 0.f);
+}
+template <int NI>
+__device__ __forceinline__ unsigned ftp_load_flags(const uint8_t* p, int left) {
+    if (NI == 3) return *reinterpret_cast<const unsigned*>(p);
+    return (unsigned)p[0] | (left > 1 ? (unsigned)p[1] << 8 : 0u) | (left > 2 ? (unsigned)p[2] << 16 : 0u) |
+           (left > 3 ? (unsigned)p[3] << 24 : 0u);
+}
+template <int NI>
+__device__ __forceinline__ void ftp_store(float* p, int left, const float (&z)[4]) {
+    if (NI == 3) {
+        *reinterpret_cast<float4*>(p) = make_float4(z[0], z[1], z[2], z[3]);
+        return;
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+        if (m < left) p[m] = z[m];
 }
 
 // Shared memory of a block and the thread's places in it.
@@ -456,13 +483,14 @@ __device__ __forceinline__ int ftp_zadj(const Dom& D, int p) {
 // Pre-smoothing (from z = 0, colours 0, 1, 0, 1) and the restriction of  scale r - A z  to the parts of the
 // level-1 blocks.  Writes z on its chunk's planes [k0, k1) and b_1.  The last half-sweep leaves the residual
 // of colour 1 zero, so only colour 0 is evaluated (one plane behind the last half-sweep).
-template <int LX>
+template <int LX, int NI>
 __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* __restrict__ rg, float* __restrict__ zg,
                                                             float scale, MGLev C1, int kchunk, const SolveScal* sc) {
     if (sc->done) return;
     extern __shared__ __align__(16) unsigned char ftp_raw[];
     const FShared<LX> S = ftp_shared<LX>(ftp_raw);
-    const FCol c = ftp_column<LX>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    const FCol<NI> c = ftp_column<LX, NI>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    const int left = D.nx - c.gx;       // cells from the quad's first to the end of the row
     const int k0 = blockIdx.z * kchunk, k1 = min(D.nz, k0 + kchunk);
     const int tlo = max(0, k0 - 4), thi = k1 + 3;
     const int row0 = c.gx + D.sy * c.gy;
@@ -477,12 +505,12 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
         if (t >= D.nz) return;
         const long long P = row0 + D.sz * t;
         if (c.in0) {
-            nr0 = *reinterpret_cast<const float4*>(rg + P);
-            if (D.flags) nf0 = *reinterpret_cast<const unsigned*>(D.flags + P);
+            nr0 = ftp_load<NI>(rg + P, left);
+            if (D.flags) nf0 = ftp_load_flags<NI>(D.flags + P, left);
         }
         if (c.in1) {
-            nr1 = *reinterpret_cast<const float4*>(rg + P + D.sy);
-            if (D.flags) nf1 = *reinterpret_cast<const unsigned*>(D.flags + P + D.sy);
+            nr1 = ftp_load<NI>(rg + P + D.sy, left);
+            if (D.flags) nf1 = ftp_load_flags<NI>(D.flags + P + D.sy, left);
         }
     };
     fetch(tlo);
@@ -510,7 +538,7 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
             for (int row = 0; row < 2; ++row)
 #pragma unroll
                 for (int w = 0; w < 2; ++w) {
-                    const int m = (row ? 1 - D0 : D0) + 2 * w, mi = m == 0 ? 0 : (m == 3 ? 2 : 1);
+                    const int m = (row ? 1 - D0 : D0) + 2 * w, mi = FCol<NI>::at(m);
                     float iv = c.inv[row][mi];
                     if (gen & 1u) {
                         const unsigned f = (row ? ft.y : ft.x) >> (8 * m);
@@ -528,7 +556,7 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
             if (p >= tlo && p < D.nz) {
                 const int sl = ftp_back(slot, k);
                 const bool g = (gen >> k) & 1u;
-                ftp_sweep<LX, D0>(c, Z[k], Z[k + 1], Z[k - 1], S.below(k - 1, pr), S.above(k - 1, pr), S.rhs(sl, 0, k & 1),
+                ftp_sweep<LX, D0, NI>(c, Z[k], Z[k + 1], Z[k - 1], S.below(k - 1, pr), S.above(k - 1, pr), S.rhs(sl, 0, k & 1),
                                   S.rhs(sl, 1, k & 1), scale, g, S.f + sl * FTP_NT + threadIdx.x, g ? ftp_zadj(D, p) : 0, S.rcp);
                 S.publish(k, pw, Z[k], D0);
             }
@@ -537,8 +565,8 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
         const int tw = t - 3;
         if (tw >= k0 && tw < k1) {
             float* zo = zg + row0 + D.sz * tw;
-            if (c.own0) *reinterpret_cast<float4*>(zo) = make_float4(Z[3][0][0], Z[3][0][1], Z[3][0][2], Z[3][0][3]);
-            if (c.own1) *reinterpret_cast<float4*>(zo + D.sy) = make_float4(Z[3][1][0], Z[3][1][1], Z[3][1][2], Z[3][1][3]);
+            if (c.own0) ftp_store<NI>(zo, left, Z[3][0]);
+            if (c.own1) ftp_store<NI>(zo + D.sy, left, Z[3][1]);
         }
         // residual of colour 0 on plane t - 4
         const int tr = t - 4;
@@ -547,12 +575,13 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
             const bool g = (gen >> 4) & 1u;
             const float2 yb = S.below(3, pr), yt = S.above(3, pr), r0 = S.rhs(sl, 0, 0), r1 = S.rhs(sl, 1, 0);
             float e0, e1;
-            ftp_xside<LX, D0>(c, Z[4], e0, e1);
+            ftp_xside<LX, D0, NI>(c, Z[4], e0, e1);
             const uint2 ff = g ? S.f[sl * FTP_NT + threadIdx.x] : make_uint2(0u, 0u);
             const int zadj = g ? ftp_zadj(D, tr) : 0;
             float res[2][2];
             auto cell = [&](int row, int m, float a, float b, float p, float q, float l, float u, float r) {
-                int d = c.dg[row][m == 0 ? 0 : (m == 3 ? 2 : 1)];
+                int d = c.dg[row][FCol<NI>::at(m)];
+                if (NI == 4 && d == 0) return 0.f;                // outside the domain
                 float s;
                 if (!g) {
                     s = ((a + b) + (p + q)) + (l + u);
@@ -583,27 +612,29 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
             }
             if ((D0 == 1 || lastp) && c.own0) {
                 const long long q = (c.gx >> 1) + (long long)C1.px * ((c.gy >> 1) + (long long)C1.py * (tr >> 1));
-                const int2 o = *reinterpret_cast<const int2*>(C1.off + q);
+                const bool two = NI == 3 || left > 2;    // the second position lies in the domain
+                const int2 o = NI == 3 ? *reinterpret_cast<const int2*>(C1.off + q) : make_int2(C1.off[q], two ? C1.off[q + 1] : 0);
                 const bool odd = D0 == 1;                // both planes of the block are there
                 // a warp without a cut link in the two planes: whole blocks
                 if (!((gen >> 4) & 1u) && !(odd && ((gen >> 5) & 1u))) {
                     put_b1<float>(C1, o.x, odd ? (er[0][0] + er[1][0]) + (res[0][0] + res[1][0]) : er[0][0] + er[1][0]);
-                    put_b1<float>(C1, o.y, odd ? (er[0][1] + er[1][1]) + (res[0][1] + res[1][1]) : er[0][1] + er[1][1]);
+                    if (two) put_b1<float>(C1, o.y, odd ? (er[0][1] + er[1][1]) + (res[0][1] + res[1][1]) : er[0][1] + er[1][1]);
                 } else {
                     const long long Pe = row0 + D.sz * (tr & ~1);
                     unsigned fe[2], fo[2];
-                    fe[0] = D.flags ? *reinterpret_cast<const unsigned*>(D.flags + Pe) : 0u;
-                    fe[1] = D.flags && c.in1 ? *reinterpret_cast<const unsigned*>(D.flags + Pe + D.sy) : 0u;
-                    fo[0] = D.flags && odd ? *reinterpret_cast<const unsigned*>(D.flags + Pe + D.sz) : 0u;
-                    fo[1] = D.flags && odd && c.in1 ? *reinterpret_cast<const unsigned*>(D.flags + Pe + D.sz + D.sy) : 0u;
+                    fe[0] = D.flags ? ftp_load_flags<NI>(D.flags + Pe, left) : 0u;
+                    fe[1] = D.flags && c.in1 ? ftp_load_flags<NI>(D.flags + Pe + D.sy, left) : 0u;
+                    fo[0] = D.flags && odd ? ftp_load_flags<NI>(D.flags + Pe + D.sz, left) : 0u;
+                    fo[1] = D.flags && odd && c.in1 ? ftp_load_flags<NI>(D.flags + Pe + D.sz + D.sy, left) : 0u;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
+                        if (h == 1 && !two) break;
                         unsigned fl[8], in = 0;
                         float rv[8];
 #pragma unroll
                         for (int m = 0; m < 8; ++m) {
                             const int di = m & 1, dj = (m >> 1) & 1, dk = m >> 2;
-                            const bool ok = (dj == 0 || c.in1) && (dk == 0 || odd);
+                            const bool ok = (dj == 0 || c.in1) && (dk == 0 || odd) && (NI == 3 || 2 * h + di < left);
                             fl[m] = ok ? ((dk ? fo[dj] : fe[dj]) >> (8 * (2 * h + di))) & 0xffu : 0u;
                             in |= (ok ? 1u : 0u) << m;
                             // colour 0: x + y + z even within the block
@@ -638,14 +669,15 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
 // Post-smoothing (colours 1, 0, 1, 0) of the iterate the coarse correction left, read from zin (an array
 // this pass does not write: neighbouring tiles read each other's cells), into z; then (r, z) over the grid:
 // rz_old = rz, rz = (r, z).
-template <int LX>
+template <int LX, int NI>
 __global__ void __launch_bounds__(FTP_NT, 1) k_mg_post_fused(Dom D, const float* __restrict__ rg, const float* __restrict__ zin,
                                                              float* __restrict__ zg, float scale, int kchunk, SolveScal* sc,
                                                              double* partials, unsigned* counter) {
     if (sc->done) return;
     extern __shared__ __align__(16) unsigned char ftp_raw[];
     const FShared<LX> S = ftp_shared<LX>(ftp_raw);
-    const FCol c = ftp_column<LX>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    const FCol<NI> c = ftp_column<LX, NI>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    const int left = D.nx - c.gx;       // cells from the quad's first to the end of the row
     const int k0 = blockIdx.z * kchunk, k1 = min(D.nz, k0 + kchunk);
     const int tlo = max(0, k0 - 4), thi = k1 + 2;
     const int row0 = c.gx + D.sy * c.gy;
@@ -659,20 +691,20 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_post_fused(Dom D, const float*
         if (t >= D.nz) return;
         const long long P = row0 + D.sz * t;
         if (c.in0) {
-            nr0 = *reinterpret_cast<const float4*>(rg + P);
-            if (D.flags) nf0 = *reinterpret_cast<const unsigned*>(D.flags + P);
+            nr0 = ftp_load<NI>(rg + P, left);
+            if (D.flags) nf0 = ftp_load_flags<NI>(D.flags + P, left);
         }
         if (c.in1) {
-            nr1 = *reinterpret_cast<const float4*>(rg + P + D.sy);
-            if (D.flags) nf1 = *reinterpret_cast<const unsigned*>(D.flags + P + D.sy);
+            nr1 = ftp_load<NI>(rg + P + D.sy, left);
+            if (D.flags) nf1 = ftp_load_flags<NI>(D.flags + P + D.sy, left);
         }
     };
     auto fetch_z = [&](int t) {
         nz0 = nz1 = zero4;
         if (t >= D.nz) return;
         const long long P = row0 + D.sz * t;
-        if (c.in0) nz0 = *reinterpret_cast<const float4*>(zin + P);
-        if (c.in1) nz1 = *reinterpret_cast<const float4*>(zin + P + D.sy);
+        if (c.in0) nz0 = ftp_load<NI>(zin + P, left);
+        if (c.in1) nz1 = ftp_load<NI>(zin + P + D.sy, left);
     };
 #pragma unroll
     for (int q = 1; q < 5; ++q) ftp_zero(Z[q]);
@@ -707,7 +739,7 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_post_fused(Dom D, const float*
             if (p >= tlo && p < D.nz) {
                 const int sl = ftp_back(slot, k);
                 const bool g = (gen >> k) & 1u;
-                ftp_sweep<LX, D0>(c, Z[k], Z[k + 1], k ? Z[k > 0 ? k - 1 : 0] : zn, S.below(k, pr), S.above(k, pr),
+                ftp_sweep<LX, D0, NI>(c, Z[k], Z[k + 1], k ? Z[k > 0 ? k - 1 : 0] : zn, S.below(k, pr), S.above(k, pr),
                                   S.rhs(sl, 0, (k + 1) & 1), S.rhs(sl, 1, (k + 1) & 1), scale, g,
                                   S.f + sl * FTP_NT + threadIdx.x, g ? ftp_zadj(D, p) : 0, S.rcp);
                 if (k < 3) S.publish(k + 1, pw, Z[k], D0);
@@ -719,12 +751,12 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_post_fused(Dom D, const float*
             float* zo = zg + row0 + D.sz * tf;
             // row 0 of plane t - 3: colour 0 holds the cells D0, D0 + 2; row 1 the others
             if (c.own0) {
-                *reinterpret_cast<float4*>(zo) = make_float4(Z[3][0][0], Z[3][0][1], Z[3][0][2], Z[3][0][3]);
+                ftp_store<NI>(zo, left, Z[3][0]);
                 const float2 a = S.rhs(sl, 0, 0), b = S.rhs(sl, 0, 1);
                 part += (a.x * Z[3][0][D0] + a.y * Z[3][0][D0 + 2]) + (b.x * Z[3][0][1 - D0] + b.y * Z[3][0][3 - D0]);
             }
             if (c.own1) {
-                *reinterpret_cast<float4*>(zo + D.sy) = make_float4(Z[3][1][0], Z[3][1][1], Z[3][1][2], Z[3][1][3]);
+                ftp_store<NI>(zo + D.sy, left, Z[3][1]);
                 const float2 a = S.rhs(sl, 1, 0), b = S.rhs(sl, 1, 1);
                 part += (a.x * Z[3][1][1 - D0] + a.y * Z[3][1][3 - D0]) + (b.x * Z[3][1][D0] + b.y * Z[3][1][D0 + 2]);
             }
@@ -1652,7 +1684,7 @@ void fused_plan(const LesCtx& c, MG& mg, int sb) {
     const Dom& D = c.D;
     bool per = false;
     for (int f = 0; f < 6; ++f) per = per || D.bc[f] == IBM_BC_PERIODIC;
-    mg.fused = mg.allow_fused && sb == 4 && mg.sweeps == 2 && mg.nlev > 1 && !per && D.nx % 4 == 0;
+    mg.fused = mg.allow_fused && sb == 4 && mg.sweeps == 2 && mg.nlev > 1 && !per;
     if (!mg.fused) return;
     long long best = -1;
     for (int lx = 16; lx <= 32; lx *= 2) {
@@ -1661,7 +1693,7 @@ void fused_plan(const LesCtx& c, MG& mg, int sb) {
         for (int ch = 1; ch <= 64; ++ch) {
             int k = (D.nz + ch - 1) / ch;
             k += k & 1;
-            if (k < 4 && ch > 1) break;
+            if (k < 2 && ch > 1) break;
             const long long nchunk = (D.nz + k - 1) / k;
             const long long waves = (tx * ty * nchunk + IBM_NSM - 1) / IBM_NSM;
             const long long cost = waves * (k + 8);
@@ -2011,6 +2043,15 @@ static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStrea
     return IBM_OK;
 }
 
+// Calls f(quads along x of a tile, values per row of a column) with the plan's constants.
+template <class Fn>
+static void fused_dispatch(const LesCtx& c, const MG& mg, Fn f) {
+    using std::integral_constant;
+    const bool vec = c.D.nx % 4 == 0;
+    if (mg.flx == 16) vec ? f(integral_constant<int, 16>{}, integral_constant<int, 3>{}) : f(integral_constant<int, 16>{}, integral_constant<int, 4>{});
+    else vec ? f(integral_constant<int, 32>{}, integral_constant<int, 3>{}) : f(integral_constant<int, 32>{}, integral_constant<int, 4>{});
+}
+
 // V-cycle with the fused fine-grid passes: pre-smoothing + restriction, the coarse levels,
 // prolongation, post-smoothing + (r, z).
 static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z, SolveScal* sc, cudaStream_t s) {
@@ -2019,8 +2060,11 @@ static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z,
     const MGLev& L1 = mg.lev[1];
     int launches = 0;
     prof_begin(c.prof, PS_MG_FINE, s);
-    if (mg.flx == 16) k_mg_pre_fused<16><<<mg.fgrid, FTP_NT, FTile<16>::smem(), s>>>(c.D, r, z2, scale, L1, mg.fz_chunk, sc);
-    else k_mg_pre_fused<32><<<mg.fgrid, FTP_NT, FTile<32>::smem(), s>>>(c.D, r, z2, scale, L1, mg.fz_chunk, sc);
+    auto pre = [&](auto lx, auto ni) {
+        constexpr int LX = decltype(lx)::value, NI = decltype(ni)::value;
+        k_mg_pre_fused<LX, NI><<<mg.fgrid, FTP_NT, FTile<LX>::smem(), s>>>(c.D, r, z2, scale, L1, mg.fz_chunk, sc);
+    };
+    fused_dispatch(c, mg, pre);
     prof_end(c.prof, PS_MG_FINE, s);
     ++launches;
     prof_begin(c.prof, PS_MG_COARSE, s);
@@ -2028,14 +2072,16 @@ static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z,
     if (rc) return rc;
     prof_end(c.prof, PS_MG_COARSE, s);
     prof_begin(c.prof, PS_MG_TRANSFER, s);
-    k_mg_prolong0_x4<<<lin_blocks((c.D.nx / 4) * (long long)L1.py * L1.pz), 256, 0, s>>>(c.D, z2, L1, (float)mg.omega, sc);
+    if (x4_ok(c)) k_mg_prolong0_x4<<<lin_blocks((c.D.nx / 4) * (long long)L1.py * L1.pz), 256, 0, s>>>(c.D, z2, L1, (float)mg.omega, sc);
+    else k_mg_prolong0<float><<<lin_blocks(L1.P), 256, 0, s>>>(c.D, z2, L1, (float)mg.omega, sc);
     prof_end(c.prof, PS_MG_TRANSFER, s);
     ++launches;
     prof_begin(c.prof, PS_MG_FINE, s);
-    if (mg.flx == 16)
-        k_mg_post_fused<16><<<mg.fgrid, FTP_NT, FTile<16>::smem(), s>>>(c.D, r, z2, z, scale, mg.fz_chunk, sc, c.partials, c.counter);
-    else
-        k_mg_post_fused<32><<<mg.fgrid, FTP_NT, FTile<32>::smem(), s>>>(c.D, r, z2, z, scale, mg.fz_chunk, sc, c.partials, c.counter);
+    auto post = [&](auto lx, auto ni) {
+        constexpr int LX = decltype(lx)::value, NI = decltype(ni)::value;
+        k_mg_post_fused<LX, NI><<<mg.fgrid, FTP_NT, FTile<LX>::smem(), s>>>(c.D, r, z2, z, scale, mg.fz_chunk, sc, c.partials, c.counter);
+    };
+    fused_dispatch(c, mg, post);
     prof_end(c.prof, PS_MG_FINE, s);
     ++launches;
     IBM_LAUNCHED("mg_vcycle (fused)");
@@ -2084,10 +2130,15 @@ int mg_setup(const LesCtx& c, MG& mg, int sb) {
     fused_plan(c, mg, sb);
     if (mg.fused) {
         MG_ALLOCB(mg.z2, c.D.N * 4);
-        IBM_CUDA(cudaFuncSetAttribute(k_mg_pre_fused<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<16>::smem()));
-        IBM_CUDA(cudaFuncSetAttribute(k_mg_pre_fused<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<32>::smem()));
-        IBM_CUDA(cudaFuncSetAttribute(k_mg_post_fused<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<16>::smem()));
-        IBM_CUDA(cudaFuncSetAttribute(k_mg_post_fused<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<32>::smem()));
+        cudaError_t e = cudaSuccess;
+        auto attr = [&](auto lx, auto ni) {
+            constexpr int LX = decltype(lx)::value, NI = decltype(ni)::value;
+            e = cudaFuncSetAttribute(k_mg_pre_fused<LX, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<LX>::smem());
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_mg_post_fused<LX, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FTile<LX>::smem());
+        };
+        fused_dispatch(c, mg, attr);
+        if (e != cudaSuccess) return ibm_cuda_check(e, "multigrid set-up: fused passes");
     }
     return IBM_OK;
 }

@@ -67,7 +67,7 @@ struct MG {
     struct MGTail* tail; // small levels in one launch: first level, shared memory per block (0: not used) and layout
     int tail_first, tail_smem;
     void* tail_img;      // the blocks' constant shared memory
-    // fused fine-grid passes (FP32, two sweeps, nx a multiple of 4, no periodic axis)
+    // fused fine-grid passes (FP32, two sweeps, no periodic axis)
     int allow_fused;     // les_params.mg_passes == 0
     int fused;           // 1: the fused kernels apply to this grid and configuration
     int flx;             // quads along x of a tile (16 or 32)

@@ -102,11 +102,14 @@ def test_correction_subtracts_fp64_pressures_of_any_size(L, shape, prec, bc):
 
 @pytest.mark.parametrize("body", [True, False])
 @pytest.mark.parametrize("shape,bc", [((20, 10, 9), CHANNEL), ((64, 64, 8), (2, 2, 4, 2, 2, 1)), ((68, 66, 31), CHANNEL),
-                                      ((132, 33, 12), (1, 2, 2, 3, 4, 2)), ((1036, 5, 3), CHANNEL), ((244, 130, 40), (3, 3, 2, 3, 3, 3))])
+                                      ((132, 33, 12), (1, 2, 2, 3, 4, 2)), ((1036, 5, 3), CHANNEL), ((244, 130, 40), (3, 3, 2, 3, 3, 3)),
+                                      ((37, 20, 11), CHANNEL), ((66, 33, 12), (2, 2, 4, 2, 2, 1)), ((131, 61, 47), CHANNEL),
+                                      ((1, 70, 40), (3, 3, 2, 3, 3, 3)), ((183, 9, 30), (1, 2, 2, 3, 4, 2))])
 def test_fused_smoothing_is_the_separate_half_sweeps(L, shape, bc, body):
     """One V-cycle with the fused passes against the one-kernel-per-half-sweep form on the same vector: tiles that
-    end at, just past and far from the domain faces, one and several z-chunks, every outflow face.  Both run the
-    same FP32 updates: about 20 dependent roundings of 2^-24 per value and cycle."""
+    end at, just past and far from the domain faces, rows of every length modulo 4, one and several z-chunks,
+    every outflow face.  Both run the same FP32 updates: about 20 dependent roundings of 2^-24 per value and
+    cycle."""
     import workloads as W
     nx, ny, nz = shape
     rng = np.random.default_rng(4)
