@@ -265,6 +265,7 @@ extern "C" int les_create(const ibm_grid* g, const les_params* p, const ibm_geom
     S->c.nlaunch = &S->nlaunch;
     {
         int rc1 = flux_kernels_setup();
+        if (!rc1) rc1 = stencil4_setup();
         if (!rc1) rc1 = build_general_list(S->c, 0);
         if (rc1) {
             free_state(S);

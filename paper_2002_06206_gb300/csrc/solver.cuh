@@ -142,6 +142,7 @@ int launch_forces(const LesCtx& c, const float* tri, long long ntri, const doubl
 
 // stencil4.cu: FP32 fine-grid kernels with 4 cells per thread (nx a multiple of 4)
 bool x4_ok(const LesCtx& c);
+int stencil4_setup();      // once per process that solves: shared memory of the kernels above 48 KB
 void launch_cg_dir_spmv_x4(const LesCtx& c, const float* src, const float* pold, float* pnew, float* q, float idx2,
                            SolveScal* sc, int pcg, cudaStream_t s);
 void launch_mg_smooth0_x4(const LesCtx& c, const float* r, float* z, float scale, int col, int zero, int fin,
