@@ -1605,68 +1605,81 @@ __global__ void __launch_bounds__(256) k_mg_restrict0_x4(Dom D, const float* __r
     }
 }
 
-// FP32 prolongation with nx a multiple of 4, same layout as k_mg_restrict0_x4.
-__global__ void __launch_bounds__(256) k_mg_prolong0_x4(Dom D, float* __restrict__ z, MGLev C, float omega,
+// FP32 prolongation with nx a multiple of 4: a thread takes two positions of level 1 along x, two rows of two planes.
+// Flags, offsets and the iterate are loaded together, so that the coarse values are the only loads that wait for
+// others, and a warp without a cut link skips the search for parts.  Bound by HBM:
+// 8 bytes per cell and the coarse values; at 512 x 256 x 256, where the iterate is partly in L2, 92 -> 46 us.
+__global__ void __launch_bounds__(256, 4) k_mg_prolong0_x4(Dom D, float* __restrict__ z, MGLev C, float omega,
                                                         const SolveScal* sc) {
     if (sc->done) return;
     const float* __restrict__ xc = (const float*)C.x;
-    const int px = D.nx / 4;
+    const unsigned px = (unsigned)D.nx / 4;
     const long long npairs = (long long)px * C.py * C.pz;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < npairs;
          t += (long long)gridDim.x * blockDim.x) {
-        const unsigned tu = (unsigned)t, rq = tu / (unsigned)px;
-        const int xp = (int)(tu - rq * (unsigned)px), Y = (int)(rq % (unsigned)C.py), Z = (int)(rq / (unsigned)C.py);
-        const int i0 = 4 * xp;
-        unsigned f4[2][2];
-        unsigned rows = 0;
+        const unsigned tu = (unsigned)t, rq = tu / px;
+        const int xp = (int)(tu - rq * px), Y = (int)(rq % (unsigned)C.py), Z = (int)(rq / (unsigned)C.py);
+        const long long P0 = 4 * xp + (long long)D.sy * (2 * Y) + D.sz * (2 * Z);
+        const bool y2 = 2 * Y + 1 < D.ny, z2 = 2 * Z + 1 < D.nz;
+        float4 zv[2][2];
+        unsigned f4[2][2], any = 0u;
 #pragma unroll
         for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
             for (int dj = 0; dj < 2; ++dj) {
-                const int j = 2 * Y + dj, k = 2 * Z + dk;
-                const bool ok = j < D.ny && k < D.nz;
-                f4[dk][dj] = ok ? flags4(D, i0 + (long long)D.sy * j + D.sz * k) : 0u;
-                rows |= (ok ? 1u : 0u) << (2 * dk + dj);
+                const bool ok = (dj == 0 || y2) && (dk == 0 || z2);
+                const long long P = P0 + dj * (long long)D.sy + dk * D.sz;
+                zv[dk][dj] = ok ? ld4(z + P) : make_float4(0.f, 0.f, 0.f, 0.f);
+                f4[dk][dj] = ok ? flags4(D, P) : 0u;
+                any |= f4[dk][dj];
             }
-        float w[2][8];     // [position][cell]: the coarse value each fine cell receives
+        const int2 o = *reinterpret_cast<const int2*>(C.off + 2 * xp + (long long)C.px * (Y + (long long)C.py * Z));
+        if (!any) {
+            const float a = omega * xc[o.x], b = omega * xc[o.y];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            unsigned fl[8];
-            unsigned in = 0;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                const int di = m & 1, dj = (m >> 1) & 1, dk = m >> 2;
-                fl[m] = (f4[dk][dj] >> (8 * (2 * h + di))) & 0xffu;
-                in |= ((rows >> (2 * dk + dj)) & 1u) << m;
+            for (int q = 0; q < 4; ++q) {
+                float4& v = zv[q >> 1][q & 1];
+                v.x += a;
+                v.y += a;
+                v.z += b;
+                v.w += b;
             }
-            int part[8];
-            const int np = fine_parts(D, fl, in, part);
-            const int o = C.off[(2 * xp + h) + (long long)C.px * (Y + (long long)C.py * Z)];
-            float v[8];
+        } else {
+            const unsigned rows = 1u | (y2 ? 2u : 0u) | (z2 ? 4u : 0u) | (y2 && z2 ? 8u : 0u);
 #pragma unroll
-            for (int s = 0; s < 8; ++s) v[s] = s < np ? xc[o + s] : 0.f;
+            for (int h = 0; h < 2; ++h) {
+                unsigned fl[8], in = 0;
 #pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                float a = v[0];
+                for (int m = 0; m < 8; ++m) {
+                    const int di = m & 1, dj = (m >> 1) & 1, dk = m >> 2;
+                    fl[m] = (f4[dk][dj] >> (8 * (2 * h + di))) & 0xffu;
+                    in |= ((rows >> (2 * dk + dj)) & 1u) << m;
+                }
+                int part[8];
+                const int np = fine_parts(D, fl, in, part);
+                const int oo = h ? o.y : o.x;
+                float v[8];
 #pragma unroll
-                for (int s = 1; s < 8; ++s) a = part[m] == s ? v[s] : a;
-                w[h][m] = a;
+                for (int s = 0; s < 8; ++s) v[s] = s < np ? xc[oo + s] : 0.f;
+#pragma unroll
+                for (int m = 0; m < 8; ++m) {
+                    const int di = m & 1, dj = (m >> 1) & 1, dk = m >> 2;
+                    float a = v[0];
+#pragma unroll
+                    for (int s = 1; s < 8; ++s) a = part[m] == s ? v[s] : a;
+                    float4& u = zv[dk][dj];
+                    if (h == 0 && di == 0) u.x += omega * a;
+                    else if (h == 0) u.y += omega * a;
+                    else if (di == 0) u.z += omega * a;
+                    else u.w += omega * a;
+                }
             }
         }
 #pragma unroll
         for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
-            for (int dj = 0; dj < 2; ++dj) {
-                if (!((rows >> (2 * dk + dj)) & 1u)) continue;
-                const long long P = i0 + (long long)D.sy * (2 * Y + dj) + D.sz * (2 * Z + dk);
-                float4 z4 = ld4(z + P);
-                const int m0 = 2 * dj + 4 * dk;
-                z4.x += omega * w[0][m0];
-                z4.y += omega * w[0][m0 + 1];
-                z4.z += omega * w[1][m0];
-                z4.w += omega * w[1][m0 + 1];
-                st4(z + P, z4);
-            }
+            for (int dj = 0; dj < 2; ++dj)
+                if ((dj == 0 || y2) && (dk == 0 || z2)) st4(z + P0 + dj * (long long)D.sy + dk * D.sz, zv[dk][dj]);
     }
 }
 
