@@ -11,7 +11,7 @@
 #include "solver.cuh"
 
 #ifndef IBM_FLUX_GEN_MINB
-#define IBM_FLUX_GEN_MINB 4   // the general-cell flux kernels gather from global memory: occupancy pays for small spills
+#define IBM_FLUX_GEN_MINB 5
 #endif
 #ifndef IBM_FLUX_MINB
 #define IBM_FLUX_MINB 3
@@ -70,39 +70,13 @@ __global__ void __launch_bounds__(256) k_csm(Dom D, const T* __restrict__ u, T* 
     nut[P] = C * delta2 * sqrt(SS);
 }
 
-// Advected value on the face of P towards side s along axis a: the central value blended with a
-// fraction gam of QUICK (6 upwind + 3 downwind - far upwind)/8, the far upwind value read across the
-// upwind cell's outer link.  L and R are the lower and upper cells of the face, so both cells of a face
-// compute the same value.  Cut faces and domain faces keep the central value.
-template <class T>
-__device__ __forceinline__ T face_adv(const Dom& D, const T* __restrict__ u, int c, long long P, const int x[3],
-                                      unsigned fl, int a, int s, T uP, T uN, T Uf, T gam) {
-    const T central = (T)0.5 * (uP + uN);
-    if (gam == (T)0) return central;
-    long long off;
-    if ((fl & (1u << (2 * a + (s > 0)))) || !nb_offset(D, a, s, x[a], off)) return central;
-    const int n = a == 0 ? D.nx : (a == 1 ? D.ny : D.nz);
-    const long long Nn = P + off;
-    const long long Lc = s > 0 ? P : Nn, Rc = s > 0 ? Nn : P;
-    const int xo = x[a] + s < 0 ? n - 1 : (x[a] + s >= n ? 0 : x[a] + s);
-    const int xL = s > 0 ? x[a] : xo, xR = s > 0 ? xo : x[a];
-    const T uL = s > 0 ? uP : uN, uR = s > 0 ? uN : uP;
-    T q;
-    if (Uf >= (T)0) {
-        const T far = vel_across(D, u, c, Lc, xL, D.flags ? (unsigned)D.flags[Lc] : 0u, a, -1);
-        q = ((T)6 * uL + (T)3 * uR - far) / (T)8;
-    } else {
-        const T far = vel_across(D, u, c, Rc, xR, D.flags ? (unsigned)D.flags[Rc] : 0u, a, +1);
-        q = ((T)6 * uR + (T)3 * uL - far) / (T)8;
-    }
-    return ((T)1 - gam) * central + gam * q;
-}
-
-// L(u) of a cell per unit volume: flux-form advection with the face velocity U (central value
-// blended with QUICK), diffusion with nu + nu_t, the transpose part of the SGS stress divergence.
-// flux_general applies the ghost and boundary rules of vel_across on every link; the tiled fast path
-// evaluates the same formulas for a cell where they reduce to direct reads (fast_cell).  With D.hom set
-// the ghost values lose their wall and inflow velocities, which gives the linear part of L.
+// L(u) of a cell per unit volume: flux-form advection with the face velocity U, diffusion with nu + nu_t, the
+// transpose part of the SGS stress divergence.  The advected value is the central one blended with a fraction gam
+// of QUICK, (6 upwind + 3 downwind - far upwind) / 8, the far upwind value read across the upwind cell's outer
+// link; cut faces and domain faces keep the central value.  flux_axis applies the ghost and boundary rules of
+// vel_across on every link; the tiled fast path evaluates the same formulas for a cell where they reduce to direct
+// reads (fast_cell).  With D.hom set the ghost values lose their wall and inflow velocities, which gives the linear
+// part of L.
 
 // The cell and its six neighbours (across periodic seams too) have no cut link: its flux then needs
 // only neighbour values and the domain-boundary ghosts, which the tiles below hold.
@@ -498,57 +472,103 @@ __device__ __forceinline__ void fast_tile_march(const Dom& D, const FaceLayout& 
 template <class T>
 size_t fast_tile_smem() { return (size_t)(FT_RING * FT_NV * FT_PL + 2 * 3 * (FT_FXN + FT_FYN)) * sizeof(T); }
 
+// Values of the components a, a + 1, a + 2 (mod 3) that cell P reads across its link (a, s): vel_across for all
+// three, with the kind of the link found once.  v: the cell's own values.
 template <class T>
-__device__ __forceinline__ void flux_general(const Dom& D, const FaceLayout& F, const T* __restrict__ u,
-                                             const T* __restrict__ U, const T* __restrict__ nut, long long P, int i,
-                                             int j, int k, T nu, T gam, T (&h)[3]) {
+__device__ __forceinline__ void vel3_across(const Dom& D, const T* const (&u)[3], const int (&cm)[3], long long P, int xa,
+                                            unsigned fl, int a, int s, const T (&v)[3], T (&o)[3]) {
+    const int bit = link_bit(a, s);
+    long long off;
+    if (fl & (1u << bit)) {
+        const LinkRec& r = link_record(D, P, fl, bit);
+        const T cp = (T)r.c_p, ci = D.hom ? (T)0 : (T)r.c_ib, co = r.opp >= 0 ? (T)r.c_o : (T)0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            o[c] = (D.hom ? (T)0 : ci * (T)r.uib[cm[c]]) + cp * v[c];
+            if (r.opp >= 0) o[c] = o[c] + co * u[c][r.opp];
+        }
+    } else if (nb_offset(D, a, s, xa, off)) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) o[c] = u[c][P + off];
+    } else {
+        const int k = D.bc[bit];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (k == IBM_BC_INFLOW) o[c] = (D.hom ? (T)0 : (T)2 * (T)D.u_in[cm[c]]) - v[c];
+            else if (k == IBM_BC_OUTFLOW) o[c] = v[c];
+            else o[c] = k == IBM_BC_SLIP && c > 0 ? v[c] : -v[c];
+        }
+    }
+}
+
+// Both faces of cell P along axis a, any links: contributions to the components a, a + 1, a + 2 (mod 3), which
+// uP receives at the cell.
+template <class T>
+__device__ __forceinline__ void flux_axis(const Dom& D, const FaceLayout& F, const T* __restrict__ u,
+                                          const T* __restrict__ U, const T* __restrict__ nut, long long P,
+                                          const int (&x)[3], int a, T nu, T gam, T (&h)[3], T (&uP)[3]) {
     const T inv2dx = (T)0.5 * dom_idx<T>(D), invdx = dom_idx<T>(D);
-    const int n[3] = {D.nx, D.ny, D.nz};
+    const int b = a == 2 ? 0 : a + 1, d = b == 2 ? 0 : b + 1, cm[3] = {a, b, d};
+    const T* const uc[3] = {u + a * D.N, u + b * D.N, u + d * D.N};
+    const int xa = a == 0 ? x[0] : (a == 1 ? x[1] : x[2]), xb = a == 0 ? x[1] : (a == 1 ? x[2] : x[0]),
+              xd = a == 0 ? x[2] : (a == 1 ? x[0] : x[1]), na = a == 0 ? D.nx : (a == 1 ? D.ny : D.nz);
     const unsigned fl = flags_at(D, P);
-    const int x[3] = {i, j, k};
     const T nutP = nut[P];
-    h[0] = h[1] = h[2] = (T)0;
-        T GP[3][3];
-        grad_at(D, u, P, x, fl, inv2dx, GP);
+    const long long f0 = F.index(a, x[0], x[1], x[2]);
+    const long long fs = a == 0 ? 1 : (a == 1 ? F.dim[1][0] : (long long)F.dim[2][0] * F.dim[2][1]);
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+    for (int c = 0; c < 3; ++c) {
+        uP[c] = uc[c][P];
+        h[c] = (T)0;
+    }
+    // d u_a / d b and d u_a / d d at a cell with coordinates (.., xb, xd)
+    auto cross = [&](long long Q, unsigned f, T& gb, T& gd) {
+        gb = (vel_across(D, u, a, Q, xb, f, b, +1) - vel_across(D, u, a, Q, xb, f, b, -1)) * inv2dx;
+        gd = (vel_across(D, u, a, Q, xd, f, d, +1) - vel_across(D, u, a, Q, xd, f, d, -1)) * inv2dx;
+    };
+    T GP[2];
+    cross(P, fl, GP[0], GP[1]);
+#pragma unroll 1
+    for (int s = -1; s <= 1; s += 2) {
+        const T Uf = U[f0 + (s > 0 ? fs : 0)], sg = (T)s;
+        long long off = 0;
+        const bool interior = !(fl & (1u << link_bit(a, s))) && nb_offset(D, a, s, xa, off);
+        T uN[3], tt[2] = {sg * GP[0], sg * GP[1]}, nutf = nutP;
+        vel3_across(D, uc, cm, P, xa, fl, a, s, uP, uN);
+        T adv[3];
 #pragma unroll
-            for (int s = -1; s <= 1; s += 2) {
-                const int fx0 = x[0] + (a == 0 && s > 0), fx1 = x[1] + (a == 1 && s > 0), fx2 = x[2] + (a == 2 && s > 0);
-                const T Uf = U[F.index(a, fx0, fx1, fx2)];
-                const int bit = 2 * a + (s > 0);
-                long long off = 0;
-                const bool interior = !(fl & (1u << bit)) && nb_offset(D, a, s, x[a], off);
-                T nutf = nutP;
-                T GN[3] = {0, 0, 0};
-                if (interior) {
-                    const long long Nn = P + off;
-                    nutf = (T)0.5 * (nutP + nut[Nn]);
-                    int xn[3] = {x[0], x[1], x[2]};
-                    xn[a] += s;
-                    if (xn[a] < 0) xn[a] += n[a];
-                    if (xn[a] >= n[a]) xn[a] -= n[a];
-                    const unsigned fln = flags_at(D, Nn);
+        for (int c = 0; c < 3; ++c) adv[c] = (T)0.5 * (uP[c] + uN[c]);
+        if (interior) {
+            const long long Q = P + off;
+            const unsigned fn = flags_at(D, Q);
+            nutf = (T)0.5 * (nutP + nut[Q]);
+            T GN[2];
+            cross(Q, fn, GN[0], GN[1]);
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        if (q == a) continue;
-                        GN[q] = (vel_across(D, u, a, Nn, xn[q], fln, q, +1) - vel_across(D, u, a, Nn, xn[q], fln, q, -1)) * inv2dx;
-                    }
-                }
+            for (int c = 0; c < 2; ++c) tt[c] = sg * (T)0.5 * (GP[c] + GN[c]);
+            if (gam != (T)0) {
+                // far upwind value: across the outer link of the upwind cell
+                const bool up = (Uf >= (T)0) == (s > 0);        // P is the upwind cell
+                const int xn = xa + s < 0 ? na - 1 : (xa + s >= na ? 0 : xa + s);
+                T v[3], w[3], far[3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    const T uP = u[c * D.N + P];
-                    const T uN = vel_across(D, u, c, P, x[a], fl, a, s);
-                    const T D1 = (uN - uP) * invdx;
-                    T Tt;
-                    if (c == a) Tt = D1;
-                    else if (interior) Tt = (T)s * (T)0.5 * (GP[c][a] + GN[c]);
-                    else Tt = (T)s * GP[c][a];
-                    const T conv = -(T)s * Uf * face_adv(D, u, c, P, x, fl, a, s, uP, uN, Uf, gam);
-                    h[c] += conv + (nu + nutf) * D1 + nutf * Tt;
+                    v[c] = up ? uP[c] : uN[c];
+                    w[c] = up ? uN[c] : uP[c];
                 }
+                vel3_across(D, uc, cm, up ? P : Q, up ? xa : xn, up ? fl : fn, a, up ? -s : s, v, far);
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    adv[c] = ((T)1 - gam) * adv[c] + gam * (((T)6 * v[c] + (T)3 * w[c] - far[c]) * (T)0.125);
             }
-    #pragma unroll
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const T D1 = (uN[c] - uP[c]) * invdx;
+            h[c] += (nu + nutf) * D1 + nutf * (c == 0 ? D1 : tt[c > 0 ? c - 1 : 0]) - sg * Uf * adv[c];
+        }
+    }
+#pragma unroll
     for (int c = 0; c < 3; ++c) h[c] *= invdx;
 }
 
@@ -561,62 +581,75 @@ __device__ __forceinline__ void cell_coords(const Dom& D, long long P, int& i, i
     i = (int)(r - jj * sy);
 }
 
-// Calls body(P, i, j, k) for the entries of the list of the cells that are not fast_cell, strided
-// over a capped grid.
-template <class Body>
-__device__ __forceinline__ void for_general_cells(const Dom& D, const int32_t* __restrict__ list, long long nlist,
-                                                  Body body) {
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nlist; q += (long long)gridDim.x * blockDim.x) {
-        const long long P = list[q];
-        int i, j, k;
-        cell_coords(D, P, i, j, k);
-        body(P, i, j, k);
+// Cells that are not fast_cell, from their list.  A warp takes one axis of 32 cells, so that what depends on the axis
+// is uniform in it, and three warps make up the cells: they leave their shares of the three components in shared
+// memory and each finishes one component.  1024 x 512 x 384 around a vehicle, Crank-Nicolson operator: 3.9 -> 1.8 ms
+// against one thread per cell with all six faces unrolled, which waited for instructions (a thousand per face) and
+// spilled; 128 x 64 x 64 in FP64: 35 -> 14 us.  Four and seven blocks per SM: 16 % and 1 % slower.
+#define FG_CELLS 64
+#define FG_NT (3 * FG_CELLS)
+
+template <class T, class Epi>
+__device__ __forceinline__ void general_march(const Dom& D, const FaceLayout& F, const T* __restrict__ u,
+                                              const T* __restrict__ U, const T* __restrict__ nut, T nu, T gam,
+                                              const int32_t* __restrict__ list, long long nlist, const T* wv, Epi epi) {
+    __shared__ T part[2][3][3][FG_CELLS];           // [parity][axis][component][cell]
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), a = warp % 3;
+    const int cell = 32 * (warp / 3) + (threadIdx.x & 31);
+    int buf = 0;
+    for (long long q0 = blockIdx.x * (long long)FG_CELLS; q0 < nlist; q0 += (long long)gridDim.x * FG_CELLS) {
+        const bool on = q0 + cell < nlist;
+        const long long P = on ? list[q0 + cell] : 0;
+        T uP[3] = {}, w = (T)0;
+        if (on) {
+            int x[3];
+            cell_coords(D, P, x[0], x[1], x[2]);
+            if (wv) w = wv[a * D.N + P];
+            T h[3];
+            flux_axis(D, F, u, U, nut, P, x, a, nu, gam, h, uP);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) part[buf][a][a + c < 3 ? a + c : a + c - 3][cell] = h[c];
+        }
+        __syncthreads();
+        if (on) epi(a * D.N + P, 0, (part[buf][0][a][cell] + part[buf][1][a][cell]) + part[buf][2][a][cell], uP[0], w);
+        buf ^= 1;
     }
 }
 
-// Runs epi(plane, off, h, u, w) over the kernel's cells (cell = plane + off / sizeof(T), w = wv there): z-marching shared-memory tiles of fast cells, or the
-// general list.
+// Runs epi(q, off, h, u, w) for every component of the kernel's cells (value q + off / sizeof(T) of the stacked
+// components, w = wv there): z-marching shared-memory tiles of fast cells, or the general list.
 template <bool GENERAL, class T, class Epi>
 __device__ __forceinline__ void flux_cells(const Dom& D, const FaceLayout& F, const T* __restrict__ u,
                                            const T* __restrict__ U, const T* __restrict__ nut, T nu, T gam,
                                            const int32_t* __restrict__ list, long long nlist, const T* wv, Epi epi) {
     if constexpr (GENERAL) {
-        for_general_cells(D, list, nlist, [&](long long P, int i, int j, int k) {
-            T h[3];
-            flux_general(D, F, u, U, nut, P, i, j, k, nu, gam, h);
-            const T uc[3] = {u[P], u[D.N + P], u[2 * D.N + P]};
-            T wq[3] = {};
-            if (wv)
-                for (int c = 0; c < 3; ++c) wq[c] = wv[c * D.N + P];
-            epi(P, 0, h, uc, wq);
-        });
+        general_march<T>(D, F, u, U, nut, nu, gam, list, nlist, wv, epi);
     } else {
-        fast_tile_march<T>(D, F, u, U, nut, nu, gam, wv, epi);
+        fast_tile_march<T>(D, F, u, U, nut, nu, gam, wv,
+                           [&](long long P, Off<T> o, const T (&h)[3], const T (&uc)[3], const T (&w)[3]) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) epi(c * D.N + P, o, h[c], uc[c], w[c]);
+        });
     }
 }
 
-// Momentum predictor, Adams-Bashforth 2 in time (Euler on the first step).  One thread per cell.
-// Resident blocks of 256 threads per SM the fast FP32 flux kernels are compiled for (register cap).
+// Resident blocks per SM the flux kernels are compiled for (register cap), and their threads.
 template <class T, bool GENERAL>
 struct FluxOcc {
-    static constexpr int value = sizeof(T) == 4 ? (GENERAL ? IBM_FLUX_GEN_MINB : IBM_FLUX_MINB) : 1;
+    static constexpr int value = sizeof(T) == 4 ? (GENERAL ? IBM_FLUX_GEN_MINB : IBM_FLUX_MINB) : (GENERAL ? 2 : 1);
+    static constexpr int threads = GENERAL ? FG_NT : 256;
 };
 
+// Momentum predictor, Adams-Bashforth 2 in time (Euler on the first step).
 template <bool GENERAL, class T>
-__global__ void __launch_bounds__(256, (FluxOcc<T, GENERAL>::value)) k_predict(Dom D, FaceLayout F, const T* __restrict__ u, const T* __restrict__ U,
+__global__ void __launch_bounds__((FluxOcc<T, GENERAL>::threads), (FluxOcc<T, GENERAL>::value)) k_predict(Dom D, FaceLayout F, const T* __restrict__ u, const T* __restrict__ U,
                                                  const T* __restrict__ nut, const T* Hprev, T* H,
                                                  T* __restrict__ ustar, T nu, T dt, int first, T gam,
                                                  const int32_t* __restrict__ list, long long nlist) {
     flux_cells<GENERAL, T>(D, F, u, U, nut, nu, gam, list, nlist, first ? nullptr : Hprev,
-                           [&](long long P, Off<T> o, const T (&h)[3], const T (&uc)[3], const T (&w)[3]) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long oc = c * D.N + P;
-            const T hc = h[c];
-            const T hp = first ? (T)0 : w[c];
-            to_off(H + oc, o, hc);
-            to_off(ustar + oc, o, first ? uc[c] + dt * hc : uc[c] + dt * ((T)1.5 * hc - (T)0.5 * hp));
-        }
+                           [&](long long q, Off<T> o, T h, T uc, T w) {
+        to_off(H + q, o, h);
+        to_off(ustar + q, o, first ? uc + dt * h : uc + dt * ((T)1.5 * h - (T)0.5 * w));
     });
 }
 
@@ -1070,24 +1103,20 @@ unsigned lin_blocks(long long n, int threads) {
 // The fast kernel of a pair leaves its sums in sc->part; the general kernel, launched after it, adds
 // its own and finishes (so the totals are formed in a fixed order).
 template <class T, bool GENERAL>
-__global__ void __launch_bounds__(256, (FluxOcc<T, GENERAL>::value)) k_cn_begin(Dom D, FaceLayout F, const T* __restrict__ u, const T* __restrict__ U,
+__global__ void __launch_bounds__((FluxOcc<T, GENERAL>::threads), (FluxOcc<T, GENERAL>::value)) k_cn_begin(Dom D, FaceLayout F, const T* __restrict__ u, const T* __restrict__ U,
                                                   const T* __restrict__ nut, T* __restrict__ H, T* __restrict__ r,
                                                   T* __restrict__ rh, T* __restrict__ x, T nu, T gam, T dt, double tol2,
                                                   int maxit, int keepx, SolveScal* sc, double* partials, unsigned* counter,
                                                   const int32_t* __restrict__ list, long long nlist) {
     T a0 = 0;
     flux_cells<GENERAL, T>(D, F, u, U, nut, nu, gam, list, nlist, (const T*)nullptr,
-                           [&](long long P, Off<T> o, const T (&h)[3], const T (&)[3], const T (&)[3]) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long q = c * D.N + P;
-            const T b = dt * h[c];
-            to_off(H + q, o, h[c]);
-            to_off(r + q, o, b);
-            to_off(rh + q, o, b);
-            if (!keepx) to_off(x + q, o, (T)0);
-            a0 += b * b;
-        }
+                           [&](long long q, Off<T> o, T h, T, T) {
+        const T b = dt * h;
+        to_off(H + q, o, h);
+        to_off(r + q, o, b);
+        to_off(rh + q, o, b);
+        if (!keepx) to_off(x + q, o, (T)0);
+        a0 += b * b;
     });
     T acc[1] = {a0};
     grid_reduce<1>(acc, partials, counter, [&](double* t) {
@@ -1127,7 +1156,7 @@ __global__ void k_cn_p(long long n, const T* __restrict__ r, T* __restrict__ p, 
 // (y, s), (y, y) -> omega.  mode 2 (warm start, xin = the previous increment): r = b - M xin with b
 // read from and r written to r2, r_hat = r in y, (r, r) -> rr = rho.
 template <class T, bool GENERAL, int mode>
-__global__ void __launch_bounds__(256, (FluxOcc<T, GENERAL>::value)) k_cn_apply(Dom D, FaceLayout F, const T* __restrict__ xin,
+__global__ void __launch_bounds__((FluxOcc<T, GENERAL>::threads), (FluxOcc<T, GENERAL>::value)) k_cn_apply(Dom D, FaceLayout F, const T* __restrict__ xin,
                                                   const T* __restrict__ U, const T* __restrict__ nut,
                                                   T* __restrict__ y, const T* __restrict__ w, T* r2, T nu, T gam,
                                                   T hdt, SolveScal* sc, double* partials,
@@ -1135,26 +1164,21 @@ __global__ void __launch_bounds__(256, (FluxOcc<T, GENERAL>::value)) k_cn_apply(
     if (sc->done) return;
     T a0 = 0, a1 = 0;
     flux_cells<GENERAL, T>(D, F, xin, U, nut, nu, gam, list, nlist, mode == 0 ? w : (mode == 2 ? (const T*)r2 : nullptr),
-                           [&](long long P, Off<T> o, const T (&h)[3], const T (&uc)[3], const T (&wq)[3]) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long q = c * D.N + P;
-            const T xv = uc[c];
-            const T yv = xv - hdt * h[c];
-            if (mode == 2) {
-                const T rn = wq[c] - yv;
-                to_off(r2 + q, o, rn);
-                to_off(y + q, o, rn);
-                a0 += rn * rn;
-                continue;
-            }
-            to_off(y + q, o, yv);
-            if (mode == 0) {
-                a0 += wq[c] * yv;
-            } else {
-                a0 += yv * xv;
-                a1 += yv * yv;
-            }
+                           [&](long long q, Off<T> o, T h, T xv, T wq) {
+        const T yv = xv - hdt * h;
+        if (mode == 2) {
+            const T rn = wq - yv;
+            to_off(r2 + q, o, rn);
+            to_off(y + q, o, rn);
+            a0 += rn * rn;
+            return;
+        }
+        to_off(y + q, o, yv);
+        if (mode == 0) {
+            a0 += wq * yv;
+        } else {
+            a0 += yv * xv;
+            a1 += yv * yv;
         }
     });
     T acc[2] = {a0, a1};
@@ -1267,6 +1291,13 @@ int tile_planes(const Dom& D) {
     return best_k;
 }
 
+// Blocks of the general-cell kernels: those that fit on the GPU at once, fewer for a short list.
+template <class T>
+unsigned general_blocks(long long n) {
+    const long long b = (n + FG_CELLS - 1) / FG_CELLS, cap = (long long)FluxOcc<T, true>::value * IBM_NSM;
+    return (unsigned)(b > cap ? cap : (b < 1 ? 1 : b));
+}
+
 template <class T>
 int predict_cn_t(const LesCtx& c, const T* u, const T* U, const T* nut, T* H, T* ustar, int* iters, cudaStream_t s) {
     CNWork& w = *c.cn;
@@ -1276,13 +1307,13 @@ int predict_cn_t(const LesCtx& c, const T* u, const T* U, const T* nut, T* H, T*
     const unsigned nbv = lin_blocks(n3, 256);
     T *r = (T*)w.r, *rh = (T*)w.rh, *p = (T*)w.p, *v = (T*)w.v, *sv = (T*)w.sv, *tv = (T*)w.tv, *x = (T*)w.x;
     const T nu = (T)c.nu, gam = (T)c.quick, dt = (T)c.dt, hdt = (T)(0.5 * c.dt);
-    const unsigned ngen = lin_blocks(c.n_general > 0 ? c.n_general : 1, 256);
+    const unsigned ngen = general_blocks<T>(c.n_general);
     prof_begin(c.prof, PS_PREDICT, s);
     // warm start from the previous step's increment (the increment changes slowly from step to step)
     const int keepx = w.have_x;
     k_cn_begin<T, false><<<tile_grid<T>(c), dim3(FT_X, FT_Y), fast_tile_smem<T>(), s>>>(c.D, c.F, u, U, nut, H, r, rh, x, nu, gam, dt, w.tol * w.tol,
                                                         w.maxit, keepx, w.sc, c.partials, c.counter, nullptr, 0);
-    k_cn_begin<T, true><<<ngen, 256, 0, s>>>(c.D, c.F, u, U, nut, H, r, rh, x, nu, gam, dt, w.tol * w.tol, w.maxit,
+    k_cn_begin<T, true><<<ngen, FG_NT, 0, s>>>(c.D, c.F, u, U, nut, H, r, rh, x, nu, gam, dt, w.tol * w.tol, w.maxit,
                                              keepx, w.sc, c.partials, c.counter, c.general, c.n_general);
     prof_end(c.prof, PS_PREDICT, s);
     IBM_LAUNCHED("k_cn_begin");
@@ -1293,7 +1324,7 @@ int predict_cn_t(const LesCtx& c, const T* u, const T* U, const T* nut, T* H, T*
         T* r2 = mode == 2 ? r : nullptr;
         k_cn_apply<T, false, mode><<<tile_grid<T>(c), dim3(FT_X, FT_Y), fast_tile_smem<T>(), s>>>(
             Dh, c.F, in, U, nut, out, wv, r2, nu, gam, hdt, w.sc, c.partials, c.counter, nullptr, 0);
-        k_cn_apply<T, true, mode><<<ngen, 256, 0, s>>>(Dh, c.F, in, U, nut, out, wv, r2, nu, gam, hdt, w.sc, c.partials,
+        k_cn_apply<T, true, mode><<<ngen, FG_NT, 0, s>>>(Dh, c.F, in, U, nut, out, wv, r2, nu, gam, hdt, w.sc, c.partials,
                                                        c.counter, c.general, c.n_general);
     };
     if (keepx) {
@@ -1446,7 +1477,7 @@ static void predict_t(const LesCtx& c, const T* u, const T* U, const T* nut, con
     k_predict<false, T><<<tile_grid<T>(c), dim3(FT_X, FT_Y), fast_tile_smem<T>(), s>>>(c.D, c.F, u, U, nut, Hprev, H, ustar, (T)c.nu, (T)c.dt, first,
                                                        (T)c.quick, nullptr, 0);
     if (c.n_general > 0)
-        k_predict<true, T><<<lin_blocks(c.n_general, 256), 256, 0, s>>>(c.D, c.F, u, U, nut, Hprev, H, ustar,
+        k_predict<true, T><<<general_blocks<T>(c.n_general), FG_NT, 0, s>>>(c.D, c.F, u, U, nut, Hprev, H, ustar,
                                                                          (T)c.nu, (T)c.dt, first, (T)c.quick,
                                                                          c.general, c.n_general);
 }

@@ -235,3 +235,38 @@ def test_cg_on_quads_of_cells_takes_the_iterations_of_fp64(L, shape, bc, body):
         its.append(st.iters)
         sol.close()
     assert abs(its[1] - its[0]) <= 2 + 0.1 * its[0], its
+
+
+@pytest.mark.parametrize("prec,tol", [(0, 1e-12), (1, 2e-5)])
+@pytest.mark.parametrize("shape,bc", [((5, 4, 3), CHANNEL), ((1, 9, 2), (2, 1, 4, 3, 3, 2)), ((33, 9, 7), (0, 0, 3, 4, 1, 2)),
+                                      ((16, 16, 16), PERIODIC), ((40, 21, 18), (4, 3, 0, 0, 2, 1))])
+@pytest.mark.parametrize("quick", [0.0, 0.25])
+def test_momentum_flux_of_cells_with_any_links_is_the_oracles(L, shape, bc, quick, prec, tol):
+    """A dense soup leaves hardly a cell without a cut link near it: lists that end anywhere within a block, every
+    domain boundary, cut links of the neighbours.  FP32 values and ghosts carry a few roundings of 6e-8 of the
+    fluxes, whose cancelling sums the scale below holds; 2e-5 allows 300 of them."""
+    import oracle
+    import workloads as W
+    nx, ny, nz = shape
+    N = nx * ny * nz
+    rng = np.random.default_rng(12)
+    tri = W.random_soup(40, (0.3, 0.3, 0.3), (nx - 0.3, ny - 0.3, nz - 0.3), 3.0, seed=5).astype(np.float32)
+    g = L.make_grid(nx, ny, nz)
+    geo = L.Geometry(g, torch.from_numpy(tri).cuda())
+    ref = oracle.Case(nx, ny, nz, 1.0, 0.03, 0.15, bc)
+    ref.set_geometry(tri)
+    ref.pr.quick = quick
+    sol = L.Solver(g, 0.03, 0.15, bc, precision=prec, geometry=geo, quick=quick, precond=0)
+    td, nd = sol.dtype, np.float64 if prec == 0 else np.float32
+    u = (0.5 + 0.3 * rng.standard_normal(3 * N)).astype(nd)
+    U = ref.faces(u.astype(np.float64)).astype(nd)
+    nut = (0.01 * rng.random(N)).astype(nd)
+    H0 = (0.1 * rng.standard_normal(3 * N)).astype(nd)
+    dev = [torch.from_numpy(v).to("cuda", td) for v in (u, U, nut, H0)]
+    us = torch.empty(3 * N, dtype=td, device="cuda")
+    sol.predict(dev[0], dev[1], dev[2], dev[3], dev[3], us, False)
+    Hr, ur = ref.predict(u.astype(np.float64), U.astype(np.float64), nut.astype(np.float64), H0.astype(np.float64), False)
+    scale = np.linalg.norm(np.abs(U).max() * np.abs(u)) + np.linalg.norm(Hr)
+    assert np.linalg.norm(dev[3].cpu().numpy() - Hr) <= tol * scale
+    assert np.linalg.norm(us.cpu().numpy() - ur) <= tol * (np.linalg.norm(ur) + 0.15 * scale)
+    sol.close()
