@@ -221,6 +221,52 @@ __device__ __forceinline__ T link_sum7(const Dom& D, long long P, int i, int j, 
     return sum;
 }
 
+// The links of a cell without a branch, so that a warp with a cell on a domain face or a cut link runs the same
+// instructions as any other: `open`, the links to another cell (bit order x-, x+, y-, ..), `out`, the outflow faces,
+// and the neighbours' offsets (0 where there is none).
+struct CellLinks {
+    unsigned open, out;
+    long long off[6];
+};
+
+__device__ __forceinline__ CellLinks cell_links(const Dom& D, int i, int j, int k, unsigned fl) {
+    CellLinks L;
+    L.open = L.out = 0u;
+    const int x[3] = {i, j, k}, n[3] = {D.nx, D.ny, D.nz};
+    const long long st[3] = {1, (long long)D.sy, D.sz};
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+        const int a = b >> 1, s = (b & 1) ? 1 : -1;
+        const bool in = s > 0 ? x[a] + 1 < n[a] : x[a] > 0, per = D.bc[b] == IBM_BC_PERIODIC;
+        L.open |= (in || per) ? 1u << b : 0u;
+        L.out |= (!in && D.bc[b] == IBM_BC_OUTFLOW) ? 1u << b : 0u;
+        L.off[b] = in ? s * st[a] : (per ? -s * (n[a] - 1) * st[a] : 0);
+    }
+    L.open &= ~fl;
+    return L;
+}
+
+// Sum of a value over the open links.
+template <class T, class Get>
+__device__ __forceinline__ T open_sum(const CellLinks& L, long long P, Get get) {
+    T v[6];
+#pragma unroll
+    for (int b = 0; b < 6; ++b) v[b] = (L.open >> b) & 1u ? get(P + L.off[b]) : (T)0;
+    return ((v[0] + v[1]) + (v[2] + v[3])) + (v[4] + v[5]);
+}
+
+// 0 .. 12 and their reciprocals (0 for 0) in the working precision: an FP64 division costs more than the rest of a
+// cell's update, a conversion to FP64 as much as an addition.
+__constant__ double c_num64[13] = {0., 1., 2., 3., 4., 5., 6., 7., 8., 9., 10., 11., 12.};
+__constant__ double c_rcp64[13] = {0.,      1.,      1. / 2., 1. / 3., 1. / 4.,  1. / 5., 1. / 6.,
+                                   1. / 7., 1. / 8., 1. / 9., 1. / 10., 1. / 11., 1. / 12.};
+template <class T> __device__ __forceinline__ T small_num(int n);
+template <> __device__ __forceinline__ float small_num<float>(int n) { return (float)n; }
+template <> __device__ __forceinline__ double small_num<double>(int n) { return c_num64[n]; }
+template <class T> __device__ __forceinline__ T over_num(T v, int n);
+template <> __device__ __forceinline__ float over_num<float>(float v, int n) { return n == 6 ? v * (1.f / 6.f) : v / (float)n; }
+template <> __device__ __forceinline__ double over_num<double>(double v, int n) { return v * c_rcp64[n]; }
+
 // Launch geometry of the cell kernels.
 struct CellGrid {
     dim3 grid, block;

@@ -93,46 +93,30 @@ __device__ __forceinline__ long long pos_index(const MGLev& L, const int X[3]) {
 
 // ---- fine-grid smoothing ----------------------------------------------------------------------
 
-// Gauss-Seidel value of a fine cell:  z_P = (sum_links g z_N - scale r_P) / dg, with the interior
-// fast path (six uncut links, dg = 6).  Returns false for an isolated cell (dg = 0).
+// Gauss-Seidel value of a fine cell:  z_P = (sum_links z_N - scale r_P) / dg, 0 for an isolated cell (dg = 0).
 template <class T>
 __device__ __forceinline__ T gs_value(const Dom& D, const T* __restrict__ r, const T* z, T scale, long long P, int i,
                                       int j, int k, bool zero) {
-    const unsigned fl = flags_at(D, P);
-    if (fl == 0u && i > 0 && i < D.nx - 1 && j > 0 && j < D.ny - 1 && k > 0 && k < D.nz - 1) {
-        const T s = zero ? (T)0
-                         : ((z[P - 1] + z[P + 1]) + (z[P - D.sy] + z[P + D.sy])) + (z[P - D.sz] + z[P + D.sz]);
-        return (s - scale * r[P]) * (T)(1.0 / 6.0);
-    }
-    const int x[3] = {i, j, k};
-    float g[6], d;
-    long long off[6];
-    fine_links(D, P, x, fl, g, off, d);
-    const float dg = g[0] + g[1] + g[2] + g[3] + g[4] + g[5] + d;
-    if (dg == 0.f) return (T)0;
-    T s = 0;
-    if (!zero) {
-#pragma unroll
-        for (int b = 0; b < 6; ++b)
-            if (g[b] != 0.f) s += z[P + off[b]];
-    }
-    return (s - scale * r[P]) / (T)dg;
+    const CellLinks L = cell_links(D, i, j, k, flags_at(D, P));
+    const int dg = __popc(L.open) + 2 * __popc(L.out);
+    const T s = zero ? (T)0 : open_sum<T>(L, P, [&](long long c) { return z[c]; });
+    return dg == 0 ? (T)0 : over_num<T>(s - scale * r[P], dg);
 }
 
-// One red-black Gauss-Seidel pass of colour `col` on level 0 for  A^ z = scale * r.  Each thread takes
-// IBM_KU pairs of planes of one (i, j) column and updates the cell of colour `col` in each pair.
-// With `zero` the iterate is taken as 0 (first pass of a V-cycle) and the other cell of each pair is
-// cleared.
-template <class T>
+// One red-black Gauss-Seidel pass of colour `col` on level 0 for  A^ z = scale * r.  Each thread takes KU pairs of
+// planes of one (i, j) column and updates the cell of colour `col` in each pair.  With `zero` the iterate is taken
+// as 0 (first pass of a V-cycle) and the other cell of each pair is cleared.  64 x 32 x 32 in FP64, KU = 1: 2.7 us, with four
+// pairs and an FP64 division at every domain face 9.5 us.
+template <class T, int KU>
 __global__ void __launch_bounds__(256) k_mg_smooth0(Dom D, const T* __restrict__ r, T* __restrict__ z, T scale,
                                                     int col, int zero, const SolveScal* sc) {
     if (sc->done) return;
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
     if (i >= D.nx || j >= D.ny) return;
-    const int kb = blockIdx.z * (2 * IBM_KU);
+    const int kb = blockIdx.z * (2 * KU);
     const int par = (col + i + j) & 1;
 #pragma unroll
-    for (int u = 0; u < IBM_KU; ++u) {
+    for (int u = 0; u < KU; ++u) {
         const int k = kb + 2 * u + par;
         const long long P = i + (long long)D.sy * j + D.sz * k;
         if (k < D.nz) z[P] = gs_value<T>(D, r, z, scale, P, i, j, k, zero != 0);
@@ -144,18 +128,18 @@ __global__ void __launch_bounds__(256) k_mg_smooth0(Dom D, const T* __restrict__
 }
 
 // Last pass of the V-cycle on level 0 (colour 0) fused with rho = (r, z) over both colours.
-template <class T>
+template <class T, int KU>
 __global__ void __launch_bounds__(256) k_mg_final0(Dom D, const T* __restrict__ r, T* __restrict__ z, T scale,
                                                    SolveScal* sc, double* partials, unsigned* counter) {
     if (sc->done) return;
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
     const bool active = i < D.nx && j < D.ny;
-    const int kb = blockIdx.z * (2 * IBM_KU);
+    const int kb = blockIdx.z * (2 * KU);
     const int par = (i + j) & 1;                 // plane offset of the colour-0 cell in each pair
     T part = 0;
     if (active) {
 #pragma unroll
-        for (int u = 0; u < IBM_KU; ++u) {
+        for (int u = 0; u < KU; ++u) {
             const int k = kb + 2 * u + par, k2 = kb + 2 * u + (par ^ 1);
             if (k < D.nz) {
                 const long long P = i + (long long)D.sy * j + D.sz * k;
@@ -1461,33 +1445,49 @@ __global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant
 // ---- transfer between the fine grid and level 1 -------------------------------------------------
 
 // b_1 of each part of a level-1 block = the sum of the fine residuals  scale r - (A z)  of its cells, and the
-// first half-sweep of level 1, x_1 = -b_1 / dg.
+// first half-sweep of level 1, x_1 = -b_1 / dg.  Eight lanes per block, one per cell: 64 x 32 x 32 in FP64
+// 4.8 us, 21.5 us
+// with one lane.
 template <class T>
 __global__ void __launch_bounds__(256) k_mg_restrict0(Dom D, const T* __restrict__ r, const T* __restrict__ z, T scale,
                                                       MGLev C, const SolveScal* sc) {
     if (sc->done) return;
+    const int m = threadIdx.x & 7;
+    const unsigned gm = 0xffu << (threadIdx.x & 24);
     auto zv = [&](long long c) { return z[c]; };
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < C.P; q += (long long)gridDim.x * blockDim.x) {
+    for (long long q = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3; q < C.P;
+         q += ((long long)gridDim.x * blockDim.x) >> 3) {
         int X[3];
         coords3(q, C.px, C.py, X);
-        unsigned fl[8];
-        long long P[8];
-        const unsigned in = block_flags(D, X, fl, P);
-        int part[8];
-        const int np = fine_parts(D, fl, in, part);
-        T acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            if (!((in >> m) & 1u)) continue;
-            const int x0 = 2 * X[0] + (m & 1), x1 = 2 * X[1] + ((m >> 1) & 1), x2 = 2 * X[2] + (m >> 2);
-            const T res = scale * r[P[m]] - link_sum7<T>(D, P[m], x0, x1, x2, fl[m], z[P[m]], zv);
-#pragma unroll
-            for (int s = 0; s < 8; ++s) acc[s] += part[m] == s ? res : (T)0;
-        }
+        const int i = 2 * X[0] + (m & 1), j = 2 * X[1] + ((m >> 1) & 1), k = 2 * X[2] + (m >> 2);
+        const bool on = i < D.nx && j < D.ny && k < D.nz;
+        const long long P = i + (long long)D.sy * j + D.sz * k;
         const int o = C.off[q];
+        unsigned f = 0u;
+        T res = (T)0;
+        if (on) {
+            f = flags_at(D, P);
+            const CellLinks L = cell_links(D, i, j, k, f);
+            const int dg = __popc(L.open) + 2 * __popc(L.out & ~f);
+            res = scale * r[P] - (open_sum<T>(L, P, zv) - small_num<T>(dg) * z[P]);
+        }
+        const unsigned in = (__ballot_sync(gm, on) >> (threadIdx.x & 24)) & 0xffu;
+        int np = 1, mine = 0;
+        if (__ballot_sync(gm, f != 0u) != 0u || in != 0xffu) {
+            unsigned fl[8];
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
-            if (s < np) put_b1<T>(C, o + s, acc[s]);
+            for (int e = 0; e < 8; ++e) fl[e] = __shfl_sync(gm, f, e, 8);
+            int part[8];
+            np = fine_parts(D, fl, in, part);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) mine = m == e ? part[e] : mine;
+        }
+        for (int s = 0; s < np; ++s) {
+            T v = mine == s ? res : (T)0;
+#pragma unroll
+            for (int d = 1; d < 8; d *= 2) v += __shfl_xor_sync(gm, v, d);
+            if (m == s) put_b1<T>(C, o + s, v);
+        }
     }
 }
 
@@ -2169,13 +2169,22 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
     if constexpr (std::is_same<T, float>::value) {
         if (mg.fused) return vcycle_fused(c, mg, r, z, sc, s);
     }
+    // one pair of planes per thread where four would leave SMs idle
+    const bool few = (long long)c.cgrid.x * c.cgrid.y * c.cgrid.z < 4 * IBM_NSM;
+    auto pairs = [&](auto f) {
+        if (few) f(std::integral_constant<int, 1>{}, flat_grid(c.D.nx, c.D.ny, c.D.nz, 2));
+        else f(std::integral_constant<int, IBM_KU>{}, c.cgrid);
+    };
     auto fine = [&](int col, int zero) {
+        auto smooth = [&](auto ku, dim3 grid) {
+            k_mg_smooth0<T, decltype(ku)::value><<<grid, g.block, 0, s>>>(c.D, r, z, scale, col, zero, sc);
+        };
         prof_begin(c.prof, PS_MG_FINE, s);
         if constexpr (std::is_same<T, float>::value) {
             if (vec) launch_mg_smooth0_x4(c, r, z, scale, col, zero, 0, sc, s);
-            else k_mg_smooth0<T><<<c.cgrid, g.block, 0, s>>>(c.D, r, z, scale, col, zero, sc);
+            else pairs(smooth);
         } else {
-            k_mg_smooth0<T><<<c.cgrid, g.block, 0, s>>>(c.D, r, z, scale, col, zero, sc);
+            pairs(smooth);
         }
         prof_end(c.prof, PS_MG_FINE, s);
         ++launches;
@@ -2189,9 +2198,9 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
         prof_begin(c.prof, PS_MG_TRANSFER, s);
         if constexpr (std::is_same<T, float>::value) {
             if (vec) k_mg_restrict0_x4<<<lin_blocks((c.D.nx / 4) * (long long)L1.py * L1.pz), 256, 0, s>>>(c.D, r, z, scale, L1, sc);
-            else k_mg_restrict0<T><<<lin_blocks(L1.P), 256, 0, s>>>(c.D, r, z, scale, L1, sc);
+            else k_mg_restrict0<T><<<lin_blocks(8 * L1.P), 256, 0, s>>>(c.D, r, z, scale, L1, sc);
         } else {
-            k_mg_restrict0<T><<<lin_blocks(L1.P), 256, 0, s>>>(c.D, r, z, scale, L1, sc);
+            k_mg_restrict0<T><<<lin_blocks(8 * L1.P), 256, 0, s>>>(c.D, r, z, scale, L1, sc);
         }
         prof_end(c.prof, PS_MG_TRANSFER, s);
         ++launches;
@@ -2213,12 +2222,15 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
         fine(1, 0);
         if (q + 1 < S) fine(0, 0);
     }
+    auto final = [&](auto ku, dim3 grid) {
+        k_mg_final0<T, decltype(ku)::value><<<grid, g.block, 0, s>>>(c.D, r, z, scale, sc, c.partials, c.counter);
+    };
     prof_begin(c.prof, PS_MG_FINE, s);
     if constexpr (std::is_same<T, float>::value) {
         if (vec) launch_mg_smooth0_x4(c, r, z, scale, 0, 0, 1, sc, s);
-        else k_mg_final0<T><<<c.cgrid, g.block, 0, s>>>(c.D, r, z, scale, sc, c.partials, c.counter);
+        else pairs(final);
     } else {
-        k_mg_final0<T><<<c.cgrid, g.block, 0, s>>>(c.D, r, z, scale, sc, c.partials, c.counter);
+        pairs(final);
     }
     prof_end(c.prof, PS_MG_FINE, s);
     ++launches;
