@@ -43,6 +43,7 @@ struct MGTail {
     MGTailLev t[IBM_MG_MAXLEV];
     MGLev lev[IBM_MG_MAXLEV];
     int first, nlev, coarse_sweeps;
+    int ctas, shift;         // blocks of the cluster; a place is block << shift | index
     int image;               // bytes of a block's constant arrays (the first in its shared memory)
     const uint4* img;        // their image in global memory, block after block
     double omega;
@@ -50,7 +51,7 @@ struct MGTail {
 
 namespace {
 
-#define MG_TAIL_CTAS 8          // portable cluster size
+#define MG_TAIL_BIG 16          // blocks of the tail's cluster where the GPU can hold it; 8, the portable size, elsewhere
 #define MG_TAIL_MAX (1LL << 14) // levels with at most this many unknowns run in the one-launch tail
 #define MG_COARSE_TARGET 1024   // coarsening stops at this many unknowns (or one position)
 #define MG_ELL 6                // links of an unknown kept in the padded rows (more: its CSR row)
@@ -1150,26 +1151,27 @@ __global__ void __launch_bounds__(256) k_gup(MGLev F, MGLev C, T omega, const So
     gup<T>(F, C, omega, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
-// The small levels first .. nlev-1 of a V-cycle in one launch of one cluster of MG_TAIL_CTAS blocks.  Every
+// The small levels first .. nlev-1 of a V-cycle in one launch of one cluster of M.ctas blocks.  Every
 // block keeps its share of each level (half of it of either colour) in shared memory; neighbours are read
 // from the other blocks' shared memory and a cluster barrier (hardware, release/acquire at cluster scope)
 // separates dependent passes.  The coarsest level belongs to block 0 as a whole and is solved there with
 // barriers of the warps it needs, its rows in registers.  All of it is latency: five passes per level and 32
 // on the coarsest.  So everything that does not change between V-cycles (rows, parents of neighbours,
-// children, as places: block << 13 | index) is laid out once as an image of the blocks' shared memory and
+// children, as places: block << M.shift | index) is laid out once as an image of the blocks' shared memory and
 // copied in by 16-byte loads that are all in flight at once, and a row's reads do not wait for one another.
-// Levels of 8227, 1032 and 136 unknowns: 20 us (FP64 38), 48 us through L2 with device-wide fences and rows read
-// where they are used (FP64 80).
+// Levels of 8227, 1032 and 136 unknowns: 18 us (FP64 32, of which the FP64 units of 16 SMs are half); with eight
+// blocks 20 us (FP64 38), 48 us through L2 with device-wide fences and rows read where they are used (FP64 80).
 #define MG_TAIL_NT 512
 #define MG_FAR 0xffffu          // first place of a row with more than MG_ELL links: start and count follow
 
 struct TailPlace {
     MGTailLev t;
+    int shift;
     __device__ __forceinline__ unsigned operator()(int u) const {
         const bool c = u >= t.M0;
         const unsigned w = (unsigned)(c ? u - t.M0 : u), s = (unsigned)(c ? t.s1 : t.s0);
         const unsigned r = __umulhi(w, c ? t.i1 : t.i0);
-        return r << 13 | ((c ? (unsigned)t.s0 : 0u) + w - r * s);
+        return r << shift | ((c ? (unsigned)t.s0 : 0u) + w - r * s);
     }
 };
 
@@ -1177,8 +1179,9 @@ template <class T>
 struct TailLevel {
     MGTailLev t;
     unsigned char* sm;
-    int rank;
-    __device__ __forceinline__ TailLevel(const MGTail& M, int l, unsigned char* s, int r) : t(M.t[l]), sm(s), rank(r) {}
+    int rank, shift;
+    __device__ __forceinline__ TailLevel(const MGTail& M, int l, unsigned char* s, int r)
+        : t(M.t[l]), sm(s), rank(r), shift(M.shift) {}
     template <class V>
     __device__ __forceinline__ V* arr(int o) const { return reinterpret_cast<V*>(sm + o); }
     __device__ __forceinline__ T* x() const { return arr<T>(t.x); }
@@ -1196,7 +1199,7 @@ struct TailLevel {
     }
     // value of an array (a pointer into this block's shared memory) at a place
     __device__ __forceinline__ T at(const T* a, unsigned place) const {
-        return *cg::this_cluster().map_shared_rank(const_cast<T*>(a) + (place & 8191u), place >> 13);
+        return *cg::this_cluster().map_shared_rank(const_cast<T*>(a) + (place & ((1u << shift) - 1u)), place >> shift);
     }
     // sum over the links of local unknown i of g f(place of the neighbour, place of its parent)
     template <bool PARENT, class Fn>
@@ -1235,7 +1238,7 @@ __global__ void __launch_bounds__(256) k_tail_image(MGTail M, unsigned char* img
     for (int l = M.first; l <= last; ++l) {
         const TailLevel<T> A(M, l, sm, rank);
         const MGLev& L = M.lev[l];
-        const TailPlace here{A.t}, up{M.t[l < last ? l + 1 : l]}, below{M.t[l > M.first ? l - 1 : l]};
+        const TailPlace here{A.t, M.shift}, up{M.t[l < last ? l + 1 : l], M.shift}, below{M.t[l > M.first ? l - 1 : l], M.shift};
         const int S = A.t.s0 + A.t.s1;
         int nch = 0;
         for (int c = 0; c < 2; ++c) {
@@ -1799,7 +1802,7 @@ int build_ell(MGLev& L) {
 
 // Shares and shared-memory layout of the tail for levels first .. nlev - 1; its bytes per block (0: too large).
 long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
-    const int last = mg.nlev - 1, blocks = first < last ? MG_TAIL_CTAS : 1;
+    const int last = mg.nlev - 1, blocks = first < last ? M.ctas : 1, most = (1 << M.shift) - 1;
     long long o = 0;
     auto take = [&](long long bytes) {
         const long long at = o;
@@ -1811,7 +1814,7 @@ long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
         const MGLev& L = mg.lev[l];
         MGTailLev& t = M.t[l];
         const long long M1 = L.M - L.M0;
-        if (L.M > 8191LL * MG_TAIL_CTAS || (l == last && L.M > 8191)) return 0;
+        if (L.M > (long long)most * M.ctas || (l == last && L.M > most)) return 0;
         t.M = (int)L.M;
         t.M0 = (int)L.M0;
         const int nb = l < last ? blocks : 1;
@@ -1825,7 +1828,7 @@ long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
         if (t.s0 == 1) t.i0 = 0;
         if (t.s1 == 1) t.i1 = 0;
         const long long S = t.s0 + t.s1;
-        if (S > 8191) return 0;
+        if (S > most) return 0;
         t.col = take(S * 2 * MG_ELL);
         t.pc = take(l < last ? S * 2 * MG_ELL : 0);
         t.g = take(S * sb * MG_ELL);
@@ -1877,6 +1880,31 @@ long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
     return o <= 220 * 1024 ? o : 0;
 }
 
+cudaLaunchConfig_t tail_config(int blocks, int smem, cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(MG_TAIL_NT);
+    cfg.dynamicSmemBytes = smem;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Whether the GPU can hold a cluster of MG_TAIL_BIG blocks (above the portable size).
+bool tail_fits(int sb, int smem) {
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = tail_config(MG_TAIL_BIG, smem, at);
+    int n = 0;
+    const cudaError_t e = sb == 8 ? cudaOccupancyMaxActiveClusters(&n, k_mg_tail<double>, &cfg)
+                                  : cudaOccupancyMaxActiveClusters(&n, k_mg_tail<float>, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && n > 0;
+}
+
 // The tail starts at the first level whose shares fit, of those with at most MG_TAIL_MAX unknowns; a coarsest
 // level too large for one block's shared memory runs from global memory (tail_smem = 0).
 int tail_plan(MG& mg, int sb) {
@@ -1884,6 +1912,10 @@ int tail_plan(MG& mg, int sb) {
     mg.tail_first = last;
     mg.tail_smem = 0;
     if (last < 1) return IBM_OK;
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     mg.tail = (MGTail*)calloc(1, sizeof(MGTail));
     if (!mg.tail) return ibm_fail(IBM_E_NOMEM, "multigrid set-up: host allocation");
     for (int l = 0; l < IBM_MG_MAXLEV; ++l) mg.tail->lev[l] = mg.lev[l];
@@ -1892,21 +1924,24 @@ int tail_plan(MG& mg, int sb) {
     mg.tail->omega = mg.omega;
     for (int l = 1; l <= last; ++l) {
         if (l < last && mg.lev[l].M > MG_TAIL_MAX) continue;
-        int rc;
-        const long long bytes = tail_layout(mg, *mg.tail, l, sb, rc);
-        if (rc) return rc;
-        if (bytes > 0) {
+        for (int big = 1; big >= 0 && mg.tail_smem == 0; --big) {
+            int rc;
+            mg.tail->ctas = big ? MG_TAIL_BIG : 8;
+            mg.tail->shift = big ? 12 : 13;
+            const long long bytes = tail_layout(mg, *mg.tail, l, sb, rc);
+            if (rc) return rc;
+            if (bytes == 0 || (big && l < last && !tail_fits(sb, (int)bytes))) continue;
             mg.tail->first = mg.tail_first = l;
             mg.tail_smem = (int)bytes;
-            break;
         }
+        if (mg.tail_smem > 0) break;
     }
     if (mg.tail_smem > 0) {
-        const int blocks = mg.tail_first < last ? MG_TAIL_CTAS : 1;
+        const int blocks = mg.tail_first < last ? mg.tail->ctas : 1;
         int* cur = nullptr;
         MG_ALLOCB(mg.tail_img, (size_t)blocks * mg.tail->image);
-        MG_ALLOC(cur, MG_TAIL_CTAS * IBM_MG_MAXLEV);
-        cudaError_t e = cudaMemset(cur, 0, sizeof(int) * MG_TAIL_CTAS * IBM_MG_MAXLEV);
+        MG_ALLOC(cur, blocks * IBM_MG_MAXLEV);
+        cudaError_t e = cudaMemset(cur, 0, sizeof(int) * blocks * IBM_MG_MAXLEV);
         if (e == cudaSuccess) e = cudaMemset(mg.tail_img, 0, (size_t)blocks * mg.tail->image);
         if (e == cudaSuccess) {
             mg.tail->img = (const uint4*)mg.tail_img;
@@ -1918,8 +1953,6 @@ int tail_plan(MG& mg, int sb) {
         cudaFree(cur);
         if (e != cudaSuccess) return ibm_cuda_check(e, "multigrid set-up: tail");
     }
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
     return IBM_OK;
 }
 
@@ -2030,18 +2063,9 @@ static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStrea
         launches += 2;
     }
     if (mg.tail_smem > 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(tf < last ? MG_TAIL_CTAS : 1);
-        cfg.blockDim = dim3(MG_TAIL_NT);
-        cfg.dynamicSmemBytes = mg.tail_smem;
-        cfg.stream = s;
         cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = cfg.gridDim.x;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
+        cudaLaunchConfig_t cfg = tail_config(tf < last ? mg.tail->ctas : 1, mg.tail_smem, at);
+        cfg.stream = s;
         IBM_CUDA(cudaLaunchKernelEx(&cfg, k_mg_tail<T>, *mg.tail, (const SolveScal*)sc));
     } else {
         k_gcoarsest<T><<<1, 1024, 0, s>>>(mg.lev[last], mg.coarse_sweeps, sc);
