@@ -170,7 +170,7 @@ static int check_params(const les_params* p) {
 
 #define ALLOC(ptr, bytes)                                                                \
     do {                                                                                 \
-        cudaError_t e_ = cudaMalloc((void**)&(ptr), (bytes) > 0 ? (bytes) : 16);          \
+        cudaError_t e_ = ibm_malloc(&(ptr), (bytes) > 0 ? (bytes) : 16);          \
         if (e_ != cudaSuccess) {                                                         \
             free_state(S);                                                               \
             return ibm_fail(IBM_E_NOMEM, "les_create: %s (%zu bytes)", cudaGetErrorString(e_), (size_t)(bytes)); \
@@ -332,8 +332,8 @@ extern "C" int les_attach_guess(les_state* S, ibm_net* net) {
     if (net && !S->p_prev) {
         const size_t N = (size_t)S->c.D.N;
         cudaError_t e;
-        if ((e = cudaMalloc(&S->p_prev, N * 8)) != cudaSuccess || (e = cudaMalloc(&S->p_keep, N * 8)) != cudaSuccess ||
-            (e = cudaMalloc(&S->x_guess, N * 8)) != cudaSuccess || (e = cudaMalloc(&S->two_res, 2 * 8)) != cudaSuccess)
+        if ((e = ibm_malloc(&S->p_prev, N * 8)) != cudaSuccess || (e = ibm_malloc(&S->p_keep, N * 8)) != cudaSuccess ||
+            (e = ibm_malloc(&S->x_guess, N * 8)) != cudaSuccess || (e = ibm_malloc(&S->two_res, 2 * 8)) != cudaSuccess)
             return ibm_fail(IBM_E_NOMEM, "les_attach_guess: %s", cudaGetErrorString(e));
         S->steps = 0;
     }

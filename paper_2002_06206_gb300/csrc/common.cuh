@@ -21,6 +21,11 @@ struct LinkRec {
     double uib[3];
 };
 
+// cudaMalloc that gives freed geometry memory back (classify.cu) before it fails.
+cudaError_t ibm_malloc_bytes(void** p, size_t bytes);
+template <class T>
+inline cudaError_t ibm_malloc(T** p, size_t bytes) { return ibm_malloc_bytes((void**)p, bytes); }
+
 // Everything a cell kernel needs to know about the grid, the boundaries and the immersed body.
 struct Dom {
     int nx, ny, nz;

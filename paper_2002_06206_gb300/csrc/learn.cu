@@ -434,11 +434,11 @@ static int net_reserve(ibm_net* n, long long N) {
     n->cap_cells = 0;
     const size_t act = (size_t)N * NN_C * sizeof(__nv_bfloat16);
     cudaError_t e;
-    if ((e = cudaMalloc(&n->x0, act)) != cudaSuccess || (e = cudaMalloc(&n->y1, act)) != cudaSuccess ||
-        (e = cudaMalloc(&n->y2, act)) != cudaSuccess || (e = cudaMalloc(&n->d3, act)) != cudaSuccess ||
-        (e = cudaMalloc(&n->d2, act)) != cudaSuccess || (e = cudaMalloc(&n->d1, act)) != cudaSuccess ||
-        (e = cudaMalloc(&n->out, (size_t)N * sizeof(float))) != cudaSuccess ||
-        (e = cudaMalloc(&n->wpart, (size_t)WG_BLOCKS * WG_STRIDE * sizeof(float))) != cudaSuccess)
+    if ((e = ibm_malloc(&n->x0, act)) != cudaSuccess || (e = ibm_malloc(&n->y1, act)) != cudaSuccess ||
+        (e = ibm_malloc(&n->y2, act)) != cudaSuccess || (e = ibm_malloc(&n->d3, act)) != cudaSuccess ||
+        (e = ibm_malloc(&n->d2, act)) != cudaSuccess || (e = ibm_malloc(&n->d1, act)) != cudaSuccess ||
+        (e = ibm_malloc(&n->out, (size_t)N * sizeof(float))) != cudaSuccess ||
+        (e = ibm_malloc(&n->wpart, (size_t)WG_BLOCKS * WG_STRIDE * sizeof(float))) != cudaSuccess)
         return ibm_fail(IBM_E_NOMEM, "ibm_net: %s", cudaGetErrorString(e));
     n->cap_cells = N;
     return IBM_OK;
@@ -469,16 +469,16 @@ extern "C" int ibm_net_create(const float* h_params, ibm_net** out) {
     cudaError_t e;
     const size_t pb = (NN_NPARAM + 16) * sizeof(float);   // padded: layer 3's bias is read as 8 lanes
     const size_t fb = NN_KSTEPS * 32 * 2 * sizeof(uint32_t);
-    if ((e = cudaMalloc(&n->master, pb)) != cudaSuccess || (e = cudaMalloc(&n->grad, pb)) != cudaSuccess ||
-        (e = cudaMalloc(&n->m, pb)) != cudaSuccess || (e = cudaMalloc(&n->v, pb)) != cudaSuccess ||
-        (e = cudaMalloc(&n->scal, 8 * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&n->partials, 8 * 8 * IBM_NSM * sizeof(double) * 2)) != cudaSuccess ||
-        (e = cudaMalloc(&n->counter, 4 * sizeof(unsigned))) != cudaSuccess) {
+    if ((e = ibm_malloc(&n->master, pb)) != cudaSuccess || (e = ibm_malloc(&n->grad, pb)) != cudaSuccess ||
+        (e = ibm_malloc(&n->m, pb)) != cudaSuccess || (e = ibm_malloc(&n->v, pb)) != cudaSuccess ||
+        (e = ibm_malloc(&n->scal, 8 * sizeof(double))) != cudaSuccess ||
+        (e = ibm_malloc(&n->partials, 8 * 8 * IBM_NSM * sizeof(double) * 2)) != cudaSuccess ||
+        (e = ibm_malloc(&n->counter, 4 * sizeof(unsigned))) != cudaSuccess) {
         ibm_net_destroy(n);
         return ibm_fail(IBM_E_NOMEM, "ibm_net_create: %s", cudaGetErrorString(e));
     }
     for (int l = 0; l < 3; ++l)
-        if ((e = cudaMalloc(&n->frag_fwd[l], fb)) != cudaSuccess || (e = cudaMalloc(&n->frag_bwd[l], fb)) != cudaSuccess) {
+        if ((e = ibm_malloc(&n->frag_fwd[l], fb)) != cudaSuccess || (e = ibm_malloc(&n->frag_bwd[l], fb)) != cudaSuccess) {
             ibm_net_destroy(n);
             return ibm_fail(IBM_E_NOMEM, "ibm_net_create: %s", cudaGetErrorString(e));
         }

@@ -1435,9 +1435,9 @@ int flux_kernels_setup() {
 int build_general_list(LesCtx& c, cudaStream_t s) {
     const long long nrows = (long long)c.D.ny * c.D.nz;
     unsigned long long* rc = nullptr;
-    IBM_CUDA(cudaMalloc((void**)&rc, (size_t)(nrows + 1) * sizeof(unsigned long long)));
+    IBM_CUDA(ibm_malloc(&rc, (size_t)(nrows + 1) * sizeof(unsigned long long)));
     dim3 rows((unsigned)c.D.ny, (unsigned)c.D.nz);
-    cudaError_t e0 = cudaMalloc((void**)&c.fastmask, (size_t)c.D.N);
+    cudaError_t e0 = ibm_malloc(&c.fastmask, (size_t)c.D.N);
     if (e0 != cudaSuccess) {
         cudaFree(rc);
         return ibm_fail(IBM_E_NOMEM, "momentum flux: fast-cell mask (%lld bytes)", (long long)c.D.N);
@@ -1447,7 +1447,7 @@ int build_general_list(LesCtx& c, cudaStream_t s) {
     unsigned long long total = 0;
     cudaError_t e = cudaMemcpyAsync(&total, rc + nrows, sizeof(total), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&c.general, (size_t)(total > 0 ? total : 1) * sizeof(int32_t));
+    if (e == cudaSuccess) e = ibm_malloc(&c.general, (size_t)(total > 0 ? total : 1) * sizeof(int32_t));
     if (e == cudaSuccess && total > 0) {
         k_list_general<<<rows, 32, 0, s>>>(c.D, rc, c.general);
         e = cudaGetLastError();

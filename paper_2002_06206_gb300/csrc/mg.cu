@@ -1753,12 +1753,12 @@ void free_level(MGLev& L) {
 
 #define MG_ALLOC(ptr, n)                                                                         \
     do {                                                                                         \
-        cudaError_t e_ = cudaMalloc((void**)&(ptr), ((n) > 0 ? (size_t)(n) : 1) * sizeof(*(ptr))); \
+        cudaError_t e_ = ibm_malloc(&(ptr), ((n) > 0 ? (size_t)(n) : 1) * sizeof(*(ptr))); \
         if (e_ != cudaSuccess) return ibm_cuda_check(e_, "multigrid set-up: " #ptr);              \
     } while (0)
 #define MG_ALLOCB(ptr, bytes)                                                                    \
     do {                                                                                         \
-        cudaError_t e_ = cudaMalloc((void**)&(ptr), (size_t)(bytes) > 0 ? (size_t)(bytes) : 16); \
+        cudaError_t e_ = ibm_malloc(&(ptr), (size_t)(bytes) > 0 ? (size_t)(bytes) : 16); \
         if (e_ != cudaSuccess) return ibm_cuda_check(e_, "multigrid set-up: " #ptr);              \
     } while (0)
 

@@ -261,7 +261,7 @@ extern "C" int ibm_surface_create(const ibm_grid* g, const float* d_tri, int64_t
     long long* tiles = nullptr;
     cudaError_t e = cudaSuccess;
 #define SALLOC(p, bytes)                                                     \
-    if (e == cudaSuccess) e = cudaMalloc((void**)&(p), (size_t)(bytes))
+    if (e == cudaSuccess) e = ibm_malloc(&(p), (size_t)(bytes))
     SALLOC(S->off, (nb + 1) * sizeof(long long));
     SALLOC(cnt, nb * sizeof(unsigned));
     SALLOC(tiles, (nt + 1) * sizeof(long long));
@@ -286,7 +286,7 @@ extern "C" int ibm_surface_create(const ibm_grid* g, const float* d_tri, int64_t
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) {
         S->nent = total;
-        e = cudaMalloc((void**)&S->ent, (size_t)(total > 0 ? total : 1) * sizeof(int32_t));
+        e = ibm_malloc(&S->ent, (size_t)(total > 0 ? total : 1) * sizeof(int32_t));
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, nb * sizeof(unsigned), s);
     if (e == cudaSuccess && ntri > 0) {

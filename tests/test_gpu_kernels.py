@@ -270,3 +270,35 @@ def test_momentum_flux_of_cells_with_any_links_is_the_oracles(L, shape, bc, quic
     assert np.linalg.norm(dev[3].cpu().numpy() - Hr) <= tol * scale
     assert np.linalg.norm(us.cpu().numpy() - ur) <= tol * (np.linalg.norm(ur) + 0.15 * scale)
     sol.close()
+
+
+def test_geometries_made_and_destroyed_on_several_threads_and_streams(L):
+    """Tables made from memory that another geometry gave back are the same as the first ones."""
+    import threading
+    import workloads as W
+    shapes = [(40, 30, 20), (64, 64, 64), (9, 8, 7)]
+    soups = [torch.from_numpy(W.random_soup(80, (1, 1, 1), tuple(n - 1 for n in s), 4.0, seed=3).astype(np.float32)).cuda()
+             for s in shapes]
+
+    def tables(q):
+        geo = L.Geometry(L.make_grid(*shapes[q]), soups[q])
+        out = [v.cpu().numpy() for v in geo.export()]
+        geo.close()
+        return out
+
+    first = [tables(q) for q in range(3)]
+    wrong = []
+
+    def work(seed):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for n in range(8):
+                q = (seed + n) % 3
+                if not all(np.array_equal(a, b) for a, b in zip(tables(q), first[q])):
+                    wrong.append((seed, n))
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
