@@ -34,40 +34,135 @@ __device__ __forceinline__ void grad_at(const Dom& D, const T* __restrict__ u, l
 
 __device__ __forceinline__ unsigned flags_at(const Dom& D, long long P) { return D.flags ? (unsigned)D.flags[P] : 0u; }
 
-// Eq. Smagorinsky with the coherent-structure coefficient of Eq. Q / Eq. FCS.  One thread per cell.
+// Domain-boundary ghost of component c across face (a, s) of the cell holding v (vel_across's rules).
 template <class T>
-__global__ void __launch_bounds__(256) k_csm(Dom D, const T* __restrict__ u, T* __restrict__ nut) {
-    const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y, k = blockIdx.z;
-    if (i >= D.nx || j >= D.ny) return;
-    const T inv2dx = (T)0.5 * dom_idx<T>(D), delta2 = dom_dx<T>(D) * dom_dx<T>(D);
-    const long long P = i + (long long)D.sy * j + D.sz * k;
-    const unsigned fl = flags_at(D, P);
-    const int x[3] = {i, j, k};
-    T G[3][3];
-    if (fl == 0u && i > 0 && i < D.nx - 1 && j > 0 && j < D.ny - 1 && k > 0 && k < D.nz - 1) {
-        const long long o[3] = {1, (long long)D.sy, D.sz};
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) G[a][b] = (u[b * D.N + P + o[a]] - u[b * D.N + P - o[a]]) * inv2dx;
-    } else {
-        grad_at(D, u, P, x, fl, inv2dx, G);
+__device__ __forceinline__ T bc_ghost(const Dom& D, int a, int s, int c, T v) {
+    switch (D.bc[2 * a + (s > 0)]) {
+        case IBM_BC_INFLOW: return (D.hom ? (T)0 : (T)2 * (T)D.u_in[c]) - v;
+        case IBM_BC_OUTFLOW: return v;
+        case IBM_BC_SLIP: return c == a ? -v : v;
+        default: return -v;
     }
-    T SS = 0, WW = 0;
+}
+
+// base is the same for the whole block, the byte offset within a plane fixed per thread (a plane has less
+// than 2^31/3 cells: 32 bits for FP32): one add per access.
+template <class T>
+using Off = std::conditional_t<sizeof(T) == 4, unsigned, unsigned long long>;
+
+template <class T>
+__device__ __forceinline__ T at_off(const T* base, Off<T> off) {
+    return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
+}
+
+template <class T>
+__device__ __forceinline__ void to_off(T* base, Off<T> off, T v) {
+    *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off) = v;
+}
+
+// Eq. Smagorinsky with the coherent-structure coefficient of Eq. Q / Eq. FCS.
+//
+// A thread marches through kz planes of one (x, y) column with the velocity of three planes in registers; the x
+// neighbours come by shuffle, the rows above and below from L1.  Cells on a domain face take the boundary's ghosts
+// in place; only cells with a cut link go through vel_across.  With g = the undivided central differences,
+// 4 dx^2 S:S = A + B / 2 and 4 dx^2 W:W = C / 2 for A = sum g_aa^2, B = sum (g_ab + g_ba)^2, C = sum (g_ab - g_ba)^2.
+// 512 x 256 x 256 in FP32: 266 us, of 270 instructions per cell (addresses mostly; 16 bytes per cell would take 80);
+// 338 us with one thread per cell and 18 loads.  251 x 127 x 93, two planes per thread: 39 -> 35 us (55 with eight, 44
+// with one).  FP64 128 x 64 x 64: 110 -> 59 us, one square root in place of two and half of the products.
+template <class T>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_csm(Dom D, const T* __restrict__ u, T* __restrict__ nut, int kz) {
+    const int i0 = blockIdx.x * IBM_TX + threadIdx.x, j0 = blockIdx.y * IBM_TY + threadIdx.y;
+    const bool active = i0 < D.nx && j0 < D.ny;
+    const int i = min(i0, D.nx - 1), j = min(j0, D.ny - 1);
+    const int k0 = blockIdx.z * kz, k1 = min(k0 + kz, D.nz);
+    const T scale = (T)(1.0 / 40.0) * dom_dx<T>(D);              // C / F^(3/2), dx^2 and 1 / (2 dx)
+    long long xl = 0, xh = 0, yl = 0, yh = 0, zo = 0;
+    const bool hxl = nb_offset(D, 0, -1, i, xl), hxh = nb_offset(D, 0, 1, i, xh);
+    const bool hyl = nb_offset(D, 1, -1, j, yl), hyh = nb_offset(D, 1, 1, j, yh);
+    const bool endl = threadIdx.x == 0 || i == 0, endh = threadIdx.x == 31 || i == D.nx - 1, both = endl && endh;
+    // byte offsets within a plane: the cell, its y neighbours, the x neighbour a warp's end needs (the cell itself
+    // where there is none)
+    const int p = i + D.sy * j;
+    const Off<T> o = (Off<T>)p * sizeof(T), oyl = (Off<T>)(p + (int)yl) * sizeof(T), oyh = (Off<T>)(p + (int)yh) * sizeof(T),
+                 oe = (Off<T>)(p + (int)(endl ? xl : xh)) * sizeof(T), oh = (Off<T>)(p + (int)xh) * sizeof(T);
+    const bool hx = hxl && hxh && hyl && hyh;
+    const T* U0 = u + D.sz * k0;
+    T m[3], v[3], n[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int c = 0; c < 3; ++c) v[c] = at_off(U0 + c * D.N, o);
+    const bool hzl = nb_offset(D, 2, -1, k0, zo);
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const T S = (T)0.5 * (G[a][b] + G[b][a]);
-            const T W = (T)0.5 * (G[a][b] - G[b][a]);
-            SS += S * S;
-            WW += W * W;
+    for (int c = 0; c < 3; ++c) m[c] = hzl ? at_off(U0 + c * D.N + zo, o) : bc_ghost(D, 2, -1, c, v[c]);
+    for (int k = k0; k < k1; ++k) {
+        zo = 0;
+        const bool hzh = nb_offset(D, 2, 1, k, zo);
+        const T* Uk = u + D.sz * k;
+        T gx[3], gy[3], gz[3], b[3], t[3], e[3] = {}, g[3] = {};
+        // loads first, from the cell itself where there is no neighbour
+#pragma unroll
+        for (int c = 0; c < 3; ++c) n[c] = at_off(Uk + c * D.N + zo, o);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) b[c] = at_off(Uk + c * D.N, oyl);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) t[c] = at_off(Uk + c * D.N, oyh);
+        if (endl || endh) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) e[c] = at_off(Uk + c * D.N, oe);
         }
-    const T Q = (T)0.5 * (WW - SS), E = (T)0.5 * (WW + SS);
-    const T F = E > (T)0 ? Q / E : (T)0;
-    const T aF = F < (T)0 ? -F : F;
-    const T C = (T)(1.0 / 20.0) * (aF * sqrt(aF));
-    nut[P] = C * delta2 * sqrt(SS);
+        if (both) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) g[c] = at_off(Uk + c * D.N, oh);
+        }
+        const unsigned fl = D.flags ? (D.flags + D.sz * k)[(unsigned)p] & 63u : 0u;
+        T l[3], h[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            l[c] = __shfl_up_sync(0xffffffffu, v[c], 1);
+            h[c] = __shfl_down_sync(0xffffffffu, v[c], 1);
+            if (endl) l[c] = e[c];
+            if (endh) h[c] = both ? g[c] : e[c];
+        }
+        if (__any_sync(0xffffffffu, !(hx && hzh))) {    // ghosts of the domain faces
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (!hxl) l[c] = bc_ghost(D, 0, -1, c, v[c]);
+                if (!hxh) h[c] = bc_ghost(D, 0, 1, c, v[c]);
+                if (!hyl) b[c] = bc_ghost(D, 1, -1, c, v[c]);
+                if (!hyh) t[c] = bc_ghost(D, 1, 1, c, v[c]);
+                if (!hzh) n[c] = bc_ghost(D, 2, 1, c, v[c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            gx[c] = h[c] - l[c];
+            gy[c] = t[c] - b[c];
+            gz[c] = n[c] - m[c];
+        }
+        if (__any_sync(0xffffffffu, fl != 0u) && fl != 0u) {
+            const int x[3] = {i, j, k};
+            T G[3][3];
+            grad_at(D, u, p + D.sz * k, x, fl, (T)1, G);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                gx[c] = G[0][c];
+                gy[c] = G[1][c];
+                gz[c] = G[2][c];
+            }
+        }
+        const T s0 = gx[1] + gy[0], s1 = gx[2] + gz[0], s2 = gy[2] + gz[1];
+        const T w0 = gx[1] - gy[0], w1 = gx[2] - gz[0], w2 = gy[2] - gz[1];
+        const T A = gx[0] * gx[0] + gy[1] * gy[1] + gz[2] * gz[2];
+        const T SS = A + (T)0.5 * (s0 * s0 + s1 * s1 + s2 * s2), WW = (T)0.5 * (w0 * w0 + w1 * w1 + w2 * w2);
+        const T E = WW + SS;
+        const T F = E > (T)0 ? (WW - SS) / E : (T)0;
+        const T aF = F < (T)0 ? -F : F;
+        if (active) to_off(nut + D.sz * k, o, scale * (aF * sqrt(aF * SS)));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            m[c] = v[c];
+            v[c] = n[c];
+        }
+    }
 }
 
 // L(u) of a cell per unit volume: flux-form advection with the face velocity U, diffusion with nu + nu_t, the
@@ -127,17 +222,6 @@ __device__ __forceinline__ bool fast_cell(const Dom& D, long long P, int i, int 
 #define FT_NT (FT_X * FT_Y)
 #define FT_FXN (FT_Y * (FT_X + 1))     // x faces of a tile plane, per component
 #define FT_FYN ((FT_Y + 1) * FT_X)     // y faces
-
-// Domain-boundary ghost of component c across face (a, s) of the cell holding v (vel_across's rules).
-template <class T>
-__device__ __forceinline__ T bc_ghost(const Dom& D, int a, int s, int c, T v) {
-    switch (D.bc[2 * a + (s > 0)]) {
-        case IBM_BC_INFLOW: return (D.hom ? (T)0 : (T)2 * (T)D.u_in[c]) - v;
-        case IBM_BC_OUTFLOW: return v;
-        case IBM_BC_SLIP: return c == a ? -v : v;
-        default: return -v;
-    }
-}
 
 // Coefficients of the faces of one axis at one place.
 template <class T>
@@ -200,21 +284,6 @@ __device__ __forceinline__ void face_inplane(const FaceW<T>& w, const FaceK<T>& 
     const T db = w.wl * (s[B - E] - s[-B - E]) + w.wr * (s[B] - s[-B]);
     const T dzs = w.wl * (Sp[A * FT_PL + q - E] - Sm[A * FT_PL + q - E]) + w.wr * dz;
     face_phi<T, A>(w, K, Uf, l, r, far, db, dzs, S0[3 * FT_PL + q - E] + nr, phi);
-}
-
-// base is the same for the whole block, the byte offset within a plane fixed per thread (a plane has less
-// than 2^31/3 cells: 32 bits for FP32): one add per access.
-template <class T>
-using Off = std::conditional_t<sizeof(T) == 4, unsigned, unsigned long long>;
-
-template <class T>
-__device__ __forceinline__ T at_off(const T* base, Off<T> off) {
-    return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
-}
-
-template <class T>
-__device__ __forceinline__ void to_off(T* base, Off<T> off, T v) {
-    *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off) = v;
 }
 
 // Calls epi(plane, off, h, u, w) for the fast cells: the cell is plane + off / sizeof(T), plane uniform; w holds
@@ -724,11 +793,11 @@ __device__ __forceinline__ double cut_face_velocity(const Dom& D, long long L, l
 }
 
 // A thread of the face and correction kernels takes one (x, y) column of `kz` planes, so the z neighbour
-// of a plane is the register of the next; kz falls to 1 on grids that would not fill the GPU otherwise.
-inline dim3 column_grid(const Dom& D, int& kz) {
+// of a plane is the register of the next; kz falls to 1 on grids that would give fewer than `least` blocks.
+inline dim3 column_grid(const Dom& D, int& kz, long long least = 8LL * IBM_NSM) {
     const long long bxy = (long long)((D.nx + IBM_TX - 1) / IBM_TX) * ((D.ny + IBM_TY - 1) / IBM_TY);
     kz = 8;
-    while (kz > 1 && bxy * ((D.nz + kz - 1) / kz) < 8LL * IBM_NSM) kz >>= 1;
+    while (kz > 1 && bxy * ((D.nz + kz - 1) / kz) < least) kz >>= 1;
     return flat_grid(D.nx, D.ny, D.nz, kz);
 }
 
@@ -1462,10 +1531,10 @@ int build_general_list(LesCtx& c, cudaStream_t s) {
 }
 
 int launch_csm(const LesCtx& c, const void* u, void* nut, cudaStream_t s) {
-    if (c.prec == IBM_FP64)
-        k_csm<double><<<c.pgrid, c.cg.block, 0, s>>>(c.D, (const double*)u, (double*)nut);
-    else
-        k_csm<float><<<c.pgrid, c.cg.block, 0, s>>>(c.D, (const float*)u, (float*)nut);
+    int kz = 1;
+    const dim3 g = column_grid(c.D, kz, 24LL * IBM_NSM);        // four rounds of six blocks per SM
+    if (c.prec == IBM_FP64) k_csm<double><<<g, c.cg.block, 0, s>>>(c.D, (const double*)u, (double*)nut, kz);
+    else k_csm<float><<<g, c.cg.block, 0, s>>>(c.D, (const float*)u, (float*)nut, kz);
     IBM_LAUNCHED("k_csm");
     IBM_COUNT(c, 1);
     return IBM_OK;

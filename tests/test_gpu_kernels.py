@@ -265,6 +265,11 @@ def test_momentum_flux_of_cells_with_any_links_is_the_oracles(L, shape, bc, quic
     dev = [torch.from_numpy(v).to("cuda", td) for v in (u, U, nut, H0)]
     us = torch.empty(3 * N, dtype=td, device="cuda")
     sol.predict(dev[0], dev[1], dev[2], dev[3], dev[3], us, False)
+    # eddy viscosity: ghosts at every boundary and cut link, the first and last planes of a column
+    nut_dev = torch.empty(N, dtype=td, device="cuda")
+    sol.csm(dev[0], nut_dev)
+    nut_ref = ref.csm(u.astype(np.float64))
+    assert np.linalg.norm(nut_dev.cpu().numpy() - nut_ref) <= tol * np.linalg.norm(nut_ref)
     Hr, ur = ref.predict(u.astype(np.float64), U.astype(np.float64), nut.astype(np.float64), H0.astype(np.float64), False)
     scale = np.linalg.norm(np.abs(U).max() * np.abs(u)) + np.linalg.norm(Hr)
     assert np.linalg.norm(dev[3].cpu().numpy() - Hr) <= tol * scale
