@@ -54,37 +54,48 @@ __global__ void __launch_bounds__(256) k_apply(Dom D, const T* __restrict__ p, T
     CELL_LOOP_END
 }
 
-// r = b - A x in FP64; stores r in the working precision; res2 = ||r||^2 (FP64), rr = ||(Tr) r||^2.
-template <class Tr>
+// r = b - A x in FP64; stores r in the working precision; res2 = rr = ||(Tr) r||^2.
+// Bound by the FP64 units: five additions, two fused multiply-adds and the rounding to FP32 per cell, at cells with
+// a cut link or a domain face too (count of links from a table).  512 x 256 x 256 to FP32: 740 -> 565 us (the eight
+// operations take 500), 256 x 128 x 128 around a dirty sphere 115 -> 73 us.
+template <class Tr, int KU>
 __global__ void __launch_bounds__(256) k_residual(Dom D, const double* __restrict__ b, const double* __restrict__ x64,
                                                   Tr* __restrict__ r, double idx2, SolveScal* sc, double* partials,
                                                   unsigned* counter) {
-    Tr part0 = 0, part1 = 0;     // norms accumulated per thread in the working precision
+    Tr part = 0;                 // accumulated per thread in the working precision
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
-    const int kb = blockIdx.z * IBM_KU;
+    const int kb = blockIdx.z * KU;
     const bool active = i < D.nx && j < D.ny;
     auto xv = [&](long long n) { return x64[n]; };
 #pragma unroll
-    for (int u = 0; u < IBM_KU; ++u) {
+    for (int u = 0; u < KU; ++u) {
         const int k = kb + u;
         if (active && k < D.nz) {
             const long long P = i + (long long)D.sy * j + D.sz * k;
             const unsigned fl = D.flags ? (unsigned)D.flags[P] : 0u;
-            const double ap = link_sum7<double>(D, P, i, j, k, fl, x64[P], xv) * idx2;
-            const double rv = b[P] - ap;
+            const CellLinks L = cell_links(D, i, j, k, fl);
+            const int dg = __popc(L.open) + 2 * __popc(L.out & ~fl);
+            const double rv = fma(-idx2, fma(-small_num<double>(dg), x64[P], open_sum<double>(L, P, xv)), b[P]);
             const Tr rt = (Tr)rv;
             if (r) r[P] = rt;
-            if constexpr (std::is_same<Tr, double>::value) part0 += rv * rv;
-            else part0 += rt * rt;
-            part1 += rt * rt;
+            part += rt * rt;
         }
     }
-    decltype(part0) acc[2] = {part0, part1};
-    grid_reduce<2>(acc, partials, counter, [&](double* t) {
+    decltype(part) acc[1] = {part};
+    grid_reduce<1>(acc, partials, counter, [&](double* t) {
         sc->res2 = t[0];
-        sc->rr = t[1];
+        sc->rr = t[0];
         if (!isfinite(t[0])) sc->nonfinite = 1;
     });
+}
+
+template <class Tr>
+void launch_residual(const LesCtx& c, const double* b, const double* x, Tr* r, double idx2, SolveScal* sc, cudaStream_t s) {
+    // one plane per thread where four would leave SMs idle
+    if ((long long)c.fgrid.x * c.fgrid.y * c.fgrid.z < IBM_NSM)
+        k_residual<Tr, 1><<<flat_grid(c.D.nx, c.D.ny, c.D.nz, 1), c.cg.block, 0, s>>>(c.D, b, x, r, idx2, sc, c.partials, c.counter);
+    else
+        k_residual<Tr, IBM_KU><<<c.fgrid, c.cg.block, 0, s>>>(c.D, b, x, r, idx2, sc, c.partials, c.counter);
 }
 
 __global__ void __launch_bounds__(256) k_dot_bb(Dom D, const double* __restrict__ b, SolveScal* sc, double* partials,
@@ -225,9 +236,20 @@ __global__ void __launch_bounds__(256) k_cg_update(long long N, const T* __restr
     });
 }
 
-__global__ void k_add_correction(long long N, double* __restrict__ x, const float* __restrict__ e) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x)
-        x[c] += (double)e[c];
+__global__ void __launch_bounds__(256) k_add_correction(long long N, double* __restrict__ x, const float* __restrict__ e) {
+    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
+    const long long nv = ((uintptr_t)x & 15u) == 0 ? N / 4 : 0;       // (x is the caller's, e begins an allocation)
+    for (long long v = tid; v < nv; v += nth) {
+        const float4 f = reinterpret_cast<const float4*>(e)[v];
+        double2 a = reinterpret_cast<const double2*>(x)[2 * v], b = reinterpret_cast<const double2*>(x)[2 * v + 1];
+        a.x += (double)f.x;
+        a.y += (double)f.y;
+        b.x += (double)f.z;
+        b.y += (double)f.w;
+        reinterpret_cast<double2*>(x)[2 * v] = a;
+        reinterpret_cast<double2*>(x)[2 * v + 1] = b;
+    }
+    for (long long c = 4 * nv + tid; c < N; c += nth) x[c] += (double)e[c];
 }
 
 // Red-black SOR sweep of one colour ((i + j + k) mod 2), in place on the FP64 iterate.
@@ -588,14 +610,9 @@ int run_poisson(const LesCtx& c, PoissonWork& w, const double* b, double* x, dou
     for (;;) {
         // true residual in FP64; the Krylov residual array receives it in the working precision
         prof_begin(c.prof, PS_RESIDUAL, s);
-        if (solver == IBM_SOLVER_RBSOR)
-            k_residual<double><<<c.fgrid, c.cg.block, 0, s>>>(c.D, b, x, (double*)nullptr, idx2, w.sc, c.partials,
-                                                              c.counter);
-        else if (c.prec == IBM_FP64)
-            k_residual<double><<<c.fgrid, c.cg.block, 0, s>>>(c.D, b, x, (double*)w.r, idx2, w.sc, c.partials,
-                                                              c.counter);
-        else
-            k_residual<float><<<c.fgrid, c.cg.block, 0, s>>>(c.D, b, x, (float*)w.r, idx2, w.sc, c.partials, c.counter);
+        if (solver == IBM_SOLVER_RBSOR) launch_residual<double>(c, b, x, nullptr, idx2, w.sc, s);
+        else if (c.prec == IBM_FP64) launch_residual<double>(c, b, x, (double*)w.r, idx2, w.sc, s);
+        else launch_residual<float>(c, b, x, (float*)w.r, idx2, w.sc, s);
         prof_end(c.prof, PS_RESIDUAL, s);
         IBM_LAUNCHED("k_residual");
         IBM_COUNT(c, 1);
