@@ -818,9 +818,10 @@ __device__ __forceinline__ T domain_face(const Dom& D, int a, int s, T in, const
 // One thread per cell writes its three lower faces (and the upper one of the last cell of an axis), so the
 // three components are read once and no face index has to be taken apart.  A cell knows a cut lower face
 // from its own flags: ibm_setup accepts only flags in which both cells of a face agree.  512x256x256 FP32:
-// 260 us (3.2 TB/s of the 25 bytes per cell), 660 us as one grid-stride kernel per axis with 64-bit divisions.
+// 181 us (4.6 TB/s of the 25 bytes per cell; bound by latency: six blocks per SM and two planes in flight; four planes
+// at three blocks took 260), 660 us as one grid-stride kernel per axis with 64-bit divisions.
 template <class T>
-__global__ void __launch_bounds__(256) k_faces(Dom D, FaceLayout F, const T* __restrict__ us, T* __restrict__ Us, int kz) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_faces(Dom D, FaceLayout F, const T* __restrict__ us, T* __restrict__ Us, int kz) {
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
     const int k0 = blockIdx.z * kz, k1 = min(k0 + kz, D.nz);
     if (i >= D.nx || j >= D.ny) return;
@@ -837,7 +838,7 @@ __global__ void __launch_bounds__(256) k_faces(Dom D, FaceLayout F, const T* __r
     const bool edge = i == 0 || j == 0 || i == D.nx - 1 || j == D.ny - 1;
     T zm = k0 > 0 ? u2[-D.sz] : (T)0;
     const int nk = k1 - k0;
-#pragma unroll 4
+#pragma unroll 2
     for (int q = 0; q < nk; ++q) {
         const long long o = q * D.sz;
         const unsigned fl = D.flags ? (unsigned)D.flags[P0 + o] : 0u;
@@ -919,20 +920,27 @@ __global__ void k_outflow_shift(Dom D, FaceLayout F, T* __restrict__ Us, const d
 }
 
 // Eq. poisson right-hand side: b = div(U*) / dt, evaluated in the working precision and stored in
-// FP64 (the pressure solve's FP64 residual b - A p starts from it).
+// FP64 (the pressure solve's FP64 residual b - A p starts from it).  A thread marches a column and keeps the z face
+// it shares with the next cell.  512x256x256 FP32: 110 us (20 bytes per cell would take 99), 157 us with one thread
+// per cell and a 64-bit index for each of its six faces.
 template <class T>
-__global__ void __launch_bounds__(256) k_rhs(Dom D, FaceLayout F, const T* __restrict__ Us, double* __restrict__ b,
-                                             double inv_dxdt) {
-    const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y, k = blockIdx.z;
+__global__ void __launch_bounds__(256, 8) k_rhs(Dom D, FaceLayout F, const T* __restrict__ Us, double* __restrict__ b,
+                                                double inv_dxdt, int kz) {
+    const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
+    const int k0 = blockIdx.z * kz, nk = min(kz, D.nz - k0);
     if (i >= D.nx || j >= D.ny) return;
     const T inv = (T)inv_dxdt;
-    {
-        const long long P = i + (long long)D.sy * j + D.sz * k;
-        T div = 0;
-        div += Us[F.index(0, i + 1, j, k)] - Us[F.index(0, i, j, k)];
-        div += Us[F.index(1, i, j + 1, k)] - Us[F.index(1, i, j, k)];
-        div += Us[F.index(2, i, j, k + 1)] - Us[F.index(2, i, j, k)];
-        b[P] = (double)(div * inv);
+    const T* __restrict__ X = Us + F.index(0, i, j, k0);
+    const T* __restrict__ Y = Us + F.index(1, i, j, k0);
+    const T* __restrict__ Z = Us + F.index(2, i, j, k0);
+    double* __restrict__ o = b + i + (long long)D.sy * j + D.sz * k0;
+    const long long sfx = (long long)F.dim[0][0] * F.dim[0][1], sfy = (long long)F.dim[1][0] * F.dim[1][1];
+    T z = Z[0];
+#pragma unroll 4
+    for (int q = 0; q < nk; ++q, X += sfx, Y += sfy, Z += D.sz, o += D.sz) {
+        const T x0 = X[0], x1 = X[1], y0 = Y[0], y1 = Y[D.nx], z1 = Z[D.sz];
+        *o = (double)((((x1 - x0) + (y1 - y0)) + (z1 - z)) * inv);
+        z = z1;
     }
 }
 
@@ -974,10 +982,10 @@ template <> struct PVal<float> {
 // Eq. correction: cells by the central pressure difference through the link values (c = dt / (2 dx)), faces
 // by the compact difference across uncut interior and outflow faces (dtdx = dt / dx).  One thread per cell
 // updates the cell, its three lower faces and the upper one of the last cell of an axis, marching a column:
-// p, u*, U* and the flags are read once.  512x256x256 FP32: 403 us (4.7 TB/s of the 57 bytes per cell), 930 us
-// as one cell and three face kernels in FP64 differences.
+// p, u*, U* and the flags are read once.  512x256x256 FP32: 363 us (5.3 TB/s of the 57 bytes per cell; 403 us at
+// three blocks per SM), 930 us as one cell and three face kernels in FP64 differences.
 template <class T>
-__global__ void __launch_bounds__(256) k_correct(Dom D, FaceLayout F, const T* __restrict__ us, const T* __restrict__ Us,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_correct(Dom D, FaceLayout F, const T* __restrict__ us, const T* __restrict__ Us,
                                                  const double* __restrict__ p, T* __restrict__ u, T* __restrict__ U, T c,
                                                  T dtdx, int kz) {
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
@@ -1614,10 +1622,10 @@ int launch_faces(const LesCtx& c, const void* ustar, void* Ustar, cudaStream_t s
 
 int launch_rhs(const LesCtx& c, const void* Ustar, double* b, cudaStream_t s) {
     const double inv = 1.0 / (c.D.dx * c.dt);
-    if (c.prec == IBM_FP64)
-        k_rhs<double><<<c.pgrid, c.cg.block, 0, s>>>(c.D, c.F, (const double*)Ustar, b, inv);
-    else
-        k_rhs<float><<<c.pgrid, c.cg.block, 0, s>>>(c.D, c.F, (const float*)Ustar, b, inv);
+    int kz = 1;
+    const dim3 g = column_grid(c.D, kz);
+    if (c.prec == IBM_FP64) k_rhs<double><<<g, c.cg.block, 0, s>>>(c.D, c.F, (const double*)Ustar, b, inv, kz);
+    else k_rhs<float><<<g, c.cg.block, 0, s>>>(c.D, c.F, (const float*)Ustar, b, inv, kz);
     IBM_LAUNCHED("k_rhs");
     IBM_COUNT(c, 1);
     return IBM_OK;
