@@ -204,13 +204,14 @@ __device__ __forceinline__ bool fast_cell(const Dom& D, long long P, int i, int 
 // the z face stays in registers for the next plane.  A plane's sums run one step later, so a single
 // barrier per plane orders both the face buffers (two of them, by plane parity) and the ring.
 //
-// Bound by instruction issue.  Per face and component: the advected value is c0 (u_L + u_R) + kq (3 (u_L +
-// u_R + u_up) - u_far), the scale factors of the differences are taken out of the components, addresses are a
+// Bound by instruction issue.  Per face and component: the advected value is c_L u_L + c_R u_R - kq u_far with
+// coefficients chosen once per face by the sign of its velocity, the scale factors of the differences are taken out of the components, addresses are a
 // block-uniform plane plus a fixed thread offset.  512x256x256 FP32, Crank-Nicolson operator: 660 us (530
 // thread instructions per cell, 2.6 per cycle and SM; its 41 bytes per cell would take 205 us), 1540 us with
 // per-component face forms, 64-bit face indexes and velocities loaded where they are used.  Two rows per
 // thread (455 instructions, 16 resident warps) and four blocks per SM (64 registers) measured 660 and 694 us.
-// FP64: 212 us at 128x64x64, three quarters of the FP64 rate for its 160 operations per cell.
+// FP64: 183 us at 128x64x64 (212 with 20 operations per cell more: per-component upwind sums, weighted cross
+// derivatives), three quarters of the FP64 rate.
 #define FT_X 32
 #define FT_Y 8
 #define FT_H 2
@@ -226,13 +227,19 @@ __device__ __forceinline__ bool fast_cell(const Dom& D, long long P, int i, int 
 // Coefficients of the faces of one axis at one place.
 template <class T>
 struct FaceW {
-    T wl, wr;      // weights of the two cells in the cross derivatives (sum 2)
-    T c0, kq;      // central and QUICK coefficients of the advected value
+    T cu, cd, kq;  // the advected value is cu u_up + cd u_down - kq u_far
+    T wl, wr;      // FP32: weights of the two cells in the cross derivatives (sum 2)
+    bool lo, hi;   // domain face below, above: only the cell inside counts
+    // wl a + wr b; by selection in FP64, where an operation costs more than four integer ones
+    __device__ __forceinline__ T cross(T a, T b) const {
+        if constexpr (sizeof(T) == 4) return wl * a + wr * b;
+        else return (lo ? b : a) + (hi ? a : b);
+    }
 };
 
 template <class T>
 struct FaceK {
-    T c0, kq;              // interior faces
+    T cu, cd, kq;          // interior faces
     T nui, h, e;           // nu / dx, 1 / (2 dx), 1 / (8 dx)
 };
 
@@ -241,7 +248,10 @@ __device__ __forceinline__ FaceW<T> face_w(const FaceK<T>& K, bool dlo, bool dhi
     FaceW<T> w;
     w.wl = dlo ? (T)0 : (dhi ? (T)2 : (T)1);
     w.wr = dlo ? (T)2 : (dhi ? (T)0 : (T)1);
-    w.c0 = dlo || dhi ? (T)0.5 : K.c0;
+    w.lo = dlo;
+    w.hi = dhi;
+    w.cu = dlo || dhi ? (T)0.5 : K.cu;
+    w.cd = dlo || dhi ? (T)0.5 : K.cd;
     w.kq = dlo || dhi ? (T)0 : K.kq;
     return w;
 }
@@ -254,14 +264,13 @@ template <class T, int A>
 __device__ __forceinline__ void face_phi(const FaceW<T>& w, const FaceK<T>& K, T Uf, const T (&l)[3], const T (&r)[3],
                                          const T (&far)[3], T d0, T d1, T nn, T (&phi)[3]) {
     const T a = K.nui + K.h * nn, x = K.e * nn, aa = a + K.h * nn;
-    const T uc = Uf * w.c0, uq = Uf * w.kq;
     const bool up = Uf >= (T)0;
+    const T cl = Uf * (up ? w.cu : w.cd), cr = Uf * (up ? w.cd : w.cu), cf = Uf * w.kq;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const T s = l[c] + r[c];
-        const T q = (T)3 * (s + (up ? l[c] : r[c])) - far[c];
-        T v = (c == A ? aa : a) * (r[c] - l[c]) - uc * s;
-        v -= uq * q;
+        T v = (c == A ? aa : a) * (r[c] - l[c]) + cf * far[c];
+        v -= cl * l[c];
+        v -= cr * r[c];
         if (c != A) v += x * (c == (A == 0 ? 1 : 0) ? d0 : d1);
         phi[c] = v;
     }
@@ -281,8 +290,8 @@ __device__ __forceinline__ void face_inplane(const FaceW<T>& w, const FaceK<T>& 
         far[c] = sf[c * FT_PL];
     }
     const T* s = S0 + A * FT_PL + q;
-    const T db = w.wl * (s[B - E] - s[-B - E]) + w.wr * (s[B] - s[-B]);
-    const T dzs = w.wl * (Sp[A * FT_PL + q - E] - Sm[A * FT_PL + q - E]) + w.wr * dz;
+    const T db = w.cross(s[B - E] - s[-B - E], s[B] - s[-B]);
+    const T dzs = w.cross(Sp[A * FT_PL + q - E] - Sm[A * FT_PL + q - E], dz);
     face_phi<T, A>(w, K, Uf, l, r, far, db, dzs, S0[3 * FT_PL + q - E] + nr, phi);
 }
 
@@ -297,8 +306,9 @@ __device__ __forceinline__ void fast_tile_march(const Dom& D, const FaceLayout& 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + FT_X * ty;
     const T invdx = dom_idx<T>(D);
     FaceK<T> K;
-    K.c0 = (T)0.5 * ((T)1 - gam);
     K.kq = gam * (T)0.125;
+    K.cd = (T)0.5 * ((T)1 - gam) + (T)3 * K.kq;
+    K.cu = K.cd + (T)3 * K.kq;
     K.nui = nu * invdx;
     K.h = (T)0.5 * invdx;
     K.e = (T)0.125 * invdx;
@@ -428,8 +438,8 @@ __device__ __forceinline__ void fast_tile_march(const Dom& D, const FaceLayout& 
             const T *m = Sm + 2 * FT_PL + cidx, *o = S0 + 2 * FT_PL + cidx;
             ex = o[1] - o[-1];
             ey = o[FT_SX] - o[-FT_SX];
-            face_phi<T, 2>(wz, K, Uf, um, uc, far, wz.wl * (m[1] - m[-1]) + wz.wr * ex,
-                           wz.wl * (m[FT_SX] - m[-FT_SX]) + wz.wr * ey, Sm[3 * FT_PL + cidx] + nc, zlo);
+            face_phi<T, 2>(wz, K, Uf, um, uc, far, wz.cross(m[1] - m[-1], ex),
+                           wz.cross(m[FT_SX] - m[-FT_SX], ey), Sm[3 * FT_PL + cidx] + nc, zlo);
         }
         // face velocities of the step's faces, loaded a step ahead
         T Ufx, Ufy, Ufz, Ufe;
@@ -495,7 +505,7 @@ __device__ __forceinline__ void fast_tile_march(const Dom& D, const FaceLayout& 
                 const T np = Sp[3 * FT_PL + cidx];
                 const T* o = Sp + 2 * FT_PL + cidx;
                 const T nx_ = o[1] - o[-1], ny_ = o[FT_SX] - o[-FT_SX];
-                face_phi<T, 2>(wz, K, Ufz, uc, up, far, wz.wl * ex + wz.wr * nx_, wz.wl * ey + wz.wr * ny_, nc + np, zhi);
+                face_phi<T, 2>(wz, K, Ufz, uc, up, far, wz.cross(ex, nx_), wz.cross(ey, ny_), nc + np, zhi);
                 ex = nx_;
                 ey = ny_;
                 nc = np;
