@@ -1023,13 +1023,24 @@ struct ArrEmit {
 
 // Padded rows of the V-cycle: link e of unknown u at [e M + u], so a warp's rows are read whole; padding has
 // g = 0.  A row with more than MG_ELL links stores -1 as its first column and is read from the CSR arrays.
-__global__ void k_ell(MGLev L) {
+// A conductance counts the fine faces between two parts: where all of a level's are whole numbers below 256 the
+// V-cycle reads them as bytes, a row's six in one load (eg8), else as floats (eg).  `wide` is set if one is not.
+__global__ void k_ell(MGLev L, int* wide) {
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < L.M; u += (long long)gridDim.x * blockDim.x) {
         const int k0 = L.rp[u], n = L.rp[u + 1] - k0;
+        unsigned w[2] = {0u, 0u};
         for (int e = 0; e < MG_ELL; ++e) {
+            const float g = n <= MG_ELL && e < n ? L.g[k0 + e] : 0.f;
+            if (L.eg) {
+                L.eg[e * L.M + u] = g;
+                continue;
+            }
             L.ecol[e * L.M + u] = n > MG_ELL ? -1 : (e < n ? L.col[k0 + e] : (int)u);
-            L.eg[e * L.M + u] = n <= MG_ELL && e < n ? L.g[k0 + e] : 0.f;
+            const unsigned q = g >= 0.f && g < 256.f ? (unsigned)g : 0u;
+            if ((float)q != g) atomicExch(wide, 1);
+            w[e >> 2] |= q << (8 * (e & 3));
         }
+        if (!L.eg) L.eg8[u] = make_uint2(w[0], w[1]);
     }
 }
 
@@ -1048,9 +1059,14 @@ __device__ __forceinline__ T row_sum(const MGLev& L, long long u, Fn f) {
     int c[MG_ELL];
     float g[MG_ELL];
 #pragma unroll
-    for (int e = 0; e < MG_ELL; ++e) {
-        c[e] = L.ecol[e * L.M + u];
-        g[e] = L.eg[e * L.M + u];
+    for (int e = 0; e < MG_ELL; ++e) c[e] = L.ecol[e * L.M + u];
+    if (!L.eg) {
+        const uint2 w = L.eg8[u];
+#pragma unroll
+        for (int e = 0; e < MG_ELL; ++e) g[e] = (float)(((e < 4 ? w.x : w.y) >> (8 * (e & 3))) & 255u);
+    } else {
+#pragma unroll
+        for (int e = 0; e < MG_ELL; ++e) g[e] = L.eg[e * L.M + u];
     }
     if (c[0] < 0) {
         for (int e = L.rp[u]; e < L.rp[u + 1]; ++e) s += (T)L.g[e] * f(L.col[e]);
@@ -1743,7 +1759,7 @@ struct SetupTmp {
 
 void free_level(MGLev& L) {
     cudaFree(L.off); cudaFree(L.cnt); cudaFree(L.pos); cudaFree(L.rp); cudaFree(L.col); cudaFree(L.g);
-    cudaFree(L.ecol); cudaFree(L.eg); cudaFree(L.d); cudaFree(L.invdg); cudaFree(L.parent); cudaFree(L.cp); cudaFree(L.ch); cudaFree(L.b);
+    cudaFree(L.ecol); cudaFree(L.eg); cudaFree(L.eg8); cudaFree(L.d); cudaFree(L.invdg); cudaFree(L.parent); cudaFree(L.cp); cudaFree(L.ch); cudaFree(L.b);
     cudaFree(L.x);
     const int px = L.px, py = L.py, pz = L.pz;
     const long long P = L.P;
@@ -1792,10 +1808,19 @@ int scan_in_place(int32_t* a, long long n, SetupTmp& t, long long* total) {
     return IBM_OK;
 }
 
-int build_ell(MGLev& L) {
+int build_ell(MGLev& L, SetupTmp& t) {
     MG_ALLOC(L.ecol, MG_ELL * L.M);
+    MG_ALLOC(L.eg8, L.M);
+    IBM_CUDA(cudaMemset(t.ovf, 0, sizeof(int)));
+    k_ell<<<lin_blocks(L.M), 256>>>(L, t.ovf);
+    IBM_LAUNCHED("k_ell");
+    int wide = 0;
+    IBM_CUDA(cudaMemcpy(&wide, t.ovf, sizeof(int), cudaMemcpyDeviceToHost));
+    if (!wide) return IBM_OK;
+    cudaFree(L.eg8);
+    L.eg8 = nullptr;
     MG_ALLOC(L.eg, MG_ELL * L.M);
-    k_ell<<<lin_blocks(L.M), 256>>>(L);
+    k_ell<<<lin_blocks(L.M), 256>>>(L, t.ovf);
     IBM_LAUNCHED("k_ell");
     return IBM_OK;
 }
@@ -1989,7 +2014,7 @@ int build_level1(const LesCtx& c, MGLev& L, int sb, SetupTmp& t) {
     if (h) return ibm_fail(IBM_E_INVALID, "multigrid set-up: a level-1 block has too many links");
     MG_ALLOC(t.lab, L.M);           // the largest level: reused by the others
     MG_ALLOC(t.num, L.M);
-    return build_ell(L);
+    return build_ell(L, t);
 }
 
 // Level C from level F; returns 1 (and leaves C empty) when the level would not shrink enough or
@@ -2042,7 +2067,7 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
     MG_ALLOC(C.g, C.nnz);
     k_links_next<<<lin_blocks(C.P), 256>>>(F, C, 1, all, t.ovf);
     IBM_LAUNCHED("k_links_next");
-    if ((rc = build_ell(C))) return -rc;
+    if ((rc = build_ell(C, t))) return -rc;
     IBM_CUDA(cudaDeviceSynchronize());
     return 0;
 }

@@ -48,7 +48,8 @@ struct MGLev {
     int32_t* col;        // [nnz] neighbour unknown
     float* g;            // [nnz] conductance: sum of the fine conductances between the two aggregates
     int32_t* ecol;       // padded rows read by the V-cycle (mg.cu), column-major
-    float* eg;
+    float* eg;           // their conductances, if eg8 cannot hold them
+    uint2* eg8;          // their conductances as bytes
     float* d;            // [M] Dirichlet (outflow) diagonal term
     float* invdg;        // [M] 1 / (sum of g + d), 0 for an isolated unknown
     int32_t* parent;     // [M] unknown of level l + 1 that contains this one
