@@ -22,6 +22,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "scan.cuh"
@@ -470,13 +471,15 @@ __device__ __forceinline__ int ftp_zadj(const Dom& D, int p) {
 // of colour 1 zero, so only colour 0 is evaluated (one plane behind the last half-sweep).
 template <int LX, int NI>
 __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* __restrict__ rg, float* __restrict__ zg,
-                                                            float scale, MGLev C1, int kchunk, const SolveScal* sc) {
+                                                            float scale, MGLev C1, const int4* __restrict__ chunks, int ntx,
+                                                            int nty, const SolveScal* sc) {
     if (sc->done) return;
     extern __shared__ __align__(16) unsigned char ftp_raw[];
     const FShared<LX> S = ftp_shared<LX>(ftp_raw);
-    const FCol<NI> c = ftp_column<LX, NI>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    const int4 item = chunks[blockIdx.x];       // tile, its planes
+    const FCol<NI> c = ftp_column<LX, NI>(D, item.x, item.y, ntx, nty);
     const int left = D.nx - c.gx;       // cells from the quad's first to the end of the row
-    const int k0 = blockIdx.z * kchunk, k1 = min(D.nz, k0 + kchunk);
+    const int k0 = item.z, k1 = item.w;
     const int tlo = max(0, k0 - 4), thi = k1 + 3;
     const int row0 = c.gx + D.sy * c.gy;
     float Z[6][2][4];
@@ -656,14 +659,16 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
 // rz_old = rz, rz = (r, z).
 template <int LX, int NI>
 __global__ void __launch_bounds__(FTP_NT, 1) k_mg_post_fused(Dom D, const float* __restrict__ rg, const float* __restrict__ zin,
-                                                             float* __restrict__ zg, float scale, int kchunk, SolveScal* sc,
+                                                             float* __restrict__ zg, float scale, const int4* __restrict__ chunks,
+                                                             int ntx, int nty, SolveScal* sc,
                                                              double* partials, unsigned* counter) {
     if (sc->done) return;
     extern __shared__ __align__(16) unsigned char ftp_raw[];
     const FShared<LX> S = ftp_shared<LX>(ftp_raw);
-    const FCol<NI> c = ftp_column<LX, NI>(D, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    const int4 item = chunks[blockIdx.x];       // tile, its planes
+    const FCol<NI> c = ftp_column<LX, NI>(D, item.x, item.y, ntx, nty);
     const int left = D.nx - c.gx;       // cells from the quad's first to the end of the row
-    const int k0 = blockIdx.z * kchunk, k1 = min(D.nz, k0 + kchunk);
+    const int k0 = item.z, k1 = item.w;
     const int tlo = max(0, k0 - 4), thi = k1 + 2;
     const int row0 = c.gx + D.sy * c.gy;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1709,34 +1714,137 @@ unsigned lin_blocks(long long n) {
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-// Whether the fused passes apply, and their launch shape: of the two tile widths (64 x 64 or 128 x 32 cells,
-// halo included) and the z-chunks, the one with the fewest plane steps over all waves (one block per SM; a
-// chunk of k planes takes k + 8 steps).  64 x 64 has the smaller halo, 128 x 32 fits some grids better.
-void fused_plan(const LesCtx& c, MG& mg, int sb) {
+// Planes of a tile (halo included) with a cut link: the passes take the general half-sweeps there.
+__global__ void __launch_bounds__(256) k_tile_marks(Dom D, int w, int h, uint8_t* marks) {
+    const int x0 = blockIdx.y * (w - 8), y0 = blockIdx.z * (h - 8), k = blockIdx.x;
+    unsigned any = 0u;
+    for (int q = threadIdx.x; q < w * h; q += blockDim.x) {
+        const int x = x0 + q % w, y = y0 + q / w;
+        if (x < D.nx && y < D.ny) any |= D.flags[x + (long long)D.sy * y + D.sz * k] & 63u;
+    }
+    any = __syncthreads_or(any != 0u);
+    if (threadIdx.x == 0) marks[blockIdx.y + (long long)gridDim.y * (blockIdx.z + (long long)gridDim.z * k)] = any ? 1 : 0;
+}
+
+// The launch of the fused passes: of the two tile widths (64 x 64 or 128 x 32 cells, halo included; 64 x 64 has the
+// smaller halo, 128 x 32 fits some grids better), each tile cut into chunks of whole pairs of planes.  A chunk costs
+// its planes and eight more, planes with cut links FZ_GENERAL as much as others (measured: 2.57 and 1.57 us), and
+// blocks run one per SM; for eight numbers of rounds the limit on a chunk's cost is bisected that lets the
+// chunks fit the rounds, and the cheapest is kept.  With chunks of equal height the tiles around a body came last: the
+// two passes take 43 and 34 us in place of 52 and 42 on 256 x 128 x 128 cells around a dirty sphere, 836 and 624 in place
+// of 896 and 681 on 1024 x 512 x 384 around a vehicle (1.3 for FZ_GENERAL: 928 and 679; 2.5: 917 and 663).
+#define FZ_GENERAL 1.65f
+
+struct FzPlan {
+    int tx, ty, nz;
+    const float* sum;           // [tile][nz + 9] sums of the planes' costs from plane -4 on, nz + 4 the last
+    // chunks of at most `limit` (a pair of planes at least); their number, or -1 if more than `most`
+    long long cut(float limit, long long most, int4* out, float* cost) const {
+        long long n = 0;
+        for (int t = 0; t < tx * ty; ++t) {
+            const float* s = sum + (long long)t * (nz + 9);
+            for (int k0 = 0; k0 < nz;) {
+                int k1 = k0 + 2;
+                while (k1 < nz && at(s, k0, k1 + 2) <= limit) k1 += 2;
+                if (k1 > nz) k1 = nz;
+                if (n == most) return -1;
+                if (out) {
+                    out[n] = make_int4(t % tx, t / tx, k0, k1);
+                    cost[n] = at(s, k0, k1);
+                }
+                ++n;
+                k0 = k1;
+            }
+        }
+        return n;
+    }
+    float at(const float* s, int k0, int k1) const { return s[(k1 > nz ? nz : k1) + 8] - s[k0]; }
+};
+
+int fused_plan(const LesCtx& c, MG& mg, int sb) {
     const Dom& D = c.D;
     bool per = false;
     for (int f = 0; f < 6; ++f) per = per || D.bc[f] == IBM_BC_PERIODIC;
     mg.fused = mg.allow_fused && sb == 4 && mg.sweeps == 2 && mg.nlev > 1 && !per;
-    if (!mg.fused) return;
-    long long best = -1;
+    if (!mg.fused) return IBM_OK;
+    float best = -1.f;
     for (int lx = 16; lx <= 32; lx *= 2) {
         const int w = 4 * lx, h = 2 * (FTP_NT / lx);
-        const long long tx = D.nx > w ? (D.nx - 8 + w - 9) / (w - 8) : 1, ty = D.ny > h ? (D.ny - 8 + h - 9) / (h - 8) : 1;
-        for (int ch = 1; ch <= 64; ++ch) {
-            int k = (D.nz + ch - 1) / ch;
-            k += k & 1;
-            if (k < 2 && ch > 1) break;
-            const long long nchunk = (D.nz + k - 1) / k;
-            const long long waves = (tx * ty * nchunk + IBM_NSM - 1) / IBM_NSM;
-            const long long cost = waves * (k + 8);
-            if (best < 0 || cost < best) {
-                best = cost;
-                mg.fz_chunk = k;
+        FzPlan p;
+        p.tx = D.nx > w ? (D.nx - 8 + w - 9) / (w - 8) : 1;
+        p.ty = D.ny > h ? (D.ny - 8 + h - 9) / (h - 8) : 1;
+        p.nz = D.nz;
+        const long long tiles = (long long)p.tx * p.ty, cap = tiles * ((D.nz + 1) / 2);
+        uint8_t *dev = nullptr, *marks = (uint8_t*)calloc(tiles, D.nz);
+        float* sum = (float*)malloc(sizeof(float) * tiles * (D.nz + 9));
+        int4* out = (int4*)malloc(sizeof(int4) * cap);
+        float* cost = (float*)malloc(sizeof(float) * cap);
+        int* order = (int*)malloc(sizeof(int) * cap);
+        cudaError_t e = marks && sum && out && cost && order ? cudaSuccess : cudaErrorMemoryAllocation;
+        if (e == cudaSuccess && D.flags) {
+            e = ibm_malloc(&dev, tiles * D.nz);
+            if (e == cudaSuccess) {
+                k_tile_marks<<<dim3(D.nz, p.tx, p.ty), 256>>>(D, w, h, dev);
+                e = cudaMemcpy(marks, dev, tiles * D.nz, cudaMemcpyDeviceToHost);
+            }
+            cudaFree(dev);
+        }
+        if (e == cudaSuccess) {
+            for (long long t = 0; t < tiles; ++t) {
+                float* s = sum + t * (D.nz + 9);
+                float a = 0.f;
+                for (int k = -4; k < D.nz + 4; ++k) {
+                    s[k + 4] = a;
+                    if (k < 0) continue;
+                    a += k == 0 || k == D.nz - 1 || (k < D.nz && marks[t + tiles * k]) ? FZ_GENERAL : 1.f;
+                }
+                s[D.nz + 8] = a;
+            }
+            p.sum = sum;
+            const int first = (int)((tiles + IBM_NSM - 1) / IBM_NSM);
+            for (int rounds = first; rounds < first + 8; ++rounds) {
+                float lo = 0.f, hi = FZ_GENERAL * (D.nz + 9);
+                const long long most = (long long)rounds * IBM_NSM;
+                if (p.cut(hi, most, nullptr, nullptr) < 0) continue;
+                for (int it = 0; it < 14; ++it) {
+                    const float mid = 0.5f * (lo + hi);
+                    if (p.cut(mid, most, nullptr, nullptr) >= 0) hi = mid;
+                    else lo = mid;
+                }
+                long long n = p.cut(hi, most, out, cost);
+                float worst = 0.f;
+                for (long long q = 0; q < n; ++q) {
+                    worst = cost[q] > worst ? cost[q] : worst;
+                    order[q] = (int)q;
+                }
+                const float total = worst * ((n + IBM_NSM - 1) / IBM_NSM);
+                if (best >= 0.f && total >= 0.999f * best) continue;
+                // the dearest first
+                std::sort(order, order + n, [&](int a, int b) { return cost[a] != cost[b] ? cost[a] > cost[b] : a < b; });
+                int4* sorted = (int4*)malloc(sizeof(int4) * n);
+                if (!sorted) { e = cudaErrorMemoryAllocation; break; }
+                for (long long q = 0; q < n; ++q) sorted[q] = out[order[q]];
+                cudaFree(mg.fz);
+                mg.fz = nullptr;
+                e = ibm_malloc(&mg.fz, sizeof(int4) * n);
+                if (e == cudaSuccess) e = cudaMemcpy(mg.fz, sorted, sizeof(int4) * n, cudaMemcpyHostToDevice);
+                free(sorted);
+                if (e != cudaSuccess) break;
+                best = total;
                 mg.flx = lx;
-                mg.fgrid = dim3((unsigned)tx, (unsigned)ty, (unsigned)nchunk);
+                mg.fz_items = (int)n;
+                mg.fz_tx = p.tx;
+                mg.fz_ty = p.ty;
             }
         }
+        free(marks);
+        free(sum);
+        free(out);
+        free(cost);
+        free(order);
+        if (e != cudaSuccess) return ibm_cuda_check(e, "multigrid set-up: plan of the fused passes");
     }
+    return IBM_OK;
 }
 
 // ---- host side of the set-up --------------------------------------------------------------------
@@ -2124,7 +2232,7 @@ static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z,
     prof_begin(c.prof, PS_MG_FINE, s);
     auto pre = [&](auto lx, auto ni) {
         constexpr int LX = decltype(lx)::value, NI = decltype(ni)::value;
-        k_mg_pre_fused<LX, NI><<<mg.fgrid, FTP_NT, FTile<LX>::smem(), s>>>(c.D, r, z2, scale, L1, mg.fz_chunk, sc);
+        k_mg_pre_fused<LX, NI><<<mg.fz_items, FTP_NT, FTile<LX>::smem(), s>>>(c.D, r, z2, scale, L1, mg.fz, mg.fz_tx, mg.fz_ty, sc);
     };
     fused_dispatch(c, mg, pre);
     prof_end(c.prof, PS_MG_FINE, s);
@@ -2141,7 +2249,7 @@ static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z,
     prof_begin(c.prof, PS_MG_FINE, s);
     auto post = [&](auto lx, auto ni) {
         constexpr int LX = decltype(lx)::value, NI = decltype(ni)::value;
-        k_mg_post_fused<LX, NI><<<mg.fgrid, FTP_NT, FTile<LX>::smem(), s>>>(c.D, r, z2, z, scale, mg.fz_chunk, sc, c.partials, c.counter);
+        k_mg_post_fused<LX, NI><<<mg.fz_items, FTP_NT, FTile<LX>::smem(), s>>>(c.D, r, z2, z, scale, mg.fz, mg.fz_tx, mg.fz_ty, sc, c.partials, c.counter);
     };
     fused_dispatch(c, mg, post);
     prof_end(c.prof, PS_MG_FINE, s);
@@ -2154,6 +2262,8 @@ static int vcycle_fused(const LesCtx& c, const MG& mg, const float* r, float* z,
 void mg_free(MG& mg) {
     for (int l = 1; l < IBM_MG_MAXLEV; ++l) free_level(mg.lev[l]);
     cudaFree(mg.z2);
+    cudaFree(mg.fz);
+    mg.fz = nullptr;
     cudaFree(mg.tail_img);
     mg.tail_img = nullptr;
     free(mg.tail);
@@ -2189,7 +2299,7 @@ int mg_setup(const LesCtx& c, MG& mg, int sb) {
         mg.nlev = l + 2;
     }
     if ((rc = tail_plan(mg, sb))) return rc;
-    fused_plan(c, mg, sb);
+    if ((rc = fused_plan(c, mg, sb))) return rc;
     if (mg.fused) {
         MG_ALLOCB(mg.z2, c.D.N * 4);
         cudaError_t e = cudaSuccess;

@@ -72,8 +72,8 @@ struct MG {
     int allow_fused;     // les_params.mg_passes == 0
     int fused;           // 1: the fused kernels apply to this grid and configuration
     int flx;             // quads along x of a tile (16 or 32)
-    int fz_chunk;        // planes per z-chunk of a fused launch (even)
-    dim3 fgrid;          // tiles x, tiles y, z-chunks
+    int4* fz;            // blocks of a fused launch: tile x, tile y, first plane (even), end
+    int fz_items, fz_tx, fz_ty;   // their number, tiles along x and y
     void* z2;            // [N] working precision: pre-smoothed and prolongated z, read by the post-smoothing
                          // pass (which writes z): no block reads what another block of the pass writes
 };
