@@ -68,21 +68,42 @@ __device__ __forceinline__ void mma_bf16(float d[4], const uint32_t a[4], const 
 }
 
 // Convolution of a channel-last BF16 field with 27 taps on the tensor cores (implicit GEMM, K = 27
-// taps x 8 channels padded to 224).  sgn = +1: forward (input at c + off); sgn = -1: input gradient
-// (input at c - off, transposed weights).  mode 0: store BF16 relu(acc + bias); mode 1: store FP32
-// channel 0 of acc + bias; mode 2: store BF16 acc masked by (mask > 0) at the output cell (ReLU
+// taps x 8 channels padded to 224).  SGN = +1: forward (input at c + off); SGN = -1: input gradient
+// (input at c - off, transposed weights).  MODE 0: store BF16 relu(acc + bias); 1: store FP32
+// channel 0 of acc + bias; 2: store BF16 acc masked by (mask > 0) at the output cell (ReLU
 // derivative).  The input is staged in shared memory.  A block owns a 32 x 4 (x, y) tile
-// of output cells and walks NC_KZ planes; the input planes k - 1, k, k + 1 over the tile plus a one-cell
-// halo sit in a three-plane ring (16 bytes per cell, zero outside the grid).  Warp w computes the
+// of output cells and walks kz planes; the input planes over the tile plus a one-cell halo sit in a four-plane
+// ring (16 bytes per cell, zero outside the grid): three that are read and the one the plane loaded during the
+// previous step goes into, so a step has one barrier and no load is waited for.  Warp w computes the
 // 16 cells (w % 2) * 16 .. + 15 of row w / 2: for each k-step (two taps x 8 channels) one
 // ldmatrix.x4 gathers the A fragment straight from the ring -- each lane names one 16-byte row, the
-// input cell of its (cell, tap) -- and one mma.sync accumulates it.
+// input cell of its (cell, tap), a plane's base and a constant -- and one mma.sync accumulates it.
+// 128^3 cells: 38 us per layer (input gradients 50, with the mask), 74 with three planes, loads waited for and ring slots by
+// remainders per tap.
 #define NC_TX 32
 #define NC_TY 4
-#define NC_KZ 8
 #define NC_SX (NC_TX + 2)
 #define NC_SY (NC_TY + 2)
 #define NC_PL (NC_SX * NC_SY)
+#define NC_RING 4
+
+// The plane of the ring a thread fills: one position of the halo tile (threads beyond it: none), its value of the
+// plane in flight.
+struct RingFill {
+    long long at;        // element offset within a plane of the grid, -1 outside
+    uint4 v;
+    __device__ __forceinline__ RingFill(int tid, int x0, int y0, int nx, int ny) {
+        const int gx = x0 + tid % NC_SX - 1, gy = y0 + tid / NC_SX - 1;
+        at = tid < NC_PL && gx >= 0 && gx < nx && gy >= 0 && gy < ny ? (gx + (long long)nx * gy) * NN_C : -1;
+    }
+    __device__ __forceinline__ void fetch(const __nv_bfloat16* __restrict__ in, int k, int nz, long long plane) {
+        v = make_uint4(0u, 0u, 0u, 0u);
+        if (at >= 0 && k >= 0 && k < nz) v = *reinterpret_cast<const uint4*>(in + k * plane + at);
+    }
+    __device__ __forceinline__ void put(uint4* ring, int k, int tid) const {
+        if (tid < NC_PL) ring[((k + NC_RING) % NC_RING) * NC_PL + tid] = v;
+    }
+};
 
 __device__ __forceinline__ void ldsm_x4(uint32_t r[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
@@ -90,25 +111,17 @@ __device__ __forceinline__ void ldsm_x4(uint32_t r[4], uint32_t addr) {
                  : "r"(addr));
 }
 
-__global__ void __launch_bounds__(256) k_nn_conv_tile(int nx, int ny, int nz, const __nv_bfloat16* __restrict__ in,
-                                                      const uint32_t* __restrict__ frag, const float* __restrict__ bias,
-                                                      int sgn, int mode, __nv_bfloat16* __restrict__ outb,
-                                                      float* __restrict__ outf, const __nv_bfloat16* __restrict__ mask) {
-    __shared__ __align__(16) uint4 ring[3 * NC_PL + 1];          // + one zero row for the padding tap
+template <int SGN, int MODE>
+__global__ void __launch_bounds__(256, 4) k_nn_conv_tile(int nx, int ny, int nz, int kz, const __nv_bfloat16* __restrict__ in,
+                                                         const uint32_t* __restrict__ frag, const float* __restrict__ bias,
+                                                         __nv_bfloat16* __restrict__ outb, float* __restrict__ outf,
+                                                         const __nv_bfloat16* __restrict__ mask) {
+    __shared__ __align__(16) uint4 ring[NC_RING * NC_PL + 1];    // + one zero row for the padding tap
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int x0 = blockIdx.x * NC_TX, y0 = blockIdx.y * NC_TY, z0 = blockIdx.z * NC_KZ;
-    const int z1 = z0 + NC_KZ < nz ? z0 + NC_KZ : nz;
-    if (tid == 0) ring[3 * NC_PL] = make_uint4(0u, 0u, 0u, 0u);
-    auto load_plane = [&](int kk) {
-        uint4* dst = ring + ((kk % 3) + 3) % 3 * NC_PL;
-        for (int e = tid; e < NC_PL; e += 256) {
-            const int gx = x0 + e % NC_SX - 1, gy = y0 + e / NC_SX - 1;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (kk >= 0 && kk < nz && gx >= 0 && gx < nx && gy >= 0 && gy < ny)
-                v = *reinterpret_cast<const uint4*>(in + (gx + (long long)nx * (gy + (long long)ny * kk)) * NN_C);
-            dst[e] = v;
-        }
-    };
+    const int x0 = blockIdx.x * NC_TX, y0 = blockIdx.y * NC_TY, z0 = blockIdx.z * kz;
+    const int z1 = z0 + kz < nz ? z0 + kz : nz;
+    const long long plane = (long long)nx * ny * NN_C;
+    if (tid == 0) ring[NC_RING * NC_PL] = make_uint4(0u, 0u, 0u, 0u);
     const int g = lane >> 2, q = lane & 3;
     uint32_t bf[NN_KSTEPS][2];
 #pragma unroll
@@ -118,68 +131,99 @@ __global__ void __launch_bounds__(256) k_nn_conv_tile(int nx, int ny, int nz, co
     }
     const float b0 = bias ? bias[2 * q] : 0.f, b1 = bias ? bias[2 * q + 1] : 0.f;
     // this lane's ldmatrix row: matrix mj = lane / 8 (cells +8 for odd mj, tap +1 for mj >= 2), row lane % 8
-    const int mj = lane >> 3, mr = lane & 7;
+    const int mj = lane >> 3, mr = lane & 7, hi = mj >> 1;
     const int cx = (w & 1) * 16 + ((mj & 1) ? 8 : 0) + mr;          // tile-local output x of the row
     const int cy = w >> 1;
     const uint32_t ring_base = (uint32_t)__cvta_generic_to_shared(ring);
-    const uint32_t zero_row = ring_base + 3 * NC_PL * 16;
-    load_plane(z0 - 1);
-    load_plane(z0);
-    for (int k = z0; k < z1; ++k) {
-        load_plane(k + 1);
+    const uint32_t cell0 = ring_base + (uint32_t)(((cy + 1) * NC_SX + cx + 1) * 16), zero_row = ring_base + NC_RING * NC_PL * 16;
+    RingFill fill(tid, x0, y0, nx, ny);
+#pragma unroll
+    for (int t = -1; t <= 1; ++t) {
+        fill.fetch(in, z0 + t, nz, plane);
+        fill.put(ring, z0 + t, tid);
+    }
+    fill.fetch(in, z0 + 2, nz, plane);
+    const int i0 = x0 + (w & 1) * 16 + g, j = y0 + cy;
+    const bool on[2] = {i0 < nx && j < ny, i0 + 8 < nx && j < ny};
+    long long c = i0 + (long long)nx * (j + (long long)ny * z0);
+    for (int k = z0; k < z1; ++k, c += (long long)nx * ny) {
+        // every warp is done with plane k - 2, planes up to k + 1 are there
         __syncthreads();
+        if (k + 2 <= z1) {
+            fill.put(ring, k + 2, tid);
+            if (k + 3 <= z1) fill.fetch(in, k + 3, nz, plane);
+        }
+        uint32_t pb[3];                          // planes k - SGN, k, k + SGN: taps 0 .. 8, 9 .. 17, 18 .. 26
+#pragma unroll
+        for (int e = 0; e < 3; ++e) pb[e] = cell0 + (uint32_t)((k + SGN * (e - 1) + NC_RING) % NC_RING) * (NC_PL * 16);
         float d[4] = {0.f, 0.f, 0.f, 0.f};
+        __nv_bfloat162 mk[2] = {};
+        if (MODE == 2) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (on[h]) mk[h] = *reinterpret_cast<const __nv_bfloat162*>(mask + (c + 8 * h) * NN_C + 2 * q);
+        }
 #pragma unroll
         for (int s = 0; s < NN_KSTEPS; ++s) {
-            const int t = 2 * s + (mj >> 1);
-            uint32_t addr = zero_row;
-            if (t < NN_TAPS) {
-                int dz, dy, dx;
-                tap_off(t, dz, dy, dx);
-                const int sl = (((k + sgn * dz) % 3) + 3) % 3;
-                addr = ring_base + (uint32_t)((sl * NC_PL + (cy + sgn * dy + 1) * NC_SX + (cx + sgn * dx + 1)) * 16);
-            }
+            const int ta = 2 * s, tb = 2 * s + 1;                    // compile-time taps of the two halves
+            const uint32_t aa = pb[ta / 9] + (uint32_t)(SGN * (((ta / 3) % 3 - 1) * NC_SX + ta % 3 - 1) * 16);
+            const uint32_t ab = tb < NN_TAPS ? pb[tb < NN_TAPS ? tb / 9 : 0] + (uint32_t)(SGN * (((tb / 3) % 3 - 1) * NC_SX + tb % 3 - 1) * 16)
+                                             : zero_row;
             uint32_t a[4];
-            ldsm_x4(a, addr);
+            ldsm_x4(a, hi ? ab : aa);
             // ldmatrix returns the matrices in lane order: 0 cells 0-7 tap 2s, 1 cells 8-15 tap 2s,
             // 2 cells 0-7 tap 2s+1, 3 cells 8-15 tap 2s+1 -- the a0..a3 order of mma's A fragment
             mma_bf16(d, a, bf[s]);
         }
-        const int j = y0 + cy;
-        const long long row = (long long)nx * (j + (long long)ny * k);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int i = x0 + (w & 1) * 16 + g + 8 * h;
-            if (i >= nx || j >= ny) continue;
-            const long long c = row + i;
+            if (!on[h]) continue;
+            const long long ch = c + 8 * h;
             float v0 = d[2 * h] + b0, v1 = d[2 * h + 1] + b1;
-            if (mode == 0) {
+            if (MODE == 0) {
                 v0 = fmaxf(v0, 0.f);
                 v1 = fmaxf(v1, 0.f);
-                *reinterpret_cast<uint32_t*>(outb + c * NN_C + 2 * q) = pack_bf16(v0, v1);
-            } else if (mode == 1) {
-                if (q == 0) outf[c] = v0;
+                *reinterpret_cast<uint32_t*>(outb + ch * NN_C + 2 * q) = pack_bf16(v0, v1);
+            } else if (MODE == 1) {
+                if (q == 0) outf[ch] = v0;
             } else {
-                const __nv_bfloat162 mk = *reinterpret_cast<const __nv_bfloat162*>(mask + c * NN_C + 2 * q);
-                if (!(__bfloat162float(mk.x) > 0.f)) v0 = 0.f;
-                if (!(__bfloat162float(mk.y) > 0.f)) v1 = 0.f;
-                *reinterpret_cast<uint32_t*>(outb + c * NN_C + 2 * q) = pack_bf16(v0, v1);
+                if (!(__bfloat162float(mk[h].x) > 0.f)) v0 = 0.f;
+                if (!(__bfloat162float(mk[h].y) > 0.f)) v1 = 0.f;
+                *reinterpret_cast<uint32_t*>(outb + ch * NN_C + 2 * q) = pack_bf16(v0, v1);
             }
         }
-        __syncthreads();
     }
+}
+
+// Planes per block: the fewest plane steps over all rounds of `slots` resident blocks (a block of k planes takes
+// about k + 2).
+inline int conv_planes(int nx, int ny, int nz, long long slots) {
+    const long long xy = (long long)((nx + NC_TX - 1) / NC_TX) * ((ny + NC_TY - 1) / NC_TY);
+    long long best = -1;
+    int kz = nz;
+    for (int k = 4; k <= 128; ++k) {
+        const long long n = xy * ((nz + k - 1) / k), cost = ((n + slots - 1) / slots) * (k + 2);
+        if (best < 0 || cost < best) {
+            best = cost;
+            kz = k;
+        }
+        if (k >= nz) break;
+    }
+    return kz;
 }
 
 // Weight and bias gradients of one layer: dW[co][tap][ci] = sum_c dz[c][co] y[c + off(tap)][ci],
 // db[co] = sum_c dz[c][co], as a GEMM on the tensor cores: M = 27 taps x 8 channels (padded to 28 taps;
 // the padding tap reads a row of ones in channel 0, so its row is db), N = 8 output channels, K = the
-// cells.  The tile, the three-plane ring and the warps' cells are those of the convolution above: per
+// cells.  The tile, the ring and the warps' cells are those of the convolution above: per
 // plane a warp takes 16 cells, one ldmatrix.x2.trans gives their dz as the B fragment, and per pair of taps
 // one ldmatrix.x4.trans gathers y as the A fragment.  Each mma starts from zero and is added in FP32, so a
 // sum is a chain of one FP32 addition per 16 cells.  Blocks walk tiles of a fixed grid and write one partial
 // each.  Both operands are read once (16 + 16 bytes per cell, halo from L2).
-// 128^3 cells: 98 us per layer; one thread per (tap, channel) with serial global loads took 2.8 ms.
-#define WG_BLOCKS 608
+// 128^3 cells: 62 us per layer, 98 with loads waited for; one thread per (tap, channel) with serial global loads
+// took 2.8 ms.
+#define WG_MINB 3
+#define WG_BLOCKS (WG_MINB * IBM_NSM)       // resident at once
 #define WG_STRIDE (NN_TAPS * NN_C * NN_C + NN_C)
 
 __device__ __forceinline__ void ldsm_x4_t(uint32_t r[4], uint32_t addr) {
@@ -191,21 +235,22 @@ __device__ __forceinline__ void ldsm_x2_t(uint32_t r[2], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
 }
 
-__global__ void __launch_bounds__(256) k_nn_wgrad(int nx, int ny, int nz, int ncout,
+__global__ void __launch_bounds__(256, WG_MINB) k_nn_wgrad(int nx, int ny, int nz, int kz, int ncout,
                                                   const __nv_bfloat16* __restrict__ dz,
                                                   const __nv_bfloat16* __restrict__ y, float* __restrict__ wpart) {
-    __shared__ __align__(16) uint4 ring[3 * NC_PL + 1];          // y planes k - 1 .. k + 1, then the row of ones
+    __shared__ __align__(16) uint4 ring[NC_RING * NC_PL + 1];    // y planes as in the convolution, then the row of ones
     __shared__ __align__(16) uint4 zt[2][NC_TX * NC_TY];         // dz of the plane, double buffered
     __shared__ float red[NN_KSTEPS * 2 * NN_C * NN_C];           // [tap][ci][co]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (tid == 0) ring[3 * NC_PL] = make_uint4(0x3f80u, 0u, 0u, 0u);     // bf16 1 in channel 0
+    if (tid == 0) ring[NC_RING * NC_PL] = make_uint4(0x3f80u, 0u, 0u, 0u);     // bf16 1 in channel 0
     for (int e = tid; e < NN_KSTEPS * 2 * NN_C * NN_C; e += 256) red[e] = 0.f;
-    const int gx = (nx + NC_TX - 1) / NC_TX, gy = (ny + NC_TY - 1) / NC_TY, gz = (nz + NC_KZ - 1) / NC_KZ;
+    const int gx = (nx + NC_TX - 1) / NC_TX, gy = (ny + NC_TY - 1) / NC_TY, gz = (nz + kz - 1) / kz;
     const unsigned items = (unsigned)gx * gy * gz;
+    const long long plane = (long long)nx * ny * NN_C;
     const int mj = lane >> 3, mr = lane & 7;
     // matrix mj of the x4 gather: tap 2s + (mj & 1), cells 8 (mj >> 1) .. + 7 of the warp's 16
     const int cx = (w & 1) * 16 + (mj >> 1) * 8 + mr, cy = w >> 1;
-    const uint32_t ring_base = (uint32_t)__cvta_generic_to_shared(ring), ones = ring_base + 3 * NC_PL * 16;
+    const uint32_t ring_base = (uint32_t)__cvta_generic_to_shared(ring), ones = ring_base + NC_RING * NC_PL * 16;
     const uint32_t cell0 = (uint32_t)(((cy + 1) * NC_SX + cx + 1) * 16);
     const uint32_t zaddr = (uint32_t)__cvta_generic_to_shared(&zt[0][0]) +
                            (uint32_t)((cy * NC_TX + (w & 1) * 16 + (lane & 15)) * 16);
@@ -216,40 +261,46 @@ __global__ void __launch_bounds__(256) k_nn_wgrad(int nx, int ny, int nz, int nc
         for (int h = 0; h < 4; ++h) acc[s][h] = 0.f;
     for (unsigned it = blockIdx.x; it < items; it += gridDim.x) {
         const unsigned q = it / (unsigned)gx;
-        const int x0 = (int)(it - q * gx) * NC_TX, y0 = (int)(q % (unsigned)gy) * NC_TY, z0 = (int)(q / (unsigned)gy) * NC_KZ;
-        const int z1 = z0 + NC_KZ < nz ? z0 + NC_KZ : nz;
-        auto load_plane = [&](int kk, int slot) {
-            uint4* dst = ring + slot * NC_PL;
-            if (tid < NC_PL) {
-                const int ix = x0 + tid % NC_SX - 1, iy = y0 + tid / NC_SX - 1;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (kk >= 0 && kk < nz && ix >= 0 && ix < nx && iy >= 0 && iy < ny)
-                    v = *reinterpret_cast<const uint4*>(y + (ix + (long long)nx * (iy + (long long)ny * kk)) * NN_C);
-                dst[tid] = v;
-            }
+        const int x0 = (int)(it - q * gx) * NC_TX, y0 = (int)(q % (unsigned)gy) * NC_TY, z0 = (int)(q / (unsigned)gy) * kz;
+        const int z1 = z0 + kz < nz ? z0 + kz : nz;
+        RingFill fill(tid, x0, y0, nx, ny);
+        const int zx = x0 + (tid & (NC_TX - 1)), zy = y0 + tid / NC_TX;
+        const bool zin = tid < NC_TX * NC_TY && zx < nx && zy < ny;
+        const __nv_bfloat16* zp = dz + (zx + (long long)nx * zy) * NN_C;
+        uint4 zv;
+        auto fetch_dz = [&](int k) {
+            zv = make_uint4(0u, 0u, 0u, 0u);
+            if (zin) zv = *reinterpret_cast<const uint4*>(zp + k * plane);
         };
-        auto load_dz = [&](int kk, int buf) {
-            if (tid < NC_TX * NC_TY) {
-                const int ix = x0 + (tid & (NC_TX - 1)), iy = y0 + tid / NC_TX;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (ix < nx && iy < ny)
-                    v = *reinterpret_cast<const uint4*>(dz + (ix + (long long)nx * (iy + (long long)ny * kk)) * NN_C);
-                zt[buf][tid] = v;
-            }
+        auto put_dz = [&](int k) {
+            if (tid < NC_TX * NC_TY) zt[k & 1][tid] = zv;
         };
-        __syncthreads();                        // the previous tile's reads of the ring are done
-        load_plane(z0 - 1, 0);
-        load_plane(z0, 1);
-        int sp = 0, sc = 1, sn = 2;             // ring slots of planes k - 1, k, k + 1
+        __syncthreads();                        // the previous tile's reads are done
+#pragma unroll
+        for (int t = -1; t <= 1; ++t) {
+            fill.fetch(y, z0 + t, nz, plane);
+            fill.put(ring, z0 + t, tid);
+        }
+        fetch_dz(z0);
+        put_dz(z0);
+        fill.fetch(y, z0 + 2, nz, plane);
+        if (z0 + 1 < z1) fetch_dz(z0 + 1);
         for (int k = z0; k < z1; ++k) {
-            const int buf = k & 1;
-            load_plane(k + 1, sn);
-            load_dz(k, buf);
+            // every warp is done with plane k - 2 of y and k - 1 of dz; y up to k + 1 and dz of k are there
             __syncthreads();
+            if (k + 2 <= z1) {
+                fill.put(ring, k + 2, tid);
+                if (k + 3 <= z1) fill.fetch(y, k + 3, nz, plane);
+            }
+            if (k + 1 < z1) {
+                put_dz(k + 1);
+                if (k + 2 < z1) fetch_dz(k + 2);
+            }
             uint32_t b[2];
-            ldsm_x2_t(b, zaddr + (uint32_t)buf * (NC_TX * NC_TY * 16));
-            const uint32_t pb[3] = {cell0 + ring_base + (uint32_t)(sp * NC_PL * 16), cell0 + ring_base + (uint32_t)(sc * NC_PL * 16),
-                                    cell0 + ring_base + (uint32_t)(sn * NC_PL * 16)};
+            ldsm_x2_t(b, zaddr + (uint32_t)(k & 1) * (NC_TX * NC_TY * 16));
+            uint32_t pb[3];
+#pragma unroll
+            for (int e = 0; e < 3; ++e) pb[e] = cell0 + ring_base + (uint32_t)((k + e - 1 + NC_RING) % NC_RING) * (NC_PL * 16);
 #pragma unroll
             for (int s = 0; s < NN_KSTEPS; ++s) {
                 const int ta = 2 * s, tb = 2 * s + 1;                    // compile-time taps of the two halves
@@ -262,11 +313,6 @@ __global__ void __launch_bounds__(256) k_nn_wgrad(int nx, int ny, int nz, int nc
 #pragma unroll
                 for (int h = 0; h < 4; ++h) acc[s][h] += d[h];
             }
-            __syncthreads();                    // slot sp is overwritten by the next plane
-            const int t = sp;
-            sp = sc;
-            sc = sn;
-            sn = t;
         }
     }
     // the block's sum over its warps, in warp order
@@ -520,10 +566,13 @@ extern "C" int ibm_net_get_grads(const ibm_net* n, float* h_grads) {
 
 static void conv(const ibm_net* n, int nx, int ny, int nz, const __nv_bfloat16* in, int l, int sgn, int mode,
                  __nv_bfloat16* outb, float* outf, const __nv_bfloat16* mask, cudaStream_t s) {
-    const dim3 grid((unsigned)((nx + NC_TX - 1) / NC_TX), (unsigned)((ny + NC_TY - 1) / NC_TY),
-                    (unsigned)((nz + NC_KZ - 1) / NC_KZ));
-    k_nn_conv_tile<<<grid, 256, 0, s>>>(nx, ny, nz, in, sgn > 0 ? n->frag_fwd[l] : n->frag_bwd[l],
-                                        sgn > 0 ? n->master + offset_b(l) : nullptr, sgn, mode, outb, outf, mask);
+    const int kz = conv_planes(nx, ny, nz, 4LL * IBM_NSM);
+    const dim3 grid((unsigned)((nx + NC_TX - 1) / NC_TX), (unsigned)((ny + NC_TY - 1) / NC_TY), (unsigned)((nz + kz - 1) / kz));
+    const uint32_t* frag = sgn > 0 ? n->frag_fwd[l] : n->frag_bwd[l];
+    const float* bias = sgn > 0 ? n->master + offset_b(l) : nullptr;
+    if (mode == 0) k_nn_conv_tile<1, 0><<<grid, 256, 0, s>>>(nx, ny, nz, kz, in, frag, bias, outb, outf, mask);
+    else if (mode == 1) k_nn_conv_tile<1, 1><<<grid, 256, 0, s>>>(nx, ny, nz, kz, in, frag, bias, outb, outf, mask);
+    else k_nn_conv_tile<-1, 2><<<grid, 256, 0, s>>>(nx, ny, nz, kz, in, frag, bias, outb, outf, mask);
 }
 
 static int net_forward(ibm_net* n, const ibm_grid* g, cudaStream_t s) {
@@ -599,13 +648,13 @@ extern "C" int ibm_net_train_step(ibm_net* n, const ibm_grid* g, const double* d
     conv(n, g->nx, g->ny, g->nz, n->d3, 2, -1, 2, n->d2, nullptr, n->y2, s);
     conv(n, g->nx, g->ny, g->nz, n->d2, 1, -1, 2, n->d1, nullptr, n->y1, s);
     // weight gradients
-    const long long tiles = (long long)((g->nx + NC_TX - 1) / NC_TX) * ((g->ny + NC_TY - 1) / NC_TY) *
-                            ((g->nz + NC_KZ - 1) / NC_KZ);
+    const int kz = conv_planes(g->nx, g->ny, g->nz, WG_BLOCKS);
+    const long long tiles = (long long)((g->nx + NC_TX - 1) / NC_TX) * ((g->ny + NC_TY - 1) / NC_TY) * ((g->nz + kz - 1) / kz);
     const int nblk = (int)(tiles < WG_BLOCKS ? tiles : WG_BLOCKS);
     const __nv_bfloat16* dz[3] = {n->d1, n->d2, n->d3};
     const __nv_bfloat16* yin[3] = {n->x0, n->y1, n->y2};
     for (int l = 0; l < 3; ++l) {
-        k_nn_wgrad<<<nblk, 256, 0, s>>>(g->nx, g->ny, g->nz, cout_of(l), dz[l], yin[l], n->wpart);
+        k_nn_wgrad<<<nblk, 256, 0, s>>>(g->nx, g->ny, g->nz, kz, cout_of(l), dz[l], yin[l], n->wpart);
         k_nn_wgrad_reduce<<<(WG_STRIDE + 31) / 32, 256, 0, s>>>(n->wpart, nblk, cout_of(l), 1.f / (float)N, n->grad + offset_w(l),
                                             n->grad + offset_b(l));
     }
