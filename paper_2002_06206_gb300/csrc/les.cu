@@ -8,6 +8,7 @@
 // cells next to cut links in a separate general kernel.
 #include <type_traits>
 
+#include "scan.cuh"
 #include "solver.cuh"
 
 #ifndef IBM_FLUX_GEN_MINB
@@ -1481,17 +1482,6 @@ __global__ void k_row_counts(Dom D, unsigned long long* __restrict__ rc, uint8_t
     for (int o = 16; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
     if (threadIdx.x == 0) rc[j + (long long)D.ny * k] = n;
 }
-
-__global__ void k_row_scan(long long nrows, unsigned long long* __restrict__ rc, unsigned long long* total) {
-    // one thread: rows are few (ny * nz) and this runs once per solver state
-    unsigned long long acc = 0;
-    for (long long r = 0; r < nrows; ++r) {
-        const unsigned long long v = rc[r];
-        rc[r] = acc;
-        acc += v;
-    }
-    *total = acc;
-}
 }  // namespace
 
 int flux_kernels_setup() {
@@ -1530,7 +1520,7 @@ int build_general_list(LesCtx& c, cudaStream_t s) {
         return ibm_fail(IBM_E_NOMEM, "momentum flux: fast-cell mask (%lld bytes)", (long long)c.D.N);
     }
     k_row_counts<<<rows, 32, 0, s>>>(c.D, rc, c.fastmask);
-    k_row_scan<<<1, 1, 0, s>>>(nrows, rc, rc + nrows);
+    k_scan_tile_totals<<<1, IBM_SCAN_NT, 0, s>>>((long long*)rc, nrows, (long long*)rc + nrows);
     unsigned long long total = 0;
     cudaError_t e = cudaMemcpyAsync(&total, rc + nrows, sizeof(total), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

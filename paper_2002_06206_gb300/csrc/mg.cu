@@ -1715,15 +1715,16 @@ unsigned lin_blocks(long long n) {
 }
 
 // Planes of a tile (halo included) with a cut link: the passes take the general half-sweeps there.
-__global__ void __launch_bounds__(256) k_tile_marks(Dom D, int w, int h, uint8_t* marks) {
-    const int x0 = blockIdx.y * (w - 8), y0 = blockIdx.z * (h - 8), k = blockIdx.x;
+__global__ void __launch_bounds__(256) k_tile_marks(Dom D, int w, int h, unsigned tx, unsigned ty, uint8_t* marks) {
+    const unsigned row = blockIdx.x / tx;
+    const int x0 = (int)(blockIdx.x - row * tx) * (w - 8), y0 = (int)(row % ty) * (h - 8), k = (int)(row / ty);
     unsigned any = 0u;
     for (int q = threadIdx.x; q < w * h; q += blockDim.x) {
         const int x = x0 + q % w, y = y0 + q / w;
         if (x < D.nx && y < D.ny) any |= D.flags[x + (long long)D.sy * y + D.sz * k] & 63u;
     }
     any = __syncthreads_or(any != 0u);
-    if (threadIdx.x == 0) marks[blockIdx.y + (long long)gridDim.y * (blockIdx.z + (long long)gridDim.z * k)] = any ? 1 : 0;
+    if (threadIdx.x == 0) marks[blockIdx.x] = any ? 1 : 0;
 }
 
 // The launch of the fused passes: of the two tile widths (64 x 64 or 128 x 32 cells, halo included; 64 x 64 has the
@@ -1784,7 +1785,7 @@ int fused_plan(const LesCtx& c, MG& mg, int sb) {
         if (e == cudaSuccess && D.flags) {
             e = ibm_malloc(&dev, tiles * D.nz);
             if (e == cudaSuccess) {
-                k_tile_marks<<<dim3(D.nz, p.tx, p.ty), 256>>>(D, w, h, dev);
+                k_tile_marks<<<(unsigned)(tiles * D.nz), 256>>>(D, w, h, p.tx, p.ty, dev);
                 e = cudaMemcpy(marks, dev, tiles * D.nz, cudaMemcpyDeviceToHost);
             }
             cudaFree(dev);
@@ -1805,6 +1806,7 @@ int fused_plan(const LesCtx& c, MG& mg, int sb) {
             for (int rounds = first; rounds < first + 8; ++rounds) {
                 float lo = 0.f, hi = FZ_GENERAL * (D.nz + 9);
                 const long long most = (long long)rounds * IBM_NSM;
+                if (best >= 0.f && 0.999f * best / rounds < hi) hi = 0.999f * best / rounds;     // dearer than the best so far
                 if (p.cut(hi, most, nullptr, nullptr) < 0) continue;
                 for (int it = 0; it < 14; ++it) {
                     const float mid = 0.5f * (lo + hi);
@@ -2217,7 +2219,7 @@ static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStrea
 template <class Fn>
 static void fused_dispatch(const LesCtx& c, const MG& mg, Fn f) {
     using std::integral_constant;
-    const bool vec = c.D.nx % 4 == 0;
+    const bool vec = x4_ok(c);
     if (mg.flx == 16) vec ? f(integral_constant<int, 16>{}, integral_constant<int, 3>{}) : f(integral_constant<int, 16>{}, integral_constant<int, 4>{});
     else vec ? f(integral_constant<int, 32>{}, integral_constant<int, 3>{}) : f(integral_constant<int, 32>{}, integral_constant<int, 4>{});
 }

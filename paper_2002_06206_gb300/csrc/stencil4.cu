@@ -339,7 +339,8 @@ __global__ void __launch_bounds__(256, 4) k_mg_smooth0_x4(Dom D, const float* __
 
 }  // namespace
 
-bool x4_ok(const LesCtx& c) { return (c.D.nx % 4) == 0; }
+// (rows of the library's own arrays then start on 16-byte boundaries; the flags are the caller's)
+bool x4_ok(const LesCtx& c) { return c.D.nx % 4 == 0 && ((uintptr_t)c.D.flags & 3u) == 0; }
 
 dim3 x4_grid(const LesCtx& c) {
     const long long tiles = (long long)((c.D.nx / 4 + X4_TX - 1) / X4_TX) * ((c.D.ny + X4_TY - 1) / X4_TY) *

@@ -307,3 +307,40 @@ def test_geometries_made_and_destroyed_on_several_threads_and_streams(L):
     for t in threads:
         t.join()
     assert not wrong
+
+
+def test_a_solve_with_flags_at_any_address(L):
+    """Flags are the caller's array: at an odd address the kernels read them byte by byte."""
+    import ctypes as C
+    import workloads as W
+    nx, ny, nz = 36, 33, 20
+    N = nx * ny * nz
+    g = L.make_grid(nx, ny, nz)
+    soup = torch.from_numpy(W.random_soup(60, (1, 1, 1), (nx - 1, ny - 1, nz - 1), 4.0, seed=8).astype(np.float32)).cuda()
+    b = None
+    out = []
+    for shift in (0, 1):
+        geo = L.Geometry(g, soup)
+        if shift:
+            buf = torch.empty(N + 1, dtype=torch.uint8, device="cuda")
+            flags = buf[1:]
+            flags.copy_(geo.flags)
+            h = C.c_void_p()
+            v = lambda t: C.c_void_p(t.data_ptr())
+            assert L.lib().ibm_setup(C.byref(g), C.byref(geo.gp), v(flags), v(geo.face_id), v(geo.t_lo), v(geo.t_hi), geo.n_cut,
+                                     C.byref(h), None) == 0
+            geo.close()
+            geo.handle, geo.flags = h, flags
+        sol = L.Solver(g, 0.01, 0.2, CHANNEL, precision=1, geometry=geo, precond=1)
+        if b is None:
+            b = torch.empty(N, dtype=torch.float64, device="cuda")
+            sol.apply(torch.from_numpy(np.random.default_rng(1).standard_normal(N)).cuda(), b)
+        p = torch.zeros(N, dtype=torch.float64, device="cuda")
+        st = sol.solve(b, p, 1e-8, 1000, 0)
+        r = torch.empty_like(b)
+        sol.apply(p, r)
+        assert st.status == 0 and float((b - r).norm()) <= 1.001e-8 * float(b.norm())
+        out.append(st.iters)
+        sol.close()
+        geo.close()
+    assert abs(out[0] - out[1]) <= 1 + out[0] // 10
