@@ -505,6 +505,11 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
     unsigned gen = 0u;                  // bit k: plane t - k takes the general form in this warp
     int slot = 0;                       // ring slot of plane t
     float er[2][2] = {{0.f, 0.f}, {0.f, 0.f}};       // residuals of the even plane [row][position]
+    // the two positions of level 1: their first unknowns, loaded with the even plane, and 1 / dg, loaded a step later
+    // (at the point of use the two loads, one after the other, took a quarter of the pass)
+    const bool two = NI == 3 || left > 2;                // the second position lies in the domain
+    int2 bo = make_int2(0, 0);
+    float2 bi = make_float2(0.f, 0.f);
     auto step = [&](auto par, int t) {
         constexpr int D0 = decltype(par)::value;      // = t & 1
         const int pw = D0, pr = 1 - D0;                // exchange buffers written and read in this step
@@ -517,6 +522,15 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
         S.f[slot * FTP_NT + threadIdx.x] = ft;
         gen = (gen << 1) | ((__any_sync(0xffffffffu, ((nf0 | nf1) & 0x3f3f3f3fu) != 0u) || t == 0 || t == D.nz - 1) ? 1u : 0u);
         fetch(t + 1);
+        if (c.own0 && t - 4 >= k0 && t - 4 < k1) {
+            if (D0 == 0) {
+                const int* o = C1.off + (c.gx >> 1) + (long long)C1.px * ((c.gy >> 1) + (long long)C1.py * ((t - 4) >> 1));
+                if (NI == 3) bo = *reinterpret_cast<const int2*>(o);
+                else bo = make_int2(o[0], two ? o[1] : 0);
+            } else {
+                bi = make_float2(C1.invdg[bo.x], two ? C1.invdg[bo.y] : 0.f);
+            }
+        }
         // half-sweep 1 on plane t, from z = 0
         ftp_zero(Z[0]);
         if (t < D.nz) {
@@ -599,14 +613,17 @@ __global__ void __launch_bounds__(FTP_NT, 1) k_mg_pre_fused(Dom D, const float* 
                 }
             }
             if ((D0 == 1 || lastp) && c.own0) {
-                const long long q = (c.gx >> 1) + (long long)C1.px * ((c.gy >> 1) + (long long)C1.py * (tr >> 1));
-                const bool two = NI == 3 || left > 2;    // the second position lies in the domain
-                const int2 o = NI == 3 ? *reinterpret_cast<const int2*>(C1.off + q) : make_int2(C1.off[q], two ? C1.off[q + 1] : 0);
+                const int2 o = bo;
                 const bool odd = D0 == 1;                // both planes of the block are there
+                if (!odd) bi = make_float2(C1.invdg[o.x], two ? C1.invdg[o.y] : 0.f);
                 // a warp without a cut link in the two planes: whole blocks
                 if (!((gen >> 4) & 1u) && !(odd && ((gen >> 5) & 1u))) {
-                    put_b1<float>(C1, o.x, odd ? (er[0][0] + er[1][0]) + (res[0][0] + res[1][0]) : er[0][0] + er[1][0]);
-                    if (two) put_b1<float>(C1, o.y, odd ? (er[0][1] + er[1][1]) + (res[0][1] + res[1][1]) : er[0][1] + er[1][1]);
+                    auto put = [&](int u, float b, float inv) {
+                        ((float*)C1.b)[u] = b;
+                        ((float*)C1.x)[u] = -b * inv;
+                    };
+                    put(o.x, odd ? (er[0][0] + er[1][0]) + (res[0][0] + res[1][0]) : er[0][0] + er[1][0], bi.x);
+                    if (two) put(o.y, odd ? (er[0][1] + er[1][1]) + (res[0][1] + res[1][1]) : er[0][1] + er[1][1], bi.y);
                 } else {
                     const long long Pe = row0 + D.sz * (tr & ~1);
                     unsigned fe[2], fo[2];
