@@ -62,22 +62,6 @@ namespace {
 __device__ __forceinline__ unsigned flags_at(const Dom& D, long long P) { return D.flags ? (unsigned)D.flags[P] : 0u; }
 
 
-// Conductances and Dirichlet term of a fine (level 0) cell, links in the order x-, x+, y-, y+, z-, z+.
-__device__ __forceinline__ void fine_links(const Dom& D, long long P, const int x[3], unsigned fl, float g[6],
-                                           long long off[6], float& d) {
-    d = 0.f;
-#pragma unroll
-    for (int b = 0; b < 6; ++b) {
-        const int a = b >> 1, s = (b & 1) ? 1 : -1;
-        long long o = 0;
-        const bool in = nb_offset(D, a, s, x[a], o);
-        off[b] = o;
-        g[b] = (!(fl & (1u << b)) && in) ? 1.f : 0.f;
-        if (!in && D.bc[b] == IBM_BC_OUTFLOW) d += 2.f;
-    }
-}
-
-
 // Cell coordinates from a linear index (grids hold fewer than 2^31 cells: 32-bit division).
 __device__ __forceinline__ void coords3(long long c, int nx, int ny, int x[3]) {
     const unsigned u = (unsigned)c, unx = (unsigned)nx, uny = (unsigned)ny;
@@ -251,8 +235,8 @@ __device__ __forceinline__ void put_b1(const MGLev& C, int u, T b) {
 // with a cut link in its plane takes the general form for that plane.
 //
 // The kernels are bound by instruction issue with shared memory close behind: about 300 instructions per
-// thread and plane for 8 cells.  512x256x256: 164 us (pre) and 150 us (post), 1.9 and 2.9 TB/s of the 9.1 and
-// 13 bytes per cell.  A ring of planes in shared memory filled by TMA with one barrier per half-sweep, the
+// thread and plane for 8 cells.  512x256x256: 137 us (pre) and 149 us (post), 2.2 and 2.9 TB/s of the 9.1 and
+// 13 bytes per cell; z of the post pass through a cp.async ring two planes ahead took 180 us.  A ring of planes in shared memory filled by TMA with one barrier per half-sweep, the
 // form before, took 640 and 480 us: it issued 11 and 8.5 warp instructions per cell.
 #define FTP_NT 512
 #define FTP_RING 5
@@ -413,13 +397,13 @@ __device__ __forceinline__ unsigned ftp_load_flags(const uint8_t* p, int left) {
 }
 template <int NI>
 __device__ __forceinline__ void ftp_store(float* p, int left, const float (&z)[4]) {
-    if (NI == 3) {
+    if constexpr (NI == 3) {
         *reinterpret_cast<float4*>(p) = make_float4(z[0], z[1], z[2], z[3]);
-        return;
-    }
+    } else {
 #pragma unroll
-    for (int m = 0; m < 4; ++m)
-        if (m < left) p[m] = z[m];
+        for (int m = 0; m < 4; ++m)
+            if (m < left) p[m] = z[m];
+    }
 }
 
 // Shared memory of a block and the thread's places in it.
@@ -1750,7 +1734,8 @@ __global__ void __launch_bounds__(256) k_tile_marks(Dom D, int w, int h, unsigne
 // blocks run one per SM; for eight numbers of rounds the limit on a chunk's cost is bisected that lets the
 // chunks fit the rounds, and the cheapest is kept.  With chunks of equal height the tiles around a body came last: the
 // two passes take 43 and 34 us in place of 52 and 42 on 256 x 128 x 128 cells around a dirty sphere, 836 and 624 in place
-// of 896 and 681 on 1024 x 512 x 384 around a vehicle (1.3 for FZ_GENERAL: 928 and 679; 2.5: 917 and 663).
+// of 896 and 681 on 1024 x 512 x 384 around a vehicle (1.3 for FZ_GENERAL: 928 and 679; 2.5: 917 and 663).  With the
+// first pass's loads ahead (600 us there) 1.4, 1.9 and 2.3 are again slower.
 #define FZ_GENERAL 1.65f
 
 struct FzPlan {
