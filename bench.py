@@ -375,7 +375,7 @@ def time_classify(L, torch, name=WORKLOAD, repeats=5):
     return {"workload": name, "triangles": int(tri.shape[0]), "cells": N, "ms": ms,
             "predicate_tests": int(ntests.value), "mtests_per_s": ntests.value / (ms * 1e-3) / 1e6,
             "links_per_s": 3 * N / (ms * 1e-3), "cut_faces": int(ncut.value),
-            "note": "median of %d after one warm-up; includes the per-face table fill, compaction and the "
+            "note": "median of %d after one warm-up; includes the compaction and the "
                     "host read of the cut count" % repeats}
 
 

@@ -246,7 +246,7 @@ class Geometry:
             break
         self.n_cut = int(n_cut.value)
         self.n_tests = int(n_tests.value)
-        self.workspace = None           # 48 bytes per cell, needed by the classification only
+        self.workspace = None           # needed by the classification only
         self.face_id = self.face_id[:self.n_cut]
         self.t_lo = self.t_lo[:self.n_cut]
         self.t_hi = self.t_hi[:self.n_cut]
