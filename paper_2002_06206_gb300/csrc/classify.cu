@@ -83,7 +83,9 @@ __device__ __forceinline__ bool face_hit(const Tri& T, int a, int jb, int jc, co
 
 // FP32 test of the same line that only ever says "certainly outside": two of the barycentric weights differ
 // in sign by more than the FP32 error (every difference and product is good to a few 2^-24 of the absolute
-// products) and the edge tolerance, so the FP64 predicate rejects the line whatever the sign of their sum.
+// products) and the edge tolerance, so the FP64 predicate rejects the line whatever the sign of their sum.  It needs
+// the line's coordinates j + 1/2 exact in FP32: on grids of more than 2^23 cells along an axis every line goes to
+// the FP64 predicate (TestArgs::fp32).
 __device__ __forceinline__ bool surely_outside(float Ab, float Ac, float Bb, float Bc, float Cb, float Cc, float qb, float qc,
                                                float eps) {
     const float ab = qb - Ab, ac = qc - Ac, bb = qb - Bb, bc = qc - Bc, cb = qb - Cb, cc = qc - Cc;
@@ -117,6 +119,7 @@ struct TestArgs {
     long long ntri;
     int n[3];
     double eps_edge, eps_det;
+    int fp32;                      // surely_outside may be asked
     uint8_t* flags;
     unsigned long long *tmin, *tmax, *tests;
     HitList hits;
@@ -277,7 +280,8 @@ __global__ void __launch_bounds__(256) k_test_lines(TestArgs A, int tpb) {
                 if (g < total) {
                     l = (unsigned)(g - e0);
                     const int jc = (int)(l / (unsigned)nb), jb = (int)l - jc * nb;
-                    may = !surely_outside(q[0], q[1], q[2], q[3], q[4], q[5], (float)(b0 + jb) + 0.5f, (float)(c0 + jc) + 0.5f, epsf);
+                    may = !A.fp32 || !surely_outside(q[0], q[1], q[2], q[3], q[4], q[5], (float)(b0 + jb) + 0.5f,
+                                                     (float)(c0 + jc) + 0.5f, epsf);
                 }
                 const unsigned m = __ballot_sync(0xffffffffu, may);
                 if (may) {
@@ -503,6 +507,7 @@ extern "C" int ibm_classify(const ibm_grid* g, const float* d_tri, int64_t ntri,
         A.n[0] = g->nx; A.n[1] = g->ny; A.n[2] = g->nz;
         A.eps_edge = gp->eps_edge;
         A.eps_det = gp->eps_det;
+        A.fp32 = g->nx <= 1 << 23 && g->ny <= 1 << 23 && g->nz <= 1 << 23;
         A.flags = d_flags;
         A.tmin = w.tmin;
         A.tmax = w.tmax;
