@@ -85,7 +85,8 @@ __device__ __forceinline__ bool face_hit(const Tri& T, int a, int jb, int jc, co
 // in sign by more than the FP32 error (every difference and product is good to a few 2^-24 of the absolute
 // products) and the edge tolerance, so the FP64 predicate rejects the line whatever the sign of their sum.  It needs
 // the line's coordinates j + 1/2 exact in FP32: on grids of more than 2^23 cells along an axis every line goes to
-// the FP64 predicate (TestArgs::fp32).
+// the FP64 predicate (TestArgs::fp32).  eps >= 0: a negative tolerance (a triangle shrunk by it) counts as 0 here,
+// which rejects less.
 __device__ __forceinline__ bool surely_outside(float Ab, float Ac, float Bb, float Bc, float Cb, float Cc, float qb, float qc,
                                                float eps) {
     const float ab = qb - Ab, ac = qc - Ac, bb = qb - Bb, bc = qc - Bc, cb = qb - Cb, cc = qc - Cc;
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(256) k_test_lines(TestArgs A, int tpb) {
             store(hit, fid, bits);
             nq -= nq < 32 ? nq : 32;
         };
-        const float epsf = (float)A.eps_edge * 1.0001f;
+        const float epsf = A.eps_edge > 0.0 ? (float)A.eps_edge * 1.0001f : 0.f;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const int b = (a + 1) % 3, c = (a + 2) % 3;

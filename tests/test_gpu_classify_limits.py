@@ -41,3 +41,13 @@ def test_lines_beyond_the_whole_numbers_of_fp32(L, axis):
     tri[:, :, axis] = rng.integers(n - 38, n, (400, 1)) + rng.integers(-1, 2, (400, 3))
     tri[:40, :, axis] -= n // 2
     same_as_the_oracle(L, tuple(shape), tri.astype(np.float32))
+
+
+@pytest.mark.parametrize("eps", [-0.3, -0.05, -1e-9, 0.0, 0.02, 5.0])
+def test_edge_tolerances_of_either_sign(L, eps):
+    """A negative tolerance keeps the inner part of a triangle, a large one reaches beyond it.  Small triangles with
+    lines at any distance from their edges, and large ones."""
+    import workloads as W
+    shape = (40, 36, 33)
+    soup = np.concatenate([W.random_soup(4000, (0, 0, 0), shape, 2.5, seed=3), W.random_soup(40, (0, 0, 0), shape, 30.0, seed=4)])
+    same_as_the_oracle(L, shape, soup.astype(np.float32), eps_edge=eps)
