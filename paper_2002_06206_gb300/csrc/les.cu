@@ -956,12 +956,12 @@ __global__ void __launch_bounds__(256, 8) k_rhs(Dom D, FaceLayout F, const T* __
 }
 
 // A pressure held for differences that are rounded to the working precision.  FP64 mode: the double itself.
-// FP32 mode: hi + lo, the double's leading 24 bits and the 29 below them as two floats, taken from its bits:
-// GB300 issues an FP64 subtraction or conversion at 1/70 of the FP32 rate, and six differences per cell made
-// the correction FP64 bound.  hi - hi' is exact for values within a factor of two and rounded to 2^-24 of
-// the difference otherwise, lo carries 2^-48 of the value, so the difference is good to the FP32 rounding of
-// its result.  Values whose low part leaves the range of a float (below 2^-74, above 2^127, not finite) set
-// `odd`: the cell then takes FP64 arithmetic.
+// FP32 mode: hi + mid + lo, the double's leading 24 bits and the 16 and 13 below them as three floats, all exact,
+// taken from its bits: GB300 issues an FP64 subtraction or conversion at 1/70 of the FP32 rate, and six differences
+// per cell made the correction FP64 bound.  `minus` keeps the rounding errors of its two large terms, so the result is
+// the exact difference rounded once, however much of the two values cancels, as an FP64 subtraction rounded to FP32
+// gives it (a tie may round the other way).  Values whose low part leaves the normal range of a float (below 2^-74, above
+// 2^126, not finite) set `odd`: the cell then takes FP64 arithmetic.
 template <class T> struct PVal;
 template <> struct PVal<double> {
     double v;
@@ -970,31 +970,41 @@ template <> struct PVal<double> {
     __device__ __forceinline__ double minus(const PVal& o) const { return v - o.v; }
 };
 template <> struct PVal<float> {
-    float hi, lo;
+    float hi, mid, lo;
     __device__ __forceinline__ PVal(double x, bool& odd) {
         const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
-        // exponents 949 .. 1149 (and zero): the float's exponent is the low eight bits with the top one flipped
+        // exponents 949 .. 1148 (and zero): the float's exponent is the low eight bits with the top one flipped
         const unsigned m = h & 0x7fffffffu;
         odd = odd || (m - (949u << 20) > (200u << 20) && (m | l) != 0u);
         const unsigned b = (__funnelshift_l(l, h, 3) ^ 0x40000000u) & 0x7fffffffu;
-        const unsigned f = m == 0u ? 0u : b | (h & 0x80000000u);
+        const unsigned f = m == 0u ? 0u : b | (h & 0x80000000u), e = f & 0xff800000u;
         hi = __uint_as_float(f);
-        lo = __uint_as_float((f & 0xff800000u) - (52u << 23)) * (float)(l & 0x1fffffffu);
+        // (whole numbers below 2^23 by way of 2^23 + n: conversions run at an eighth of the FP32 rate)
+        mid = __uint_as_float(e - (39u << 23)) * (__uint_as_float(0x4b000000u | ((l >> 13) & 0xffffu)) - 8388608.f);
+        lo = __uint_as_float(e - (52u << 23)) * (__uint_as_float(0x4b000000u | (l & 0x1fffu)) - 8388608.f);
     }
     __device__ __forceinline__ PVal neg() const {
         PVal r(*this);
         r.hi = -hi;
+        r.mid = -mid;
         r.lo = -lo;
         return r;
     }
-    __device__ __forceinline__ float minus(const PVal& o) const { return (hi - o.hi) + (lo - o.lo); }
+    __device__ __forceinline__ float minus(const PVal& o) const {
+        // the rounding error of the leading difference (any order of the two) ...
+        const float d = __fsub_rn(hi, o.hi), t = __fsub_rn(d, hi), e1 = __fsub_rn(__fsub_rn(hi, __fsub_rn(d, t)), __fadd_rn(o.hi, t));
+        // ... and of the sum with the middle one, which is exact where that is the larger
+        const float m = __fsub_rn(mid, o.mid), s = __fadd_rn(d, m), e2 = __fsub_rn(m, __fsub_rn(s, d));
+        return s + ((e1 + e2) + (lo - o.lo));
+    }
 };
 
 // Eq. correction: cells by the central pressure difference through the link values (c = dt / (2 dx)), faces
 // by the compact difference across uncut interior and outflow faces (dtdx = dt / dx).  One thread per cell
 // updates the cell, its three lower faces and the upper one of the last cell of an axis, marching a column:
-// p, u*, U* and the flags are read once.  512x256x256 FP32: 363 us (5.3 TB/s of the 57 bytes per cell; 403 us at
-// three blocks per SM), 930 us as one cell and three face kernels in FP64 differences.
+// p, u*, U* and the flags are read once.  The differences along y are left to the FP64 units, which are idle beside
+// those of split pressures.  512x256x256 FP32: 416 us (4.6 TB/s of the 57 bytes per cell), 475 us with all differences
+// from split pressures; 930 us as one cell and three face kernels in FP64 differences.
 template <class T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_correct(Dom D, FaceLayout F, const T* __restrict__ us, const T* __restrict__ Us,
                                                  const double* __restrict__ p, T* __restrict__ u, T* __restrict__ U, T c,
@@ -1022,7 +1032,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_correct(Dom D, 
         return k + 1 < D.nz ? D.sz : (periodic(2) ? -(long long)k * D.sz : 0);
     };
     bool odd = false, odd_c = false;
-    V pc(p[P], odd_c), pm(p[P + zoff(k0, -1)], odd);
+    double q = p[P];
+    V pc(q, odd_c), pm(p[P + zoff(k0, -1)], odd);
     for (int k = k0; k < k1; ++k, P += D.sz, fx += sfx, fy += sfy, fz += D.sz) {
         const unsigned fl = D.flags ? (unsigned)D.flags[P] : 0u;
         const T usx = us[P], usy = us[D.N + P], usz = us[2 * D.N + P];
@@ -1030,8 +1041,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_correct(Dom D, 
         const long long oz = zoff(k, 1);
         bool odd_z = false;
         odd = odd || odd_c;
-        V zp(p[P + oz], odd_z);
-        V xm(p[P + oxm], odd), xp(p[P + oxp], odd), ym(p[P + oym], odd), yp(p[P + oyp], odd);
+        const double qz = p[P + oz];
+        double yl = p[P + oym], yh = p[P + oyp];
+        V zp(qz, odd_z);
+        V xm(p[P + oxm], odd), xp(p[P + oxp], odd);
         V zm = pm;
         const V zc = zp;
         odd = odd || odd_z;
@@ -1040,37 +1053,38 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_correct(Dom D, 
         if (side) {
             if (i == 0 && outflow(0, -1)) xm = pc.neg();
             if (i == D.nx - 1 && outflow(0, 1)) xp = pc.neg();
-            if (j == 0 && outflow(1, -1)) ym = pc.neg();
-            if (j == D.ny - 1 && outflow(1, 1)) yp = pc.neg();
+            if (j == 0 && outflow(1, -1)) yl = -q;
+            if (j == D.ny - 1 && outflow(1, 1)) yh = -q;
             if (k == 0 && outflow(2, -1)) zm = pc.neg();
             if (k == D.nz - 1 && outflow(2, 1)) zp = pc.neg();
             if (k == 0 && kept(2, -1)) keep |= 16u;
         }
         // differences: lower, upper and central of each axis; a cut link reads the cell's own pressure
-        T lo[3] = {pc.minus(xm), pc.minus(ym), pc.minus(zm)}, up[3] = {(T)0, (T)0, (T)0}, ce[3];
+        T lo[3] = {pc.minus(xm), (T)(q - yl), pc.minus(zm)}, up[3] = {(T)0, (T)0, (T)0}, ce[3];
         ce[0] = xp.minus(xm);
-        ce[1] = yp.minus(ym);
         ce[2] = zp.minus(zm);
         if (side) {
             up[0] = xp.minus(pc);
-            up[1] = yp.minus(pc);
+            up[1] = (T)(yh - q);
             up[2] = zp.minus(pc);
         }
-        if (fl & 63u) {
+        if (fl & 4u) yl = q;
+        if (fl & 8u) yh = q;
+        ce[1] = (T)(yh - yl);
+        if (fl & 51u) {
             if (fl & 3u) ce[0] = ((fl & 2u) ? pc : xp).minus((fl & 1u) ? pc : xm);
-            if (fl & 12u) ce[1] = ((fl & 8u) ? pc : yp).minus((fl & 4u) ? pc : ym);
             if (fl & 48u) ce[2] = ((fl & 32u) ? pc : zp).minus((fl & 16u) ? pc : zm);
         }
         if (sizeof(T) == 4 && odd) {
-            const double q = p[P];
-            const long long off[3][2] = {{oxm, oxp}, {oym, oyp}, {zoff(k, -1), oz}};
-            const int x[3] = {i, j, k}, n[3] = {D.nx, D.ny, D.nz};
-            for (int a = 0; a < 3; ++a) {
-                const double l = x[a] == 0 && outflow(a, -1) ? -q : p[P + off[a][0]];
-                const double h = x[a] == n[a] - 1 && outflow(a, 1) ? -q : p[P + off[a][1]];
+            const long long off[2][2] = {{oxm, oxp}, {zoff(k, -1), oz}};
+            const int x[2] = {i, k}, n[2] = {D.nx, D.nz};
+            for (int h = 0; h < 2; ++h) {
+                const int a = 2 * h;
+                const double l = x[h] == 0 && outflow(a, -1) ? -q : p[P + off[h][0]];
+                const double r = x[h] == n[h] - 1 && outflow(a, 1) ? -q : p[P + off[h][1]];
                 lo[a] = (T)(q - l);
-                up[a] = (T)(h - q);
-                ce[a] = (T)(((fl >> (2 * a + 1)) & 1u ? q : h) - ((fl >> (2 * a)) & 1u ? q : l));
+                up[a] = (T)(r - q);
+                ce[a] = (T)(((fl >> (2 * a + 1)) & 1u ? q : r) - ((fl >> (2 * a)) & 1u ? q : l));
             }
         }
         u[P] = usx - c * ce[0];
@@ -1086,6 +1100,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_correct(Dom D, 
         }
         pm = pc;
         pc = zc;
+        q = qz;
         odd = odd_c;
         odd_c = odd_z;
     }
