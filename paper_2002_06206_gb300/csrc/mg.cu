@@ -13,7 +13,10 @@
 // With piecewise-constant prolongation P and restriction R = P^T the Galerkin coarse operator R A P
 // is again a weighted graph Laplacian plus the outflow terms: the conductance between two coarse
 // unknowns is the sum of the fine conductances between their aggregates.  Links join only
-// face-neighbouring positions, so the parity of a position two-colours every level.  The V-cycle
+// face-neighbouring positions, so the parity of a position two-colours every level without an odd number of positions
+// (three or more) along a periodic axis.  On an `odd` level the seam joins positions of one colour; a half-sweep then
+// takes the values its own colour had before it (one simultaneous update of the colour), so the sweeps before and after
+// the correction stay adjoint and no thread reads what another writes.  The V-cycle
 // (pre-smoothing red then black, post-smoothing black then red, the coarse correction scaled by
 // omega < 2, symmetric sweeps on the coarsest level) is a symmetric operator, as CG requires.
 //
@@ -33,6 +36,7 @@ namespace cg = cooperative_groups;
 // Levels first .. nlev - 1 of the one-launch tail (see k_mg_tail), with each level's share of a block.
 struct MGTailLev {
     int M, M0;               // unknowns; the first M0 have colour 0
+    int odd;                 // links within a colour
     int s0, s1;              // unknowns of either colour per block (all of them for the coarsest: block 0)
     unsigned i0, i1;         // floor(2^32 / s) + 1
     int x, b, t;             // byte offsets of its arrays in shared memory: iterate, right-hand side, residual,
@@ -91,10 +95,11 @@ __device__ __forceinline__ T gs_value(const Dom& D, const T* __restrict__ r, con
 
 // One red-black Gauss-Seidel pass of colour `col` on level 0 for  A^ z = scale * r.  Each thread takes KU pairs of
 // planes of one (i, j) column and updates the cell of colour `col` in each pair.  With `zero` the iterate is taken
-// as 0 (first pass of a V-cycle) and the other cell of each pair is cleared.  64 x 32 x 32 in FP64, KU = 1: 2.7 us, with four
+// as 0 (first pass of a V-cycle) and the other cell of each pair is cleared.  zin: the iterate before the pass (z itself
+// unless the grid is odd).  64 x 32 x 32 in FP64, KU = 1: 2.7 us, with four
 // pairs and an FP64 division at every domain face 9.5 us.
 template <class T, int KU>
-__global__ void __launch_bounds__(256) k_mg_smooth0(Dom D, const T* __restrict__ r, T* __restrict__ z, T scale,
+__global__ void __launch_bounds__(256) k_mg_smooth0(Dom D, const T* __restrict__ r, T* z, const T* zin, T scale,
                                                     int col, int zero, const SolveScal* sc) {
     if (sc->done) return;
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
@@ -105,7 +110,7 @@ __global__ void __launch_bounds__(256) k_mg_smooth0(Dom D, const T* __restrict__
     for (int u = 0; u < KU; ++u) {
         const int k = kb + 2 * u + par;
         const long long P = i + (long long)D.sy * j + D.sz * k;
-        if (k < D.nz) z[P] = gs_value<T>(D, r, z, scale, P, i, j, k, zero != 0);
+        if (k < D.nz) z[P] = gs_value<T>(D, r, zin, scale, P, i, j, k, zero != 0);
         if (zero) {
             const int k2 = kb + 2 * u + (par ^ 1);
             if (k2 < D.nz) z[i + (long long)D.sy * j + D.sz * k2] = (T)0;
@@ -115,7 +120,7 @@ __global__ void __launch_bounds__(256) k_mg_smooth0(Dom D, const T* __restrict__
 
 // Last pass of the V-cycle on level 0 (colour 0) fused with rho = (r, z) over both colours.
 template <class T, int KU>
-__global__ void __launch_bounds__(256) k_mg_final0(Dom D, const T* __restrict__ r, T* __restrict__ z, T scale,
+__global__ void __launch_bounds__(256) k_mg_final0(Dom D, const T* __restrict__ r, T* z, const T* zin, T scale,
                                                    SolveScal* sc, double* partials, unsigned* counter) {
     if (sc->done) return;
     const int i = blockIdx.x * IBM_TX + threadIdx.x, j = blockIdx.y * IBM_TY + threadIdx.y;
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(256) k_mg_final0(Dom D, const T* __restrict__ 
             const int k = kb + 2 * u + par, k2 = kb + 2 * u + (par ^ 1);
             if (k < D.nz) {
                 const long long P = i + (long long)D.sy * j + D.sz * k;
-                const T zv = gs_value<T>(D, r, z, scale, P, i, j, k, false);
+                const T zv = gs_value<T>(D, r, zin, scale, P, i, j, k, false);
                 z[P] = zv;
                 part += r[P] * zv;
             }
@@ -1056,7 +1061,8 @@ __global__ void k_ell(MGLev L, int* wide) {
 // written with b by whoever forms b; the residual of colour 0 after colour 1 is then  -sum g x_w  and that
 // of colour 1 is zero, so the restriction reads colour 0 only.  After the correction colour 1 reads its
 // neighbours' prolongated values on the fly and colour 0 reads colour 1: neither needs its own old value,
-// so no pass adds the correction.  Four passes per level: colour 1, restriction, colour 1, colour 0.
+// so no pass adds the correction.  Four passes per level: colour 1, restriction, colour 1, colour 0.  An odd level's
+// residual is evaluated in full and its passes after the correction write a second array (godd).
 
 // sum over the links of u of g f(neighbour).
 template <class T, class Fn>
@@ -1087,14 +1093,14 @@ __device__ __forceinline__ T row_sum(const MGLev& L, long long u, Fn f) {
     return s;
 }
 
-// Colour `col` from its neighbours.
+// Colour `col` from its neighbours, into `out`.
 template <class T>
-__device__ __forceinline__ void gsmooth(const MGLev& L, int col, long long t0, long long nt) {
+__device__ __forceinline__ void gsmooth(const MGLev& L, int col, long long t0, long long nt, T* out) {
     const T* b = (const T*)L.b;
-    T* x = (T*)L.x;
+    const T* x = (const T*)L.x;
     const long long lo = col ? L.M0 : 0, hi = col ? L.M : L.M0;
     for (long long u = lo + t0; u < hi; u += nt)
-        x[u] = (row_sum<T>(L, u, [&](int w) { return x[w]; }) - b[u]) * (T)L.invdg[u];
+        out[u] = (row_sum<T>(L, u, [&](int w) { return x[w]; }) - b[u]) * (T)L.invdg[u];
 }
 
 // Colour 1 after the coarse correction: the neighbours (colour 0) count with x + omega x_C(parent).
@@ -1107,11 +1113,28 @@ __device__ __forceinline__ void gup(const MGLev& L, const MGLev& C, T omega, lon
         x[u] = (row_sum<T>(L, u, [&](int w) { return x[w] + omega * xc[L.parent[w]]; }) - b[u]) * (T)L.invdg[u];
 }
 
+// The passes of an odd level.  0: colour 1 before the correction (its own old value is 0); 1: colour 1 after it, into
+// y; 2: colour 0 after it, into y.  What has no new value yet counts with its old one and the correction.
+template <class T>
+__device__ __forceinline__ void godd(const MGLev& L, const MGLev& C, T omega, int pass, long long t0, long long nt) {
+    const T* b = (const T*)L.b;
+    const T* xc = (const T*)C.x;
+    T *x = (T*)L.x, *y = (T*)L.y;
+    const long long lo = pass < 2 ? L.M0 : 0, hi = pass < 2 ? L.M : L.M0;
+    for (long long u = lo + t0; u < hi; u += nt) {
+        const T s = row_sum<T>(L, u, [&](int w) {
+            if (pass == 0) return w < L.M0 ? x[w] : (T)0;
+            return pass == 2 && w >= L.M0 ? y[w] : x[w] + omega * xc[L.parent[w]];
+        });
+        (pass == 0 ? x : y)[u] = (s - b[u]) * (T)L.invdg[u];
+    }
+}
+
 // b_C[v] = -sum over the children u of v of colour 0 of  sum g x_w; x_C = -b_C / dg.  Four lanes per coarse
 // unknown (a plain 2x2x2 block has four children of each colour).  The thread count is a multiple of 32.
-// FP64: 1 / dg is stored in FP32, so the smoothed residuals vanish to 2^-24 only; they are evaluated in full
-// over all children.
-template <class T>
+// FULL (FP64, where 1 / dg is stored in FP32 and the smoothed residuals vanish to 2^-24 only, and odd levels): the
+// residuals are evaluated as they are, over all children.
+template <class T, bool FULL>
 __device__ __forceinline__ void grestrict(const MGLev& F, const MGLev& C, long long t0, long long nt) {
     const T* xf = (const T*)F.x;
     T* bc = (T*)C.b;
@@ -1124,7 +1147,7 @@ __device__ __forceinline__ void grestrict(const MGLev& F, const MGLev& C, long l
         if (v < C.M)
             for (int k = C.cp[v] + lane; k < C.cp[v + 1]; k += 4) {
                 const int u = C.ch[k];
-                if constexpr (std::is_same<T, double>::value) {
+                if constexpr (FULL) {
                     const T xu = xf[u];
                     acc += ((const T*)F.b)[u] - (row_sum<T>(F, u, [&](int w) { return xf[w] - xu; }) - (T)F.d[u] * xu);
                 } else {
@@ -1149,8 +1172,11 @@ __global__ void __launch_bounds__(1024) k_gcoarsest(MGLev L, int sweeps, const S
     for (long long u = threadIdx.x; u < L.M; u += blockDim.x) x[u] = (T)0;
     __syncthreads();
     for (int pass = 0; pass < 4 * sweeps; ++pass) {
-        const int half = pass / (2 * sweeps);
-        gsmooth<T>(L, (pass & 1) ^ half, threadIdx.x, blockDim.x);
+        const int half = pass / (2 * sweeps), col = (pass & 1) ^ half;
+        gsmooth<T>(L, col, threadIdx.x, blockDim.x, L.odd ? (T*)L.y : x);
+        __syncthreads();
+        if (!L.odd) continue;
+        for (long long u = (col ? L.M0 : 0) + threadIdx.x; u < (col ? L.M : L.M0); u += blockDim.x) x[u] = ((T*)L.y)[u];
         __syncthreads();
     }
 }
@@ -1158,13 +1184,19 @@ __global__ void __launch_bounds__(1024) k_gcoarsest(MGLev L, int sweeps, const S
 template <class T>
 __global__ void __launch_bounds__(256) k_gsmooth(MGLev L, int col, const SolveScal* sc) {
     if (sc->done) return;
-    gsmooth<T>(L, col, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
+    gsmooth<T>(L, col, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x, (T*)L.x);
 }
 
 template <class T>
+__global__ void __launch_bounds__(256) k_godd(MGLev L, MGLev C, T omega, int pass, const SolveScal* sc) {
+    if (sc->done) return;
+    godd<T>(L, C, omega, pass, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
+}
+
+template <class T, bool FULL>
 __global__ void __launch_bounds__(256) k_grestrict(MGLev F, MGLev C, const SolveScal* sc) {
     if (sc->done) return;
-    grestrict<T>(F, C, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
+    grestrict<T, FULL>(F, C, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
 template <class T>
@@ -1270,7 +1302,7 @@ __global__ void __launch_bounds__(256) k_tail_image(MGTail M, unsigned char* img
             for (int i = threadIdx.x; i < n; i += blockDim.x) {
                 const int u = lo + i, r0 = L.rp[u], nr = L.rp[u + 1] - r0;
                 A.dg()[base + i] = (T)L.invdg[u];
-                if (sizeof(T) == 8) A.d()[base + i] = (T)L.d[u];
+                if (sizeof(T) == 8 || A.t.odd) A.d()[base + i] = (T)L.d[u];
                 int at = 0;
                 if (nr > MG_ELL) {
                     at = atomicAdd(&cur[rank * IBM_MG_MAXLEV + l], nr);
@@ -1298,7 +1330,8 @@ __global__ void __launch_bounds__(256) k_tail_image(MGTail M, unsigned char* img
     }
 }
 
-template <class T>
+// ODD: a level may be odd.
+template <class T, bool ODD>
 __global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant__ MGTail M, const SolveScal* sc) {
     if (sc->done) return;                       // the flag is uniform: set by an earlier kernel
     extern __shared__ __align__(16) unsigned char tail_smem[];
@@ -1333,11 +1366,18 @@ __global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant
             for (int i = tid; i < C.t.M; i += MG_TAIL_NT) C.x()[i] = (T)0;
     }
     cl.sync();
-    // colour c of a level from its neighbours
+    // a place on level A belongs to colour 0
+    auto first = [&](const TailLevel<T>& A, unsigned q) { return (q & ((1u << A.shift) - 1u)) < (unsigned)A.t.s0; };
+    // colour c of a level from its neighbours (odd levels: colour 1 from those of colour 0, its own old value is 0)
     auto smooth = [&](const TailLevel<T>& A, int c) {
         int base, n, lo;
         A.span(c, base, n, lo);
         T* x = A.x();
+        if (ODD && A.t.odd) {
+            for (int i = base + tid; i < base + n; i += MG_TAIL_NT)
+                x[i] = (A.template row<false>(i, [&](unsigned q, unsigned) { return first(A, q) ? A.at(x, q) : (T)0; }) - A.b()[i]) * A.dg()[i];
+            return;
+        }
         for (int i = base + tid; i < base + n; i += MG_TAIL_NT)
             x[i] = (A.template row<false>(i, [&](unsigned q, unsigned) { return A.at(x, q); }) - A.b()[i]) * A.dg()[i];
     };
@@ -1346,13 +1386,14 @@ __global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant
         T* x = A.x();
         smooth(A, 1);
         cl.sync();
-        // residuals (FP64: of both colours, see grestrict)
-        for (int c = 0; c < (sizeof(T) == 8 ? 2 : 1); ++c) {
+        // residuals (in full: of both colours, see grestrict)
+        const bool full = sizeof(T) == 8 || (ODD && A.t.odd);
+        for (int c = 0; c < (full ? 2 : 1); ++c) {
             int base, n, lo;
             A.span(c, base, n, lo);
             for (int i = base + tid; i < base + n; i += MG_TAIL_NT) {
                 const T xu = x[i];
-                if (sizeof(T) == 8)
+                if (full)
                     A.tmp()[i] = A.b()[i] - (A.template row<false>(i, [&](unsigned q, unsigned) { return A.at(x, q) - xu; }) - A.d()[i] * xu);
                 else
                     A.tmp()[i] = -A.template row<false>(i, [&](unsigned q, unsigned) { return A.at(x, q); });
@@ -1407,21 +1448,28 @@ __global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant
             for (int pass = 0; pass < 2 * M.coarse_sweeps; ++pass) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
+                    // (the barriers stand outside what only some lanes of a warp run)
                     auto colour = [&](auto cc) {
                         constexpr int c = decltype(cc)::value;
-                        if (!on[c]) return;
                         const int i = (c ? A.t.s0 : 0) + tid;
                         T s = 0;
-                        if (q[c][0] == MG_FAR) {
-                            s = A.template row<false>(i, [&](unsigned p, unsigned) { return x[p]; });
-                        } else {
-                            T v[MG_ELL];
+                        if (on[c]) {
+                            if (q[c][0] == MG_FAR) {
+                                s = A.template row<false>(i, [&](unsigned p, unsigned) { return x[p]; });
+                            } else {
+                                T v[MG_ELL];
 #pragma unroll
-                            for (int e = 0; e < MG_ELL; ++e) v[e] = x[q[c][e]];
+                                for (int e = 0; e < MG_ELL; ++e) v[e] = x[q[c][e]];
 #pragma unroll
-                            for (int e = 0; e < MG_ELL; ++e) s += g[c][e] * v[e];
+                                for (int e = 0; e < MG_ELL; ++e) s += g[c][e] * v[e];
+                            }
                         }
-                        x[i] = (s - b[c]) * dg[c];
+                        if (ODD && A.t.odd) {                       // every value of the colour is read before one is written
+                            __syncwarp();
+                            asm volatile("bar.sync 1, %0;" ::"r"(nth) : "memory");
+                        }
+                        if (on[c]) x[i] = (s - b[c]) * dg[c];
+                        __syncwarp();
                     };
                     if (h ^ (pass >= M.coarse_sweeps ? 1 : 0)) colour(std::integral_constant<int, 1>{});
                     else colour(std::integral_constant<int, 0>{});
@@ -1432,15 +1480,37 @@ __global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant
             for (int pass = 0; pass < 4 * M.coarse_sweeps; ++pass) {
                 const int c = (pass & 1) ^ (pass / (2 * M.coarse_sweeps));
                 const int lo = c ? A.t.M0 : 0, hi = c ? A.t.M : A.t.M0;
+                T* out = ODD && A.t.odd ? A.tmp() : x;
                 for (int i = lo + tid; i < hi; i += MG_TAIL_NT)
-                    x[i] = (A.template row<false>(i, [&](unsigned p, unsigned) { return x[p]; }) - A.b()[i]) * A.dg()[i];
+                    out[i] = (A.template row<false>(i, [&](unsigned p, unsigned) { return x[p]; }) - A.b()[i]) * A.dg()[i];
                 __syncthreads();
+                if (ODD && A.t.odd) {
+                    for (int i = lo + tid; i < hi; i += MG_TAIL_NT) x[i] = out[i];
+                    __syncthreads();
+                }
             }
         }
     }
     cl.sync();
     for (int l = last - 1; l >= M.first; --l) {
         const TailLevel<T> A(M, l, tail_smem, rank), C(M, l + 1, tail_smem, rank);
+        if (ODD && A.t.odd) {
+            // as godd, into tmp
+            T *x = A.x(), *y = A.tmp();
+            const T om = (T)M.omega;
+            for (int c = 1; c >= 0; --c) {
+                int base, n, lo;
+                A.span(c, base, n, lo);
+                for (int i = base + tid; i < base + n; i += MG_TAIL_NT)
+                    y[i] = (A.template row<true>(i, [&](unsigned q, unsigned p) {
+                               return c == 0 && !first(A, q) ? A.at(y, q) : A.at(x, q) + om * C.at(C.x(), p);
+                           }) - A.b()[i]) * A.dg()[i];
+                cl.sync();
+            }
+            for (int i = tid; i < A.t.s0 + A.t.s1; i += MG_TAIL_NT) x[i] = y[i];
+            if (l > M.first) cl.sync();
+            continue;
+        }
         {
             // colour 1: the neighbours count with their prolongated correction
             int base, n, lo;
@@ -1872,7 +1942,7 @@ struct SetupTmp {
 void free_level(MGLev& L) {
     cudaFree(L.off); cudaFree(L.cnt); cudaFree(L.pos); cudaFree(L.rp); cudaFree(L.col); cudaFree(L.g);
     cudaFree(L.ecol); cudaFree(L.eg); cudaFree(L.eg8); cudaFree(L.d); cudaFree(L.invdg); cudaFree(L.parent); cudaFree(L.cp); cudaFree(L.ch); cudaFree(L.b);
-    cudaFree(L.x);
+    cudaFree(L.x); cudaFree(L.y);
     const int px = L.px, py = L.py, pz = L.pz;
     const long long P = L.P;
     memset(&L, 0, sizeof(L));
@@ -1950,6 +2020,7 @@ long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
     for (int l = first; l <= last; ++l) {
         const MGLev& L = mg.lev[l];
         MGTailLev& t = M.t[l];
+        t.odd = L.odd;
         const long long M1 = L.M - L.M0;
         if (L.M > (long long)most * M.ctas || (l == last && L.M > most)) return 0;
         t.M = (int)L.M;
@@ -1970,7 +2041,7 @@ long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
         t.pc = take(l < last ? S * 2 * MG_ELL : 0);
         t.g = take(S * sb * MG_ELL);
         t.dg = take(S * sb);
-        t.d = take(sb == 8 ? S * 8 : 0);
+        t.d = take(sb == 8 || t.odd ? S * sb : 0);
         // the most children and the most links of long rows that any block holds
         int32_t *cp = nullptr, *rp = (int32_t*)malloc(sizeof(int32_t) * (L.M + 1));
         if (l > first) cp = (int32_t*)malloc(sizeof(int32_t) * (L.M + 1));
@@ -2012,7 +2083,7 @@ long long tail_layout(const MG& mg, MGTail& M, int first, int sb, int& rc) {
         const long long S = t.s0 + t.s1;
         t.x = take(S * sb);
         t.b = take(S * sb);
-        t.t = take(l < last ? S * sb : 0);
+        t.t = take(l < last || t.odd ? S * sb : 0);
     }
     return o <= 220 * 1024 ? o : 0;
 }
@@ -2031,13 +2102,16 @@ cudaLaunchConfig_t tail_config(int blocks, int smem, cudaLaunchAttribute* at) {
     return cfg;
 }
 
+template <class T>
+auto tail_kernel(bool odd) { return odd ? k_mg_tail<T, true> : k_mg_tail<T, false>; }
+
 // Whether the GPU can hold a cluster of MG_TAIL_BIG blocks (above the portable size).
-bool tail_fits(int sb, int smem) {
+bool tail_fits(int sb, int smem, bool odd) {
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = tail_config(MG_TAIL_BIG, smem, at);
     int n = 0;
-    const cudaError_t e = sb == 8 ? cudaOccupancyMaxActiveClusters(&n, k_mg_tail<double>, &cfg)
-                                  : cudaOccupancyMaxActiveClusters(&n, k_mg_tail<float>, &cfg);
+    const cudaError_t e = sb == 8 ? cudaOccupancyMaxActiveClusters(&n, tail_kernel<double>(odd), &cfg)
+                                  : cudaOccupancyMaxActiveClusters(&n, tail_kernel<float>(odd), &cfg);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess && n > 0;
 }
@@ -2049,10 +2123,12 @@ int tail_plan(MG& mg, int sb) {
     mg.tail_first = last;
     mg.tail_smem = 0;
     if (last < 1) return IBM_OK;
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    IBM_CUDA(cudaFuncSetAttribute(k_mg_tail<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    bool odd = false;
+    for (int l = 1; l <= last; ++l) odd = odd || mg.lev[l].odd;
+    mg.tail_odd = odd;
+    const void* const kernel = sb == 8 ? (const void*)tail_kernel<double>(odd) : (const void*)tail_kernel<float>(odd);
+    IBM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    IBM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     mg.tail = (MGTail*)calloc(1, sizeof(MGTail));
     if (!mg.tail) return ibm_fail(IBM_E_NOMEM, "multigrid set-up: host allocation");
     for (int l = 0; l < IBM_MG_MAXLEV; ++l) mg.tail->lev[l] = mg.lev[l];
@@ -2067,7 +2143,7 @@ int tail_plan(MG& mg, int sb) {
             mg.tail->shift = big ? 12 : 13;
             const long long bytes = tail_layout(mg, *mg.tail, l, sb, rc);
             if (rc) return rc;
-            if (bytes == 0 || (big && l < last && !tail_fits(sb, (int)bytes))) continue;
+            if (bytes == 0 || (big && l < last && !tail_fits(sb, (int)bytes, odd))) continue;
             mg.tail->first = mg.tail_first = l;
             mg.tail_smem = (int)bytes;
         }
@@ -2093,12 +2169,21 @@ int tail_plan(MG& mg, int sb) {
     return IBM_OK;
 }
 
+// Whether a level's periodic axes join positions of one colour.
+int odd_level(const Dom& D, int px, int py, int pz) {
+    const int n[3] = {px, py, pz};
+    for (int a = 0; a < 3; ++a)
+        if (D.bc[2 * a] == IBM_BC_PERIODIC && n[a] > 1 && n[a] % 2 == 1) return 1;
+    return 0;
+}
+
 int build_level1(const LesCtx& c, MGLev& L, int sb, SetupTmp& t) {
     const Dom& D = c.D;
     L.px = (D.nx + 1) / 2;
     L.py = (D.ny + 1) / 2;
     L.pz = (D.nz + 1) / 2;
     L.P = (long long)L.px * L.py * L.pz;
+    L.odd = odd_level(D, L.px, L.py, L.pz);
     MG_ALLOC(L.off, L.P);
     MG_ALLOC(L.cnt, L.P);
     k_parts1<<<lin_blocks(L.P), 256>>>(D, L, t.sub0);
@@ -2112,6 +2197,7 @@ int build_level1(const LesCtx& c, MGLev& L, int sb, SetupTmp& t) {
     MG_ALLOC(L.parent, L.M);
     MG_ALLOCB(L.b, L.M * sb);
     MG_ALLOCB(L.x, L.M * sb);
+    if (L.odd) MG_ALLOCB(L.y, L.M * sb);
     IBM_CUDA(cudaMemset(t.ovf, 0, sizeof(int)));
     k_links1<<<lin_blocks(L.P), 256>>>(D, L, t.sub0, 0, t.ovf);
     IBM_LAUNCHED("k_links1");
@@ -2131,11 +2217,12 @@ int build_level1(const LesCtx& c, MGLev& L, int sb, SetupTmp& t) {
 
 // Level C from level F; returns 1 (and leaves C empty) when the level would not shrink enough or
 // a row would not fit, 0 when built, < 0 on error (negated status).
-int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
+int build_next(const Dom& D, MGLev& F, MGLev& C, int sb, SetupTmp& t) {
     C.px = (F.px + 1) / 2;
     C.py = (F.py + 1) / 2;
     C.pz = (F.pz + 1) / 2;
     C.P = (long long)C.px * C.py * C.pz;
+    C.odd = odd_level(D, C.px, C.py, C.pz);
     MG_ALLOC(C.off, C.P);
     MG_ALLOC(C.cnt, C.P);
     k_uf_init<<<lin_blocks(F.M), 256>>>(F.M, t.lab, t.num);
@@ -2153,7 +2240,7 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
     MG_ALLOC(C.pos, C.M);
     MG_ALLOC(C.rp, C.M + 1);
     MG_ALLOC(C.cp, C.M + 1);
-    const int all = sb == 8;
+    const int all = sb == 8 || F.odd;
     const long long nchild = all ? F.M : F.M0;
     MG_ALLOC(C.ch, nchild);
     MG_ALLOC(C.d, C.M);
@@ -2161,6 +2248,7 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
     MG_ALLOC(C.parent, C.M);
     MG_ALLOCB(C.b, C.M * sb);
     MG_ALLOCB(C.x, C.M * sb);
+    if (C.odd) MG_ALLOCB(C.y, C.M * sb);
     IBM_CUDA(cudaMemset(t.ovf, 0, sizeof(int)));
     k_links_next<<<lin_blocks(C.P), 256>>>(F, C, 0, all, t.ovf);
     IBM_LAUNCHED("k_links_next");
@@ -2186,6 +2274,13 @@ int build_next(MGLev& F, MGLev& C, int sb, SetupTmp& t) {
 
 }  // namespace
 
+// Level l with x as its passes left it (an odd level's separate ones end in y).
+static MGLev solved(const MG& mg, int l) {
+    MGLev L = mg.lev[l];
+    if (L.odd && l < mg.tail_first) L.x = L.y;
+    return L;
+}
+
 // Coarse levels of a V-cycle (level 1 holds the restricted residual and its first half-sweep; on return level 1
 // holds the coarse correction): descent, coarsest solve and ascent, as separate kernels on the large levels
 // and one cluster launch for the small ones (and always for the coarsest).
@@ -2194,24 +2289,34 @@ static int coarse_levels(const LesCtx& c, const MG& mg, SolveScal* sc, cudaStrea
     const T om = (T)mg.omega;
     const int last = mg.nlev - 1, tf = mg.tail_first;
     for (int l = 1; l < tf; ++l) {
-        const MGLev& L = mg.lev[l];
-        k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, sc);
-        k_grestrict<T><<<lin_blocks(4 * mg.lev[l + 1].M), 256, 0, s>>>(L, mg.lev[l + 1], sc);
+        const MGLev &L = mg.lev[l], &C = mg.lev[l + 1];
+        if (L.odd) k_godd<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, C, om, 0, sc);
+        else k_gsmooth<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, 1, sc);
+        const unsigned nb = lin_blocks(4 * C.M);
+        if constexpr (sizeof(T) == 8) k_grestrict<T, true><<<nb, 256, 0, s>>>(L, C, sc);
+        else if (L.odd) k_grestrict<T, true><<<nb, 256, 0, s>>>(L, C, sc);
+        else k_grestrict<T, false><<<nb, 256, 0, s>>>(L, C, sc);
         launches += 2;
     }
     if (mg.tail_smem > 0) {
         cudaLaunchAttribute at[1];
         cudaLaunchConfig_t cfg = tail_config(tf < last ? mg.tail->ctas : 1, mg.tail_smem, at);
         cfg.stream = s;
-        IBM_CUDA(cudaLaunchKernelEx(&cfg, k_mg_tail<T>, *mg.tail, (const SolveScal*)sc));
+        IBM_CUDA(cudaLaunchKernelEx(&cfg, tail_kernel<T>(mg.tail_odd), *mg.tail, (const SolveScal*)sc));
     } else {
         k_gcoarsest<T><<<1, 1024, 0, s>>>(mg.lev[last], mg.coarse_sweeps, sc);
     }
     ++launches;
     for (int l = tf - 1; l >= 1; --l) {
         const MGLev& L = mg.lev[l];
-        k_gup<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, mg.lev[l + 1], om, sc);
-        k_gsmooth<T><<<lin_blocks(L.M0), 256, 0, s>>>(L, 0, sc);
+        const MGLev C = solved(mg, l + 1);
+        if (L.odd) {
+            k_godd<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, C, om, 1, sc);
+            k_godd<T><<<lin_blocks(L.M0), 256, 0, s>>>(L, C, om, 2, sc);
+        } else {
+            k_gup<T><<<lin_blocks(L.M - L.M0), 256, 0, s>>>(L, C, om, sc);
+            k_gsmooth<T><<<lin_blocks(L.M0), 256, 0, s>>>(L, 0, sc);
+        }
         launches += 2;
     }
     return IBM_OK;
@@ -2285,6 +2390,8 @@ int mg_setup(const LesCtx& c, MG& mg, int sb) {
     L0.pz = c.D.nz;
     L0.P = L0.M = c.D.N;
     mg.nlev = 1;
+    mg.odd = odd_level(c.D, c.D.nx, c.D.ny, c.D.nz);
+    if (mg.odd) MG_ALLOCB(mg.z2, c.D.N * sb);
     if (c.D.N <= MG_COARSE_TARGET) return IBM_OK;      // fine smoothing alone
     SetupTmp t;
     t.nt = scan_tiles(c.D.N);
@@ -2297,7 +2404,7 @@ int mg_setup(const LesCtx& c, MG& mg, int sb) {
     for (int l = 1; l + 1 < IBM_MG_MAXLEV; ++l) {
         MGLev& F = mg.lev[l];
         if (F.M <= MG_COARSE_TARGET || F.P == 1) break;
-        const int r2 = build_next(F, mg.lev[l + 1], sb, t);
+        const int r2 = build_next(c.D, F, mg.lev[l + 1], sb, t);
         if (r2 < 0) return -r2;
         if (r2 > 0) break;
         mg.nlev = l + 2;
@@ -2338,13 +2445,18 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
         if (few) f(std::integral_constant<int, 1>{}, flat_grid(c.D.nx, c.D.ny, c.D.nz, 2));
         else f(std::integral_constant<int, IBM_KU>{}, c.cgrid);
     };
+    // an odd grid's passes read a copy of the iterate
+    const T* zin = mg.odd ? (const T*)mg.z2 : z;
+    cudaError_t kept = cudaSuccess;
+    auto keep = [&]() { return mg.odd ? cudaMemcpyAsync(mg.z2, z, sizeof(T) * c.D.N, cudaMemcpyDeviceToDevice, s) : cudaSuccess; };
     auto fine = [&](int col, int zero) {
         auto smooth = [&](auto ku, dim3 grid) {
-            k_mg_smooth0<T, decltype(ku)::value><<<grid, g.block, 0, s>>>(c.D, r, z, scale, col, zero, sc);
+            k_mg_smooth0<T, decltype(ku)::value><<<grid, g.block, 0, s>>>(c.D, r, z, zin, scale, col, zero, sc);
         };
         prof_begin(c.prof, PS_MG_FINE, s);
+        if (!zero && kept == cudaSuccess) kept = keep();
         if constexpr (std::is_same<T, float>::value) {
-            if (vec) launch_mg_smooth0_x4(c, r, z, scale, col, zero, 0, sc, s);
+            if (vec) launch_mg_smooth0_x4(c, r, z, zin, scale, col, zero, 0, sc, s);
             else pairs(smooth);
         } else {
             pairs(smooth);
@@ -2357,7 +2469,7 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
         fine(1, 0);
     }
     if (mg.nlev > 1) {
-        const MGLev& L1 = mg.lev[1];
+        const MGLev &L1 = mg.lev[1], X1 = solved(mg, 1);
         prof_begin(c.prof, PS_MG_TRANSFER, s);
         if constexpr (std::is_same<T, float>::value) {
             if (vec) k_mg_restrict0_x4<<<lin_blocks((c.D.nx / 4) * (long long)L1.py * L1.pz), 256, 0, s>>>(c.D, r, z, scale, L1, sc);
@@ -2373,10 +2485,10 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
         prof_end(c.prof, PS_MG_COARSE, s);
         prof_begin(c.prof, PS_MG_TRANSFER, s);
         if constexpr (std::is_same<T, float>::value) {
-            if (vec) k_mg_prolong0_x4<<<lin_blocks((c.D.nx / 4) * (long long)L1.py * L1.pz), 256, 0, s>>>(c.D, z, L1, om, sc);
-            else k_mg_prolong0<T><<<lin_blocks(L1.P), 256, 0, s>>>(c.D, z, L1, om, sc);
+            if (vec) k_mg_prolong0_x4<<<lin_blocks((c.D.nx / 4) * (long long)L1.py * L1.pz), 256, 0, s>>>(c.D, z, X1, om, sc);
+            else k_mg_prolong0<T><<<lin_blocks(L1.P), 256, 0, s>>>(c.D, z, X1, om, sc);
         } else {
-            k_mg_prolong0<T><<<lin_blocks(L1.P), 256, 0, s>>>(c.D, z, L1, om, sc);
+            k_mg_prolong0<T><<<lin_blocks(L1.P), 256, 0, s>>>(c.D, z, X1, om, sc);
         }
         prof_end(c.prof, PS_MG_TRANSFER, s);
         ++launches;
@@ -2386,11 +2498,13 @@ int mg_vcycle(const LesCtx& c, const MG& mg, const T* r, T* z, SolveScal* sc, cu
         if (q + 1 < S) fine(0, 0);
     }
     auto final = [&](auto ku, dim3 grid) {
-        k_mg_final0<T, decltype(ku)::value><<<grid, g.block, 0, s>>>(c.D, r, z, scale, sc, c.partials, c.counter);
+        k_mg_final0<T, decltype(ku)::value><<<grid, g.block, 0, s>>>(c.D, r, z, zin, scale, sc, c.partials, c.counter);
     };
     prof_begin(c.prof, PS_MG_FINE, s);
+    if (kept == cudaSuccess) kept = keep();
+    if (kept != cudaSuccess) return ibm_cuda_check(kept, "mg_vcycle");
     if constexpr (std::is_same<T, float>::value) {
-        if (vec) launch_mg_smooth0_x4(c, r, z, scale, 0, 0, 1, sc, s);
+        if (vec) launch_mg_smooth0_x4(c, r, z, zin, scale, 0, 0, 1, sc, s);
         else pairs(final);
     } else {
         pairs(final);

@@ -38,6 +38,7 @@ void prof_end(Prof* p, int slot, cudaStream_t s);
 #define IBM_MG_MAXLEV 16
 struct MGLev {
     int px, py, pz;      // positions along x, y, z
+    int odd;             // a periodic axis joins positions of one colour
     long long P;         // positions
     long long M, M0;     // unknowns; the first M0 have colour 0
     long long nnz;       // stored links (each link once from either end)
@@ -53,10 +54,11 @@ struct MGLev {
     float* d;            // [M] Dirichlet (outflow) diagonal term
     float* invdg;        // [M] 1 / (sum of g + d), 0 for an isolated unknown
     int32_t* parent;     // [M] unknown of level l + 1 that contains this one
-    int32_t* cp;         // [M + 1] first child (levels >= 2: unknowns of level l - 1, in FP32 those of colour 0)
+    int32_t* cp;         // [M + 1] first child (levels >= 2: unknowns of level l - 1, in FP32 those of colour 0 unless odd)
     int32_t* ch;         // children, grouped by parent
     void* b;             // right-hand side (working precision)
     void* x;             // iterate
+    void* y;             // odd levels: the iterate after the coarse correction
 };
 struct MGTail;
 struct MG {
@@ -67,6 +69,7 @@ struct MG {
     MGLev lev[IBM_MG_MAXLEV];
     struct MGTail* tail; // small levels in one launch: first level, shared memory per block (0: not used) and layout
     int tail_first, tail_smem;
+    bool tail_odd;       // one of the levels is odd
     void* tail_img;      // the blocks' constant shared memory
     // fused fine-grid passes (FP32, two sweeps, no periodic axis)
     int allow_fused;     // les_params.mg_passes == 0
@@ -74,7 +77,8 @@ struct MG {
     int flx;             // quads along x of a tile (16 or 32)
     int4* fz;            // blocks of a fused launch: tile x, tile y, first plane (even), end
     int fz_items, fz_tx, fz_ty;   // their number, tiles along x and y
-    void* z2;            // [N] working precision: pre-smoothed and prolongated z, read by the post-smoothing
+    int odd;             // a periodic axis of the fine grid joins cells of one colour
+    void* z2;            // [N] working precision; odd grids: the iterate before a half-sweep.  Fused passes: pre-smoothed and prolongated z, read by the post-smoothing
                          // pass (which writes z): no block reads what another block of the pass writes
 };
 
@@ -146,7 +150,7 @@ bool x4_ok(const LesCtx& c);
 int stencil4_setup();      // once per process that solves: shared memory of the kernels above 48 KB
 void launch_cg_dir_spmv_x4(const LesCtx& c, const float* src, const float* pold, float* pnew, float* q, float idx2,
                            SolveScal* sc, int pcg, cudaStream_t s);
-void launch_mg_smooth0_x4(const LesCtx& c, const float* r, float* z, float scale, int col, int zero, int fin,
+void launch_mg_smooth0_x4(const LesCtx& c, const float* r, float* z, const float* zin, float scale, int col, int zero, int fin,
                           SolveScal* sc, cudaStream_t s);
 
 // Builds the levels (allocates them; synchronises the device).  mg.sweeps, omega and coarse_sweeps

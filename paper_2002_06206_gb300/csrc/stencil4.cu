@@ -286,9 +286,9 @@ __device__ __forceinline__ void gs_plain(float (&zc)[4], const float4& r4, const
 }
 
 // One red-black pass of colour `col` (see mg.cu), 4 cells per thread: the cells of the other colour
-// are read and written back unchanged, which no other thread modifies during the pass.  With `fin`
+// are read and written back unchanged, which no other thread modifies during the pass (zin: the iterate before it).  With `fin`
 // this is the last pass of the V-cycle (colour 0) and (r, z) over all cells is reduced as well.
-__global__ void __launch_bounds__(256, 4) k_mg_smooth0_x4(Dom D, const float* __restrict__ r, float* z, float scale,
+__global__ void __launch_bounds__(256, 4) k_mg_smooth0_x4(Dom D, const float* __restrict__ r, float* z, const float* zin, float scale,
                                                        int col, int zero, int fin, SolveScal* sc, double* partials,
                                                        unsigned* counter) {
     if (sc->done) return;
@@ -306,19 +306,19 @@ __global__ void __launch_bounds__(256, 4) k_mg_smooth0_x4(Dom D, const float* __
         if (zero) {
             zc[0] = zc[1] = zc[2] = zc[3] = 0.f;
         } else {
-            const float4 z4 = ld4(z + P);
+            const float4 z4 = ld4(zin + P);
             zc[0] = z4.x; zc[1] = z4.y; zc[2] = z4.z; zc[3] = z4.w;
         }
         if (plain_chunk(D, i0, j, k, fl4)) {
             // the colour's two cells are m = c0 and c0 + 2; c0 is uniform across a warp (same j, k)
-            if (c0 == 0) gs_plain<0>(zc, r4, z, P, D, scale, zero != 0);
-            else gs_plain<1>(zc, r4, z, P, D, scale, zero != 0);
+            if (c0 == 0) gs_plain<0>(zc, r4, zin, P, D, scale, zero != 0);
+            else gs_plain<1>(zc, r4, zin, P, D, scale, zero != 0);
         } else {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int m = c0 + 2 * h;
                 const unsigned fl = (fl4 >> (8 * m)) & 0xffu;
-                const float g = gs_generic(D, r, z, scale, P + m, i0 + m, j, k, fl, zero != 0);
+                const float g = gs_generic(D, r, zin, scale, P + m, i0 + m, j, k, fl, zero != 0);
                 if (m == 0) zc[0] = g;
                 else if (m == 1) zc[1] = g;
                 else if (m == 2) zc[2] = g;
@@ -374,8 +374,8 @@ void launch_cg_dir_spmv_x4(const LesCtx& c, const float* src, const float* pold,
         c.D, src, pold, pnew, q, idx2, sc, c.partials, c.counter, pcg, kz);
 }
 
-void launch_mg_smooth0_x4(const LesCtx& c, const float* r, float* z, float scale, int col, int zero, int fin,
+void launch_mg_smooth0_x4(const LesCtx& c, const float* r, float* z, const float* zin, float scale, int col, int zero, int fin,
                           SolveScal* sc, cudaStream_t s) {
-    k_mg_smooth0_x4<<<x4_grid(c), dim3(X4_TX, X4_TY), 0, s>>>(c.D, r, z, scale, col, zero, fin, sc, c.partials,
+    k_mg_smooth0_x4<<<x4_grid(c), dim3(X4_TX, X4_TY), 0, s>>>(c.D, r, z, zin, scale, col, zero, fin, sc, c.partials,
                                                               c.counter);
 }
