@@ -146,7 +146,9 @@ int ibm_classify_noalloc(const ibm_grid* grid, const float* d_tri, int64_t ntri,
 /* Setup (Sec. 2.4.1 Eq. dummy_cell_region, Sec. 2.4.2 Eq. q_axis and Eq. distribution_function):
  * sets flags bits 6-7 in place and builds two link records per cut face (one per side) with the
  * ghost branch, its coefficients and the forcing weights.  The returned geometry owns its device
- * memory; d_flags must stay alive and unchanged while the geometry is used. */
+ * memory; d_flags must stay alive and unchanged while the geometry is used.  Host synchronisation.
+ * The memory of destroyed geometries (up to 2 GiB per device) stays with the library for the next
+ * ones until an allocation of this library fails or ibm_geom_trim is called. */
 int ibm_setup(const ibm_grid* grid, const ibm_geom_params* gp, uint8_t* d_flags,
               const int64_t* d_face_id, const double* d_t_lo, const double* d_t_hi, int64_t n_cut,
               ibm_geom** out, void* stream);
@@ -163,6 +165,9 @@ int ibm_geom_export(const ibm_geom* geom, int64_t* d_idx, double* d_coef, int64_
  * flux, or its Poisson block has no solution and the solve ends with IBM_E_NOCONV. */
 int ibm_set_boundary_velocity(ibm_geom* geom, const double* d_uib, void* stream);
 void ibm_geom_destroy(ibm_geom* geom);
+/* Give the memory that destroyed geometries left on the current device back to it, for callers that
+ * run short of memory elsewhere.  Synchronises the device. */
+int ibm_geom_trim(void);
 
 /* ---------------------------------------------------------------------------------------------- */
 /* Flow solver.  les_create allocates every workspace once; no later call allocates. `geom` may be  */

@@ -556,6 +556,7 @@ struct ibm_geom {
     ibm_geom_params gp;
     long long N;
     long long n_cut, n_rec, n_inc;
+    int pooled;            // cellrec and rec are from the pool
     uint8_t* flags;        // caller-owned
     int32_t* cellrec;      // [N]
     LinkRec* rec;          // [n_rec]
@@ -753,19 +754,19 @@ __global__ void k_set_uib(LinkRec* __restrict__ rec, long long n, const double* 
 // A moving body is classified again and again; mapping and unmapping the tables (0.8 GB for 201 M cells) took 1.4
 // of the 3.4 ms of a vehicle and 160 of the 420 us of a small sphere.  They come from a pool of the stream-ordered
 // allocator that keeps up to kPoolKeep bytes of freed memory per device; what lies beyond goes back at the next
-// synchronisation, the rest when any allocation of this library fails (ibm_malloc).  A handle may have been used on
-// any stream, so freeing waits for the device, as cudaFree does.
+// synchronisation, the rest when any allocation of this library fails (ibm_malloc) or the caller asks for it
+// (ibm_geom_trim).  A handle may have been used on any stream, so freeing waits for the device, as cudaFree does.
 const unsigned long long kPoolKeep = 2ULL << 30;
 const int kPoolDevices = 64;
 std::mutex g_pool_mutex;
 cudaMemPool_t g_pool[kPoolDevices];
 bool g_pool_tried[kPoolDevices];          // a device without pools takes cudaMalloc and cudaFree throughout
 
-cudaMemPool_t device_pool() {
+cudaMemPool_t device_pool(bool create) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= kPoolDevices) return nullptr;
     std::lock_guard<std::mutex> lock(g_pool_mutex);
-    if (!g_pool_tried[dev]) {
+    if (create && !g_pool_tried[dev]) {
         g_pool_tried[dev] = true;
         cudaMemPoolProps p = {};
         p.allocType = cudaMemAllocationTypePinned;
@@ -782,41 +783,50 @@ cudaMemPool_t device_pool() {
     return g_pool[dev];
 }
 
-cudaError_t geom_alloc(void** p, size_t bytes, cudaStream_t s) {
-    const cudaMemPool_t q = device_pool();
+// What freed tables hold goes back to the device.
+cudaError_t pool_trim() {
+    const cudaMemPool_t q = device_pool(false);
+    if (!q) return cudaSuccess;
+    const cudaError_t e = cudaDeviceSynchronize();
+    return e != cudaSuccess ? e : cudaMemPoolTrimTo(q, 0);
+}
+
+cudaError_t geom_alloc(ibm_geom* G, void** p, size_t bytes, cudaStream_t s) {
+    const cudaMemPool_t q = device_pool(true);
+    G->pooled = q != nullptr;
     if (!q) return cudaMalloc(p, bytes);
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, q, s);
     if (e == cudaErrorMemoryAllocation) {               // memory the pool holds may be in pieces
         cudaGetLastError();
-        cudaDeviceSynchronize();
-        cudaMemPoolTrimTo(q, 0);
+        pool_trim();
         e = cudaMallocFromPoolAsync(p, bytes, q, s);
+        if (e != cudaSuccess) cudaGetLastError();
     }
     return e;
 }
 
-void geom_free(void* a, void* b) {
-    if (!a && !b) return;
+void geom_free(ibm_geom* G) {
     cudaDeviceSynchronize();
-    if (!device_pool()) {
-        cudaFree(a);
-        cudaFree(b);
-        return;
-    }
-    if (a) cudaFreeAsync(a, 0);
-    if (b) cudaFreeAsync(b, 0);
+    for (void* p : {(void*)G->cellrec, (void*)G->rec})
+        if (p && G->pooled) cudaFreeAsync(p, 0);
+        else if (p) cudaFree(p);
 }
 
 }  // namespace
 
 cudaError_t ibm_malloc_bytes(void** p, size_t bytes) {
-    cudaError_t e = cudaMalloc(p, bytes);
+    const cudaError_t e = cudaMalloc(p, bytes);
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();
-    const cudaMemPool_t q = device_pool();
-    cudaDeviceSynchronize();
-    if (!q || cudaMemPoolTrimTo(q, 0) != cudaSuccess) return e;
-    return cudaMalloc(p, bytes);
+    if (pool_trim() != cudaSuccess) return e;
+    const cudaError_t again = cudaMalloc(p, bytes);
+    if (again != cudaSuccess) cudaGetLastError();
+    return again;
+}
+
+extern "C" int ibm_geom_trim(void) {
+    IBM_CUDA(pool_trim());
+    return IBM_OK;
 }
 
 extern "C" void ibm_geom_destroy(ibm_geom* G) {
@@ -824,7 +834,7 @@ extern "C" void ibm_geom_destroy(ibm_geom* G) {
     int dev = -1;
     cudaGetDevice(&dev);
     if (dev != G->device) cudaSetDevice(G->device);
-    geom_free(G->cellrec, G->rec);
+    geom_free(G);
     if (dev != G->device && dev >= 0) cudaSetDevice(dev);
     free(G);
 }
@@ -853,7 +863,7 @@ extern "C" int ibm_setup(const ibm_grid* g, const ibm_geom_params* gp, uint8_t* 
     const bool words = g->nx % 4 == 0 && ((uintptr_t)d_flags & 3u) == 0;
     // one allocation for the cell table with the scan's tile totals behind it, one for the cell list and records
     const size_t cellb = (sizeof(int32_t) * (size_t)G->N + 15) & ~(size_t)15;
-    if ((e = geom_alloc((void**)&G->cellrec, cellb + sizeof(long long) * (nt + 2), s)) != cudaSuccess) goto nomem;
+    if ((e = geom_alloc(G, (void**)&G->cellrec, cellb + sizeof(long long) * (nt + 2), s)) != cudaSuccess) goto nomem;
     tiles = (long long*)((char*)G->cellrec + cellb);
     if (words) k_region_bits<4><<<blocks_for(G->N / 4, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, d_flags);
     else k_region_bits<1><<<blocks_for(G->N, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, d_flags);
@@ -871,7 +881,7 @@ extern "C" int ibm_setup(const ibm_grid* g, const ibm_geom_params* gp, uint8_t* 
         return ibm_fail(IBM_E_INVALID, "ibm_setup: flags name %lld cut links but the list has %lld faces",
                         host & 0xffffffffLL, (long long)n_cut);
     }
-    if ((e = geom_alloc((void**)&G->rec, sizeof(LinkRec) * (size_t)G->n_rec + sizeof(int32_t) * (size_t)(G->n_inc + 4), s)) != cudaSuccess)
+    if ((e = geom_alloc(G, (void**)&G->rec, sizeof(LinkRec) * (size_t)G->n_rec + sizeof(int32_t) * (size_t)(G->n_inc + 4), s)) != cudaSuccess)
         goto nomem;
     G->inc = (int32_t*)(G->rec + G->n_rec);
     if (n_cut > 0) {
