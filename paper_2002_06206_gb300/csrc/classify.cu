@@ -756,43 +756,66 @@ __global__ void k_set_uib(LinkRec* __restrict__ rec, long long n, const double* 
 // allocator that keeps up to kPoolKeep bytes of freed memory per device; what lies beyond goes back at the next
 // synchronisation, the rest when any allocation of this library fails (ibm_malloc) or the caller asks for it
 // (ibm_geom_trim).  A handle may have been used on any stream, so freeing waits for the device, as cudaFree does.
+// A pool lives as long as its context: cudaDeviceReset ends it, so pools are found by the context's id, which no later
+// context repeats.
 const unsigned long long kPoolKeep = 2ULL << 30;
-const int kPoolDevices = 64;
+const int kPools = 64;                    // contexts with a pool; the ones after them take cudaMalloc
+struct ContextPool {
+    unsigned long long ctx;
+    cudaMemPool_t pool;                   // null: the device has none
+};
 std::mutex g_pool_mutex;
-cudaMemPool_t g_pool[kPoolDevices];
-bool g_pool_tried[kPoolDevices];          // a device without pools takes cudaMalloc and cudaFree throughout
+ContextPool g_pool[kPools];
+int g_pools;
 
-cudaMemPool_t device_pool(bool create) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kPoolDevices) return nullptr;
+// Id of the current context (made if the device has none), 0 if it cannot be told.
+unsigned long long context_id() {
+    typedef int (*GetId)(void*, unsigned long long*);         // cuCtxGetId
+    static const GetId get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &r);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && r == cudaDriverEntryPointSuccess ? (GetId)f : (GetId) nullptr;
+    }();
+    unsigned long long id = 0;
+    if (!get) return 0;
+    if (get(nullptr, &id) == 0) return id;
+    return cudaFree(nullptr) == cudaSuccess && get(nullptr, &id) == 0 ? id : 0;
+}
+
+cudaMemPool_t context_pool(bool create) {
+    const unsigned long long ctx = context_id();
+    if (!ctx) return nullptr;
     std::lock_guard<std::mutex> lock(g_pool_mutex);
-    if (create && !g_pool_tried[dev]) {
-        g_pool_tried[dev] = true;
-        cudaMemPoolProps p = {};
-        p.allocType = cudaMemAllocationTypePinned;
-        p.location.type = cudaMemLocationTypeDevice;
-        p.location.id = dev;
-        cudaMemPool_t q = nullptr;
-        unsigned long long keep = kPoolKeep;
-        if (cudaMemPoolCreate(&q, &p) != cudaSuccess || cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        g_pool[dev] = q;
+    for (int k = 0; k < g_pools; ++k)
+        if (g_pool[k].ctx == ctx) return g_pool[k].pool;
+    int dev = 0;
+    if (!create || g_pools == kPools || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    cudaMemPoolProps p = {};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = dev;
+    cudaMemPool_t q = nullptr;
+    unsigned long long keep = kPoolKeep;
+    if (cudaMemPoolCreate(&q, &p) != cudaSuccess || cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        q = nullptr;
     }
-    return g_pool[dev];
+    g_pool[g_pools++] = ContextPool{ctx, q};
+    return q;
 }
 
 // What freed tables hold goes back to the device.
 cudaError_t pool_trim() {
-    const cudaMemPool_t q = device_pool(false);
+    const cudaMemPool_t q = context_pool(false);
     if (!q) return cudaSuccess;
     const cudaError_t e = cudaDeviceSynchronize();
     return e != cudaSuccess ? e : cudaMemPoolTrimTo(q, 0);
 }
 
 cudaError_t geom_alloc(ibm_geom* G, void** p, size_t bytes, cudaStream_t s) {
-    const cudaMemPool_t q = device_pool(true);
+    const cudaMemPool_t q = context_pool(true);
     G->pooled = q != nullptr;
     if (!q) return cudaMalloc(p, bytes);
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, q, s);
