@@ -131,3 +131,23 @@ def test_levels_whose_conductances_are_no_bytes(L, prec):
     assert M[4] == 36 * 32 * 16 and info[0] == 7
     ref = dense_vcycle(r.double().view(256, 512, 576) * 0.25, 7, 1.6).flatten()
     assert float((torch.from_numpy(z).cuda() - ref).norm()) <= (2e-5 if prec else 1e-12) * float(ref.norm())
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("shape,bc", [((37, 33, 29), BOX), ((36, 33, 28), (1, 2, 0, 0, 0, 0)), ((62, 58, 50), BOX), ((44, 44, 20), (0, 0, 0, 0, 3, 3))])
+def test_solves_on_grids_whose_seams_join_a_colour(L, shape, bc, prec):
+    """The V-cycle inside the replayed iteration: a symmetric preconditioner of this strength takes about a digit per two
+    iterations (the oracle's takes at most 12 to 1e-8 on smaller boxes)."""
+    import workloads as W
+    g = L.make_grid(*shape)
+    soup = W.random_soup(40, (0.5, 0.5, 0.5), tuple(n - 0.5 for n in shape), 5.0, seed=8).astype(np.float32)
+    geo = L.Geometry(g, torch.from_numpy(soup).cuda())
+    s = L.Solver(g, 0.01, 0.2, bc, precision=prec, geometry=geo, precond=L.MULTIGRID)
+    x = torch.from_numpy(np.random.default_rng(7).standard_normal(int(np.prod(shape)))).cuda()
+    b, r, p = torch.empty_like(x), torch.empty_like(x), torch.zeros_like(x)
+    s.apply(x, b)
+    st = s.solve(b, p, 1e-8, 400)
+    s.apply(p, r)
+    assert st.status == 0 and float((b - r).norm()) <= 1.001e-8 * float(b.norm())
+    assert st.iters <= 40, st.iters
+    s.close()
