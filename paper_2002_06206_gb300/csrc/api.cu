@@ -213,7 +213,6 @@ extern "C" int les_create(const ibm_grid* g, const les_params* p, const ibm_geom
     c.NF = c.F.off[2] + (long long)c.F.dim[2][0] * c.F.dim[2][1] * c.F.dim[2][2];
     c.cg = cell_grid(g->nx, g->ny, g->nz);
     c.fgrid = flat_grid(g->nx, g->ny, g->nz);
-    c.pgrid = flat_grid(g->nx, g->ny, g->nz, 1);
     c.cgrid = flat_grid(g->nx, g->ny, g->nz, 2 * IBM_KU);
     c.prec = p->precision;
     c.nu = p->nu;

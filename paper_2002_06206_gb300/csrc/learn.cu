@@ -47,12 +47,6 @@ struct ibm_net {
 
 namespace {
 
-__device__ __forceinline__ int tap_off(int t, int& dz, int& dy, int& dx) {
-    dz = t / 9 - 1;
-    dy = (t / 3) % 3 - 1;
-    dx = t % 3 - 1;
-    return 0;
-}
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);

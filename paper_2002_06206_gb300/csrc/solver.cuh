@@ -98,7 +98,6 @@ struct LesCtx {
     FaceLayout F;
     CellGrid cg;
     dim3 fgrid;               // flat launch (IBM_KU planes per thread)
-    dim3 pgrid;               // flat launch, one cell per thread
     dim3 cgrid;               // flat launch over same-colour cell pairs (2 * IBM_KU planes per thread)
     int prec;                 // IBM_FP64 / IBM_FP32_REFINE64
     double nu, dt;

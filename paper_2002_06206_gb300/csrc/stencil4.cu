@@ -27,7 +27,6 @@ namespace {
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ float el(const float4& v, int m) { return m == 0 ? v.x : (m == 1 ? v.y : (m == 2 ? v.z : v.w)); }
 
 // The chunk [i0, i0 + 4) of row (j, k) has no cut link and all its neighbours inside the domain.
 __device__ __forceinline__ bool plain_chunk(const Dom& D, int i0, int j, int k, unsigned fl4) {
