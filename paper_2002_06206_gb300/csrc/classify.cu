@@ -814,9 +814,8 @@ cudaError_t pool_trim() {
     return e != cudaSuccess ? e : cudaMemPoolTrimTo(q, 0);
 }
 
-cudaError_t geom_alloc(ibm_geom* G, void** p, size_t bytes, cudaStream_t s) {
-    const cudaMemPool_t q = context_pool(true);
-    G->pooled = q != nullptr;
+// q: the context's pool, or null.
+cudaError_t geom_alloc(cudaMemPool_t q, void** p, size_t bytes, cudaStream_t s) {
     if (!q) return cudaMalloc(p, bytes);
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, q, s);
     if (e == cudaErrorMemoryAllocation) {               // memory the pool holds may be in pieces
@@ -883,10 +882,12 @@ extern "C" int ibm_setup(const ibm_grid* g, const ibm_geom_params* gp, uint8_t* 
     int herr = 0;
     const long long nt = list_tiles(G->N);
     cudaError_t e;
+    const cudaMemPool_t pool = context_pool(true);
+    G->pooled = pool != nullptr;
     const bool words = g->nx % 4 == 0 && ((uintptr_t)d_flags & 3u) == 0;
     // one allocation for the cell table with the scan's tile totals behind it, one for the cell list and records
     const size_t cellb = (sizeof(int32_t) * (size_t)G->N + 15) & ~(size_t)15;
-    if ((e = geom_alloc(G, (void**)&G->cellrec, cellb + sizeof(long long) * (nt + 2), s)) != cudaSuccess) goto nomem;
+    if ((e = geom_alloc(pool, (void**)&G->cellrec, cellb + sizeof(long long) * (nt + 2), s)) != cudaSuccess) goto nomem;
     tiles = (long long*)((char*)G->cellrec + cellb);
     if (words) k_region_bits<4><<<blocks_for(G->N / 4, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, d_flags);
     else k_region_bits<1><<<blocks_for(G->N, 256), 256, 0, s>>>(g->nx, g->ny, g->nz, d_flags);
@@ -904,7 +905,7 @@ extern "C" int ibm_setup(const ibm_grid* g, const ibm_geom_params* gp, uint8_t* 
         return ibm_fail(IBM_E_INVALID, "ibm_setup: flags name %lld cut links but the list has %lld faces",
                         host & 0xffffffffLL, (long long)n_cut);
     }
-    if ((e = geom_alloc(G, (void**)&G->rec, sizeof(LinkRec) * (size_t)G->n_rec + sizeof(int32_t) * (size_t)(G->n_inc + 4), s)) != cudaSuccess)
+    if ((e = geom_alloc(pool, (void**)&G->rec, sizeof(LinkRec) * (size_t)G->n_rec + sizeof(int32_t) * (size_t)(G->n_inc + 4), s)) != cudaSuccess)
         goto nomem;
     G->inc = (int32_t*)(G->rec + G->n_rec);
     if (n_cut > 0) {

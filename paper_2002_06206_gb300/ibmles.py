@@ -180,15 +180,6 @@ def trim():
     _check(lib().ibm_geom_trim())
 
 
-def _empty(*shape, **kw):
-    """torch.empty, once more after trim() where the device is full."""
-    try:
-        return torch.empty(*shape, **kw)
-    except torch.cuda.OutOfMemoryError:
-        trim()
-        return torch.empty(*shape, **kw)
-
-
 def num_faces(nx, ny, nz):
     return (nx + 1) * ny * nz + nx * (ny + 1) * nz + nx * ny * (nz + 1)
 
@@ -233,6 +224,13 @@ class Geometry:
     """Classified triangle soup + link records (ibm_classify + ibm_setup) on the current device."""
 
     def __init__(self, grid, tri, eps_edge=1e-9, eps_det=0.0, deadend_on=0, stream=None, cap=None):
+        try:
+            self._classify(grid, tri, eps_edge, eps_det, deadend_on, stream, cap)
+        except torch.cuda.OutOfMemoryError:      # once more without what destroyed geometries left
+            trim()
+            self._classify(grid, tri, eps_edge, eps_det, deadend_on, stream, cap)
+
+    def _classify(self, grid, tri, eps_edge, eps_det, deadend_on, stream, cap):
         self.grid = grid
         self.N = grid.nx * grid.ny * grid.nz
         self.gp = GeomParams(eps_edge, eps_det, deadend_on, 0)
@@ -240,15 +238,15 @@ class Geometry:
         tri = tri.to(dev, torch.float32).contiguous().view(-1, 3, 3) if isinstance(tri, torch.Tensor) \
             else torch.as_tensor(tri, dtype=torch.float32).to(dev).contiguous().view(-1, 3, 3)
         self.tri = tri
-        self.flags = _empty(self.N, dtype=torch.uint8, device=dev)
+        self.flags = torch.empty(self.N, dtype=torch.uint8, device=dev)
         ws = lib().ibm_classify_workspace_bytes(C.byref(grid), tri.shape[0])
-        self.workspace = _empty(max(int(ws), 1), dtype=torch.uint8, device=dev)
+        self.workspace = torch.empty(max(int(ws), 1), dtype=torch.uint8, device=dev)
         cap = cap if cap is not None else max(1024, 2 * int(tri.shape[0]) + 1024)
         s = _stream(stream)
         while True:
-            self.face_id = _empty(cap, dtype=torch.int64, device=dev)
-            self.t_lo = _empty(cap, dtype=torch.float64, device=dev)
-            self.t_hi = _empty(cap, dtype=torch.float64, device=dev)
+            self.face_id = torch.empty(cap, dtype=torch.int64, device=dev)
+            self.t_lo = torch.empty(cap, dtype=torch.float64, device=dev)
+            self.t_hi = torch.empty(cap, dtype=torch.float64, device=dev)
             n_cut = C.c_int64(0)
             n_tests = C.c_int64(0)
             rc = lib().ibm_classify(C.byref(grid), _ptr(tri), tri.shape[0], C.byref(self.gp), _ptr(self.flags),
