@@ -159,8 +159,7 @@ __device__ __forceinline__ void use_hit(const TestArgs& A, long long fid, unsign
 // take the FP64 predicate together: the pass is bound by its FP64 instructions (about 80 with the
 // conversions and the division).  An item of more than kBigItem tests goes to the whole block; gridDim.y
 // slices share such items when the soup has few triangles.
-// Vehicle assembly (2.03 M triangles, 6.0 M tests): 1.01 ms, 2.4 ms without the FP32 test and the queue; one
-// thread per test with offsets in memory took 1.07 ms after 1.3 ms of counting and 1.4 ms of table clearing.
+// Vehicle assembly (2.03 M triangles, 6.0 M tests): 1.01 ms, 2.4 ms without the FP32 test and the queue.
 constexpr int kBigItem = 1024;
 
 template <int PASS>

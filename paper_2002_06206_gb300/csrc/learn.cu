@@ -72,8 +72,8 @@ __device__ __forceinline__ void mma_bf16(float d[4], const uint32_t a[4], const 
 // 16 cells (w % 2) * 16 .. + 15 of row w / 2: for each k-step (two taps x 8 channels) one
 // ldmatrix.x4 gathers the A fragment straight from the ring -- each lane names one 16-byte row, the
 // input cell of its (cell, tap), a plane's base and a constant -- and one mma.sync accumulates it.
-// 128^3 cells: 38 us per layer (input gradients 50, with the mask), 74 with three planes, loads waited for and ring slots by
-// remainders per tap.
+// Bound by the gathers, 27 shared-memory reads of every row per layer: 128^3 cells 38 us (input gradients 50, with the
+// mask); 74 us with three planes, loads waited for and ring slots by remainders per tap.
 #define NC_TX 32
 #define NC_TY 4
 #define NC_SX (NC_TX + 2)

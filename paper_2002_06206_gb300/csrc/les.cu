@@ -67,9 +67,8 @@ __device__ __forceinline__ void to_off(T* base, Off<T> off, T v) {
 // neighbours come by shuffle, the rows above and below from L1.  Cells on a domain face take the boundary's ghosts
 // in place; only cells with a cut link go through vel_across.  With g = the undivided central differences,
 // 4 dx^2 S:S = A + B / 2 and 4 dx^2 W:W = C / 2 for A = sum g_aa^2, B = sum (g_ab + g_ba)^2, C = sum (g_ab - g_ba)^2.
-// 512 x 256 x 256 in FP32: 266 us, of 270 instructions per cell (addresses mostly; 16 bytes per cell would take 80);
-// 338 us with one thread per cell and 18 loads.  251 x 127 x 93, two planes per thread: 39 -> 35 us (55 with eight, 44
-// with one).  FP64 128 x 64 x 64: 110 -> 59 us, one square root in place of two and half of the products.
+// Bound by issue (87 %): 270 instructions per cell, addresses mostly; 266 us at 512 x 256 x 256 in FP32 (its 16 bytes per
+// cell would take 80), 338 us with one thread per cell and 18 loads.
 template <class T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_csm(Dom D, const T* __restrict__ u, T* __restrict__ nut, int kz) {
     const int i0 = blockIdx.x * IBM_TX + threadIdx.x, j0 = blockIdx.y * IBM_TY + threadIdx.y;
@@ -191,8 +190,9 @@ __device__ __forceinline__ bool fast_cell(const Dom& D, long long P, int i, int 
     return (m & 63u) == 0u;
 }
 
-// Fast cells run in z-marching tiles: a block of 32 x 8 threads owns an (x, y) tile and walks D.tile_z planes.  u (three components) and nu_t of the planes k-1 .. k+2 over the tile plus a two-cell halo sit in a
-// ring in shared memory; a thread holds its own column in registers.  Halo positions across a periodic
+// Fast cells run in z-marching tiles: a block of 32 x 8 threads owns an (x, y) tile and walks D.tile_z planes.  u
+// (three components) and nu_t of the planes k-1 .. k+2 over the tile plus a two-cell halo sit in a ring in shared
+// memory; a thread holds its own column in registers.  Halo positions across a periodic
 // seam hold the wrapped cell; one cell beyond a non-periodic domain face they hold the boundary ghost of
 // vel_across (a function of the cell across that face alone), so cells on the domain faces are fast too.
 // A domain face takes the near cell's nu_t and cross derivative and the central advected value: weights
@@ -205,14 +205,12 @@ __device__ __forceinline__ bool fast_cell(const Dom& D, long long P, int i, int 
 // the z face stays in registers for the next plane.  A plane's sums run one step later, so a single
 // barrier per plane orders both the face buffers (two of them, by plane parity) and the ring.
 //
-// Bound by instruction issue.  Per face and component: the advected value is c_L u_L + c_R u_R - kq u_far with
-// coefficients chosen once per face by the sign of its velocity, the scale factors of the differences are taken out of the components, addresses are a
-// block-uniform plane plus a fixed thread offset.  512x256x256 FP32, Crank-Nicolson operator: 660 us (530
-// thread instructions per cell, 2.6 per cycle and SM; its 41 bytes per cell would take 205 us), 1540 us with
-// per-component face forms, 64-bit face indexes and velocities loaded where they are used.  Two rows per
-// thread (455 instructions, 16 resident warps) and four blocks per SM (64 registers) measured 660 and 694 us.
-// FP64: 183 us at 128x64x64 (212 with 20 operations per cell more: per-component upwind sums, weighted cross
-// derivatives), three quarters of the FP64 rate.
+// Bound by instruction issue (65 %) and the latency of its barriers.  Per face and component the advected value is
+// c_L u_L + c_R u_R - kq u_far with coefficients chosen once per face by the sign of its velocity, the scale factors of
+// the differences are taken out of the components, and addresses are a block-uniform plane plus a fixed thread offset.
+// 512x256x256 FP32, Crank-Nicolson operator: 660 us (490 thread instructions per cell; its 41 bytes per cell would take
+// 205 us), 1540 us with per-component face forms, 64-bit face indexes and velocities loaded where they are used.  FP64:
+// 183 us at 128x64x64, three quarters of the FP64 rate.
 #define FT_X 32
 #define FT_Y 8
 #define FT_H 2
@@ -663,9 +661,9 @@ __device__ __forceinline__ void cell_coords(const Dom& D, long long P, int& i, i
 
 // Cells that are not fast_cell, from their list.  A warp takes one axis of 32 cells, so that what depends on the axis
 // is uniform in it, and three warps make up the cells: they leave their shares of the three components in shared
-// memory and each finishes one component.  1024 x 512 x 384 around a vehicle, Crank-Nicolson operator: 3.9 -> 1.8 ms
-// against one thread per cell with all six faces unrolled, which waited for instructions (a thousand per face) and
-// spilled; 128 x 64 x 64 in FP64: 35 -> 14 us.  Four and seven blocks per SM: 16 % and 1 % slower.
+// memory and each finishes one component.  Bound by the latency of the scattered reads.  1024 x 512 x 384 around a
+// vehicle, Crank-Nicolson operator: 1.8 ms; 3.9 ms with one thread per cell and all six faces unrolled, which waited for
+// instructions (a thousand per face) and spilled.
 #define FG_CELLS 64
 #define FG_NT (3 * FG_CELLS)
 

@@ -96,8 +96,8 @@ __device__ __forceinline__ T gs_value(const Dom& D, const T* __restrict__ r, con
 // One red-black Gauss-Seidel pass of colour `col` on level 0 for  A^ z = scale * r.  Each thread takes KU pairs of
 // planes of one (i, j) column and updates the cell of colour `col` in each pair.  With `zero` the iterate is taken
 // as 0 (first pass of a V-cycle) and the other cell of each pair is cleared.  zin: the iterate before the pass (z itself
-// unless the grid is odd).  64 x 32 x 32 in FP64, KU = 1: 2.7 us, with four
-// pairs and an FP64 division at every domain face 9.5 us.
+// unless the grid is odd).  Small grids are bound by latency: 64 x 32 x 32 in FP64 takes 2.7 us with one pair per
+// thread, 9.5 us with four and an FP64 division at every domain face.
 template <class T, int KU>
 __global__ void __launch_bounds__(256) k_mg_smooth0(Dom D, const T* __restrict__ r, T* z, const T* zin, T scale,
                                                     int col, int zero, const SolveScal* sc) {
@@ -239,10 +239,9 @@ __device__ __forceinline__ void put_b1(const MGLev& C, int u, T b) {
 // = 1 / (open links + outflow terms), fixed per column: neighbours outside the domain hold z = 0.  A warp
 // with a cut link in its plane takes the general form for that plane.
 //
-// The kernels are bound by instruction issue with shared memory close behind: about 300 instructions per
-// thread and plane for 8 cells.  512x256x256: 137 us (pre) and 149 us (post), 2.2 and 2.9 TB/s of the 9.1 and
-// 13 bytes per cell; z of the post pass through a cp.async ring two planes ahead took 180 us.  A ring of planes in shared memory filled by TMA with one barrier per half-sweep, the
-// form before, took 640 and 480 us: it issued 11 and 8.5 warp instructions per cell.
+// Neither issue (65 and 54 % of the active cycles) nor HBM (35 and 39 %) is full: what is left is the latency of one
+// barrier per plane with 16 warps on an SM.  512x256x256 under ncu: 132 us (pre) and 149 us (post) for 9.1 and 13 bytes
+// per cell; 744 and 585 us with planes in a TMA ring and one barrier per half-sweep.
 #define FTP_NT 512
 #define FTP_RING 5
 
@@ -1540,9 +1539,8 @@ __global__ void __launch_bounds__(MG_TAIL_NT, 1) k_mg_tail(const __grid_constant
 // ---- transfer between the fine grid and level 1 -------------------------------------------------
 
 // b_1 of each part of a level-1 block = the sum of the fine residuals  scale r - (A z)  of its cells, and the
-// first half-sweep of level 1, x_1 = -b_1 / dg.  Eight lanes per block, one per cell: 64 x 32 x 32 in FP64
-// 4.8 us, 21.5 us
-// with one lane.
+// first half-sweep of level 1, x_1 = -b_1 / dg.  Eight lanes per block, one per cell, for the latency of small grids:
+// 64 x 32 x 32 in FP64 4.8 us, 21.5 us with one lane.
 template <class T>
 __global__ void __launch_bounds__(256) k_mg_restrict0(Dom D, const T* __restrict__ r, const T* __restrict__ z, T scale,
                                                       MGLev C, const SolveScal* sc) {
@@ -1702,8 +1700,8 @@ __global__ void __launch_bounds__(256) k_mg_restrict0_x4(Dom D, const float* __r
 
 // FP32 prolongation with nx a multiple of 4: a thread takes two positions of level 1 along x, two rows of two planes.
 // Flags, offsets and the iterate are loaded together, so that the coarse values are the only loads that wait for
-// others, and a warp without a cut link skips the search for parts.  Bound by HBM:
-// 8 bytes per cell and the coarse values; at 512 x 256 x 256, where the iterate is partly in L2, 92 -> 46 us.
+// others, and a warp without a cut link skips the search for parts.  Bound by HBM (71 %): 8 bytes per cell and the
+// coarse values, 49 us at 512 x 256 x 256; 92 us with loads that wait for one another.
 __global__ void __launch_bounds__(256, 4) k_mg_prolong0_x4(Dom D, float* __restrict__ z, MGLev C, float omega,
                                                         const SolveScal* sc) {
     if (sc->done) return;
@@ -1800,12 +1798,11 @@ __global__ void __launch_bounds__(256) k_tile_marks(Dom D, int w, int h, unsigne
 
 // The launch of the fused passes: of the two tile widths (64 x 64 or 128 x 32 cells, halo included; 64 x 64 has the
 // smaller halo, 128 x 32 fits some grids better), each tile cut into chunks of whole pairs of planes.  A chunk costs
-// its planes and eight more, planes with cut links FZ_GENERAL as much as others (measured: 2.57 and 1.57 us), and
+// its planes and eight more, planes with cut links FZ_GENERAL as much as others (measured 2.57 and 1.57 us), and
 // blocks run one per SM; for eight numbers of rounds the limit on a chunk's cost is bisected that lets the
-// chunks fit the rounds, and the cheapest is kept.  With chunks of equal height the tiles around a body came last: the
-// two passes take 43 and 34 us in place of 52 and 42 on 256 x 128 x 128 cells around a dirty sphere, 836 and 624 in place
-// of 896 and 681 on 1024 x 512 x 384 around a vehicle (1.3 for FZ_GENERAL: 928 and 679; 2.5: 917 and 663).  With the
-// first pass's loads ahead (600 us there) 1.4, 1.9 and 2.3 are again slower.
+// chunks fit the rounds, and the cheapest is kept.  With chunks of equal height the tiles around a body came last: 52
+// and 42 us in place of 43 and 34 on 256 x 128 x 128 cells around a dirty sphere.  1.3 to 1.4 and 1.9 to 2.5 for
+// FZ_GENERAL are slower there and around the vehicle.
 #define FZ_GENERAL 1.65f
 
 struct FzPlan {

@@ -55,9 +55,9 @@ __global__ void __launch_bounds__(256) k_apply(Dom D, const T* __restrict__ p, T
 }
 
 // r = b - A x in FP64; stores r in the working precision; res2 = rr = ||(Tr) r||^2.
-// Bound by the FP64 units: five additions, two fused multiply-adds and the rounding to FP32 per cell, at cells with
-// a cut link or a domain face too (count of links from a table).  512 x 256 x 256 to FP32: 740 -> 565 us (the eight
-// operations take 500), 256 x 128 x 128 around a dirty sphere 115 -> 73 us.
+// Bound by the FP64 units (85 % busy): five additions, two fused multiply-adds and the rounding to FP32 per cell, at
+// cells with a cut link or a domain face too (count of links from a table).  512 x 256 x 256 to FP32: 565 us, of which
+// the eight operations take 500; 740 us with twelve.
 template <class Tr, int KU>
 __global__ void __launch_bounds__(256) k_residual(Dom D, const double* __restrict__ b, const double* __restrict__ x64,
                                                   Tr* __restrict__ r, double idx2, SolveScal* sc, double* partials,
@@ -126,9 +126,8 @@ __global__ void k_reset(SolveScal* sc) {
 
 // CG, first half: direction p = r + beta p_old (recomputed where a neighbour needs it, so p never
 // needs a pass of its own), q = A p, and (p, q).  Flat launch: each thread takes KU planes of one
-// (i, j) column, unrolled, so its loads are all independent; one plane where four would leave SMs idle.
-// 64 x 32 x 32 in FP64: 15.8 -> 8.4 us
-// (with the links found without a branch); at 131 x 61 x 47 in FP32 one plane takes 12.2 us, four 11.2.
+// (i, j) column, unrolled, so its loads are all independent; one plane where four would leave SMs idle (64 x 32 x 32
+// in FP64: 8.4 against 15.8 us), four elsewhere (131 x 61 x 47 in FP32: 11.2 against 12.2 us).
 template <class T, int KU>
 __global__ void __launch_bounds__(256) k_cg_dir_spmv(Dom D, const T* __restrict__ r, const T* __restrict__ pold,
                                                      T* __restrict__ pnew, T* __restrict__ q, T idx2, SolveScal* sc,

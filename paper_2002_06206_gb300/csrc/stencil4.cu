@@ -46,9 +46,9 @@ __device__ __forceinline__ unsigned flags4(const Dom& D, long long P) {
 // outermost warps form the row beyond it as well), the x neighbours outside a quad come by shuffle (the
 // warp's end lanes copy one value each).  The first iteration of a solve does not read p_old.  Cells with a cut link
 // take the same neighbour values with their closed links left out; domain faces change the neighbour's place
-// (periodic) or the count of links.  Bound by HBM (17 bytes per cell): at 512 x 256 x 256 118 us, 84 us at the copy
-// rate; 232 us with p formed at every neighbour, 170 us marching with plain loads.  Three blocks per SM with rings of
-// three planes take the same there and 8 % more at 256 x 128 x 128.
+// (periodic) or the count of links.  Bound by the chain of a wait, a barrier and the arithmetic per plane with 16 warps
+// on an SM (DRAM 57 %): 118 us at 512 x 256 x 256, 1.4 times what its 17 bytes per cell take at the copy rate; 232 us with
+// p formed at every neighbour.  Three blocks per SM with rings of three planes are 8 % slower at 256 x 128 x 128.
 #define SP_TY 8                  // row pairs per block
 #define SP_ROWS (2 * SP_TY)
 #define SP_MINB 2                // resident blocks per SM
